@@ -167,13 +167,14 @@ __device__ __forceinline__ void load8(const float* p, float* x) {
     float4 a = __ldg(q), b = __ldg(q + 1);
     x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
 }
-// eight floats with one 256-bit read-only global load (sm_100 and later).  p must be 32-byte aligned (callers
-// check it, or pass the context's own buffers) and no thread may write the data during the kernel before
-// this read.
-__device__ __forceinline__ void load8_v8(const float* p, float* x) {
-    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]), "=f"(x[4]), "=f"(x[5]), "=f"(x[6]), "=f"(x[7])
-        : "l"(p));
+// a * b + c on a pair of float32 values in one instruction (each rounded as fmaf rounds)
+__device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;"
+        : "=l"(r)
+        : "l"(*reinterpret_cast<unsigned long long*>(&a)), "l"(*reinterpret_cast<unsigned long long*>(&b)),
+          "l"(*reinterpret_cast<unsigned long long*>(&c)));
+    return *reinterpret_cast<float2*>(&r);
 }
 __device__ __forceinline__ void store8(double* p, const double* x) {
     double2* q = reinterpret_cast<double2*>(p);
@@ -184,6 +185,40 @@ __device__ __forceinline__ void store8(float* p, const float* x) {
     float4* q = reinterpret_cast<float4*>(p);
     q[0] = make_float4(x[0], x[1], x[2], x[3]);
     q[1] = make_float4(x[4], x[5], x[6], x[7]);
+}
+
+// ------------------------------------------------------------------------------------------------
+// Krylov vectors (the basis r_k and q) are chunk-planar: [8][V][4], plane c = 2 mu + h holding the colours 4 h .. 4 h + 3
+// of component mu.  Consecutive sites are adjacent in a plane, so a warp of 32 consecutive sites reads a component of
+// any of their neighbours as two contiguous 512-byte segments, and its links without duplicates; with the sites' 128-byte
+// rows of the [V][4][8] layout either the links are read four times (four lanes per site) or every load touches 32
+// lines (one).
+// ------------------------------------------------------------------------------------------------
+template <typename T> __device__ __forceinline__ const T* plane_at(const T* X, int V, int s, int c) {
+    return X + ((size_t)c * V + s) * 4;
+}
+template <typename T> __device__ __forceinline__ T* plane_at(T* X, int V, int s, int c) {
+    return X + ((size_t)c * V + s) * 4;
+}
+__device__ __forceinline__ void load4(const float* p, float* x) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+    x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+}
+__device__ __forceinline__ void load4(const double* p, double* x) {
+    const double2 a = __ldg(reinterpret_cast<const double2*>(p)), b = __ldg(reinterpret_cast<const double2*>(p) + 1);
+    x[0] = a.x; x[1] = a.y; x[2] = b.x; x[3] = b.y;
+}
+__device__ __forceinline__ void store4(float* p, const float* x) {
+    *reinterpret_cast<float4*>(p) = make_float4(x[0], x[1], x[2], x[3]);
+}
+__device__ __forceinline__ void store4(double* p, const double* x) {
+    reinterpret_cast<double2*>(p)[0] = make_double2(x[0], x[1]);
+    reinterpret_cast<double2*>(p)[1] = make_double2(x[2], x[3]);
+}
+// the eight colours of component mu at site s
+template <typename T> __device__ __forceinline__ void load_plane8(const T* X, int V, int s, int mu, T* x) {
+    load4(plane_at(X, V, s, 2 * mu), x);
+    load4(plane_at(X, V, s, 2 * mu + 1), x + 4);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -319,10 +354,9 @@ struct rmhmc_ctx {
     std::string graph_note;
     // autotuned stencil shapes per (precision bytes * 100 + link format): components per lane, block size
     std::map<int, std::pair<int, int>> tune;
-    // kernel of the kinetic-force contraction (rmhmc_set_stencil_shape, RMHMC_SHAPE_KFORCE): 0 four lanes per link,
-    // own basis rows from global memory (the fastest at 32^4: 9.9 ms per kinetic evaluation against 11.2 and
-    // 11.5 ms); 1 the same with the rows staged in shared memory; 2 eight lanes per link
-    int lg_mode = 0;
+    // kernel of the kinetic-force contraction (rmhmc_set_stencil_shape, RMHMC_SHAPE_KFORCE): 4 the fused one (the default),
+    // 0 four lanes per link
+    int lg_mode = 4;
     // float64 link update in float-float arithmetic (rmhmc_set_stencil_shape, RMHMC_SHAPE_LINKUPDATE)
     bool link_update_ff = true;
     // z-extent of the multi-field adjoint kernel's slabs (rmhmc_set_stencil_shape, RMHMC_SHAPE_ADJOINT); 0 chosen

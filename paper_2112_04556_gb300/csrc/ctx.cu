@@ -5,6 +5,7 @@
 #include <string.h>
 
 #include "common.cuh"
+#include "ops.cuh"
 
 namespace rm {
 
@@ -236,10 +237,10 @@ extern "C" int rmhmc_set_stencil_shape(rmhmc_ctx* ctx, int kernel, int prec, int
         return RMHMC_OK;
     }
     if (kernel == RMHMC_SHAPE_KFORCE) {
-        if (prec != RMHMC_FP32 || linkfmt != 18 || nmu < 0 || nmu > 3 || block != (nmu == 2 ? 256 : 128))
+        if (prec != RMHMC_FP32 || linkfmt != 18 || nmu < 0 || nmu > 4 || block != (nmu == 2 || nmu == 4 ? 256 : 128))
             return set_err(ctx, RMHMC_EINVAL,
-                           "kinetic-force contraction: RMHMC_FP32, 18, nmu 0/1/3 with block 128 or 2 with 256");
-        ctx->lg_mode = nmu;
+                           "kinetic-force contraction: RMHMC_FP32, 18, nmu 0/1/3 with block 128 or 2/4 with 256");
+        ctx->lg_mode = nmu == kLgFused ? kLgFused : 0;   // 1, 2 and 3 name former variants of 0
         return RMHMC_OK;
     }
     if (kernel == RMHMC_SHAPE_ADJOINT) {

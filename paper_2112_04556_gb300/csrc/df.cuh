@@ -26,6 +26,19 @@ __device__ __forceinline__ dfl quick_two_sum(float a, float b) {
     const float s = __fadd_rn(a, b);
     return df_make(s, __fsub_rn(b, __fsub_rn(s, a)));
 }
+// float64-accurate running sum of squares in float32 arithmetic: the rounding errors of the products (fma) and of the
+// sum (TwoSum) are collected in c
+struct SumSq32 {
+    float s = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float x) {
+        const float p = __fmul_rn(x, x), e = __fmaf_rn(x, x, -p);
+        const dfl t = two_sum(s, p);
+        s = t.hi;
+        c = __fadd_rn(c, __fadd_rn(t.lo, e));
+    }
+    __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+};
+
 // Conversions between float64 and float pairs from the IEEE-754 bit fields, with integer operations and no
 // float64 arithmetic (float64 runs at a small fraction of the float32 rate on this part).  df_split: hi = x
 // rounded to 24 significant bits (its 29 low significand bits dropped, rounding half away from zero, a carry
@@ -50,6 +63,19 @@ __device__ __forceinline__ dfl df_split(double x) {
         if (sign) lo = -lo;
     }
     return df_make(hi, lo);
+}
+// the nearest float of a value, without a float64 conversion (|x| below 2^-126 gives 0)
+__device__ __forceinline__ float to_f32(float x) { return x; }
+__device__ __forceinline__ float to_f32(double x) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
+    const int e = (int)((b >> 52) & 0x7ff);
+    if (e < 1023 - 126) return __uint_as_float(sign);
+    if (e > 1023 + 127) return __uint_as_float(sign | (e == 0x7ff && (b << 12) ? 0x7fc00000u : 0x7f800000u));
+    // round half to even at bit 29; a carry moves into the exponent (up to infinity)
+    const unsigned long long m = b & 0x7fffffffffffffffull;
+    const unsigned long long r = m + 0x0fffffffull + ((m >> 29) & 1ull);
+    return __uint_as_float(sign | (unsigned)((r >> 29) - (unsigned long long)((1023 - 127) << 23)));
 }
 // a float as a double, from its bit fields (normal numbers, zero, inf and NaN; subnormals give 0)
 __device__ __forceinline__ double f_to_d_bits(float f) {

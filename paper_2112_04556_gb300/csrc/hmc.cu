@@ -1117,8 +1117,9 @@ static int md_graph_run(rmhmc_ctx* ctx, double* U, double* P, const rmhmc_params
     memcpy(st, ctx->h_pinned, sizeof st);
     memcpy(ints, (char*)ctx->h_pinned + 128, sizeof ints);
     *used = true;
-    // kernels the graph ran: 3 + 6 per step outside the loops, 8 per fixed-point iteration, 2 per Krylov iteration
-    ctx->launches += 3 + 6LL * p->nsteps + 8 * (st[1] + st[2]) + 2 * st[0];
+    // kernels the graph ran: 3 + 6 per step outside the loops, 7 per fixed-point iteration (8 with the velocity in a
+    // kernel of its own), 2 per Krylov iteration
+    ctx->launches += 3 + 6LL * p->nsteps + (ctx->lg_mode == kLgFused ? 7 : 8) * (st[1] + st[2]) + 2 * st[0];
     ctx->krylov_iters += st[0];
     ctx->links_valid = true;
     if (r) {

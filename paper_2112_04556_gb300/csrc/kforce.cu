@@ -11,6 +11,8 @@
 // where coef_a(M) = Tr(lambda^a (-i)(M - M^dag)/2) (antiherm_coef).
 #include <algorithm>
 
+#include "df.cuh"
+#include "fcontract.cuh"
 #include "krylov.cuh"
 #include "ops.cuh"
 #include "stencil.cuh"
@@ -107,22 +109,6 @@ int link_grad_launch(rmhmc_ctx* ctx, int prec, const void* X, const void* Z, int
 // 8 n^2 + 256 n + 1400 FMA per link against 576 npole per link for the direct form.
 // ------------------------------------------------------------------------------------------------
 
-// G_a += sum_c f_acd rc_c for one column d (d a compile-time constant after unrolling)
-template <typename T>
-__device__ __forceinline__ void f_contract(int d, const T (&rc)[8], T (&G)[8]) {
-    constexpr int tr[9][3] = {{0, 1, 2}, {0, 3, 6}, {0, 4, 5}, {1, 3, 5}, {1, 4, 6},
-                              {2, 3, 4}, {2, 5, 6}, {3, 4, 7}, {5, 6, 7}};
-    constexpr double fv[9] = {1.0, 0.5, -0.5, 0.5, 0.5, 0.5, -0.5, 0.86602540378443864676, 0.86602540378443864676};
-#pragma unroll
-    for (int t = 0; t < 9; t++) {
-        const int i = tr[t][0], j = tr[t][1], k = tr[t][2];
-        const T v = (T)fv[t];
-        if (d == k) { G[i] = fma(v, rc[j], G[i]); G[j] = fma(-v, rc[i], G[j]); }
-        else if (d == j) { G[k] = fma(v, rc[i], G[k]); G[i] = fma(-v, rc[k], G[i]); }
-        else if (d == i) { G[j] = fma(v, rc[k], G[j]); G[k] = fma(-v, rc[j], G[k]); }
-    }
-}
-
 // eight values from shared memory (plain loads: the read-only global path does not apply to shared memory)
 __device__ __forceinline__ void lds8(const float* p, float* x) {
     const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
@@ -199,7 +185,7 @@ __global__ void __launch_bounds__(kLgSites * 4, 4) k_link_grad_krylov(Geom g, ty
             if (live) {
                 for (int l = 0; l < n; l++) {
                     T r[8];
-                    load8_v8(R + (size_t)l * fs + (size_t)y * 32 + q * 8, r);
+                    load_plane8(R + (size_t)l * fs, g.V, y, q, r);
 #pragma unroll
                     for (int kk = 0; kk < kLgKC; kk++) {
                         const T s = Ss[kk * kBasisCap + l];
@@ -214,11 +200,11 @@ __global__ void __launch_bounds__(kLgSites * 4, 4) k_link_grad_krylov(Geom g, ty
             if (live) {
                 const int kc = min(kLgKC, n - k0);
                 for (int kk = 0; kk < kc; kk++) {
-                    const T* rk = R + (size_t)(k0 + kk) * fs + (size_t)yn * 32;
+                    const T* rk = R + (size_t)(k0 + kk) * fs;
 #pragma unroll
                     for (int mu = 0; mu < 4; mu++) {
                         T rp[8], wv[8];
-                        load8_v8(rk + mu * 8, rp);
+                        load_plane8(rk, g.V, yn, mu, rp);
                         lds8(wrow + kk * 32 + mu * 8, wv);
 #pragma unroll
                         for (int b = 0; b < 8; b++)
@@ -250,106 +236,157 @@ __global__ void __launch_bounds__(kLgSites * 4, 4) k_link_grad_krylov(Geom g, ty
     }
 }
 
-// The same contraction with the block's own basis rows staged once in shared memory (for n <= kLgStage):
-// the kernel above reads r_l(y) for all l once per chunk of kLgKC basis vectors, i.e. n / kLgKC times from
-// L2; here the 32 sites' n rows are copied in once (coalesced 16-byte loads, site records padded to 36
-// floats so that a warp's 128-bit reads fall on distinct bank quads) and every chunk reads them from shared
-// memory.  In the C phase the next neighbour row is loaded before the arithmetic of the current one.
-// Longer runs (n > kLgStage, read on the device) take the global reads of the kernel above.
-constexpr int kLgStage = 20;
-constexpr int kLgRow = 36;   // floats per staged site row (32 + 4)
+// The contraction in one pass with the velocity and the energy (the default).  Block: 32 consecutive sites, one per
+// lane; warp: component mu (phase W) or link direction nu (phase C), so that every load of the planes is two contiguous
+// 512-byte segments.  Phase W holds the site's own row of up to kLbN basis vectors in registers, four colours at a time, and
+// leaves W_k,mu = sum_l S_kl r_l,mu of all of them in shared memory; phase C adds r_k,mu(y+nu) W_k,mu(y)^T to the lane's
+// 8 x 8 accumulator, the neighbours' rows loaded one vector ahead.
+//
+// What bounds it.  The kernel above re-reads the own rows and S for every four vectors, between two barriers each, with
+// its accumulators live: at 128 registers it waits on that chain of loads (long scoreboard 5.5 per issue, 34 % of the
+// FMA pipe).  Here the own rows are read once, all in flight together, and 8 warps with 255 registers each take the
+// place of 16 with 128.  At 32^4 and 18 vectors: 2.47 ms with the velocity and the energy, against 2.75 ms and two
+// combinations of 0.48 ms each; at 16^4 0.164 ms (40 % of the FMA pipe; 42 % of the issue slots).
+// VEL: Vel = sum_k cvel[k] r_k; EN: |sum_k cen[k] r_k|^2 to *out (float64-accurate sum): both from the rows in registers.
+// Runs longer than kLbN take a pass per kLbN x kLbN block of S.  Tiles are taken in the order (z block of bz planes, t,
+// position in the slab): the t + 1 rows of a slab are then still in L2 when the sweep reaches them.
+constexpr int kLbSites = 32;
+constexpr int kLbN = 20;           // the workloads' runs have 13 to 18 vectors
+constexpr int kLbSmem = (kLbN * kLbN + 2 * kBasisCap + kLbN * 32 * kLbSites) * (int)sizeof(float);
 
-inline size_t lg_staged_smem() {
-    return sizeof(float) * ((size_t)kLgStage * kLgSites * kLgRow + kLgSites * kLgPad + kLgKC * kBasisCap);
-}
-
-template <int LF>
-__global__ void __launch_bounds__(kLgSites * 4, 2) k_link_grad_staged(Geom g, Links32 U, const float* __restrict__ R,
-                                                                      size_t fs, const int* __restrict__ flags, int n,
-                                                                      const double* __restrict__ S, int ld,
-                                                                      double* __restrict__ G) {
-    extern __shared__ __align__(16) float lgs[];
-    float* Rs = lgs;                                          // [kLgStage][kLgSites][kLgRow]
-    float* Ws = Rs + (size_t)kLgStage * kLgSites * kLgRow;    // [kLgSites][kLgPad]
-    float* Ss = Ws + kLgSites * kLgPad;                       // [kLgKC][kBasisCap]
+template <int LF, bool VEL, bool EN>
+__global__ void __launch_bounds__(128, 2)
+    k_link_grad_basis(Geom g, Links32 U, const float* __restrict__ R, size_t fs, const int* __restrict__ flags, int n,
+                      const double* __restrict__ S, int ld, double* __restrict__ G, const double* __restrict__ cvel,
+                      double* __restrict__ Vel, const double* __restrict__ cen, int bz, double* partials, unsigned* counter,
+                      double* out) {
+    extern __shared__ __align__(16) float lbs[];
+    float* Ss = lbs;                                      // [k][l] of the current block of S
+    float* cv = Ss + kLbN * kLbN;
+    float* ce = cv + kBasisCap;
+    float4* W = reinterpret_cast<float4*>(ce + kBasisCap);   // [k][plane][site]
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (flags) n = flags[1];
-    const bool staged = n <= kLgStage;
-    const int sl = threadIdx.x >> 2, q = threadIdx.x & 3;
-    float* const wrow = Ws + sl * kLgPad;
-    for (int base = blockIdx.x * kLgSites; base < g.V; base += gridDim.x * kLgSites) {
-        const int y = base + sl;
-        const bool live = y < g.V;
-        const int yn = live ? step_site(g, y, q, 1) : 0;
-        if (staged) {
-            __syncthreads();   // the previous tile's reads of Rs are done
-            const int nsite = min(kLgSites, g.V - base);
-            for (int idx = threadIdx.x; idx < n * kLgSites * 8; idx += blockDim.x) {
-                const int l = idx / (kLgSites * 8), rem = idx - l * (kLgSites * 8);
-                const int ss = rem >> 3, c4 = rem & 7;
-                if (ss < nsite) {
-                    const float4 v = __ldg(reinterpret_cast<const float4*>(R + (size_t)l * fs + (size_t)(base + ss) * 32) + c4);
-                    *reinterpret_cast<float4*>(Rs + ((size_t)l * kLgSites + ss) * kLgRow + c4 * 4) = v;
-                }
-            }
+    auto load_s = [&](int k0, int l0) {
+        for (int i = threadIdx.x; i < kLbN * kLbN; i += blockDim.x) {
+            const int k = k0 + i / kLbN, l = l0 + i % kLbN;
+            Ss[i] = k < n && l < n ? (float)S[(size_t)k * ld + l] : 0.f;
         }
-        float C[8][8];
+    };
+    const bool single = n <= kLbN;
+    if (single) load_s(0, 0);
+    for (int k = threadIdx.x; k < kBasisCap; k += blockDim.x) {
+        if (VEL) cv[k] = k < n ? (float)cvel[k] : 0.f;
+        if (EN) ce[k] = k < n ? (float)cen[k] : 0.f;
+    }
+    __syncthreads();
+    SumSq32 energy;
+    const int P = g.stride[2], V3 = g.stride[3];
+    const int nts = (P * bz + kLbSites - 1) / kLbSites;
+    const int nunit = nts * g.L[3] * ((g.L[2] + bz - 1) / bz);
+    const size_t ps = (size_t)g.V * 4;                    // plane stride
+    for (int u = blockIdx.x; u < nunit; u += gridDim.x) {
+        const int jt = u % nts, ru = u / nts, tt = ru % g.L[3], z0 = (ru / g.L[3]) * bz;
+        const int first = jt * kLbSites + lane;
+        const bool live = first < P * min(bz, g.L[2] - z0);
+        const int y = live ? tt * V3 + z0 * P + first : 0;
+        const float* const own = R + (size_t)y * 4 + 2 * w * ps;
+        const float* const nbr = R + (size_t)step_site(g, y, w, 1) * 4;
+        float2 C[8][4];                                   // C[b][d], pairs of d
 #pragma unroll
         for (int b = 0; b < 8; b++)
 #pragma unroll
-            for (int d = 0; d < 8; d++) C[b][d] = 0.f;
-        for (int k0 = 0; k0 < n; k0 += kLgKC) {
-            __syncthreads();
-            for (int t = threadIdx.x; t < kLgKC * n; t += blockDim.x) {
-                const int kk = t / n, l = t - kk * n;
-                Ss[kk * kBasisCap + l] = k0 + kk < n ? (float)S[(size_t)(k0 + kk) * ld + l] : 0.f;
-            }
-            __syncthreads();
-            float w[kLgKC][8];
+            for (int d = 0; d < 4; d++) C[b][d] = make_float2(0.f, 0.f);
+        const int nk = max(n, 1);   // an empty run (zero momenta) still writes its zeros
+        for (int k0 = 0; k0 < nk; k0 += kLbN) {
+            const int kc = min(kLbN, n - k0);
+            // neighbours' rows of the first vector, on their way during phase W
+            const float* rk = nbr + (size_t)k0 * fs;
+            float4 ra[4][2];
+            if (kc > 0)
 #pragma unroll
-            for (int kk = 0; kk < kLgKC; kk++)
+                for (int mu = 0; mu < 4; mu++)
 #pragma unroll
-                for (int a = 0; a < 8; a++) w[kk][a] = 0.f;
-            if (live) {
-                for (int l = 0; l < n; l++) {
-                    float r[8];
-                    if (staged) lds8(Rs + ((size_t)l * kLgSites + sl) * kLgRow + q * 8, r);
-                    else load8_v8(R + (size_t)l * fs + (size_t)y * 32 + q * 8, r);
+                    for (int h = 0; h < 2; h++) ra[mu][h] = __ldg(reinterpret_cast<const float4*>(rk + (2 * mu + h) * ps));
+#pragma unroll 1
+            for (int h = 0; h < 2; h++) {
+                float4 va = make_float4(0.f, 0.f, 0.f, 0.f), ea = va;
+                for (int l0 = 0; l0 < nk; l0 += kLbN) {
+                    if (!single) {
+                        __syncthreads();
+                        load_s(k0, l0);
+                        __syncthreads();
+                    }
+                    float4 r[kLbN];
 #pragma unroll
-                    for (int kk = 0; kk < kLgKC; kk++) {
-                        const float sv = Ss[kk * kBasisCap + l];
+                    for (int l = 0; l < kLbN; l++)
+                        r[l] = l0 + l < n ? __ldg(reinterpret_cast<const float4*>(own + h * ps + (size_t)(l0 + l) * fs))
+                                          : make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int k = 0; k < kc; k++) {
+                        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+                        float4* dst = W + (k * 8 + 2 * w + h) * kLbSites + lane;
+                        if (l0 > 0) a = *dst;
 #pragma unroll
-                        for (int a = 0; a < 8; a++) w[kk][a] = fmaf(sv, r[a], w[kk][a]);
+                        for (int l = 0; l < kLbN; l += 4) {
+                            const float4 s = *reinterpret_cast<const float4*>(Ss + k * kLbN + l);
+                            const float sv[4] = {s.x, s.y, s.z, s.w};
+#pragma unroll
+                            for (int q = 0; q < 4; q++) {
+                                a.x = fmaf(sv[q], r[l + q].x, a.x); a.y = fmaf(sv[q], r[l + q].y, a.y);
+                                a.z = fmaf(sv[q], r[l + q].z, a.z); a.w = fmaf(sv[q], r[l + q].w, a.w);
+                            }
+                        }
+                        *dst = a;
+                    }
+                    if ((VEL || EN) && k0 == 0)
+#pragma unroll
+                        for (int l = 0; l < kLbN; l++) {
+                            if (VEL) {
+                                const float c = cv[l0 + l];
+                                va.x = fmaf(c, r[l].x, va.x); va.y = fmaf(c, r[l].y, va.y);
+                                va.z = fmaf(c, r[l].z, va.z); va.w = fmaf(c, r[l].w, va.w);
+                            }
+                            if (EN) {
+                                const float c = ce[l0 + l];
+                                ea.x = fmaf(c, r[l].x, ea.x); ea.y = fmaf(c, r[l].y, ea.y);
+                                ea.z = fmaf(c, r[l].z, ea.z); ea.w = fmaf(c, r[l].w, ea.w);
+                            }
+                        }
+                }
+                if ((VEL || EN) && k0 == 0 && live) {
+                    if (VEL) {
+                        const double o[4] = {(double)va.x, (double)va.y, (double)va.z, (double)va.w};
+                        store4(Vel + (size_t)y * 32 + w * 8 + h * 4, o);
+                    }
+                    if (EN) {
+                        energy.add(ea.x); energy.add(ea.y);
+                        energy.add(ea.z); energy.add(ea.w);
                     }
                 }
             }
-#pragma unroll
-            for (int kk = 0; kk < kLgKC; kk++) store8(wrow + kk * 32 + q * 8, w[kk]);
             __syncthreads();
-            if (live) {
-                const int kc = min(kLgKC, n - k0);
-                // neighbour rows of the chunk, one (k, mu) ahead: iterations it = 4 kk + mu in pairs, the even
-                // one in ra, the odd one in rb
-                const float* rn = R + (size_t)k0 * fs + (size_t)yn * 32;   // (k0 + kk, mu) at rn + kk fs + 8 mu
-                auto contract = [&](const float (&rv)[8], int it) {
-                    float wv[8];
-                    lds8(wrow + (it >> 2) * 32 + (it & 3) * 8, wv);
+            for (int k = 0; k < kc; k++) {
+                rk += fs;
+#pragma unroll
+                for (int mu = 0; mu < 4; mu++) {
+                    const float a[8] = {ra[mu][0].x, ra[mu][0].y, ra[mu][0].z, ra[mu][0].w,
+                                        ra[mu][1].x, ra[mu][1].y, ra[mu][1].z, ra[mu][1].w};
+                    if (k + 1 < kc)
+#pragma unroll
+                        for (int h = 0; h < 2; h++) ra[mu][h] = __ldg(reinterpret_cast<const float4*>(rk + (2 * mu + h) * ps));
+                    const float4 w0 = W[(k * 8 + 2 * mu) * kLbSites + lane], w1 = W[(k * 8 + 2 * mu + 1) * kLbSites + lane];
+                    const float2 wp[4] = {make_float2(w0.x, w0.y), make_float2(w0.z, w0.w), make_float2(w1.x, w1.y),
+                                          make_float2(w1.z, w1.w)};
 #pragma unroll
                     for (int b = 0; b < 8; b++)
 #pragma unroll
-                        for (int d = 0; d < 8; d++) C[b][d] = fmaf(rv[b], wv[d], C[b][d]);
-                };
-                float ra[8], rb[8];
-                load8_v8(rn, ra);
-                for (int it = 0; it < 4 * kc; it += 2) {
-                    load8_v8(rn + (size_t)((it + 1) >> 2) * fs + ((it + 1) & 3) * 8, rb);   // it + 1 < 4 kc always
-                    contract(ra, it);
-                    if (it + 2 < 4 * kc) load8_v8(rn + (size_t)((it + 2) >> 2) * fs + ((it + 2) & 3) * 8, ra);
-                    contract(rb, it + 1);
+                        for (int d = 0; d < 4; d++) C[b][d] = ffma2(make_float2(a[b], a[b]), wp[d], C[b][d]);
                 }
             }
+            __syncthreads();   // W is rewritten
         }
         if (live) {
-            const mat3<float> u = LinkLoad<float, LF>::load(U, y, q);
+            const mat3<float> m = LinkLoad<float, LF>::load(U, y, w);
             float Gk[8];
 #pragma unroll
             for (int a = 0; a < 8; a++) Gk[a] = 0.f;
@@ -357,254 +394,50 @@ __global__ void __launch_bounds__(kLgSites * 4, 2) k_link_grad_staged(Geom g, Li
             for (int d = 0; d < 8; d++) {
                 float col[8], rc[8];
 #pragma unroll
-                for (int b = 0; b < 8; b++) col[b] = C[b][d];
+                for (int b = 0; b < 8; b++) col[b] = d & 1 ? C[b][d >> 1].y : C[b][d >> 1].x;
                 herm<float> E = h_zero<float>();
-                acc_uxud_tl(E, u, coef_to_herm2(col));   // 2 sum_c (R C)_cd T^c
+                acc_uxud_tl(E, m, coef_to_herm2(col));   // 2 sum_c (R C)_cd T^c
                 herm2_to_coef_tl(E, rc);                  // (R C)_cd
                 f_contract(d, rc, Gk);
             }
-            double* out = G + (size_t)y * 32 + q * 8;
+            double o[8];
 #pragma unroll
-            for (int a = 0; a < 8; a++) out[a] = (double)Gk[a] * (1.0 / 16.0);
+            for (int a = 0; a < 8; a++) o[a] = (double)Gk[a] * (1.0 / 16.0);
+            store8(G + (size_t)y * 32 + w * 8, o);
         }
+    }
+    if (EN) {
+        __shared__ double sh[4];
+        double v[1] = {energy.value()};
+        block_sum<1>(v, sh);
+        grid_sum_finish<1>(v, partials, counter, out, gridDim.x, blockIdx.x, sh);
     }
 }
 
-// The same contraction with eight lanes per link pair: the two halves of each (site, direction) split the rows b
-// of C (C[b][d], b = 4 h + i), so that a lane holds 32 accumulators instead of 64 and chunks of 8 basis vectors
-// (instead of 4) halve the passes over the site's own basis rows.  The half h is uniform per warp (threads
-// 0..127: h = 0, 128..255: h = 1), so no branch on it diverges; the two halves' force contributions meet in
-// shared memory in a fixed order.  The conjugation by the link uses the adjoint matrix (the lane's four
-// columns of Ad(U_nu(y))).
-constexpr int kLsSites = 32;             // sites per block: 4 directions x 2 halves = 8 lanes each
-constexpr int kLsKC = 8;                 // basis vectors per chunk of W
-constexpr int kLsPad = kLsKC * 32 + 4;   // W per site: [kk][mu][8] + 4
-
-template <int LF>
-__global__ void __launch_bounds__(kLsSites * 8, 2) k_link_grad_split(Geom g, Links32 U, const float* __restrict__ R,
-                                                                     size_t fs, const int* __restrict__ flags, int n,
-                                                                     const double* __restrict__ S, int ld,
-                                                                     double* __restrict__ G) {
-    __shared__ __align__(16) float Ws[kLsSites * kLsPad];
-    __shared__ float Ss[kLsKC * kBasisCap];
-    __shared__ float Gh[kLsSites * 4 * 8];   // the h = 1 halves' contributions
-    if (flags) n = flags[1];
-    const int h = threadIdx.x >> 7, sl = (threadIdx.x & 127) >> 2, nu = threadIdx.x & 3;
-    float* const wrow = Ws + sl * kLsPad;
-    for (int base = blockIdx.x * kLsSites; base < g.V; base += gridDim.x * kLsSites) {
-        const int y = base + sl;
-        const bool live = y < g.V;
-        const int yn = live ? step_site(g, y, nu, 1) : 0;
-        float C[4][8];
-#pragma unroll
-        for (int i = 0; i < 4; i++)
-#pragma unroll
-            for (int d = 0; d < 8; d++) C[i][d] = 0.f;
-        for (int k0 = 0; k0 < n; k0 += kLsKC) {
-            __syncthreads();
-            for (int t = threadIdx.x; t < kLsKC * n; t += blockDim.x) {
-                const int kk = t / n, l = t - kk * n;
-                Ss[kk * kBasisCap + l] = k0 + kk < n ? (float)S[(size_t)(k0 + kk) * ld + l] : 0.f;
-            }
-            __syncthreads();
-            // W_k,mu(y) = sum_l S_kl r_l,mu(y) for this half's four k of the chunk (mu = nu)
-            float w[4][8];
-#pragma unroll
-            for (int i = 0; i < 4; i++)
-#pragma unroll
-                for (int a = 0; a < 8; a++) w[i][a] = 0.f;
-            if (live) {
-                for (int l = 0; l < n; l++) {
-                    float r[8];
-                    load8_v8(R + (size_t)l * fs + (size_t)y * 32 + nu * 8, r);
-#pragma unroll
-                    for (int i = 0; i < 4; i++) {
-                        const float sv = Ss[(4 * h + i) * kBasisCap + l];
-#pragma unroll
-                        for (int a = 0; a < 8; a++) w[i][a] = fmaf(sv, r[a], w[i][a]);
-                    }
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < 4; i++) store8(wrow + (4 * h + i) * 32 + nu * 8, w[i]);
-            __syncthreads();
-            // C[b][d] += r_k,mu(y+nu)[b] W_k,mu(y)[d] for the rows b = 4 h + i
-            if (live) {
-                const int kc = min(kLsKC, n - k0);
-                for (int kk = 0; kk < kc; kk++) {
-                    const float* rk = R + (size_t)(k0 + kk) * fs + (size_t)yn * 32 + 4 * h;
-#pragma unroll
-                    for (int mu = 0; mu < 4; mu++) {
-                        const float4 rp = __ldg(reinterpret_cast<const float4*>(rk + mu * 8));
-                        float wv[8];
-                        lds8(wrow + kk * 32 + mu * 8, wv);
-                        const float rb[4] = {rp.x, rp.y, rp.z, rp.w};
-#pragma unroll
-                        for (int i = 0; i < 4; i++)
-#pragma unroll
-                            for (int d = 0; d < 8; d++) C[i][d] = fmaf(rb[i], wv[d], C[i][d]);
-                    }
-                }
-            }
-        }
-        // G^a = (1/16) sum_cd f_acd (Ad C)_cd; this half contributes the columns b = 4 h + i of Ad
-        float Gk[8];
-#pragma unroll
-        for (int a = 0; a < 8; a++) Gk[a] = 0.f;
-        if (live) {
-            const mat3<float> u = LinkLoad<float, LF>::load(U, y, nu);
-            float cols[4][8];
-            adjoint_columns(u, [&](int bcol, const float (&col)[8]) {
-                if ((bcol >> 2) == h)
-#pragma unroll
-                    for (int c = 0; c < 8; c++) cols[bcol & 3][c] = col[c];
-            });
-#pragma unroll
-            for (int d = 0; d < 8; d++) {
-                float rc[8];
-#pragma unroll
-                for (int c = 0; c < 8; c++) {
-                    float v = 0.f;
-#pragma unroll
-                    for (int i = 0; i < 4; i++) v = fmaf(cols[i][c], C[i][d], v);
-                    rc[c] = v;
-                }
-                f_contract(d, rc, Gk);
-            }
-        }
-        if (h == 1) {
-#pragma unroll
-            for (int a = 0; a < 8; a++) Gh[(sl * 4 + nu) * 8 + a] = Gk[a];
-        }
-        __syncthreads();
-        if (h == 0 && live) {
-            double* out = G + (size_t)y * 32 + nu * 8;
-#pragma unroll
-            for (int a = 0; a < 8; a++) out[a] = (double)(Gk[a] + Gh[(sl * 4 + nu) * 8 + a]) * (1.0 / 16.0);
-        }
-        __syncthreads();   // Gh is rewritten by the next tile
-    }
-}
-
-// The contraction of k_link_grad_krylov with the neighbour rows staged: in the C phase, lane (y, nu) needs
-// the whole row r_k(y + nu) (128 bytes); read lane by lane, one load instruction of a warp touches 32
-// different rows (one 32-byte sector each).  Here the 4 lanes of a site instead load the 4 chunks of each of
-// its 4 neighbour rows (one instruction: 8 whole rows), store them to shared memory (rows padded to 36
-// floats: a warp's 128-bit accesses fall on distinct bank quads), and after a warp barrier (the four lanes of a
-// site are in one warp) every lane reads its own row there.
-constexpr int kNbRow = 36;
-template <int LF>
-__global__ void __launch_bounds__(kLgSites * 4, 4) k_link_grad_nbs(Geom g, Links32 U, const float* __restrict__ R,
-                                                                size_t fs, const int* __restrict__ flags, int n,
-                                                                const double* __restrict__ S, int ld,
-                                                                double* __restrict__ G) {
-    __shared__ __align__(16) float Ws[kLgSites * kLgPad];
-    __shared__ float Ss[kLgKC * kBasisCap];
-    __shared__ __align__(16) float Nb[4 * kLgSites * kNbRow];   // [nu][site][kNbRow]
-    if (flags) n = flags[1];
-    const int sl = threadIdx.x >> 2, q = threadIdx.x & 3;
-    float* const wrow = Ws + sl * kLgPad;
-    for (int base = blockIdx.x * kLgSites; base < g.V; base += gridDim.x * kLgSites) {
-        const int y = base + sl;
-        const bool live = y < g.V;
-        int fwd[4] = {0, 0, 0, 0}, bwd[4];
-        if (live) neighbours(g, y, fwd, bwd);
-        float C[8][8];
-#pragma unroll
-        for (int b = 0; b < 8; b++)
-#pragma unroll
-            for (int d = 0; d < 8; d++) C[b][d] = 0.f;
-        // chunk q of the 4 neighbour rows of basis vector k: registers, then shared memory
-        float t[4][8];
-        auto gload = [&](int k) {
-            const float* rk = R + (size_t)k * fs + q * 8;
-#pragma unroll
-            for (int nu = 0; nu < 4; nu++) load8_v8(rk + (size_t)fwd[nu] * 32, t[nu]);
-        };
-        auto sstore = [&]() {
-#pragma unroll
-            for (int nu = 0; nu < 4; nu++) {
-                float4* d = reinterpret_cast<float4*>(Nb + (nu * kLgSites + sl) * kNbRow + q * 8);
-                d[0] = make_float4(t[nu][0], t[nu][1], t[nu][2], t[nu][3]);
-                d[1] = make_float4(t[nu][4], t[nu][5], t[nu][6], t[nu][7]);
-            }
-        };
-        const float* const nrow = Nb + (q * kLgSites + sl) * kNbRow;
-        for (int k0 = 0; k0 < n; k0 += kLgKC) {
-            __syncthreads();
-            for (int i = threadIdx.x; i < kLgKC * n; i += blockDim.x) {
-                const int kk = i / n, l = i - kk * n;
-                Ss[kk * kBasisCap + l] = k0 + kk < n ? (float)S[(size_t)(k0 + kk) * ld + l] : 0.f;
-            }
-            __syncthreads();
-            float w[kLgKC][8];
-#pragma unroll
-            for (int kk = 0; kk < kLgKC; kk++)
-#pragma unroll
-                for (int a = 0; a < 8; a++) w[kk][a] = 0.f;
-            if (live) {
-                for (int l = 0; l < n; l++) {
-                    float r[8];
-                    load8_v8(R + (size_t)l * fs + (size_t)y * 32 + q * 8, r);
-#pragma unroll
-                    for (int kk = 0; kk < kLgKC; kk++) {
-                        const float sv = Ss[kk * kBasisCap + l];
-#pragma unroll
-                        for (int a = 0; a < 8; a++) w[kk][a] = fmaf(sv, r[a], w[kk][a]);
-                    }
-                }
-            }
-#pragma unroll
-            for (int kk = 0; kk < kLgKC; kk++) store8(wrow + kk * 32 + q * 8, w[kk]);
-            const int kc = min(kLgKC, n - k0);   // uniform over the block
-            for (int kk = 0; kk < kc; kk++) {
-                if (live) {
-                    gload(k0 + kk);
-                    sstore();
-                }
-                __syncwarp();   // the rows of k (and, for kk = 0, the chunk's W) are in place: a site's
-                                // rows and W are written and read by its own four lanes, within one warp
-                if (live) {
-#pragma unroll
-                    for (int mu = 0; mu < 4; mu++) {
-                        float rp[8], wv[8];
-                        lds8(nrow + mu * 8, rp);
-                        lds8(wrow + kk * 32 + mu * 8, wv);
-#pragma unroll
-                        for (int b = 0; b < 8; b++)
-#pragma unroll
-                            for (int d = 0; d < 8; d++) C[b][d] = fmaf(rp[b], wv[d], C[b][d]);
-                    }
-                }
-                __syncwarp();   // the site's lanes have read the rows of k
-            }
-        }
-        if (live) {
-            const mat3<float> u = LinkLoad<float, LF>::load(U, y, q);
-            float Gk[8];
-#pragma unroll
-            for (int a = 0; a < 8; a++) Gk[a] = 0.f;
-#pragma unroll
-            for (int d = 0; d < 8; d++) {
-                float col[8], rc[8];
-#pragma unroll
-                for (int b = 0; b < 8; b++) col[b] = C[b][d];
-                herm<float> E = h_zero<float>();
-                acc_uxud_tl(E, u, coef_to_herm2(col));   // 2 sum_c (R C)_cd T^c
-                herm2_to_coef_tl(E, rc);                  // (R C)_cd
-                f_contract(d, rc, Gk);
-            }
-            double* out = G + (size_t)y * 32 + q * 8;
-#pragma unroll
-            for (int a = 0; a < 8; a++) out[a] = (double)Gk[a] * (1.0 / 16.0);
-        }
-    }
+template <bool VEL, bool EN>
+static int launch_basis(rmhmc_ctx* ctx, const float* R, const int* flags, int n, const double* S, double* G,
+                        const double* cvel, double* Vel, const double* cen, int slot, cudaStream_t st) {
+    auto kern = k_link_grad_basis<18, VEL, EN>;
+    RM_CHECK(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kLbSmem));
+    // slabs of z whose two t-slices of 20 basis vectors take at most a third of L2
+    const size_t slice = (size_t)ctx->g.stride[3] * 32 * sizeof(float) * 20 * 2, room = (size_t)40 << 20;
+    const int nzb = (int)std::min<size_t>(ctx->g.L[2], (slice + room - 1) / room);
+    const int bz = (ctx->g.L[2] + nzb - 1) / nzb;
+    const int nunit = (ctx->g.stride[2] * bz + kLbSites - 1) / kLbSites * ctx->g.L[3] * ((ctx->g.L[2] + bz - 1) / bz);
+    const int grid = std::max(1, std::min(std::min(nunit, (int)ctx->num_sms * 2), ctx->max_blocks * 2));
+    kern<<<grid, 128, kLbSmem, st>>>(ctx->g, links32(ctx), R, field_elems(ctx), flags, n, S, kBasisCap, G, cvel, Vel, cen, bz,
+                                     EN ? red_slot_partials(ctx, slot) : nullptr,
+                                     EN ? red_slot_counter(ctx, slot) : nullptr, EN ? red_slot_out(ctx, slot) : nullptr);
+    ++ctx->launches;
+    RM_LAUNCH_CHECK(ctx);
+    return RMHMC_OK;
 }
 
 // F_K from the basis rows (X_j rows 0..ns-1, Z_j rows ns..2ns-1, row stride ldr, device float64) of the
 // float32 basis R; n on the host, or read on the device from flags[1] when flags is given
 int link_grad_krylov_launch(rmhmc_ctx* ctx, const float* R, const double* rows, int ldr, int ns, const double* alpha,
-                            const int* flags, int n, double* F, cudaStream_t st) {
+                            const int* flags, int n, double* F, const double* cvel, double* Vel, const double* cen,
+                            int slot, cudaStream_t st) {
     if (ns > kMaxPairs) return set_err(ctx, RMHMC_EINVAL, "at most %d poles", kMaxPairs);
     int status = RMHMC_OK;
     double* S = (double*)workspace(ctx, "kf_pairs", sizeof(double) * kBasisCap * kBasisCap, &status);
@@ -613,35 +446,15 @@ int link_grad_krylov_launch(rmhmc_ctx* ctx, const float* R, const double* rows, 
     for (int j = 0; j < ns; j++) pw.w[j] = alpha[j];
     k_pair_matrix<<<ctx->num_sms / 4 > 1 ? ctx->num_sms / 4 : 1, 256, 0, st>>>(rows, ldr, ns, pw, flags, n, S, kBasisCap);
     ++ctx->launches;
-    if (ctx->lg_mode == 3) {
-        const int grid = capped_grid(ctx, (size_t)ctx->g.V * 4, kLgSites * 4);
-        k_link_grad_nbs<18><<<grid, kLgSites * 4, 0, st>>>(ctx->g, links32(ctx), R, field_elems(ctx), flags, n, S,
-                                                           kBasisCap, F);
-    } else if (ctx->lg_mode == 2) {
-        const int ntile = (ctx->g.V + kLsSites - 1) / kLsSites;
-        const int grid = std::max(1, std::min(ntile, (int)ctx->num_sms * 2));
-        k_link_grad_split<18><<<grid, kLsSites * 8, 0, st>>>(ctx->g, links32(ctx), R, field_elems(ctx), flags, n, S,
-                                                             kBasisCap, F);
-    } else if (ctx->lg_mode == 1) {
-        static bool configured[64] = {};
-        if (ctx->device < 0 || ctx->device >= 64) return set_err(ctx, RMHMC_EINVAL, "device index too large");
-        if (!configured[ctx->device]) {
-            RM_CHECK(ctx, cudaFuncSetAttribute(k_link_grad_staged<18>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)lg_staged_smem()));
-            configured[ctx->device] = true;
-        }
-        int per_sm = 0;
-        RM_CHECK(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_link_grad_staged<18>, kLgSites * 4,
-                                                                    lg_staged_smem()));
-        const int ntile = (ctx->g.V + kLgSites - 1) / kLgSites;
-        const int grid = std::max(1, std::min(ntile, (int)ctx->num_sms * std::max(per_sm, 1)));
-        k_link_grad_staged<18><<<grid, kLgSites * 4, lg_staged_smem(), st>>>(ctx->g, links32(ctx), R, field_elems(ctx),
-                                                                             flags, n, S, kBasisCap, F);
-    } else {
-        const int grid = capped_grid(ctx, (size_t)ctx->g.V * 4, kLgSites * 4);
-        k_link_grad_krylov<float, 18><<<grid, kLgSites * 4, 0, st>>>(ctx->g, links32(ctx), R, field_elems(ctx), flags, n,
-                                                                     S, kBasisCap, F);
+    if (ctx->lg_mode == kLgFused) {
+        if (Vel && cen) return launch_basis<true, true>(ctx, R, flags, n, S, F, cvel, Vel, cen, slot, st);
+        if (Vel) return launch_basis<true, false>(ctx, R, flags, n, S, F, cvel, Vel, cen, slot, st);
+        if (cen) return launch_basis<false, true>(ctx, R, flags, n, S, F, cvel, Vel, cen, slot, st);
+        return launch_basis<false, false>(ctx, R, flags, n, S, F, cvel, Vel, cen, slot, st);
     }
+    const int grid = capped_grid(ctx, (size_t)ctx->g.V * 4, kLgSites * 4);
+    k_link_grad_krylov<float, 18><<<grid, kLgSites * 4, 0, st>>>(ctx->g, links32(ctx), R, field_elems(ctx), flags, n, S,
+                                                                 kBasisCap, F);
     ++ctx->launches;
     RM_LAUNCH_CHECK(ctx);
     return RMHMC_OK;
@@ -651,18 +464,18 @@ int link_grad_krylov_launch(rmhmc_ctx* ctx, const float* R, const double* rows, 
 // kinetic pieces from a single Krylov run on P
 // ------------------------------------------------------------------------------------------------
 template <typename T>
-static int kinetic_t(rmhmc_ctx* ctx, const MassTerm& m, const T* P, const double* P64, double tol, int maxiter, double* F,
-                     double* Vel, double* Tkin, int* iters, cudaStream_t st) {
+static int kinetic_t(rmhmc_ctx* ctx, const MassTerm& m, const double* P, double tol, int maxiter, double* F, double* Vel,
+                     double* Tkin, int* iters, cudaStream_t st) {
     const int ns = m.npole();
     const size_t fs = field_elems(ctx);
     int status = RMHMC_OK;
     if (ns == 0) {
         // M = c^{-2}: V = c^2 P, F_K = 0, T = c^2 |P|^2 / 2
         if (F) RM_CHECK(ctx, cudaMemsetAsync(F, 0, sizeof(double) * fs, st));
-        if (Vel) RM_TRY(axpby64(ctx, m.c * m.c, P64, 0.0, nullptr, Vel, fs, st));
+        if (Vel) RM_TRY(axpby64(ctx, m.c * m.c, P, 0.0, nullptr, Vel, fs, st));
         if (Tkin) {
             double n2 = 0.0;
-            RM_TRY(norm2_64(ctx, P64, fs, &n2, st));
+            RM_TRY(norm2_64(ctx, P, fs, &n2, st));
             *Tkin = 0.5 * m.c * m.c * n2;
         }
         if (iters) *iters = 0;
@@ -670,7 +483,7 @@ static int kinetic_t(rmhmc_ctx* ctx, const MassTerm& m, const T* P, const double
     }
     const double s0 = *std::min_element(m.sigma.begin(), m.sigma.end());
     KrylovResult kr;
-    RM_TRY(krylov_run<T>(ctx, P, s0, tol, maxiter, kr, st));
+    RM_TRY((krylov_run<T, double>(ctx, P, s0, tol, maxiter, kr, st)));
     if (kr.status == 2) return set_err(ctx, RMHMC_ENOCONV, "kinetic force: Krylov run hit its cap (%d)", kr.n);
     if (iters) *iters = kr.n;
     Tridiag tri;
@@ -690,7 +503,9 @@ static int kinetic_t(rmhmc_ctx* ctx, const MassTerm& m, const T* P, const double
         v[k] = m.c * g[k];
         for (int j = 0; j < ns; j++) v[k] += m.alpha[j] * zs[j][k];
     }
-    if (Tkin) {
+    // float32 basis: force, velocity and energy in one pass over the basis
+    const bool fused = F && sizeof(T) == 4 && ctx->lg_mode == kLgFused;
+    if (Tkin && !fused) {
         // T = 1/2 |R P|^2 from the explicitly formed R P (float64 sum), not from |g|, which would
         // assume exactly orthonormal Lanczos vectors
         double* Y = (double*)workspace(ctx, "kf_y", sizeof(double) * fs, &status);
@@ -706,7 +521,7 @@ static int kinetic_t(rmhmc_ctx* ctx, const MassTerm& m, const T* P, const double
         RM_TRY(norm2_64(ctx, Y, fs, &y2, st));
         *Tkin = 0.5 * y2;
     }
-    if (Vel) {
+    if (Vel && !fused) {
         CombineSpec spec;
         spec.n = n;
         spec.M = 1;
@@ -717,16 +532,25 @@ static int kinetic_t(rmhmc_ctx* ctx, const MassTerm& m, const T* P, const double
     }
     if (F && sizeof(T) == 4) {
         // float32 basis: the force straight from the basis (rows of X_j and Z_j on the stored residuals)
-        double* rows = (double*)workspace(ctx, "kf_rows", sizeof(double) * (size_t)2 * ns * kBasisCap, &status);
+        double* rows = (double*)workspace(ctx, "kf_rows", sizeof(double) * (size_t)(2 * ns + 2) * kBasisCap, &status);
         if (!rows) return status;
-        std::vector<double> h((size_t)2 * ns * n, 0.0);
+        std::vector<double> h((size_t)(2 * ns + 2) * n, 0.0);
         for (int j = 0; j < ns; j++) {
             tri.to_basis(ys[j], h.data() + (size_t)j * n);
             tri.to_basis(zs[j], h.data() + (size_t)(ns + j) * n);
         }
+        tri.to_basis(v, h.data() + (size_t)2 * ns * n);
+        tri.to_basis(g, h.data() + (size_t)(2 * ns + 1) * n);
         RM_TRY(upload(ctx, rows, h.data(), sizeof(double) * h.size(), st));
-        RM_TRY(link_grad_krylov_launch(ctx, (const float*)krylov_basis<T>(ctx), rows, n, ns, m.alpha.data(), nullptr, n,
-                                       F, st));
+        RM_TRY(link_grad_krylov_launch(ctx, (const float*)krylov_basis<T>(ctx), rows, n, ns, m.alpha.data(), nullptr, n, F,
+                                       rows + (size_t)2 * ns * n, Vel, Tkin ? rows + (size_t)(2 * ns + 1) * n : nullptr,
+                                       kSlotNorm, st));
+        if (fused && Tkin) {
+            // |R P|^2 of the explicitly formed R P, as above
+            double y2 = 0.0;
+            RM_TRY(fetch(ctx, red_slot_out(ctx, kSlotNorm), &y2, 1, st));
+            *Tkin = 0.5 * y2;
+        }
     } else if (F) {
         T* XZ = (T*)workspace(ctx, "kf_xz64", sizeof(T) * fs * 2 * ns, &status);
         if (!XZ) return status;
@@ -750,13 +574,8 @@ static int kinetic_t(rmhmc_ctx* ctx, const MassTerm& m, const T* P, const double
 
 int kinetic_from_krylov(rmhmc_ctx* ctx, const MassTerm& m, const double* P, double tol, int maxiter, int prec,
                         double* F, double* Vel, double* T, int* iters, cudaStream_t st) {
-    if (prec == RMHMC_FP64) return kinetic_t<double>(ctx, m, P, P, tol, maxiter, F, Vel, T, iters, st);
-    int status = RMHMC_OK;
-    const size_t fs = field_elems(ctx);
-    float* P32 = (float*)workspace(ctx, "kf_p32", sizeof(float) * fs, &status);
-    if (!P32) return status;
-    RM_TRY(to_float(ctx, P, P32, fs, st));
-    return kinetic_t<float>(ctx, m, P32, P, tol, maxiter, F, Vel, T, iters, st);
+    if (prec == RMHMC_FP64) return kinetic_t<double>(ctx, m, P, tol, maxiter, F, Vel, T, iters, st);
+    return kinetic_t<float>(ctx, m, P, tol, maxiter, F, Vel, T, iters, st);
 }
 
 }  // namespace rm
@@ -795,7 +614,21 @@ extern "C" int kinetic_force(rmhmc_ctx* ctx, const double* U, const double* P, c
     MassTerm m;
     RM_TRY(parse_mass(ctx, mass, m));
     RM_TRY(ensure_links(ctx, U, stream));
-    return kinetic_from_krylov(ctx, m, P, tol, 1000, prec, F, Vout, T, nullptr, stream);
+    // the kernels read and write float64 fields 16 bytes at a time: a field at an odd multiple of 8 bytes goes through
+    // the workspace
+    const size_t bytes = sizeof(double) * field_elems(ctx);
+    int status = RMHMC_OK;
+    auto aligned = [&](const void* p, const char* name) -> double* {
+        return (uintptr_t)p % 16 ? (double*)workspace(ctx, name, bytes, &status) : (double*)p;
+    };
+    const double* Pa = aligned(P, "kf_p16");
+    double *Fa = aligned(F, "kf_f16"), *Va = aligned(Vout, "kf_v16");
+    RM_TRY(status);
+    if (Pa != P) RM_CHECK(ctx, cudaMemcpyAsync((void*)Pa, P, bytes, cudaMemcpyDeviceToDevice, stream));
+    RM_TRY(kinetic_from_krylov(ctx, m, Pa, tol, 1000, prec, Fa, Va, T, nullptr, stream));
+    if (Fa != F) RM_CHECK(ctx, cudaMemcpyAsync(F, Fa, bytes, cudaMemcpyDeviceToDevice, stream));
+    if (Va != Vout) RM_CHECK(ctx, cudaMemcpyAsync(Vout, Va, bytes, cudaMemcpyDeviceToDevice, stream));
+    return RMHMC_OK;
 }
 
 extern "C" int rmhmc_heatbath(rmhmc_ctx* ctx, const double* U, const double* xi, const rmhmc_mass* mass, double tol,

@@ -7,6 +7,7 @@
 
 #include <algorithm>
 
+#include "df.cuh"
 #include "krylov.cuh"
 #include "ops.cuh"
 #include "stencil.cuh"
@@ -35,42 +36,61 @@ template <> struct Vec<double> {
     __device__ __forceinline__ static type make(const double* x) { return make_double2(x[0], x[1]); }
 };
 
-// r_0 = b, rho_0 = |b|^2 (one vector element per thread, coalesced)
-template <typename T>
-__global__ void __launch_bounds__(kBlock) k_cg_start(const T* __restrict__ b, T* __restrict__ r0, size_t nvec, int* flags,
+// r_0 = b rounded to T and re-laid from [V][4][8] to the planes, rho_0 = |r_0|^2; thread: four colours of a component.
+// The sum of a float32 run and the rounding use no float64 arithmetic, which took longer than the bytes (32^4: a
+// conversion pass of 75 us and this one of 139 us, together 60 us of traffic)
+template <typename T, typename TI>
+__device__ __forceinline__ double start_pass(const TI* __restrict__ b, T* __restrict__ r0, int V) {
+    const size_t n4 = (size_t)V * 8;
+    SumSq32 sf;
+    double sd = 0.0;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
+        TI v[4];
+        load4(b + i * 4, v);
+        T x[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            if constexpr (sizeof(T) == 4) {
+                x[k] = to_f32(v[k]);
+                sf.add(x[k]);
+            } else {
+                x[k] = v[k];
+                sd = fma(x[k], x[k], sd);
+            }
+        }
+        store4(plane_at(r0, V, (int)(i >> 3), (int)(i & 7)), x);
+    }
+    return sizeof(T) == 4 ? sf.value() : sd;
+}
+
+template <typename T, typename TI>
+__global__ void __launch_bounds__(kBlock) k_cg_start(const TI* __restrict__ b, T* __restrict__ r0, int V, int* flags,
                                                      double* rho, double* partials, unsigned* counter) {
     __shared__ double sh[kBlock / 32];
-    using VT = Vec<T>;
-    double acc = 0.0;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nvec; i += (size_t)gridDim.x * blockDim.x) {
-        const typename VT::type v = reinterpret_cast<const typename VT::type*>(b)[i];
-        reinterpret_cast<typename VT::type*>(r0)[i] = v;
-        T x[VT::n];
-        VT::get(v, x);
-#pragma unroll
-        for (int k = 0; k < VT::n; k++) acc += (double)x[k] * (double)x[k];
-    }
-    double v[1] = {acc};
+    double v[1] = {start_pass(b, r0, V)};
     block_sum<1>(v, sh);
-    {
-        double out[1];
-        if (grid_sum_finish<1>(v, partials, counter, out, gridDim.x, blockIdx.x, sh)) {
-            rho[0] = out[0];
-            flags[1] = 0;
-            flags[0] = isfinite(out[0]) ? (out[0] == 0.0 ? 1 : 0) : 3;
-        }
+    double out[1];
+    if (grid_sum_finish<1>(v, partials, counter, out, gridDim.x, blockIdx.x, sh)) {
+        rho[0] = out[0];
+        flags[1] = 0;
+        flags[0] = isfinite(out[0]) ? (out[0] == 0.0 ? 1 : 0) : 3;
     }
 }
 
 // CG without the search direction: q_k = (A + sigma0) p_k is carried as q_k = (A + sigma0) r_k + beta_{k-1} q_{k-1}
 // (p_k = r_k + beta_{k-1} p_{k-1}), so the stencil reads only r_k; gamma_k = <p_k, A p_k> = <r_k, q_k> by
 // A-conjugacy of the directions, alpha_k = rho_k / gamma_k.  q is updated in place at the lane's own site.
+// At 32^4: 0.212 ms (two components per lane, 256 threads) against 0.225 ms with the vectors as site rows (one component,
+// four lanes a site); at 16^4 22.3 against 23.4 us.  What is left is DRAM traffic (1.25 times the 672 bytes a site) and the
+// latency of the neighbour loads.
+// One lane per site and group of NC components: a warp holds 32 consecutive sites of one group, and the blocks run
+// through the groups of a site range together, so that its links come from DRAM once.
 template <typename T, int LF, int NMU>
 __global__ void __launch_bounds__(kBlockMax, (stencil_min_blocks<T, NMU>())) k_cg_A(Geom g, typename LinksOf<T>::type U, const T* __restrict__ R, size_t fs,
                                                      T* __restrict__ q, T diag, const int* __restrict__ flags,
                                                      double* vals, int maxit, double* partials, unsigned* counter) {
     constexpr int NC = NMU == 0 ? 1 : NMU;   // components per lane
-    constexpr int LPS = 4 / NC;
+    constexpr int NG = 4 / NC;               // lanes (groups of components) per site
     __shared__ double sh[kBlockMax / 32];
     if (flags[0]) return;
     const int k = flags[1];
@@ -81,22 +101,20 @@ __global__ void __launch_bounds__(kBlockMax, (stencil_min_blocks<T, NMU>())) k_c
     const double* beta = alpha + maxit;
     const T b = k > 0 ? (T)beta[k - 1] : T(0);
     T dot = T(0);
-    const int nlane = g.V * LPS;
-    for (int lane = blockIdx.x * blockDim.x + threadIdx.x; lane < nlane; lane += gridDim.x * blockDim.x) {
-        const int s = lane / LPS, mu0 = (lane % LPS) * NC;
+    const int nunit = (g.V + 31) / 32 * NG, wpb = blockDim.x >> 5;   // warp units: (32 sites, group)
+    for (int u = blockIdx.x * wpb + (threadIdx.x >> 5); u < nunit; u += gridDim.x * wpb) {
+        const int s = u / NG * 32 + (threadIdx.x & 31), mu0 = (u % NG) * NC;
+        if (s >= g.V) continue;
         herm<T> acc[NC];
-        if constexpr (sizeof(T) == 4 && NMU == 1) hop_sum_shape<T, LF, NMU>(g, U, s, mu0, SrcFieldV8{r}, acc);
-        else hop_sum_shape<T, LF, NMU>(g, U, s, mu0, SrcField<T>{r}, acc);
+        hop_sum_shape<T, LF, NMU>(g, U, s, mu0, SrcPlanar<T>{r, g.V}, acc);
 #pragma unroll
         for (int m = 0; m < NC; m++) {
             const int mu = mu0 + m;
             T h[8], x[8], y[8];
             herm2_to_coef_tl(acc[m], h);
-            if constexpr (sizeof(T) == 4 && NMU == 1) load8_v8(r + (size_t)s * 32 + mu * 8, x);
-            else load8(r + (size_t)s * 32 + mu * 8, x);
-            T* qs = q + (size_t)s * 32 + mu * 8;
+            load_plane8(r, g.V, s, mu, x);
             if (k > 0) {
-                load8(qs, y);
+                load_plane8((const T*)q, g.V, s, mu, y);
 #pragma unroll
                 for (int a = 0; a < 8; a++) y[a] = fma(b, y[a], fma(T(-0.0625), h[a], diag * x[a]));
             } else {
@@ -105,7 +123,8 @@ __global__ void __launch_bounds__(kBlockMax, (stencil_min_blocks<T, NMU>())) k_c
             }
 #pragma unroll
             for (int a = 0; a < 8; a++) dot = fma(x[a], y[a], dot);
-            store8(qs, y);
+            store4(plane_at(q, g.V, s, 2 * mu), y);
+            store4(plane_at(q, g.V, s, 2 * mu + 1), y + 4);
         }
     }
     double v[1] = {0.0};
@@ -133,7 +152,9 @@ __global__ void __launch_bounds__(kBlockMax, (stencil_min_blocks<T, NMU>())) k_c
 template <typename T, int NMU>
 static void launch_cg_A(rmhmc_ctx* ctx, const StencilShape& shp, typename LinksOf<T>::type U, T* R, size_t fs, T* q,
                         T diag, int* flags, double* vals, int maxit, cudaStream_t st) {
-    k_cg_A<T, 18, NMU><<<stencil_blocks(ctx, shp), shp.block, 0, st>>>(ctx->g, U, R, fs, q, diag, flags, vals, maxit,
+    // whole warps of 32 sites per group
+    const size_t lanes = (size_t)((ctx->g.V + 31) / 32 * 32) * lanes_per_site(NMU);
+    k_cg_A<T, 18, NMU><<<std::min(capped_grid(ctx, lanes, shp.block), ctx->max_blocks * 2), shp.block, 0, st>>>(ctx->g, U, R, fs, q, diag, flags, vals, maxit,
                                                                       red_slot_partials(ctx, 0), red_slot_counter(ctx, 0));
     ++ctx->launches;
 }
@@ -154,9 +175,12 @@ static int cg_stencil(rmhmc_ctx* ctx, const StencilShape& shp, typename LinksOf<
     return RMHMC_OK;
 }
 
-// Launch shape of the CG stencil, tuned on its own (its loads differ from the plain stencil's: it also reads
-// and writes q, and the one-component shape reads the basis with 256-bit loads): every shape is timed on the
-// context's lattice (k = 0 on zeroed scratch, three repetitions after a warm-up) at first use.
+// Launch shape of the CG stencil, tuned on its own (its loads differ from the plain stencil's: planes, and it also reads
+// and writes q): every shape is timed on the context's lattice (k = 0 on zeroed scratch, three repetitions after a
+// warm-up) at first use.  Below kCgTuneMin sites there is nothing to time: a launch is a chain of latencies, shortest
+// with one component per lane (8^4: 9.1 us against 11.1 and 13.2 us with two and four), and timings that differ by
+// their noise alone would let two contexts sum in different orders.
+constexpr int kCgTuneMin = 16384;
 template <typename T>
 static int cg_shape(rmhmc_ctx* ctx, cudaStream_t st, StencilShape& out) {
     const int key = 10000 + (int)sizeof(T) * 100 + 18;
@@ -166,8 +190,10 @@ static int cg_shape(rmhmc_ctx* ctx, cudaStream_t st, StencilShape& out) {
         out.block = it->second.second;
         return RMHMC_OK;
     }
-    StencilShape base;
-    RM_TRY((stencil_shape<T, 18>(ctx, st, base)));
+    if (ctx->g.V < kCgTuneMin) {
+        out = StencilShape{1, 128};
+        return RMHMC_OK;
+    }
     int status = RMHMC_OK;
     const size_t fs = field_elems(ctx);
     T* X = (T*)workspace(ctx, "tune_x", sizeof(double) * fs, &status);
@@ -270,7 +296,7 @@ __global__ void __launch_bounds__(kBlock) k_cg_B(T* __restrict__ R, size_t fs, c
     }
 }
 
-// out[m] = sum_{k < n} coef[m][k] basis_k for m < M <= MB.  Every coefficient is staged in shared memory
+// out[m] = sum_{k < n} coef[m][k] basis_k for m < M <= MB, re-laid from planes to [V][4][8].  Every coefficient is staged in shared memory
 // once per block; the grid strides over vectors of 16 bytes (float4 / double2) so every basis vector is
 // read with 128-bit loads, four vectors in flight per step.  n is read from flags[1] when flags is given
 // (device-decided Krylov length); coefficient row stride ldc.
@@ -300,6 +326,9 @@ __global__ void __launch_bounds__(kBlock) k_combine(const T* __restrict__ R, siz
     const size_t nvec = fs / VN;
     const typename VT::type* Rv = reinterpret_cast<const typename VT::type*>(R);
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nvec; i += (size_t)gridDim.x * blockDim.x) {
+        // the outputs are [V][4][8]: element e of plane c at site s goes to 32 s + 4 c + e
+        const size_t c = (i * VN) / (fs >> 3), e = i * VN - c * (fs >> 3);
+        const size_t aos = (e >> 2) * 32 + c * 4 + (e & 3);
         T acc[MB][VN];
 #pragma unroll
         for (int m = 0; m < MB; m++)
@@ -337,7 +366,7 @@ __global__ void __launch_bounds__(kBlock) k_combine(const T* __restrict__ R, siz
                 TO o[VN];
 #pragma unroll
                 for (int v = 0; v < VN; v++) o[v] = (TO)acc[m][v];
-                TO* dst = outs.p[m] + i * VN;
+                TO* dst = outs.p[m] + aos;
                 if (sizeof(TO) == sizeof(T)) store_vec<TO>(dst, o);
                 else {
 #pragma unroll
@@ -505,8 +534,8 @@ T* krylov_basis(rmhmc_ctx* ctx) {
     return it == ctx->bufs.end() ? nullptr : (T*)it->second.p;
 }
 
-template <typename T>
-int krylov_run(rmhmc_ctx* ctx, const T* b, double sigma0, double tol, int maxit, KrylovResult& out, cudaStream_t st) {
+template <typename T, typename TI>
+int krylov_run(rmhmc_ctx* ctx, const TI* b, double sigma0, double tol, int maxit, KrylovResult& out, cudaStream_t st) {
     if (maxit < 1) return set_err(ctx, RMHMC_EINVAL, "maxiter must be >= 1");
     if (!(sigma0 > 0.0)) return set_err(ctx, RMHMC_EINVAL, "shifts must be > 0");
     maxit = std::min(maxit, kBasisCap);
@@ -518,7 +547,7 @@ int krylov_run(rmhmc_ctx* ctx, const T* b, double sigma0, double tol, int maxit,
     const int nb = capped_grid(ctx, nvec, kBlock);
     StencilShape shp;
     RM_TRY(cg_shape<T>(ctx, st, shp));
-    k_cg_start<T><<<nb, kBlock, 0, st>>>(b, R, nvec, w.flags, w.vals, red_slot_partials(ctx, kSlotRho),
+    k_cg_start<T, TI><<<capped_grid(ctx, fs / 4, kBlock), kBlock, 0, st>>>(b, R, ctx->g.V, w.flags, w.vals, red_slot_partials(ctx, kSlotRho),
                                          red_slot_counter(ctx, kSlotRho)); ++ctx->launches;
     RM_LAUNCH_CHECK(ctx);
     typename LinksOf<T>::type U;
@@ -637,8 +666,9 @@ int resid64(rmhmc_ctx* ctx, const double* b, const double* x, int nf, const doub
     return RMHMC_OK;
 }
 
-template int krylov_run<float>(rmhmc_ctx*, const float*, double, double, int, KrylovResult&, cudaStream_t);
-template int krylov_run<double>(rmhmc_ctx*, const double*, double, double, int, KrylovResult&, cudaStream_t);
+template int krylov_run<float, float>(rmhmc_ctx*, const float*, double, double, int, KrylovResult&, cudaStream_t);
+template int krylov_run<float, double>(rmhmc_ctx*, const double*, double, double, int, KrylovResult&, cudaStream_t);
+template int krylov_run<double, double>(rmhmc_ctx*, const double*, double, double, int, KrylovResult&, cudaStream_t);
 template float* krylov_basis<float>(rmhmc_ctx*);
 template double* krylov_basis<double>(rmhmc_ctx*);
 template int krylov_combine<float, float>(rmhmc_ctx*, const CombineSpec&, float* const*, cudaStream_t);
@@ -708,12 +738,9 @@ int solve_shifts(rmhmc_ctx* ctx, const MassTerm& m, const double* b, double tol,
     {
         KrylovResult kr;
         if (mixed) {
-            float* b32 = (float*)workspace(ctx, "ss_b32", fs * sizeof(float), &status);
-            if (!b32) return status;
-            RM_TRY(to_float(ctx, b, b32, fs, st));
-            RM_TRY(krylov_run<float>(ctx, b32, s0, std::max(0.5 * tol, floor32), maxiter, kr, st));
+            RM_TRY((krylov_run<float, double>(ctx, b, s0, std::max(0.5 * tol, floor32), maxiter, kr, st)));
         } else {
-            RM_TRY(krylov_run<double>(ctx, b, s0, 0.5 * tol, maxiter, kr, st));
+            RM_TRY((krylov_run<double, double>(ctx, b, s0, 0.5 * tol, maxiter, kr, st)));
         }
         total += kr.n;
         Tridiag tri;
@@ -756,10 +783,10 @@ int solve_shifts(rmhmc_ctx* ctx, const MassTerm& m, const double* b, double tol,
             const double want = std::max(0.5 * tol / rel, 1e-15);
             KrylovResult kr;
             if (mixed) {
-                RM_TRY(krylov_run<float>(ctx, r32 + (size_t)j * fs, m.sigma[j], std::max(want, floor32), maxiter, kr,
-                                         st));
+                RM_TRY((krylov_run<float, float>(ctx, r32 + (size_t)j * fs, m.sigma[j], std::max(want, floor32), maxiter,
+                                                 kr, st)));
             } else {
-                RM_TRY(krylov_run<double>(ctx, r + (size_t)j * fs, m.sigma[j], want, maxiter, kr, st));
+                RM_TRY((krylov_run<double, double>(ctx, r + (size_t)j * fs, m.sigma[j], want, maxiter, kr, st)));
             }
             total += kr.n;
             Tridiag tri;
@@ -891,24 +918,13 @@ int heatbath_apply(rmhmc_ctx* ctx, const MassTerm& m, const double* xi, double t
 // ------------------------------------------------------------------------------------------------
 // graph-capturable kinetic evaluation: every decision on the device
 // ------------------------------------------------------------------------------------------------
-// r_0 = b, rho_0; arms the conditional of the CG loop (1 unless b = 0)
-template <typename T>
-__global__ void __launch_bounds__(kBlock) k_cgg_start(const T* __restrict__ b, T* __restrict__ r0, size_t nvec,
-                                                      int* flags, double* rho, double* partials, unsigned* counter,
+// as k_cg_start from float64 momenta; arms the conditional of the CG loop (1 unless b = 0)
+__global__ void __launch_bounds__(kBlock) k_cgg_start(const double* __restrict__ b, float* __restrict__ r0, int V, int* flags,
+                                                      double* rho, double* partials, unsigned* counter,
                                                       cudaGraphConditionalHandle h) {
     __shared__ double sh[kBlock / 32];
-    using VT = Vec<T>;
     if (blockIdx.x == 0 && threadIdx.x == 0) flags[2] = 0;   // pass counter of the guard in k_cgg_B
-    double acc = 0.0;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nvec; i += (size_t)gridDim.x * blockDim.x) {
-        const typename VT::type v = reinterpret_cast<const typename VT::type*>(b)[i];
-        reinterpret_cast<typename VT::type*>(r0)[i] = v;
-        T x[VT::n];
-        VT::get(v, x);
-#pragma unroll
-        for (int k = 0; k < VT::n; k++) acc += (double)x[k] * (double)x[k];
-    }
-    double v[1] = {acc};
+    double v[1] = {start_pass(b, r0, V)};
     block_sum<1>(v, sh);
     double out[1];
     if (grid_sum_finish<1>(v, partials, counter, out, gridDim.x, blockIdx.x, sh)) {
@@ -1082,7 +1098,6 @@ int capture_while(rmhmc_ctx* ctx, cudaStream_t st, cudaGraphConditionalHandle h,
 
 // buffers of the captured kinetic evaluation (allocated before any capture)
 struct KinGraphBufs {
-    float* P32 = nullptr;
     float* R = nullptr;
     float* q = nullptr;
     int* flags = nullptr;
@@ -1097,14 +1112,13 @@ static int kin_graph_bufs(rmhmc_ctx* ctx, int ns, int maxit, KinGraphBufs& b) {
     int status = RMHMC_OK;
     const size_t fs = field_elems(ctx);
     b.maxit = std::min(maxit, kBasisCap);
-    b.P32 = (float*)workspace(ctx, "kg_p32", sizeof(float) * fs, &status);
     b.R = (float*)workspace(ctx, "kr_basis32", sizeof(float) * fs * (size_t)(kBasisCap + 1), &status);
     b.q = (float*)workspace(ctx, "kg_q32", sizeof(float) * fs, &status);
     void* sc = workspace(ctx, "kg_scal", 64 + sizeof(double) * 4 * (size_t)(kBasisCap + 2), &status);
     b.rows = (double*)workspace(ctx, "kg_rows", sizeof(double) * kBasisCap * (size_t)(2 * ns + 1), &status);
     b.work = (double*)workspace(ctx, "kg_work", sizeof(double) * kBasisCap * (size_t)(3 * ns + 1), &status);
     b.pairs = (double*)workspace(ctx, "kf_pairs", sizeof(double) * kBasisCap * kBasisCap, &status);
-    if (!b.P32 || !b.R || !b.q || !sc || !b.rows || !b.work || !b.pairs) return status;
+    if (!b.R || !b.q || !sc || !b.rows || !b.work || !b.pairs) return status;
     b.flags = (int*)sc;
     b.vals = (double*)((char*)sc + 64);
     return RMHMC_OK;
@@ -1140,11 +1154,11 @@ int kinetic_enqueue(rmhmc_ctx* ctx, const MassTerm& m, const double* P, double t
         dm.alpha[j] = m.alpha[j];
         dm.delta[j] = m.sigma[j] - s0;
     }
-    RM_TRY(to_float(ctx, P, b.P32, fs, st));
     cudaGraphConditionalHandle h;
     RM_TRY(capture_handle(ctx, st, 0u, &h));
-    k_cgg_start<float><<<nb, kBlock, 0, st>>>(b.P32, b.R, nvec, b.flags, b.vals, red_slot_partials(ctx, kSlotRho),
-                                              red_slot_counter(ctx, kSlotRho), h); ++ctx->launches;
+    k_cgg_start<<<capped_grid(ctx, fs / 4, kBlock), kBlock, 0, st>>>(P, b.R, ctx->g.V, b.flags, b.vals,
+                                                                     red_slot_partials(ctx, kSlotRho),
+                                                                     red_slot_counter(ctx, kSlotRho), h); ++ctx->launches;
     RM_LAUNCH_CHECK(ctx);
     cudaGraph_t body;
     RM_TRY(capture_while(ctx, st, h, &body));
@@ -1166,14 +1180,18 @@ int kinetic_enqueue(rmhmc_ctx* ctx, const MassTerm& m, const double* P, double t
         RM_CHECK(ctx, cudaStreamEndCapture(aux, &tmp));
     }
     k_lanczos_rows<<<1, 128, 0, st>>>(b.flags, b.vals, b.maxit, dm, b.rows, b.work, status); ++ctx->launches;
-    const int grid = capped_grid(ctx, fs / 4, kBlock);
-    OutPtrs<float, double> ov{};
-    ov.p[0] = Vel;
-    k_combine<float, double, 1><<<grid, kBlock, 0, st>>>(b.R, fs, b.flags, 0, b.rows + (size_t)2 * ns * kBasisCap,
-                                                         kBasisCap, 1, ov);
-    ++ctx->launches;
     RM_LAUNCH_CHECK(ctx);
-    return link_grad_krylov_launch(ctx, b.R, b.rows, kBasisCap, ns, m.alpha.data(), b.flags, 0, F, st);
+    const double* cvel = b.rows + (size_t)2 * ns * kBasisCap;
+    if (ctx->lg_mode != kLgFused) {
+        OutPtrs<float, double> ov{};
+        ov.p[0] = Vel;
+        k_combine<float, double, 1><<<capped_grid(ctx, fs / 4, kBlock), kBlock, 0, st>>>(b.R, fs, b.flags, 0, cvel,
+                                                                                        kBasisCap, 1, ov);
+        ++ctx->launches;
+        RM_LAUNCH_CHECK(ctx);
+    }
+    return link_grad_krylov_launch(ctx, b.R, b.rows, kBasisCap, ns, m.alpha.data(), b.flags, 0, F, cvel, Vel, nullptr,
+                                   kSlotNorm, st);
 }
 
 }  // namespace rm

@@ -46,9 +46,10 @@ struct Tridiag {
     void to_basis(const std::vector<double>& y, double* coef_row) const;
 };
 
-// run CG on (A + sigma0) x = b; b (internal precision, [V][4][8]) is copied into basis slot 0
-template <typename T>
-int krylov_run(rmhmc_ctx* ctx, const T* b, double sigma0, double tol, int maxit, KrylovResult& out, cudaStream_t st);
+// run CG in T on (A + sigma0) x = b; b ([V][4][8], T or float64) is rounded to T into basis slot 0.  The basis and q
+// are chunk-planar (common.cuh); combinations of them come out as [V][4][8]
+template <typename T, typename TI>
+int krylov_run(rmhmc_ctx* ctx, const TI* b, double sigma0, double tol, int maxit, KrylovResult& out, cudaStream_t st);
 // basis pointer of the last run
 template <typename T> T* krylov_basis(rmhmc_ctx* ctx);
 // out[m] = sum_k coef[m][k] r_k for m < M (outputs as float or double)

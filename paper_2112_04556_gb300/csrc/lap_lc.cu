@@ -84,7 +84,7 @@ __device__ __forceinline__ float quad_transpose_sum(const float (&f)[4], int nu)
 }
 
 // MODE 0: Y = a X + b H(X).  MODE 1: q = a r + b H(r) + beta q_old (k > 0), gamma = <r, q> (CG stencil;
-// X = r_k is basis vector k of R, flags/vals as in k_cg_A)
+// X = r_k is basis vector k of R and q, both chunk-planar; flags/vals as in k_cg_A)
 template <int LF, int MODE>
 __global__ void __launch_bounds__(kLcThreads, 1) k_lap_lc(Geom g, LcGeom lg, Links32 U, const float* __restrict__ Xin,
                                                           float* __restrict__ Y, float a, float b, size_t fs,
@@ -106,6 +106,11 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lap_lc(Geom g, LcGeom lg, Lin
         if (k > 0) beta = (float)vals[(maxit + 1) + 2 * maxit + (k - 1)];
     }
     const int tid = threadIdx.x, s = tid >> 2, nu = tid & 3;
+    // component m of the field at a site
+    auto load_x = [&](int site, int m, float* x) {
+        if (MODE == 1) load_plane8(X, g.V, site, m, x);
+        else load8(X + (size_t)site * 32 + m * 8, x);
+    };
     // box and t-range of this block
     int bi = blockIdx.x;
     const int tr = bi % lg.nt; bi /= lg.nt;
@@ -162,7 +167,9 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lap_lc(Geom g, LcGeom lg, Lin
         for (int idx = tid; idx < kLcSlots * 8; idx += kLcThreads) {
             const int sl = idx >> 3, c = idx & 7;
             const int v = slot_xyz[sl];
-            if (v >= 0) cp_async16(dst + sl * kLcRow + c * 4, X + ((size_t)v + (size_t)t * slice) * 32 + c * 4);
+            if (v < 0) continue;
+            const int site = v + t * slice;
+            cp_async16(dst + sl * kLcRow + c * 4, MODE == 1 ? plane_at(X, g.V, site, c) : X + (size_t)site * 32 + c * 4);
         }
     };
     // this thread's site (dead threads of a partial box compute on site 0 and store nothing)
@@ -208,7 +215,7 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lap_lc(Geom g, LcGeom lg, Lin
         const int m = nu;   // component of the t-halo task
         const mat3<float> u = LinkLoad<float, LF>::load(U, xyz + tp * slice, 3);
         float xm[8];
-        load8(X + ((size_t)xyz + (size_t)tp * slice) * 32 + m * 8, xm);
+        load_x(xyz + tp * slice, m, xm);
         float Bm[8];
 #pragma unroll
         for (int c = 0; c < 8; c++) Bm[c] = 0.f;
@@ -229,7 +236,7 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lap_lc(Geom g, LcGeom lg, Lin
     if (nu == 3) {
         const int tn = t0 + 1 == Lt ? 0 : t0 + 1;
 #pragma unroll
-        for (int m = 0; m < 4; m++) load8(X + ((size_t)xyz + (size_t)tn * slice) * 32 + m * 8, xf[m]);
+        for (int m = 0; m < 4; m++) load_x(xyz + tn * slice, m, xf[m]);
     }
     cp_async_wait_all();
     __syncthreads();
@@ -307,14 +314,14 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lap_lc(Geom g, LcGeom lg, Lin
         // ---- epilogue for component mu = nu; the next slice's links (and X(x, t+2) for nu = t) are loaded first
         const int x = xyz + t * slice;
         float qo[8];
-        if (MODE == 1 && k > 0 && live) load8(Y + (size_t)x * 32 + nu * 8, qo);
+        if (MODE == 1 && k > 0 && live) load_plane8((const float*)Y, g.V, x, nu, qo);
         if (t + 1 < t1) {
             u = LinkLoad<float, LF>::load(U, xyz + (t + 1) * slice, nu);
             if (has_halo) uh = LinkLoad<float, LF>::load(U, h_xyz + (t + 1) * slice, h_d);
             if (nu == 3) {
                 const int tn = t + 2 >= Lt ? t + 2 - Lt : t + 2;
 #pragma unroll
-                for (int m = 0; m < 4; m++) load8(X + ((size_t)xyz + (size_t)tn * slice) * 32 + m * 8, xf[m]);
+                for (int m = 0; m < 4; m++) load_x(xyz + tn * slice, m, xf[m]);
             }
         }
         if (live) {
@@ -335,7 +342,12 @@ __global__ void __launch_bounds__(kLcThreads, 1) k_lap_lc(Geom g, LcGeom lg, Lin
 #pragma unroll
                 for (int c = 0; c < 8; c++) dot = fmaf(xs[c], y[c], dot);
             }
-            store8(Y + (size_t)x * 32 + m * 8, y);
+            if (MODE == 1) {
+                store4(plane_at(Y, g.V, x, 2 * m), y);
+                store4(plane_at(Y, g.V, x, 2 * m + 1), y + 4);
+            } else {
+                store8(Y + (size_t)x * 32 + m * 8, y);
+            }
         }
         __syncthreads();
     }

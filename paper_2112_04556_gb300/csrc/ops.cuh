@@ -37,7 +37,11 @@ int link_update_launch(rmhmc_ctx* ctx, const double* Uin, const double* V, doubl
 // kinetic force G = sum_j alpha_j d<Z_j, A X_j>/dw straight from the float32 Krylov basis R (n vectors), with
 // X_j, Z_j given as rows of basis coefficients (rows j and ns + j, row stride ldr, device float64); n is
 // read on the device from flags[1] when flags is not null.  G float64 [V][4][8].
+// With cvel, cen (coefficients on the basis) the velocity sum_k cvel[k] r_k goes to Vel and |sum_k cen[k] r_k|^2 to the
+// reduction slot in the same pass, if that kernel is selected (ctx->lg_mode == kLgFused; the other one computes G only).
+constexpr int kLgFused = 4;
 int link_grad_krylov_launch(rmhmc_ctx* ctx, const float* R, const double* rows, int ldr, int ns, const double* alpha,
-                            const int* flags, int n, double* G, cudaStream_t st);
+                            const int* flags, int n, double* G, const double* cvel, double* Vel, const double* cen,
+                            int slot, cudaStream_t st);
 
 }  // namespace rm

@@ -94,27 +94,11 @@ template <typename T> struct SrcField {
     __device__ __forceinline__ void operator()(int s, int mu, T* x) const { load8(X + (size_t)s * 32 + mu * 8, x); }
 };
 
-// plain float32 field of the context's own (32-byte aligned, read-only during the kernel) buffers, read with
-// 256-bit loads
-struct SrcFieldV8 {
-    const float* X;
-    __device__ __forceinline__ void operator()(int s, int mu, float* x) const { load8_v8(X + (size_t)s * 32 + mu * 8, x); }
-};
-
-// fused source r + beta * p (conjugate-gradient search direction)
-template <typename T> struct SrcAxpy {
-    const T* r;
-    const T* p;
-    T beta;
-    __device__ __forceinline__ void operator()(int s, int mu, T* x) const {
-        load8(r + (size_t)s * 32 + mu * 8, x);
-        if (p) {
-            T y[8];
-            load8(p + (size_t)s * 32 + mu * 8, y);
-#pragma unroll
-            for (int a = 0; a < 8; a++) x[a] = fma(beta, y[a], x[a]);
-        }
-    }
+// Krylov vector (chunk-planar)
+template <typename T> struct SrcPlanar {
+    const T* X;
+    int V;
+    __device__ __forceinline__ void operator()(int s, int mu, T* x) const { load_plane8(X, V, s, mu, x); }
 };
 
 }  // namespace rm

@@ -162,3 +162,37 @@ def test_staged_contraction_matches_global(L):
         _, ref, _ = oracle.kinetic(L, U, P, m, tol=1e-13)
         for mode in (0, 1, 2, 3):
             assert rel_l2(out[(mode, 1e-9)], ref) <= 1e-5
+
+
+@pytest.mark.parametrize("L", [(8, 6, 4, 10), (5, 3, 4, 7), (2, 2, 3, 2), (33, 2, 3, 2)])
+@pytest.mark.parametrize("smooth,tol", [(False, 1e-2), (False, 3e-7), (False, 1e-9), (True, 1e-6)])
+def test_fused_contraction_matches_separate(L, smooth, tol):
+    """Force, velocity and energy from the fused pass over the Krylov basis (kernel 4) against the contraction and the
+    combinations on their own (kernel 0), for runs of a few vectors up to several blocks of 20 (smooth links and
+    poles down to 1e-3), on ragged tiles of 32 sites; fields that are only 8-byte aligned give the same values.
+    A force is a sum of products of 4 n pairs in either order: 2 sqrt(4 n) 2^-24 < 2e-6 for n <= 160."""
+    import paper_2112_04556_gb300 as rm
+    torch = torch_cuda()
+    U = inputs.random_links(L, eps=0.05 if smooth else 0.4, seed=43)
+    P = inputs.gaussian_fields(L, 1, seed=44)[0]
+    lam = (np.arange(64) + 0.5) / 64
+    m = rm.mass_fit_spectrum(lam, lam, 12, 1e-3, 10.0) if smooth else fit.mass_term(12, 0.9)
+    out = {}
+    with rm.Context(L) as ctx:
+        Ud, Pd = dev(U), dev(P)
+        for mode, block in ((0, 128), (4, 256)):
+            rm.set_stencil_shape(ctx, rm.SHAPE_KFORCE, rm.FP32, 18, mode, block)
+            F, V, T = rm.kinetic_force(ctx, Ud, Pd, m, tol=tol, prec=rm.MIXED)
+            out[mode] = host(F), host(V), T
+        only = rm.kinetic_force(ctx, None, Pd, m, tol=tol, prec=rm.MIXED, want_velocity=False)[0]
+        assert np.array_equal(host(only), out[4][0])
+        odd = torch.empty(P.size + 1, dtype=torch.float64, device="cuda")[1:].view(Pd.shape)
+        assert odd.data_ptr() % 16 == 8
+        odd.copy_(Pd)
+        F, V, T = rm.kinetic_force(ctx, None, odd, m, tol=tol, prec=rm.MIXED)
+        assert np.array_equal(host(F), out[4][0]) and np.array_equal(host(V), out[4][1]) and T == out[4][2]
+        zero = rm.kinetic_force(ctx, None, torch.zeros_like(Pd), m, tol=tol, prec=rm.MIXED)
+        assert float(zero[0].abs().max()) == 0.0 and float(zero[1].abs().max()) == 0.0 and zero[2] == 0.0
+    assert rel_l2(out[4][0], out[0][0]) <= 2e-6
+    assert rel_l2(out[4][1], out[0][1]) <= 2e-6
+    assert abs(out[4][2] - out[0][2]) <= 2e-6 * abs(out[0][2])
