@@ -362,6 +362,8 @@ struct rmhmc_ctx {
     // z-extent of the multi-field adjoint kernel's slabs (rmhmc_set_stencil_shape, RMHMC_SHAPE_ADJOINT); 0 chosen
     // from the lattice and the field count
     int ad_slab = 0;
+    // set when the device refuses the cooperative CG run
+    bool cg_run_off = false;
     // incremented by every rmhmc_set_stencil_shape: part of the key of a captured trajectory graph
     int shape_gen = 0;
     std::string tune_report;

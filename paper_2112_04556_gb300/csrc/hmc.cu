@@ -1117,9 +1117,10 @@ static int md_graph_run(rmhmc_ctx* ctx, double* U, double* P, const rmhmc_params
     memcpy(st, ctx->h_pinned, sizeof st);
     memcpy(ints, (char*)ctx->h_pinned + 128, sizeof ints);
     *used = true;
-    // kernels the graph ran: 3 + 6 per step outside the loops, 7 per fixed-point iteration (8 with the velocity in a
-    // kernel of its own), 2 per Krylov iteration
-    ctx->launches += 3 + 6LL * p->nsteps + (ctx->lg_mode == kLgFused ? 7 : 8) * (st[1] + st[2]) + 2 * st[0];
+    // kernels the graph ran: 3 + 6 per step outside the loops, 6 per fixed-point iteration (7 with the velocity in a
+    // kernel of its own), 2 per Krylov iteration unless a run is one kernel
+    ctx->launches += 3 + 6LL * p->nsteps + (ctx->lg_mode == kLgFused ? 6 : 7) * (st[1] + st[2]) +
+                     (cg_run_fits<float>(ctx) ? 0 : 2 * st[0]);
     ctx->krylov_iters += st[0];
     ctx->links_valid = true;
     if (r) {
@@ -1132,6 +1133,9 @@ static int md_graph_run(rmhmc_ctx* ctx, double* U, double* P, const rmhmc_params
     switch (ints[0]) {
         case 0: return RMHMC_OK;
         case 1: return set_err(ctx, RMHMC_ENOCONV, "MD graph: a Krylov run hit its iteration cap");
+        case 5:
+            RM_TRY(cg_run_reset(ctx, stream));
+            return set_err(ctx, RMHMC_ETIMEOUT, "MD graph: a grid barrier of a Krylov run gave up");
         case 3: return set_err(ctx, RMHMC_ENOCONV, "MD graph: a fixed point did not converge in %d iterations", p->fp_maxit);
         default: return set_err(ctx, RMHMC_ENAN, "MD graph: NaN/Inf");
     }

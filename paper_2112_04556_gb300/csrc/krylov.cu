@@ -544,58 +544,74 @@ int krylov_run(rmhmc_ctx* ctx, const TI* b, double sigma0, double tol, int maxit
     const size_t fs = field_elems(ctx);
     const size_t nvec = fs / Vec<T>::n;
     T* R = (T*)w.basis;
-    const int nb = capped_grid(ctx, nvec, kBlock);
-    StencilShape shp;
-    RM_TRY(cg_shape<T>(ctx, st, shp));
-    k_cg_start<T, TI><<<capped_grid(ctx, fs / 4, kBlock), kBlock, 0, st>>>(b, R, ctx->g.V, w.flags, w.vals, red_slot_partials(ctx, kSlotRho),
-                                         red_slot_counter(ctx, kSlotRho)); ++ctx->launches;
-    RM_LAUNCH_CHECK(ctx);
-    typename LinksOf<T>::type U;
-    if constexpr (sizeof(T) == 8) U = links64(ctx); else U = links32(ctx);
-    const T diag = (T)(0.5 + sigma0);
     const double tol2 = tol * tol;
-    // iteration count of the previous run of the same operator and tolerance: the first chunk of launches
-    // covers it, so a converged run usually stops after one host check
+    int* hflags = (int*)(ctx->h_pinned + kPinned - 16);
     char key[96];
     snprintf(key, sizeof key, "%d:%.17g:%.17g:%d", (int)sizeof(T), sigma0, tol, maxit);
-    int& pred = ctx->kr_pred[key];
-    int* hflags = (int*)(ctx->h_pinned + kPinned - 16);
-    cudaEvent_t* ev = ctx->kr_ev;
-    int launched = 0, chunk = 0;
-    bool stop = false;
-    while (launched < maxit && !stop) {
-        const int len = chunk == 0 ? (pred > 0 ? pred : kCheckChunk) : kCheckChunk / 2;
-        const int k1 = std::min(maxit, launched + len);
-        for (int k = launched; k < k1; k++) {
-            const bool timed = ctx->prof && k < kProfEvents;
-            if (timed) RM_CHECK(ctx, cudaEventRecord(ctx->prof_ev[2 * k], st));
-            // the solver streams 18-real links, in the tuned launch shape
-            RM_TRY(cg_stencil<T>(ctx, shp, U, R, fs, (T*)w.q, diag, w.flags, w.vals, maxit, st));
-            if (timed) RM_CHECK(ctx, cudaEventRecord(ctx->prof_ev[2 * k + 1], st));
-            k_cg_B<T><<<nb, kBlock, 0, st>>>(R, fs, (const T*)w.q, nvec, w.flags, w.vals, maxit, tol2,
-                                             red_slot_partials(ctx, kSlotRho), red_slot_counter(ctx, kSlotRho)); ++ctx->launches;
-        }
-        launched = k1;
-        RM_LAUNCH_CHECK(ctx);
-        const int slot = chunk & 1;
-        RM_CHECK(ctx, cudaMemcpyAsync(hflags + 2 * slot, w.flags, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
-        RM_CHECK(ctx, cudaEventRecord(ev[slot], st));
-        if (chunk == 0) {
-            // the predicted length: check at once
-            RM_CHECK(ctx, cudaEventSynchronize(ev[slot]));
-            if (hflags[2 * slot] != 0) stop = true;
-        } else if (chunk > 1) {
-            // inspect the previous chunk's flags while this chunk runs
-            RM_CHECK(ctx, cudaEventSynchronize(ev[slot ^ 1]));
-            if (hflags[2 * (slot ^ 1)] != 0) stop = true;
-        }
-        chunk++;
+    bool done = false;
+    if (cg_run_fits<T>(ctx)) {
+        RM_TRY((cg_run_launch<T, TI>(ctx, b, R, 0.5 + sigma0, w.flags, w.vals, maxit, tol2, nullptr, st)));
+        done = !ctx->cg_run_off;
     }
-    RM_CHECK(ctx, cudaMemcpyAsync(hflags, w.flags, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
-    RM_CHECK(ctx, cudaStreamSynchronize(st));
-    out.status = hflags[0];
-    out.n = hflags[1];
-    pred = out.n;
+    if (!done) {
+        const int nb = capped_grid(ctx, nvec, kBlock);
+        StencilShape shp;
+        RM_TRY(cg_shape<T>(ctx, st, shp));
+        k_cg_start<T, TI><<<capped_grid(ctx, fs / 4, kBlock), kBlock, 0, st>>>(b, R, ctx->g.V, w.flags, w.vals, red_slot_partials(ctx, kSlotRho),
+                                             red_slot_counter(ctx, kSlotRho)); ++ctx->launches;
+        RM_LAUNCH_CHECK(ctx);
+        typename LinksOf<T>::type U;
+        if constexpr (sizeof(T) == 8) U = links64(ctx); else U = links32(ctx);
+        const T diag = (T)(0.5 + sigma0);
+        // iteration count of the previous run of the same operator and tolerance: the first chunk of launches
+        // covers it, so a converged run usually stops after one host check
+        const int pred = ctx->kr_pred[key];
+        cudaEvent_t* ev = ctx->kr_ev;
+        int launched = 0, chunk = 0;
+        bool stop = false;
+        while (launched < maxit && !stop) {
+            const int len = chunk == 0 ? (pred > 0 ? pred : kCheckChunk) : kCheckChunk / 2;
+            const int k1 = std::min(maxit, launched + len);
+            for (int k = launched; k < k1; k++) {
+                const bool timed = ctx->prof && k < kProfEvents;
+                if (timed) RM_CHECK(ctx, cudaEventRecord(ctx->prof_ev[2 * k], st));
+                // the solver streams 18-real links, in the tuned launch shape
+                RM_TRY(cg_stencil<T>(ctx, shp, U, R, fs, (T*)w.q, diag, w.flags, w.vals, maxit, st));
+                if (timed) RM_CHECK(ctx, cudaEventRecord(ctx->prof_ev[2 * k + 1], st));
+                k_cg_B<T><<<nb, kBlock, 0, st>>>(R, fs, (const T*)w.q, nvec, w.flags, w.vals, maxit, tol2,
+                                                 red_slot_partials(ctx, kSlotRho), red_slot_counter(ctx, kSlotRho)); ++ctx->launches;
+            }
+            launched = k1;
+            RM_LAUNCH_CHECK(ctx);
+            const int slot = chunk & 1;
+            RM_CHECK(ctx, cudaMemcpyAsync(hflags + 2 * slot, w.flags, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
+            RM_CHECK(ctx, cudaEventRecord(ev[slot], st));
+            if (chunk == 0) {
+                // the predicted length: check at once
+                RM_CHECK(ctx, cudaEventSynchronize(ev[slot]));
+                if (hflags[2 * slot] != 0) stop = true;
+            } else if (chunk > 1) {
+                // inspect the previous chunk's flags while this chunk runs
+                RM_CHECK(ctx, cudaEventSynchronize(ev[slot ^ 1]));
+                if (hflags[2 * (slot ^ 1)] != 0) stop = true;
+            }
+            chunk++;
+        }
+    }
+    // flags and rho[0..n], alpha[0..n-1], beta[0..n-1] in one transfer of the scalar block (flags, 64 bytes; values)
+    const int nvals = (maxit + 1) + 3 * maxit;
+    if (nvals > kPinned - 64) return set_err(ctx, RMHMC_EINVAL, "Krylov run too long for the staging area");
+    std::vector<double> buf(8 + nvals);
+    RM_TRY(fetch(ctx, (const double*)w.flags, buf.data(), 8 + nvals, st));
+    int f[2];
+    memcpy(f, buf.data(), sizeof f);
+    out.status = f[0];
+    out.n = f[1];
+    if (out.status == 4) {
+        RM_TRY(cg_run_reset(ctx, st));
+        return set_err(ctx, RMHMC_ETIMEOUT, "Krylov run: a grid barrier gave up");
+    }
+    if (!done) ctx->kr_pred[key] = out.n;
     ctx->krylov_iters += out.n;
     if (ctx->prof) {
         // durations of the stencil launches that did work (iterations 0 .. n-1)
@@ -608,14 +624,10 @@ int krylov_run(rmhmc_ctx* ctx, const TI* b, double sigma0, double tol, int maxit
     }
     if (out.status == 0) out.status = 2;   // ran out of iterations without a flag (maxit reached)
     const int n = out.n;
-    // rho[0..n], alpha[0..n-1], beta[0..n-1] in one transfer of the scalar block
-    const int nvals = (maxit + 1) + 3 * maxit;
-    if (nvals > kPinned - 64) return set_err(ctx, RMHMC_EINVAL, "Krylov run too long for the staging area");
-    std::vector<double> buf(nvals);
-    RM_TRY(fetch(ctx, w.vals, buf.data(), nvals, st));
-    out.rho.assign(buf.begin(), buf.begin() + n + 1);
-    out.alpha.assign(buf.begin() + (maxit + 1) + maxit, buf.begin() + (maxit + 1) + maxit + n);
-    out.beta.assign(buf.begin() + (maxit + 1) + 2 * maxit, buf.begin() + (maxit + 1) + 2 * maxit + n);
+    const double* v = buf.data() + 8;
+    out.rho.assign(v, v + n + 1);
+    out.alpha.assign(v + (maxit + 1) + maxit, v + (maxit + 1) + maxit + n);
+    out.beta.assign(v + (maxit + 1) + 2 * maxit, v + (maxit + 1) + 2 * maxit + n);
     if (out.status == 3) return set_err(ctx, RMHMC_ENAN, "NaN/Inf in the Krylov recurrence");
     return RMHMC_OK;
 }
@@ -1017,7 +1029,7 @@ __global__ void __launch_bounds__(128) k_lanczos_rows(const int* __restrict__ fl
     const double* rho = vals;
     const double* alpha = vals + (maxit + 1) + maxit;
     const double* beta = alpha + maxit;
-    if (threadIdx.x == 0 && flags[0] >= 2) atomicMax(status, flags[0] == 2 ? 1 : 2);
+    if (threadIdx.x == 0 && flags[0] >= 2) atomicMax(status, flags[0] == 2 ? 1 : flags[0] == 4 ? 5 : 2);
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
         d[k] = 1.0 / alpha[k] + (k > 0 ? beta[k - 1] / alpha[k - 1] : 0.0);
         e[k] = k < n - 1 ? -sqrt(beta[k]) / alpha[k] : 0.0;
@@ -1127,8 +1139,9 @@ static int kin_graph_bufs(rmhmc_ctx* ctx, int ns, int maxit, KinGraphBufs& b) {
 int kinetic_graph_prepare(rmhmc_ctx* ctx, const MassTerm& m, int maxiter) {
     KinGraphBufs b;
     RM_TRY(kin_graph_bufs(ctx, m.npole(), maxiter, b));
+    RM_TRY(cg_run_prepare(ctx));
     StencilShape shp;
-    return cg_shape<float>(ctx, 0, shp);
+    return cg_run_fits<float>(ctx) ? RMHMC_OK : cg_shape<float>(ctx, 0, shp);
 }
 
 // Enqueue (on a capturing stream) one mixed-precision kinetic evaluation at the context's links:
@@ -1143,9 +1156,6 @@ int kinetic_enqueue(rmhmc_ctx* ctx, const MassTerm& m, const double* P, double t
     RM_TRY(kin_graph_bufs(ctx, ns, maxiter, b));
     const size_t fs = field_elems(ctx);
     const size_t nvec = fs / 4;
-    const int nb = capped_grid(ctx, nvec, kBlock);
-    StencilShape shp;
-    RM_TRY(cg_shape<float>(ctx, st, shp));
     const double s0 = *std::min_element(m.sigma.begin(), m.sigma.end());
     DevMass dm{};
     dm.ns = ns;
@@ -1154,30 +1164,38 @@ int kinetic_enqueue(rmhmc_ctx* ctx, const MassTerm& m, const double* P, double t
         dm.alpha[j] = m.alpha[j];
         dm.delta[j] = m.sigma[j] - s0;
     }
-    cudaGraphConditionalHandle h;
-    RM_TRY(capture_handle(ctx, st, 0u, &h));
-    k_cgg_start<<<capped_grid(ctx, fs / 4, kBlock), kBlock, 0, st>>>(P, b.R, ctx->g.V, b.flags, b.vals,
-                                                                     red_slot_partials(ctx, kSlotRho),
-                                                                     red_slot_counter(ctx, kSlotRho), h); ++ctx->launches;
-    RM_LAUNCH_CHECK(ctx);
-    cudaGraph_t body;
-    RM_TRY(capture_while(ctx, st, h, &body));
-    {
-        RM_CHECK(ctx, cudaStreamBeginCaptureToGraph(aux, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
-        const Links32 U = links32(ctx);
-        const float diag = (float)(0.5 + s0);
-        const int cs = cg_stencil<float>(ctx, shp, U, b.R, fs, b.q, diag, b.flags, b.vals, b.maxit, aux);
-        if (cs != RMHMC_OK) {
-            cudaGraph_t tmp;
-            cudaStreamEndCapture(aux, &tmp);
-            return cs;
-        }
-        k_cgg_B<float><<<nb, kBlock, 0, aux>>>(b.R, fs, b.q, nvec, b.flags, b.vals, b.maxit, tol * tol,
-                                               red_slot_partials(ctx, kSlotRho), red_slot_counter(ctx, kSlotRho), h,
-                                               stats); ++ctx->launches;
+    if (cg_run_fits<float>(ctx)) {
+        RM_TRY((cg_run_launch<float, double>(ctx, P, b.R, 0.5 + s0, b.flags, b.vals, b.maxit, tol * tol, stats, st)));
+        if (ctx->cg_run_off) return set_err(ctx, RMHMC_ECUDA, "cooperative launch refused");
+    } else {
+        const int nb = capped_grid(ctx, nvec, kBlock);
+        StencilShape shp;
+        RM_TRY(cg_shape<float>(ctx, st, shp));
+        cudaGraphConditionalHandle h;
+        RM_TRY(capture_handle(ctx, st, 0u, &h));
+        k_cgg_start<<<capped_grid(ctx, fs / 4, kBlock), kBlock, 0, st>>>(P, b.R, ctx->g.V, b.flags, b.vals,
+                                                                         red_slot_partials(ctx, kSlotRho),
+                                                                         red_slot_counter(ctx, kSlotRho), h); ++ctx->launches;
         RM_LAUNCH_CHECK(ctx);
-        cudaGraph_t tmp;
-        RM_CHECK(ctx, cudaStreamEndCapture(aux, &tmp));
+        cudaGraph_t body;
+        RM_TRY(capture_while(ctx, st, h, &body));
+        {
+            RM_CHECK(ctx, cudaStreamBeginCaptureToGraph(aux, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
+            const Links32 U = links32(ctx);
+            const float diag = (float)(0.5 + s0);
+            const int cs = cg_stencil<float>(ctx, shp, U, b.R, fs, b.q, diag, b.flags, b.vals, b.maxit, aux);
+            if (cs != RMHMC_OK) {
+                cudaGraph_t tmp;
+                cudaStreamEndCapture(aux, &tmp);
+                return cs;
+            }
+            k_cgg_B<float><<<nb, kBlock, 0, aux>>>(b.R, fs, b.q, nvec, b.flags, b.vals, b.maxit, tol * tol,
+                                                   red_slot_partials(ctx, kSlotRho), red_slot_counter(ctx, kSlotRho), h,
+                                                   stats); ++ctx->launches;
+            RM_LAUNCH_CHECK(ctx);
+            cudaGraph_t tmp;
+            RM_CHECK(ctx, cudaStreamEndCapture(aux, &tmp));
+        }
     }
     k_lanczos_rows<<<1, 128, 0, st>>>(b.flags, b.vals, b.maxit, dm, b.rows, b.work, status); ++ctx->launches;
     RM_LAUNCH_CHECK(ctx);

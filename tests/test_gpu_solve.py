@@ -240,3 +240,29 @@ def test_cg_stencil_shapes(nmu, block):
         F2, Vel2, T2 = rm.kinetic_force(ctx, None, dev(b), m, tol=1e-7, prec=rm.MIXED)
     assert rel_l2(host(F), host(F2)) <= 1e-5 and rel_l2(host(Vel), host(Vel2)) <= 1e-5
     assert abs(T - T2) <= 1e-6 * abs(T2)
+
+
+@pytest.mark.parametrize("L", [(2, 2, 2, 2), (3, 3, 3, 3), (5, 3, 4, 7), (8, 8, 8, 9), (13, 11, 9, 17), (12, 12, 14, 16)])
+@pytest.mark.parametrize("prec,tol,bound", [(0, 1e-12, 1e-10), (1, 1e-10, 1e-9)])
+def test_cg_run_matches_two_kernel_form(L, prec, tol, bound):
+    """The cooperative Krylov run against the two-kernel form (a pinned CG stencil selects it): less than one unit
+    of 32 sites, ragged units, the changes of block shape (8 and 24 units an SM) and several rounds of units.  Both
+    solve to the same tolerance, so the sums differ by tol |b| / (smallest shift + gap), below ten times tol here; a
+    run that hits its cap reports ENOCONV and the next one is unaffected."""
+    import paper_2112_04556_gb300 as rm
+    U = inputs.random_links(L, eps=0.4, seed=31)
+    b = inputs.gaussian_fields(L, 1, seed=32)[0]
+    m = rm.mass_fit(12, 0.9)
+    with rm.Context(L) as ctx:
+        Ud, bd = dev(U), dev(b)
+        y, _, iters, resid = rm.rat_mass_solve(ctx, Ud, bd, m, tol=tol, prec=prec)
+        assert np.all(resid <= tol) and iters > 0
+        with pytest.raises(rm.RmhmcError) as e:
+            rm.rat_mass_solve(ctx, Ud, bd, m, tol=tol, maxiter=2, prec=prec)
+        assert e.value.code == rm.ENOCONV
+        again = rm.rat_mass_solve(ctx, Ud, bd, m, tol=tol, prec=prec)
+        assert again[2] == iters and np.array_equal(host(again[0]), host(y))   # a fixed order of every sum
+        rm.set_stencil_shape(ctx, rm.SHAPE_CG, rm.FP64 if prec == 0 else rm.FP32, 18, 1, 128)
+        y2, _, iters2, _ = rm.rat_mass_solve(ctx, None, bd, m, tol=tol, prec=prec)
+    assert rel_l2(host(y), host(y2)) <= bound
+    assert abs(iters - iters2) <= 2 + iters // 20
