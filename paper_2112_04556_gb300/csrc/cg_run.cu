@@ -176,10 +176,9 @@ __global__ void __launch_bounds__(BLOCK, 1)
         for (int u = u0; u < u1; u += wpb, q += 8 * blockDim.x) {
             const int s = u / 4 * 32 + lane, mu = u & 3;
             if (s >= g.V) continue;
-            herm<T> acc[1];
-            hop_sum_shape<T, 18, NMU>(g, U, s, mu, src, acc);
-            T h[8], x[8], y[8], o[8];
-            herm2_to_coef_tl(acc[0], h);
+            T hc[1][8], x[8], y[8], o[8];
+            hop_coefs<T, sizeof(T) == 8 ? kLinkAd : 18, NMU>(g, U, s, mu, src, hc);
+            const T(&h)[8] = hc[0];
             src(s, mu, x);
             if (k > 0) {
                 q_load(q, o);
@@ -280,20 +279,19 @@ int cg_run_prepare(rmhmc_ctx* ctx) {
 }
 
 template <typename T, typename TI>
-int cg_run_launch(rmhmc_ctx* ctx, const TI* b, T* R, double diag, int* flags, double* vals, int maxit, double tol2,
+int cg_run_launch(rmhmc_ctx* ctx, const typename LinksOf<T>::type& links, const TI* b, T* R, double diag, int* flags, double* vals, int maxit, double tol2,
                   long long* iters, cudaStream_t st) {
     const CgRunShape s = cg_run_shape<T>(ctx);
     RM_TRY(cg_run_prepare(ctx));
     unsigned* bar = (unsigned*)ctx->bufs["cg_run"].p;
     double* part = (double*)((char*)bar + 64);
-    typename LinksOf<T>::type U;
-    if constexpr (sizeof(T) == 8) U = links64(ctx); else U = links32(ctx);
+    typename LinksOf<T>::type U = links;
     Geom g = ctx->g;
     size_t fs = field_elems(ctx);
     T d = (T)diag;
     int units = s.units;
     void* args[] = {&g, &U, &b, &R, &fs, &d, &flags, &vals, &maxit, &tol2, &iters, &units, &part, &bar};
-    const void* kern = (const void*)k_cg_run<T, TI, 0, 256>;
+    const void* kern = (const void*)k_cg_run<T, TI, sizeof(T) == 8 ? 1 : 0, 256>;
     if constexpr (sizeof(T) == 4) {
         if (s.maxw == 24) kern = (const void*)k_cg_run<T, TI, 0, 768>;
         if (s.maxw == 16) kern = (const void*)k_cg_run<T, TI, 1, 512>;
@@ -313,8 +311,8 @@ int cg_run_launch(rmhmc_ctx* ctx, const TI* b, T* R, double diag, int* flags, do
 
 template bool cg_run_fits<float>(const rmhmc_ctx*);
 template bool cg_run_fits<double>(const rmhmc_ctx*);
-template int cg_run_launch<float, float>(rmhmc_ctx*, const float*, float*, double, int*, double*, int, double, long long*, cudaStream_t);
-template int cg_run_launch<float, double>(rmhmc_ctx*, const double*, float*, double, int*, double*, int, double, long long*, cudaStream_t);
-template int cg_run_launch<double, double>(rmhmc_ctx*, const double*, double*, double, int*, double*, int, double, long long*, cudaStream_t);
+template int cg_run_launch<float, float>(rmhmc_ctx*, const Links32&, const float*, float*, double, int*, double*, int, double, long long*, cudaStream_t);
+template int cg_run_launch<float, double>(rmhmc_ctx*, const Links32&, const double*, float*, double, int*, double*, int, double, long long*, cudaStream_t);
+template int cg_run_launch<double, double>(rmhmc_ctx*, const Links64&, const double*, double*, double, int*, double*, int, double, long long*, cudaStream_t);
 
 }  // namespace rm

@@ -99,7 +99,9 @@ __device__ __forceinline__ int shifted(const Geom& g, const int c[4], int d, int
 //   FP32: u32a[(mu*3 + r) * V + s]  float4, r=0: (u00,u01) r=1: (u02,u10) r=2: (u11,u12)
 //         u32b[(mu*3 + j) * V + s]  float2, u2j (third row; unused by the 12-real format)
 // ------------------------------------------------------------------------------------------------
-struct Links64 { const double2* u; int V; };
+//   FP64, adjoint table (link "format" kLinkAd): ad[(mu*32 + 4b + h) * V + s]  double2 (Ad[2h][b], Ad[2h+1][b])
+constexpr int kLinkAd = 64;
+struct Links64 { const double2* u; int V; const double2* ad; };
 struct Links32 { const float4* a; const float2* b; int V; };
 
 template <typename T, int LF> struct LinkLoad;
@@ -325,7 +327,9 @@ struct rmhmc_ctx {
     float2* u32b = nullptr;
     bool links_valid = false;
     unsigned long long link_gen = 1;   // bumped whenever the internal link copies change
-    unsigned long long adj_gen = 0;    // link_gen the adjoint table was built for
+    unsigned long long adj_gen = 0;    // link_gen the float32-pair adjoint table was built for
+    unsigned long long adj64_gen = 0;  // and the float64 one
+    bool adj64_off = false;            // no memory for the float64 one
     // reductions
     double* red_partials = nullptr;   // [kRedSlots][max_blocks * 2]
     unsigned* red_counters = nullptr; // [kRedSlots]
@@ -407,7 +411,11 @@ inline int capped_grid(const rmhmc_ctx* ctx, size_t threads, int block) {
     const size_t g = (need + passes - 1) / passes;
     return (int)std::min(cap, (g + sms - 1) / sms * sms);   // whole blocks per SM
 }
-inline Links64 links64(const rmhmc_ctx* ctx) { return Links64{ctx->u64, ctx->g.V}; }
+inline Links64 links64(const rmhmc_ctx* ctx) { return Links64{ctx->u64, ctx->g.V, nullptr}; }
+// the links with their float64 adjoint table, built if the links changed since; ad is null where a table is not used
+// (more than kAdTableMax sites, or no memory for it)
+constexpr int kAdTableMax = 1 << 22;   // 2 KB a site
+int links64_adjoint(rmhmc_ctx* ctx, Links64* U, cudaStream_t st);
 inline Links32 links32(const rmhmc_ctx* ctx) { return Links32{ctx->u32a, ctx->u32b, ctx->g.V}; }
 double* red_slot_partials(rmhmc_ctx* ctx, int slot);
 unsigned* red_slot_counter(rmhmc_ctx* ctx, int slot);

@@ -27,16 +27,22 @@ __device__ __forceinline__ dfl quick_two_sum(float a, float b) {
     return df_make(s, __fsub_rn(b, __fsub_rn(s, a)));
 }
 // float64-accurate running sum of squares in float32 arithmetic: the rounding errors of the products (fma) and of the
-// sum (TwoSum) are collected in c
+// sum (TwoSum) are collected in c; values whose squares leave float32's range go to a float64 sum
 struct SumSq32 {
     float s = 0.f, c = 0.f;
+    double d = 0.0;
     __device__ __forceinline__ void add(float x) {
+        const float m = fabsf(x);
+        if (!(m >= 0x1p-40f && m <= 0x1p40f)) {
+            d = fma((double)x, (double)x, d);
+            return;
+        }
         const float p = __fmul_rn(x, x), e = __fmaf_rn(x, x, -p);
         const dfl t = two_sum(s, p);
         s = t.hi;
         c = __fadd_rn(c, __fadd_rn(t.lo, e));
     }
-    __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+    __device__ __forceinline__ double value() const { return (double)s + (double)c + d; }
 };
 
 // Conversions between float64 and float pairs from the IEEE-754 bit fields, with integer operations and no
@@ -44,7 +50,7 @@ struct SumSq32 {
 // rounded to 24 significant bits (its 29 low significand bits dropped, rounding half away from zero, a carry
 // moving into the exponent), lo = the signed remainder (at most 2^28 units of x's last place) as a float times
 // 2^(e - 52); |lo| <= ulp(hi) / 2 and hi + lo = x to 2^-49 |x|.  |x| below 2^-126 gives 0 and |x|
-// near or above 2^128 gives +-inf (NaN too); lo is dropped for |x| < 2^-74 (an absolute error below 2^-98).
+// near or above 2^128 gives +-inf (NaN too); lo keeps what float32's subnormals hold of it.
 __device__ __forceinline__ dfl df_split(double x) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
@@ -60,6 +66,10 @@ __device__ __forceinline__ dfl df_split(double x) {
     if (e >= 949) {   // 2^(e - 1075) is a normal float
         const int r = up ? (int)m - (1 << 29) : (int)m;
         lo = __int2float_rn(r) * __uint_as_float((unsigned)(e - 948) << 23);
+        if (sign) lo = -lo;
+    } else {   // 2^(e - 1075) in two steps: lo may end among the subnormals
+        const int r = up ? (int)m - (1 << 29) : (int)m;
+        lo = __int2float_rn(r) * __uint_as_float((unsigned)(e - 884) << 23) * 0x1p-64f;
         if (sign) lo = -lo;
     }
     return df_make(hi, lo);

@@ -19,4 +19,16 @@ __device__ __forceinline__ void f_contract(int d, const T (&rc)[8], T (&G)[8]) {
     }
 }
 
+// the same by rows: G_a = sum_t v_t (RC[c_t][d_t] - RC[d_t][c_t]) over the triples that hold a
+struct FTerm { int c, d; double v; };
+__constant__ FTerm kFTerms[8][4] = {
+    {{1, 2, 1.0}, {3, 6, 0.5}, {4, 5, -0.5}, {0, 0, 0.0}},
+    {{2, 0, 1.0}, {3, 5, 0.5}, {4, 6, 0.5}, {0, 0, 0.0}},
+    {{0, 1, 1.0}, {3, 4, 0.5}, {5, 6, -0.5}, {0, 0, 0.0}},
+    {{6, 0, 0.5}, {5, 1, 0.5}, {4, 2, 0.5}, {4, 7, 0.86602540378443864676}},
+    {{5, 0, -0.5}, {6, 1, 0.5}, {2, 3, 0.5}, {7, 3, 0.86602540378443864676}},
+    {{0, 4, -0.5}, {1, 3, 0.5}, {6, 2, -0.5}, {6, 7, 0.86602540378443864676}},
+    {{0, 3, 0.5}, {1, 4, 0.5}, {2, 5, -0.5}, {7, 5, 0.86602540378443864676}},
+    {{3, 4, 0.86602540378443864676}, {5, 6, 0.86602540378443864676}, {0, 0, 0.0}, {0, 0, 0.0}}};
+
 }  // namespace rm

@@ -105,13 +105,13 @@ __global__ void __launch_bounds__(kBlockMax, (stencil_min_blocks<T, NMU>())) k_c
     for (int u = blockIdx.x * wpb + (threadIdx.x >> 5); u < nunit; u += gridDim.x * wpb) {
         const int s = u / NG * 32 + (threadIdx.x & 31), mu0 = (u % NG) * NC;
         if (s >= g.V) continue;
-        herm<T> acc[NC];
-        hop_sum_shape<T, LF, NMU>(g, U, s, mu0, SrcPlanar<T>{r, g.V}, acc);
+        T hc[NC][8];
+        hop_coefs<T, LF, NMU>(g, U, s, mu0, SrcPlanar<T>{r, g.V}, hc);
 #pragma unroll
         for (int m = 0; m < NC; m++) {
             const int mu = mu0 + m;
-            T h[8], x[8], y[8];
-            herm2_to_coef_tl(acc[m], h);
+            T x[8], y[8];
+            const T(&h)[8] = hc[m];
             load_plane8(r, g.V, s, mu, x);
             if (k > 0) {
                 load_plane8((const T*)q, g.V, s, mu, y);
@@ -149,24 +149,27 @@ __global__ void __launch_bounds__(kBlockMax, (stencil_min_blocks<T, NMU>())) k_c
     }
 }
 
-template <typename T, int NMU>
+template <typename T, int NMU, int LF = 18>
 static void launch_cg_A(rmhmc_ctx* ctx, const StencilShape& shp, typename LinksOf<T>::type U, T* R, size_t fs, T* q,
                         T diag, int* flags, double* vals, int maxit, cudaStream_t st) {
     // whole warps of 32 sites per group
     const size_t lanes = (size_t)((ctx->g.V + 31) / 32 * 32) * lanes_per_site(NMU);
-    k_cg_A<T, 18, NMU><<<std::min(capped_grid(ctx, lanes, shp.block), ctx->max_blocks * 2), shp.block, 0, st>>>(ctx->g, U, R, fs, q, diag, flags, vals, maxit,
+    k_cg_A<T, LF, NMU><<<std::min(capped_grid(ctx, lanes, shp.block), ctx->max_blocks * 2), shp.block, 0, st>>>(ctx->g, U, R, fs, q, diag, flags, vals, maxit,
                                                                       red_slot_partials(ctx, 0), red_slot_counter(ctx, 0));
     ++ctx->launches;
 }
 
 // the CG stencil in a tuned shape: 3x3 gather kernels (nmu 1, 2, 4, 0) or, in float32, the link-centric
-// adjoint kernel (nmu 8, lap_lc.cu)
+// adjoint kernel (nmu 8, lap_lc.cu); in float64 with an adjoint table, the table (one component per lane)
 template <typename T>
 static int cg_stencil(rmhmc_ctx* ctx, const StencilShape& shp, typename LinksOf<T>::type U, T* R, size_t fs, T* q, T diag,
                       int* flags, double* vals, int maxit, cudaStream_t st) {
     if constexpr (sizeof(T) == 4) {
         if (shp.nmu == 8)
             return launch_cg_lc(ctx, R, q, diag, flags, vals, maxit, red_slot_partials(ctx, 0), red_slot_counter(ctx, 0), st);
+    } else if (U.ad) {
+        launch_cg_A<T, 1, kLinkAd>(ctx, StencilShape{1, 128}, U, R, fs, q, diag, flags, vals, maxit, st);
+        return RMHMC_OK;
     }
     if (shp.nmu == 4) launch_cg_A<T, 4>(ctx, shp, U, R, fs, q, diag, flags, vals, maxit, st);
     else if (shp.nmu == 2) launch_cg_A<T, 2>(ctx, shp, U, R, fs, q, diag, flags, vals, maxit, st);
@@ -388,10 +391,9 @@ __global__ void __launch_bounds__(kBlock) k_resid64(Geom g, Links64 U, const dou
     double nrm = 0.0;
     for (int lane = blockIdx.x * blockDim.x + threadIdx.x; lane < g.V * 4; lane += gridDim.x * blockDim.x) {
         const int s = lane >> 2, mu = lane & 3;
-        herm<double> acc;
-        hop_sum1<double, LF>(g, U, s, mu, SrcField<double>{xf}, acc);
-        double h[8], xx[8], bb[8], y[8];
-        herm2_to_coef_tl(acc, h);
+        double hc[1][8], xx[8], bb[8], y[8];
+        hop_coefs<double, LF, 1>(g, U, s, mu, SrcField<double>{xf}, hc);
+        const double(&h)[8] = hc[0];
         load8(xf + (size_t)s * 32 + mu * 8, xx);
         load8(b + (size_t)s * 32 + mu * 8, bb);
 #pragma unroll
@@ -549,19 +551,28 @@ int krylov_run(rmhmc_ctx* ctx, const TI* b, double sigma0, double tol, int maxit
     char key[96];
     snprintf(key, sizeof key, "%d:%.17g:%.17g:%d", (int)sizeof(T), sigma0, tol, maxit);
     bool done = false;
-    if (cg_run_fits<T>(ctx)) {
-        RM_TRY((cg_run_launch<T, TI>(ctx, b, R, 0.5 + sigma0, w.flags, w.vals, maxit, tol2, nullptr, st)));
+    typename LinksOf<T>::type U;
+    bool run = cg_run_fits<T>(ctx);
+    if constexpr (sizeof(T) == 8) {
+        U = links64(ctx);
+        if (!ctx->tune.count(10818)) RM_TRY(links64_adjoint(ctx, &U, st));
+        run = run && U.ad;
+    } else {
+        U = links32(ctx);
+    }
+    if (run) {
+        RM_TRY((cg_run_launch<T, TI>(ctx, U, b, R, 0.5 + sigma0, w.flags, w.vals, maxit, tol2, nullptr, st)));
         done = !ctx->cg_run_off;
     }
     if (!done) {
         const int nb = capped_grid(ctx, nvec, kBlock);
         StencilShape shp;
-        RM_TRY(cg_shape<T>(ctx, st, shp));
+        bool shaped = true;
+        if constexpr (sizeof(T) == 8) shaped = !U.ad;
+        if (shaped) RM_TRY(cg_shape<T>(ctx, st, shp));
         k_cg_start<T, TI><<<capped_grid(ctx, fs / 4, kBlock), kBlock, 0, st>>>(b, R, ctx->g.V, w.flags, w.vals, red_slot_partials(ctx, kSlotRho),
                                              red_slot_counter(ctx, kSlotRho)); ++ctx->launches;
         RM_LAUNCH_CHECK(ctx);
-        typename LinksOf<T>::type U;
-        if constexpr (sizeof(T) == 8) U = links64(ctx); else U = links32(ctx);
         const T diag = (T)(0.5 + sigma0);
         // iteration count of the previous run of the same operator and tolerance: the first chunk of launches
         // covers it, so a converged run usually stops after one host check
@@ -668,9 +679,13 @@ int resid64(rmhmc_ctx* ctx, const double* b, const double* x, int nf, const doub
     if (!dsig) return status;
     RM_TRY(upload(ctx, dsig, sigma, sizeof(double) * nf, st));
     const dim3 grid(capped_grid(ctx, (size_t)ctx->g.V * 4, kBlock), nf);
-    k_resid64<18><<<grid, kBlock, 0, st>>>(ctx->g, links64(ctx), b, x, dsig, r, field_elems(ctx),
-                                           red_slot_partials(ctx, kSlotResid), red_slot_counter(ctx, kSlotResid),
-                                           red_slot_out(ctx, kSlotResid), (size_t)ctx->max_blocks * 2); ++ctx->launches;
+    Links64 U = links64(ctx);
+    RM_TRY(links64_adjoint(ctx, &U, st));
+    auto kern = U.ad ? k_resid64<kLinkAd> : k_resid64<18>;
+    kern<<<grid, kBlock, 0, st>>>(ctx->g, U, b, x, dsig, r, field_elems(ctx), red_slot_partials(ctx, kSlotResid),
+                                  red_slot_counter(ctx, kSlotResid), red_slot_out(ctx, kSlotResid),
+                                  (size_t)ctx->max_blocks * 2);
+    ++ctx->launches;
     RM_LAUNCH_CHECK(ctx);
     std::vector<double> tmp((size_t)nf * 8);
     RM_TRY(fetch(ctx, red_slot_out(ctx, kSlotResid), tmp.data(), nf * 8, st));
@@ -1165,7 +1180,7 @@ int kinetic_enqueue(rmhmc_ctx* ctx, const MassTerm& m, const double* P, double t
         dm.delta[j] = m.sigma[j] - s0;
     }
     if (cg_run_fits<float>(ctx)) {
-        RM_TRY((cg_run_launch<float, double>(ctx, P, b.R, 0.5 + s0, b.flags, b.vals, b.maxit, tol * tol, stats, st)));
+        RM_TRY((cg_run_launch<float, double>(ctx, links32(ctx), P, b.R, 0.5 + s0, b.flags, b.vals, b.maxit, tol * tol, stats, st)));
         if (ctx->cg_run_off) return set_err(ctx, RMHMC_ECUDA, "cooperative launch refused");
     } else {
         const int nb = capped_grid(ctx, nvec, kBlock);

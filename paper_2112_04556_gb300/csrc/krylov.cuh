@@ -59,8 +59,9 @@ constexpr int kCgRunMax32 = 1 << 18, kCgRunMax64 = 1 << 17;
 template <typename T> bool cg_run_fits(const rmhmc_ctx* ctx);
 int cg_run_prepare(rmhmc_ctx* ctx);
 int cg_run_reset(rmhmc_ctx* ctx, cudaStream_t st);
+template <typename T> struct LinksOf;
 template <typename T, typename TI>
-int cg_run_launch(rmhmc_ctx* ctx, const TI* b, T* R, double diag, int* flags, double* vals, int maxit, double tol2,
+int cg_run_launch(rmhmc_ctx* ctx, const typename LinksOf<T>::type& U, const TI* b, T* R, double diag, int* flags, double* vals, int maxit, double tol2,
                   long long* iters, cudaStream_t st);
 // basis pointer of the last run
 template <typename T> T* krylov_basis(rmhmc_ctx* ctx);

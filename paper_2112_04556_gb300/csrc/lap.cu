@@ -24,16 +24,15 @@ __global__ void __launch_bounds__(kBlockMax, (stencil_min_blocks<T, NMU>())) k_l
     const int nlane = g.V * LPS;
     for (int lane = blockIdx.x * blockDim.x + threadIdx.x; lane < nlane; lane += gridDim.x * blockDim.x) {
         const int s = lane / LPS, mu0 = (lane % LPS) * NC;
-        herm<T> acc[NC];
-        hop_sum_shape<T, LF, NMU>(g, U, s, mu0, SrcField<T>{Xf}, acc);
+        T hc[NC][8];
+        hop_coefs<T, LF, NMU>(g, U, s, mu0, SrcField<T>{Xf}, hc);
 #pragma unroll
         for (int m = 0; m < NC; m++) {
             const int mu = mu0 + m;
-            T h[8], x[8], y[8];
-            herm2_to_coef_tl(acc[m], h);
+            T x[8], y[8];
             load8(Xf + (size_t)s * 32 + mu * 8, x);
 #pragma unroll
-            for (int k = 0; k < 8; k++) y[k] = fma(b, h[k], a * x[k]);
+            for (int k = 0; k < 8; k++) y[k] = fma(b, hc[m][k], a * x[k]);
             if (HAS_W) {
                 T w[8];
                 load8(W + f * fstride + (size_t)s * 32 + mu * 8, w);
@@ -70,7 +69,7 @@ __global__ void __launch_bounds__(kBlockMax, (stencil_min_blocks<T, NMU>())) k_l
 }
 
 template <typename T, int LF, int NMU>
-static void launch_lap_shape(rmhmc_ctx* ctx, const StencilShape& shp, const T* X, T* Y, int nfield, double a, double b,
+static void launch_lap_shape(rmhmc_ctx* ctx, const StencilShape& shp, const typename LinksOf<T>::type& U, const T* X, T* Y, int nfield, double a, double b,
                              const T* W, double c, int slot, cudaStream_t st) {
     const dim3 grid(stencil_blocks(ctx, shp), nfield);
     const size_t fs = field_elems(ctx);
@@ -78,8 +77,6 @@ static void launch_lap_shape(rmhmc_ctx* ctx, const StencilShape& shp, const T* X
     double* part = slot >= 0 ? red_slot_partials(ctx, slot) : nullptr;
     unsigned* cnt = slot >= 0 ? red_slot_counter(ctx, slot) : nullptr;
     double* out = slot >= 0 ? red_slot_out(ctx, slot) : nullptr;
-    typename LinksOf<T>::type U;
-    if constexpr (sizeof(T) == 8) U = links64(ctx); else U = links32(ctx);
     if (W) {
         if (slot >= 0) k_lap<T, LF, NMU, true, true><<<grid, shp.block, 0, st>>>(ctx->g, U, X, Y, W, (T)a, (T)b, (T)c, fs, part, cnt, out, ss);
         else k_lap<T, LF, NMU, true, false><<<grid, shp.block, 0, st>>>(ctx->g, U, X, Y, W, (T)a, (T)b, (T)c, fs, part, cnt, out, ss);
@@ -94,6 +91,22 @@ template <typename T, int LF>
 static int launch_lap_t(rmhmc_ctx* ctx, const T* X, T* Y, int nfield, double a, double b, const T* W, double c,
                         int slot, cudaStream_t st) {
     StencilShape shp;
+    typename LinksOf<T>::type U;
+    if constexpr (sizeof(T) == 8) {
+        U = links64(ctx);
+        // float64 with 18-real links, no shape pinned: the adjoint form, one component per lane (the arithmetic bounds every
+        // shape alike).  32^4: 3.66 ms and 2.46 ms for the table of new links, against 6.38 ms in the 3x3 form
+        if (LF == 18 && !ctx->tune.count(818)) {
+            RM_TRY(links64_adjoint(ctx, &U, st));
+            if (U.ad) {
+                launch_lap_shape<T, kLinkAd, 1>(ctx, StencilShape{1, 128}, U, X, Y, nfield, a, b, W, c, slot, st);
+                RM_LAUNCH_CHECK(ctx);
+                return RMHMC_OK;
+            }
+        }
+    } else {
+        U = links32(ctx);
+    }
     RM_TRY((stencil_shape<T, LF>(ctx, st, shp)));
     if (shp.nmu == 8) {
         // the link-centric kernel serves one plain field; with a third term or dots the gather kernel runs
@@ -101,10 +114,10 @@ static int launch_lap_t(rmhmc_ctx* ctx, const T* X, T* Y, int nfield, double a, 
             return launch_lap_lc(ctx, LF, (const float*)X, (float*)Y, a, b, st);
         shp = StencilShape{2, 256};
     }
-    if (shp.nmu == 4) launch_lap_shape<T, LF, 4>(ctx, shp, X, Y, nfield, a, b, W, c, slot, st);
-    else if (shp.nmu == 2) launch_lap_shape<T, LF, 2>(ctx, shp, X, Y, nfield, a, b, W, c, slot, st);
-    else if (shp.nmu == 0) launch_lap_shape<T, LF, 0>(ctx, shp, X, Y, nfield, a, b, W, c, slot, st);
-    else launch_lap_shape<T, LF, 1>(ctx, shp, X, Y, nfield, a, b, W, c, slot, st);
+    if (shp.nmu == 4) launch_lap_shape<T, LF, 4>(ctx, shp, U, X, Y, nfield, a, b, W, c, slot, st);
+    else if (shp.nmu == 2) launch_lap_shape<T, LF, 2>(ctx, shp, U, X, Y, nfield, a, b, W, c, slot, st);
+    else if (shp.nmu == 0) launch_lap_shape<T, LF, 0>(ctx, shp, U, X, Y, nfield, a, b, W, c, slot, st);
+    else launch_lap_shape<T, LF, 1>(ctx, shp, U, X, Y, nfield, a, b, W, c, slot, st);
     RM_LAUNCH_CHECK(ctx);
     return RMHMC_OK;
 }
@@ -127,6 +140,8 @@ int stencil_shape(rmhmc_ctx* ctx, cudaStream_t st, StencilShape& out) {
     T* Y = (T*)workspace(ctx, "tune_y", sizeof(double) * fs, &status);
     if (!X || !Y) return status;
     RM_CHECK(ctx, cudaMemsetAsync(X, 0, sizeof(T) * fs, st));
+    typename LinksOf<T>::type U;
+    if constexpr (sizeof(T) == 8) U = links64(ctx); else U = links32(ctx);
     cudaEvent_t e0, e1;
     RM_CHECK(ctx, cudaEventCreate(&e0));
     RM_CHECK(ctx, cudaEventCreate(&e1));
@@ -140,10 +155,10 @@ int stencil_shape(rmhmc_ctx* ctx, cudaStream_t st, StencilShape& out) {
             const StencilShape shp{nmu, block};
             auto run = [&]() {
                 if (nmu == 8) launch_lap_lc(ctx, LF, (const float*)X, (float*)Y, 0.5, -0.0625, st);
-                else if (nmu == 4) launch_lap_shape<T, LF, 4>(ctx, shp, X, Y, 1, 0.5, -0.0625, nullptr, 0.0, -1, st);
-                else if (nmu == 2) launch_lap_shape<T, LF, 2>(ctx, shp, X, Y, 1, 0.5, -0.0625, nullptr, 0.0, -1, st);
-                else if (nmu == 0) launch_lap_shape<T, LF, 0>(ctx, shp, X, Y, 1, 0.5, -0.0625, nullptr, 0.0, -1, st);
-                else launch_lap_shape<T, LF, 1>(ctx, shp, X, Y, 1, 0.5, -0.0625, nullptr, 0.0, -1, st);
+                else if (nmu == 4) launch_lap_shape<T, LF, 4>(ctx, shp, U, X, Y, 1, 0.5, -0.0625, nullptr, 0.0, -1, st);
+                else if (nmu == 2) launch_lap_shape<T, LF, 2>(ctx, shp, U, X, Y, 1, 0.5, -0.0625, nullptr, 0.0, -1, st);
+                else if (nmu == 0) launch_lap_shape<T, LF, 0>(ctx, shp, U, X, Y, 1, 0.5, -0.0625, nullptr, 0.0, -1, st);
+                else launch_lap_shape<T, LF, 1>(ctx, shp, U, X, Y, 1, 0.5, -0.0625, nullptr, 0.0, -1, st);
             };
             run();
             RM_CHECK(ctx, cudaEventRecord(e0, st));

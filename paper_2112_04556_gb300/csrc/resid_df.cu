@@ -15,6 +15,7 @@
 //    accurate as if computed in twice the working precision.
 // The residual is returned rounded to float32 (the correction solve's right-hand side) together with
 // its float64 squared norm.
+#include "df.cuh"
 #include "krylov.cuh"
 
 namespace rm {
@@ -28,23 +29,49 @@ __global__ void __launch_bounds__(kBlock) k_adjoint_table(Links64 U, int V, floa
     if (s >= V) return;
     const mat3<double> u = LinkLoad<double, 18>::load(U, s, nu);
     float* o = out + ((size_t)s * 4 + nu) * 128;
-#pragma unroll
-    for (int b = 0; b < 8; b++) {
-        double e[8];
-#pragma unroll
-        for (int a = 0; a < 8; a++) e[a] = a == b ? 1.0 : 0.0;
-        herm<double> H = h_zero<double>();
-        acc_uxud(H, u, coef_to_herm2(e));   // U (2 T^b) U^dag = sum_c Ad_cb (2 T^c)
-        double col[8];
-        herm2_to_coef(H, col);
+    adjoint_columns(u, [&](int b, const double (&col)[8]) {
 #pragma unroll
         for (int c = 0; c < 8; c++) {
-            const double v = col[c] * 0.0625;
-            const float hi = (float)v;
-            o[c * 8 + b] = hi;
-            o[64 + c * 8 + b] = (float)(v - (double)hi);
+            const dfl v = df_split(col[c] * 0.0625);
+            o[c * 8 + b] = v.hi;
+            o[64 + c * 8 + b] = v.lo;
         }
+    });
+}
+
+// the float64 table of Links64::ad: thread per (site, direction), consecutive sites adjacent in every plane
+__global__ void __launch_bounds__(kBlock) k_adjoint_table64(Links64 U, double2* __restrict__ out) {
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    const int nu = blockIdx.y;
+    if (s >= U.V) return;
+    const mat3<double> u = LinkLoad<double, 18>::load(U, s, nu);
+    double2* const o = out + (size_t)nu * 32 * U.V + s;
+    adjoint_columns(u, [&](int b, const double (&col)[8]) {
+#pragma unroll
+        for (int h = 0; h < 4; h++) o[(size_t)(4 * b + h) * U.V] = make_double2(col[2 * h], col[2 * h + 1]);
+    });
+}
+
+int links64_adjoint(rmhmc_ctx* ctx, Links64* U, cudaStream_t st) {
+    if (ctx->g.V > kAdTableMax || ctx->adj64_off) return RMHMC_OK;
+    int status = RMHMC_OK;
+    const unsigned long long ws = ctx->ws_gen;
+    double2* t = (double2*)workspace(ctx, "ad_table64", sizeof(double2) * (size_t)ctx->g.V * 128, &status);
+    if (status == RMHMC_ENOMEM) {
+        // no room: the 3x3 form serves as before
+        ctx->err.clear();
+        ctx->adj64_off = true;
+        return RMHMC_OK;
     }
+    if (!t) return status;
+    if (ctx->adj64_gen != ctx->link_gen || ws != ctx->ws_gen) {
+        k_adjoint_table64<<<dim3(site_blocks(ctx), 4), kBlock, 0, st>>>(links64(ctx), t);
+        ++ctx->launches;
+        RM_LAUNCH_CHECK(ctx);
+        ctx->adj64_gen = ctx->link_gen;
+    }
+    U->ad = t;
+    return RMHMC_OK;
 }
 
 // x (float64 [nf][V][4][8]) -> [nf][V][4][16] float32: hi[8] then lo[8] per component
@@ -55,8 +82,9 @@ __global__ void k_split_pairs(const double* __restrict__ x, float* __restrict__ 
         float h[8], l[8];
 #pragma unroll
         for (int a = 0; a < 8; a++) {
-            h[a] = (float)v[a];
-            l[a] = (float)(v[a] - (double)h[a]);
+            const dfl p = df_split(v[a]);   // integer operations: the float64 pipe held this pass at a third of its bandwidth
+            h[a] = p.hi;
+            l[a] = p.lo;
         }
         store8(out + i * 16, h);
         store8(out + i * 16 + 8, l);

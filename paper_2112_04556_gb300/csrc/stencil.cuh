@@ -80,12 +80,63 @@ __device__ __forceinline__ void hop_sum_shape(const Geom& g, const typename Link
     else hop_sum<T, LF, NMU>(g, U, s, mu0, src, acc);
 }
 
-template <typename T, int LF, class Src>
-__device__ __forceinline__ void hop_sum1(const Geom& g, const typename LinksOf<T>::type& U, int s, int mu,
-                                         const Src& src, herm<T>& acc) {
-    herm<T> a[1];
-    hop_sum<T, LF, 1>(g, U, s, mu, src, a);
-    acc = a[0];
+// The hop sum from the adjoint table, as coefficients: 64 FMA per hop and component where the 3x3 form takes 108 and the
+// expansions.  For float64, whose rate (0.55 TFMA/s) bounds every stencil: the table's 4 KB a site are read at a
+// tenth of that time.
+template <int NC, class Src>
+__device__ __forceinline__ void hop_sum_adjoint(const Geom& g, const Links64& U, int s, int mu0, const Src& src,
+                                                double (&h)[NC][8]) {
+    int fwd[4], bwd[4];
+    neighbours(g, s, fwd, bwd);
+#pragma unroll
+    for (int m = 0; m < NC; m++)
+#pragma unroll
+        for (int a = 0; a < 8; a++) h[m][a] = 0.0;
+#pragma unroll 1
+    for (int nu = 0; nu < 4; nu++) {
+        const int f = nu == 0 ? fwd[0] : nu == 1 ? fwd[1] : nu == 2 ? fwd[2] : fwd[3];
+        const int w = nu == 0 ? bwd[0] : nu == 1 ? bwd[1] : nu == 2 ? bwd[2] : bwd[3];
+        double x[NC][8];
+        const double2* t = U.ad + (size_t)nu * 32 * U.V;
+#pragma unroll
+        for (int m = 0; m < NC; m++) src(f, mu0 + m, x[m]);
+#pragma unroll
+        for (int b = 0; b < 8; b++)
+#pragma unroll
+            for (int a = 0; a < 4; a++) {
+                const double2 v = __ldg(t + (size_t)(4 * b + a) * U.V + s);
+#pragma unroll
+                for (int m = 0; m < NC; m++) {
+                    h[m][2 * a] = fma(v.x, x[m][b], h[m][2 * a]);
+                    h[m][2 * a + 1] = fma(v.y, x[m][b], h[m][2 * a + 1]);
+                }
+            }
+#pragma unroll
+        for (int m = 0; m < NC; m++) src(w, mu0 + m, x[m]);
+#pragma unroll
+        for (int a = 0; a < 4; a++)
+#pragma unroll
+            for (int b = 0; b < 8; b++) {
+                const double2 v = __ldg(t + (size_t)(4 * b + a) * U.V + w);
+#pragma unroll
+                for (int m = 0; m < NC; m++) h[m][b] = fma(v.y, x[m][2 * a + 1], fma(v.x, x[m][2 * a], h[m][b]));
+            }
+    }
+}
+
+// coefficients of the hop sum of a lane's components, in any link format
+template <typename T, int LF, int NMU, class Src>
+__device__ __forceinline__ void hop_coefs(const Geom& g, const typename LinksOf<T>::type& U, int s, int mu0, const Src& src,
+                                          T (&h)[NMU == 0 ? 1 : NMU][8]) {
+    if constexpr (LF == kLinkAd) {
+        hop_sum_adjoint(g, U, s, mu0, src, h);
+    } else {
+        constexpr int NC = NMU == 0 ? 1 : NMU;
+        herm<T> acc[NC];
+        hop_sum_shape<T, LF, NMU>(g, U, s, mu0, src, acc);
+#pragma unroll
+        for (int m = 0; m < NC; m++) herm2_to_coef_tl(acc[m], h[m]);
+    }
 }
 
 // plain field source: X[s][mu][8]

@@ -214,3 +214,20 @@ def test_lap_adjoint_every_shape_and_slab(L):
                 assert rel_l2(Y, ref) <= 1e-5, (ch, bz, lf, rel_l2(Y, ref))
                 rm.lap_apply(ctx, None, Xo, Yo, prec=rm.FP32, linkfmt=lf)
                 assert rel_l2(host(Yo).astype(np.float64), ref) <= 1e-5, (ch, bz, lf, "offset")
+
+
+@pytest.mark.parametrize("L,nf", [((2, 2, 2, 2), 1), ((5, 3, 4, 7), 3), ((33, 2, 3, 2), 1), ((8, 8, 8, 8), 2)])
+def test_lap_fp64_adjoint_table_matches_3x3_form(L, nf):
+    """float64 lap_apply from the adjoint table (the default) against a pinned 3x3 shape, for two configurations in turn:
+    the table follows the links.  Both are sums of 512 or 864 float64 products per coefficient: 1e-14."""
+    import paper_2112_04556_gb300 as rm
+    X = inputs.gaussian_fields(L, nf, seed=52)
+    Us = [inputs.random_links(L, eps=e, seed=53 + i) for i, e in enumerate((0.3, 1.5))]
+    with rm.Context(L) as a, rm.Context(L) as b:
+        rm.set_stencil_shape(b, rm.SHAPE_LAP, rm.FP64, 18, 1, 128)
+        for U in (Us[0], Us[1], Us[0]):
+            y = host(rm.lap_apply(a, dev(U), dev(X)))
+            assert np.array_equal(y, host(rm.lap_apply(a, None, dev(X))))
+            ref = host(rm.lap_apply(b, dev(U), dev(X)))
+            assert rel_l2(y, ref) <= 1e-14
+            assert rel_l2(y[0], oracle.lap(L, U, X[0])) <= 1e-12
