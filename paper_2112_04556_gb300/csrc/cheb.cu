@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "df.cuh"
 #include "krylov.cuh"
 #include "ops.cuh"
 #include "philox.cuh"
@@ -22,23 +23,32 @@ namespace rm {
 
 constexpr int kSlotCheb = 128;   // first reduction slot of the batched moments (kRedSlots - 128 fields)
 
+// v_0 of every field (blockIdx.y) and its squared norm, four values a thread; float32 without float64 arithmetic
 template <typename T>
 __global__ void k_copy_norms(const double* __restrict__ in, T* __restrict__ out, size_t fs, int V, double* partials,
                              unsigned* counters, double* red_out, size_t slot_stride) {
     __shared__ double sh[kBlock / 32];
     const int f = blockIdx.y;
-    double acc = 0.0;
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < V; s += gridDim.x * blockDim.x) {
-        const double* src = in + f * fs + (size_t)s * 32;
-        T* dst = out + f * fs + (size_t)s * 32;
-#pragma unroll 4
-        for (int k = 0; k < 32; k++) {
-            const T x = (T)src[k];
-            dst[k] = x;
-            acc += (double)x * (double)x;
+    SumSq32 sf;
+    double sd = 0.0;
+    const size_t n4 = (size_t)V * 8;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
+        double v[4];
+        T x[4];
+        load4(in + f * fs + i * 4, v);
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            if constexpr (sizeof(T) == 4) {
+                x[k] = to_f32(v[k]);
+                sf.add(x[k]);
+            } else {
+                x[k] = v[k];
+                sd = fma(x[k], x[k], sd);
+            }
         }
+        store4(out + f * fs + i * 4, x);
     }
-    double v[1] = {acc};
+    double v[1] = {sizeof(T) == 4 ? sf.value() : sd};
     block_sum<1>(v, sh);
     grid_sum_finish<1>(v, partials + f * slot_stride, counters + f, red_out + (size_t)f * 8, gridDim.x, blockIdx.x, sh);
 }
@@ -89,7 +99,7 @@ static int cheb_run(rmhmc_ctx* ctx, const double* fields64, int nr, int N, int p
     T* v[3] = {buf, buf + fs * nr, buf + 2 * fs * nr};
     const size_t ss = (size_t)ctx->max_blocks * 2;
     // v0 and mu_0
-    k_copy_norms<T><<<dim3(capped_grid(ctx, ctx->g.V, kBlock), nr), kBlock, 0, st>>>(fields64, v[0], fs, ctx->g.V,
+    k_copy_norms<T><<<dim3(capped_grid(ctx, fs / 4, kBlock), nr), kBlock, 0, st>>>(fields64, v[0], fs, ctx->g.V,
                                                                    red_slot_partials(ctx, kSlotCheb), red_slot_counter(ctx, kSlotCheb),
                                                                    red_slot_out(ctx, kSlotCheb), ss); ++ctx->launches;
     RM_LAUNCH_CHECK(ctx);
@@ -100,9 +110,8 @@ static int cheb_run(rmhmc_ctx* ctx, const double* fields64, int nr, int N, int p
         T* out = v[k % 3];
         const T* in = v[(k - 1) % 3];
         const T* w = k >= 2 ? v[(k - 2) % 3] : nullptr;
-        RM_TRY(launch_lap(ctx, prec, 18, in, out, nr, 0.0, k == 1 ? -0.125 : -0.25, w, -1.0, kSlotCheb, st));
-        RM_CHECK(ctx, cudaMemcpyAsync(dmom + (size_t)8 * nr * k, red_slot_out(ctx, kSlotCheb), sizeof(double) * 8 * nr,
-                                      cudaMemcpyDeviceToDevice, st));
+        RM_TRY(launch_lap(ctx, prec, 18, in, out, nr, 0.0, k == 1 ? -0.125 : -0.25, w, -1.0, kSlotCheb, st,
+                          dmom + (size_t)8 * nr * k));
     }
     std::vector<double> h((size_t)8 * nr * (K + 1));
     for (size_t off = 0; off < h.size(); off += kPinned) {

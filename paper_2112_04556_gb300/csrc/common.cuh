@@ -329,6 +329,7 @@ struct rmhmc_ctx {
     unsigned long long link_gen = 1;   // bumped whenever the internal link copies change
     unsigned long long adj_gen = 0;    // link_gen the float32-pair adjoint table was built for
     unsigned long long adj64_gen = 0;  // and the float64 one
+    bool loops_off = false;            // no memory for the gauge force's loops
     bool adj64_off = false;            // no memory for the float64 one
     // reductions
     double* red_partials = nullptr;   // [kRedSlots][max_blocks * 2]

@@ -70,13 +70,13 @@ __global__ void __launch_bounds__(kBlockMax, (stencil_min_blocks<T, NMU>())) k_l
 
 template <typename T, int LF, int NMU>
 static void launch_lap_shape(rmhmc_ctx* ctx, const StencilShape& shp, const typename LinksOf<T>::type& U, const T* X, T* Y, int nfield, double a, double b,
-                             const T* W, double c, int slot, cudaStream_t st) {
+                             const T* W, double c, int slot, cudaStream_t st, double* dots = nullptr) {
     const dim3 grid(stencil_blocks(ctx, shp), nfield);
     const size_t fs = field_elems(ctx);
     const size_t ss = (size_t)ctx->max_blocks * 2;
     double* part = slot >= 0 ? red_slot_partials(ctx, slot) : nullptr;
     unsigned* cnt = slot >= 0 ? red_slot_counter(ctx, slot) : nullptr;
-    double* out = slot >= 0 ? red_slot_out(ctx, slot) : nullptr;
+    double* out = slot < 0 ? nullptr : dots ? dots : red_slot_out(ctx, slot);
     if (W) {
         if (slot >= 0) k_lap<T, LF, NMU, true, true><<<grid, shp.block, 0, st>>>(ctx->g, U, X, Y, W, (T)a, (T)b, (T)c, fs, part, cnt, out, ss);
         else k_lap<T, LF, NMU, true, false><<<grid, shp.block, 0, st>>>(ctx->g, U, X, Y, W, (T)a, (T)b, (T)c, fs, part, cnt, out, ss);
@@ -89,7 +89,7 @@ static void launch_lap_shape(rmhmc_ctx* ctx, const StencilShape& shp, const type
 
 template <typename T, int LF>
 static int launch_lap_t(rmhmc_ctx* ctx, const T* X, T* Y, int nfield, double a, double b, const T* W, double c,
-                        int slot, cudaStream_t st) {
+                        int slot, cudaStream_t st, double* dots) {
     StencilShape shp;
     typename LinksOf<T>::type U;
     if constexpr (sizeof(T) == 8) {
@@ -99,7 +99,7 @@ static int launch_lap_t(rmhmc_ctx* ctx, const T* X, T* Y, int nfield, double a, 
         if (LF == 18 && !ctx->tune.count(818)) {
             RM_TRY(links64_adjoint(ctx, &U, st));
             if (U.ad) {
-                launch_lap_shape<T, kLinkAd, 1>(ctx, StencilShape{1, 128}, U, X, Y, nfield, a, b, W, c, slot, st);
+                launch_lap_shape<T, kLinkAd, 1>(ctx, StencilShape{1, 128}, U, X, Y, nfield, a, b, W, c, slot, st, dots);
                 RM_LAUNCH_CHECK(ctx);
                 return RMHMC_OK;
             }
@@ -114,10 +114,10 @@ static int launch_lap_t(rmhmc_ctx* ctx, const T* X, T* Y, int nfield, double a, 
             return launch_lap_lc(ctx, LF, (const float*)X, (float*)Y, a, b, st);
         shp = StencilShape{2, 256};
     }
-    if (shp.nmu == 4) launch_lap_shape<T, LF, 4>(ctx, shp, U, X, Y, nfield, a, b, W, c, slot, st);
-    else if (shp.nmu == 2) launch_lap_shape<T, LF, 2>(ctx, shp, U, X, Y, nfield, a, b, W, c, slot, st);
-    else if (shp.nmu == 0) launch_lap_shape<T, LF, 0>(ctx, shp, U, X, Y, nfield, a, b, W, c, slot, st);
-    else launch_lap_shape<T, LF, 1>(ctx, shp, U, X, Y, nfield, a, b, W, c, slot, st);
+    if (shp.nmu == 4) launch_lap_shape<T, LF, 4>(ctx, shp, U, X, Y, nfield, a, b, W, c, slot, st, dots);
+    else if (shp.nmu == 2) launch_lap_shape<T, LF, 2>(ctx, shp, U, X, Y, nfield, a, b, W, c, slot, st, dots);
+    else if (shp.nmu == 0) launch_lap_shape<T, LF, 0>(ctx, shp, U, X, Y, nfield, a, b, W, c, slot, st, dots);
+    else launch_lap_shape<T, LF, 1>(ctx, shp, U, X, Y, nfield, a, b, W, c, slot, st, dots);
     RM_LAUNCH_CHECK(ctx);
     return RMHMC_OK;
 }
@@ -189,18 +189,18 @@ template int stencil_shape<double, 18>(rmhmc_ctx*, cudaStream_t, StencilShape&);
 template int stencil_shape<double, 12>(rmhmc_ctx*, cudaStream_t, StencilShape&);
 
 int launch_lap(rmhmc_ctx* ctx, int prec, int linkfmt, const void* X, void* Y, int nfield, double a, double b,
-               const void* W, double c, int slot, cudaStream_t st) {
+               const void* W, double c, int slot, cudaStream_t st, double* dots) {
     if (slot >= 0 && slot + nfield > kRedSlots) return set_err(ctx, RMHMC_EINVAL, "too many reduced fields");
     if (prec == RMHMC_FP64) {
         if (linkfmt == 12)
-            return launch_lap_t<double, 12>(ctx, (const double*)X, (double*)Y, nfield, a, b, (const double*)W, c, slot, st);
-        return launch_lap_t<double, 18>(ctx, (const double*)X, (double*)Y, nfield, a, b, (const double*)W, c, slot, st);
+            return launch_lap_t<double, 12>(ctx, (const double*)X, (double*)Y, nfield, a, b, (const double*)W, c, slot, st, dots);
+        return launch_lap_t<double, 18>(ctx, (const double*)X, (double*)Y, nfield, a, b, (const double*)W, c, slot, st, dots);
     }
     if (nfield >= kAdMinFields)
-        return launch_lap_ad(ctx, linkfmt, (const float*)X, (float*)Y, nfield, a, b, (const float*)W, c, slot, st);
+        return launch_lap_ad(ctx, linkfmt, (const float*)X, (float*)Y, nfield, a, b, (const float*)W, c, slot, dots, st);
     if (linkfmt == 12)
-        return launch_lap_t<float, 12>(ctx, (const float*)X, (float*)Y, nfield, a, b, (const float*)W, c, slot, st);
-    return launch_lap_t<float, 18>(ctx, (const float*)X, (float*)Y, nfield, a, b, (const float*)W, c, slot, st);
+        return launch_lap_t<float, 12>(ctx, (const float*)X, (float*)Y, nfield, a, b, (const float*)W, c, slot, st, dots);
+    return launch_lap_t<float, 18>(ctx, (const float*)X, (float*)Y, nfield, a, b, (const float*)W, c, slot, st, dots);
 }
 
 }  // namespace rm

@@ -40,7 +40,8 @@ inline size_t ad_smem_bytes(int nd) {
     return kAdSmemFloats * sizeof(float) + kAdSites * 8 * sizeof(int) + (size_t)(kAdThreads / 32) * nd * 2 * sizeof(double);
 }
 
-// CH: fields per pass of phase 2; MINB: resident blocks the register budget is compiled for
+// CH: fields per pass of phase 2; MINB: resident blocks the register budget is compiled for.  (Nine or five fields a pass without the second operand
+// buffer read the adjoint records less often but are slower: 18 fields at 32^4 3.3-3.6 and 3.0 ms against 2.65 ms.)
 template <int LF, bool HAS_W, bool DOTS, int CH, int MINB>
 __global__ void __launch_bounds__(kAdThreads, MINB) k_lap_ad(Geom g, Links32 U, const float* __restrict__ X,
                                                         float* __restrict__ Y, const float* __restrict__ W, int nf,
@@ -51,7 +52,7 @@ __global__ void __launch_bounds__(kAdThreads, MINB) k_lap_ad(Geom g, Links32 U, 
     float* ad = smem;                                            // [kAdSites][kAdSiteStride]
     int* nbr = reinterpret_cast<int*>(smem + kAdSmemFloats);     // [kAdSites][8]
     double* dsum = reinterpret_cast<double*>(nbr + kAdSites * 8);   // [warps][nf][2] (DOTS)
-    __shared__ double sh[2 * (kAdThreads / 32)];
+    __shared__ int am_last;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     if (DOTS)
         for (int i = t; i < (kAdThreads / 32) * nf * 2; i += kAdThreads) dsum[i] = 0.0;
@@ -185,17 +186,28 @@ __global__ void __launch_bounds__(kAdThreads, MINB) k_lap_ad(Geom g, Links32 U, 
         __syncthreads();   // the next unit overwrites the adjoint records
     }
     if (DOTS) {
-        // per field: the warps' sums in warp order, then the deterministic grid sum
-        for (int f = 0; f < nf; f++) {
-            double v[2] = {0.0, 0.0};
-            if (t == 0)
-                for (int w = 0; w < kAdThreads / 32; w++) {
-                    v[0] += dsum[(w * nf + f) * 2];
-                    v[1] += dsum[(w * nf + f) * 2 + 1];
-                }
-            grid_sum_finish<2>(v, partials + f * slot_stride, counters + f, out + (size_t)f * 8, gridDim.x, blockIdx.x,
-                               sh);
+        // the warps' sums of every field in warp order, one ticket for all fields, and the last block adds the blocks'
+        // partials (a ticket per field cost 55 us of a spectrum's step: 16^4, 18 fields, 277 -> 222 us)
+        for (int i = t; i < 2 * nf; i += kAdThreads) {
+            double v = 0.0;
+            for (int w = 0; w < kAdThreads / 32; w++) v += dsum[w * nf * 2 + i];
+            partials[(size_t)(i >> 1) * slot_stride + 2 * blockIdx.x + (i & 1)] = v;
         }
+        __threadfence();
+        __syncthreads();
+        if (t == 0) am_last = atomicAdd(counters, 1u) == gridDim.x - 1;
+        __syncthreads();
+        if (!am_last) return;
+        __threadfence();
+        for (int i = warp; i < 2 * nf; i += kAdThreads / 32) {
+            const double* p = partials + (size_t)(i >> 1) * slot_stride + (i & 1);
+            double v = 0.0;
+            for (int b = lane; b < (int)gridDim.x; b += 32) v += __ldcg(p + 2 * b);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+            if (lane == 0) out[(size_t)(i >> 1) * 8 + (i & 1)] = v;
+        }
+        if (t == 0) *counters = 0u;
     }
 }
 
@@ -205,7 +217,7 @@ constexpr AdShape kAdShapes[2] = {{2, 3}, {3, 2}};
 
 template <int LF, bool HAS_W, bool DOTS, int CH, int MINB>
 static int launch_ad_t(rmhmc_ctx* ctx, const float* X, float* Y, int nf, double a, double b, const float* W, double c,
-                       int slot, cudaStream_t st) {
+                       int slot, double* dots, cudaStream_t st) {
     if (DOTS && nf > kRedSlots) return set_err(ctx, RMHMC_EINVAL, "too many reduced fields");
     auto kern = k_lap_ad<LF, HAS_W, DOTS, CH, MINB>;
     const size_t smem = ad_smem_bytes(DOTS ? nf : 0);
@@ -222,11 +234,11 @@ static int launch_ad_t(rmhmc_ctx* ctx, const float* X, float* Y, int nf, double 
     const int bz = ctx->ad_slab > 0 ? ctx->ad_slab : ctx->g.L[2];
     const int P = ctx->g.stride[2];
     const int nunit = (P * bz + kAdSites - 1) / kAdSites * ctx->g.L[3] * ((ctx->g.L[2] + bz - 1) / bz);
-    const int grid = std::max(1, std::min(nunit, (int)ctx->num_sms * std::max(per_sm, 1)));
+    const int grid = std::max(1, std::min(std::min(nunit, (int)ctx->num_sms * std::max(per_sm, 1)), ctx->max_blocks));
     const size_t ss = (size_t)ctx->max_blocks * 2;
     double* part = DOTS ? red_slot_partials(ctx, slot) : nullptr;
     unsigned* cnt = DOTS ? red_slot_counter(ctx, slot) : nullptr;
-    double* out = DOTS ? red_slot_out(ctx, slot) : nullptr;
+    double* out = !DOTS ? nullptr : dots ? dots : red_slot_out(ctx, slot);
     kern<<<grid, kAdThreads, smem, st>>>(ctx->g, links32(ctx), X, Y, W, nf, (float)a, (float)b, (float)c, field_elems(ctx),
                                          bz, part, cnt, out, ss);
     ++ctx->launches;
@@ -236,20 +248,20 @@ static int launch_ad_t(rmhmc_ctx* ctx, const float* X, float* Y, int nf, double 
 
 template <int LF, int CH, int MINB>
 static int launch_ad_shape(rmhmc_ctx* ctx, const float* X, float* Y, int nf, double a, double b, const float* W,
-                           double c, int slot, cudaStream_t st) {
+                           double c, int slot, double* dots, cudaStream_t st) {
     if (W) {
-        if (slot >= 0) return launch_ad_t<LF, true, true, CH, MINB>(ctx, X, Y, nf, a, b, W, c, slot, st);
-        return launch_ad_t<LF, true, false, CH, MINB>(ctx, X, Y, nf, a, b, W, c, slot, st);
+        if (slot >= 0) return launch_ad_t<LF, true, true, CH, MINB>(ctx, X, Y, nf, a, b, W, c, slot, dots, st);
+        return launch_ad_t<LF, true, false, CH, MINB>(ctx, X, Y, nf, a, b, W, c, slot, dots, st);
     }
-    if (slot >= 0) return launch_ad_t<LF, false, true, CH, MINB>(ctx, X, Y, nf, a, b, W, c, slot, st);
-    return launch_ad_t<LF, false, false, CH, MINB>(ctx, X, Y, nf, a, b, W, c, slot, st);
+    if (slot >= 0) return launch_ad_t<LF, false, true, CH, MINB>(ctx, X, Y, nf, a, b, W, c, slot, dots, st);
+    return launch_ad_t<LF, false, false, CH, MINB>(ctx, X, Y, nf, a, b, W, c, slot, dots, st);
 }
 
 template <int LF>
 static int launch_ad_idx(rmhmc_ctx* ctx, int k, const float* X, float* Y, int nf, double a, double b, const float* W,
-                         double c, int slot, cudaStream_t st) {
-    if (k == 0) return launch_ad_shape<LF, 2, 3>(ctx, X, Y, nf, a, b, W, c, slot, st);
-    return launch_ad_shape<LF, 3, 2>(ctx, X, Y, nf, a, b, W, c, slot, st);
+                         double c, int slot, double* dots, cudaStream_t st) {
+    if (k == 0) return launch_ad_shape<LF, 2, 3>(ctx, X, Y, nf, a, b, W, c, slot, dots, st);
+    return launch_ad_shape<LF, 3, 2>(ctx, X, Y, nf, a, b, W, c, slot, dots, st);
 }
 
 // the shape for this link format: on first use every shape is timed (one warm-up and three timed plain
@@ -270,9 +282,9 @@ static int ad_shape(rmhmc_ctx* ctx, const float* X, float* Y, int nf, cudaStream
     char line[96];
     std::string rep;
     for (int k = 0; k < 2; k++) {
-        RM_TRY(launch_ad_idx<LF>(ctx, k, X, Y, nf, 0.5, -0.0625, nullptr, 0.0, -1, st));
+        RM_TRY(launch_ad_idx<LF>(ctx, k, X, Y, nf, 0.5, -0.0625, nullptr, 0.0, -1, nullptr, st));
         RM_CHECK(ctx, cudaEventRecord(e0, st));
-        for (int r = 0; r < 3; r++) RM_TRY(launch_ad_idx<LF>(ctx, k, X, Y, nf, 0.5, -0.0625, nullptr, 0.0, -1, st));
+        for (int r = 0; r < 3; r++) RM_TRY(launch_ad_idx<LF>(ctx, k, X, Y, nf, 0.5, -0.0625, nullptr, 0.0, -1, nullptr, st));
         RM_CHECK(ctx, cudaEventRecord(e1, st));
         RM_CHECK(ctx, cudaEventSynchronize(e1));
         float ms = 0.f;
@@ -294,19 +306,19 @@ static int ad_shape(rmhmc_ctx* ctx, const float* X, float* Y, int nf, cudaStream
 
 template <int LF>
 static int launch_ad_lf(rmhmc_ctx* ctx, const float* X, float* Y, int nf, double a, double b, const float* W, double c,
-                        int slot, cudaStream_t st) {
+                        int slot, double* dots, cudaStream_t st) {
     // the tuner writes Y, so a call that updates W in place (Y == W) takes the tuned shape if there is one and
     // the middle shape otherwise
     int k = 1;
     if (W != Y) RM_TRY(ad_shape<LF>(ctx, X, Y, nf, st, &k));
     else if (ctx->tune.count(20000 + LF)) k = ctx->tune[20000 + LF].first;
-    return launch_ad_idx<LF>(ctx, k, X, Y, nf, a, b, W, c, slot, st);
+    return launch_ad_idx<LF>(ctx, k, X, Y, nf, a, b, W, c, slot, dots, st);
 }
 
 int launch_lap_ad(rmhmc_ctx* ctx, int linkfmt, const float* X, float* Y, int nfield, double a, double b, const float* W,
-                  double c, int slot, cudaStream_t st) {
-    if (linkfmt == 12) return launch_ad_lf<12>(ctx, X, Y, nfield, a, b, W, c, slot, st);
-    return launch_ad_lf<18>(ctx, X, Y, nfield, a, b, W, c, slot, st);
+                  double c, int slot, double* dots, cudaStream_t st) {
+    if (linkfmt == 12) return launch_ad_lf<12>(ctx, X, Y, nfield, a, b, W, c, slot, dots, st);
+    return launch_ad_lf<18>(ctx, X, Y, nfield, a, b, W, c, slot, dots, st);
 }
 
 }  // namespace rm

@@ -5,14 +5,14 @@
 namespace rm {
 
 // Y = a X + b H(X) + c W for nfield fields (prec: RMHMC_FP64 double, else float); if slot >= 0,
-// per-field float64 sums {<Y,Y>, <Y,X>} land in reduction slots slot .. slot+nfield-1.
+// per-field float64 sums {<Y,Y>, <Y,X>} land in reduction slots slot .. slot+nfield-1, or at dots + 8 f.
 int launch_lap(rmhmc_ctx* ctx, int prec, int linkfmt, const void* X, void* Y, int nfield, double a, double b,
-               const void* W, double c, int slot, cudaStream_t st);
+               const void* W, double c, int slot, cudaStream_t st, double* dots = nullptr);
 
 // the same for float32 fields in the adjoint form (lap_ad.cu): each link becomes its 8x8 adjoint matrix once per
 // application, shared by all fields; dots as launch_lap
 int launch_lap_ad(rmhmc_ctx* ctx, int linkfmt, const float* X, float* Y, int nfield, double a, double b, const float* W,
-                  double c, int slot, cudaStream_t st);
+                  double c, int slot, double* dots, cudaStream_t st);
 // the link-centric adjoint stencil (lap_lc.cu), float32, one field: Y = a X + b H(X); and the CG stencil
 // q = diag r_k + (-1/16) H(r_k) + beta q (k from flags[1], as the gather kernel of krylov.cu)
 int launch_lap_lc(rmhmc_ctx* ctx, int linkfmt, const float* X, float* Y, double a, double b, cudaStream_t st);
@@ -25,6 +25,16 @@ constexpr int kAdMinFields = 6;
 int gauge_force_launch(rmhmc_ctx* ctx, double beta, double c1, int prec, double* F, cudaStream_t st);
 // action S and average plaquette (float64, deterministic) from the context's float64 links
 int action_launch(rmhmc_ctx* ctx, double beta, double c1, double* S, double* plaq, cudaStream_t st);
+// Force (F not null) and, in float64, the loop sums of the action (act) from shared loops (gauge_loops.cu), on lattices of up
+// to kLoopsMax sites (scratch: up to 4.5 KB a site in float64); *used tells whether it ran.  The sums go to the slot kSlotLoops:
+// sum (1 - ReTr P/3), sum ReTr P/3 over plaquettes, sum (1 - ReTr R/3) over rectangles.  gauge_loops_prepare allocates the
+// scratch (before a capture)
+constexpr int kLoopsMax = 1 << 22;
+constexpr int kSlotLoops = 41, kSlotLoopsEnd = 128;   // the partials may run on into the unused slots
+int gauge_loops_launch(rmhmc_ctx* ctx, double beta, double c1, int prec, double* F, bool act, bool* used, cudaStream_t st);
+int gauge_loops_prepare(rmhmc_ctx* ctx, double c1, int prec);
+// float64 force with action and average plaquette (each pointer nullable) of the context's links
+int gauge_force_action(rmhmc_ctx* ctx, double beta, double c1, double* F, double* S, double* plaq, cudaStream_t st);
 // G = sum_f w_f d<Z_f, A X_f>/dw (X, Z in the arithmetic precision, [nf][V][4][8]); G float64 [V][4][8]
 int link_grad_launch(rmhmc_ctx* ctx, int prec, const void* X, const void* Z, int nf, const double* w, double* G,
                      cudaStream_t st);
