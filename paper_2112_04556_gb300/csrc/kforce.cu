@@ -538,7 +538,8 @@ static int kinetic_t(rmhmc_ctx* ctx, const MassTerm& m, const double* P, double 
         double* o[1] = {Vel};
         RM_TRY((krylov_combine<T, double>(ctx, spec, o, st)));
     }
-    if (F && sizeof(T) == 4) {
+    if (!F) return RMHMC_OK;
+    if constexpr (sizeof(T) == 4) {
         // float32 basis: the force straight from the basis (rows of X_j and Z_j on the stored residuals)
         double* rows = (double*)workspace(ctx, "kf_rows", sizeof(double) * (size_t)(2 * ns + 2) * kBasisCap, &status);
         if (!rows) return status;
@@ -559,7 +560,7 @@ static int kinetic_t(rmhmc_ctx* ctx, const MassTerm& m, const double* P, double 
             RM_TRY(fetch(ctx, red_slot_out(ctx, kSlotNorm), &y2, 1, st));
             *Tkin = 0.5 * y2;
         }
-    } else if (F) {
+    } else {
         T* XZ = (T*)workspace(ctx, "kf_xz64", sizeof(T) * fs * 2 * ns, &status);
         if (!XZ) return status;
         CombineSpec spec;
@@ -574,8 +575,7 @@ static int kinetic_t(rmhmc_ctx* ctx, const MassTerm& m, const double* P, double 
             outs[ns + j] = XZ + (size_t)(ns + j) * fs;
         }
         RM_TRY((krylov_combine<T, T>(ctx, spec, outs.data(), st)));
-        RM_TRY(link_grad_launch(ctx, sizeof(T) == 8 ? RMHMC_FP64 : RMHMC_FP32, XZ, XZ + (size_t)ns * fs, ns,
-                                m.alpha.data(), F, st));
+        RM_TRY(link_grad_launch(ctx, RMHMC_FP64, XZ, XZ + (size_t)ns * fs, ns, m.alpha.data(), F, st));
     }
     return RMHMC_OK;
 }

@@ -314,7 +314,8 @@ template <> __device__ __forceinline__ void store_vec<double>(double* p, const d
     *reinterpret_cast<double2*>(p) = make_double2(x[0], x[1]);
 }
 
-template <typename T, typename TO, int MB>
+// ADD (one output): out += the combination, rounded to T first.
+template <typename T, typename TO, int MB, bool ADD = false>
 __global__ void __launch_bounds__(kBlock) k_combine(const T* __restrict__ R, size_t fs, const int* __restrict__ flags, int n,
                                                      const double* __restrict__ coef, int ldc, int M, OutPtrs<T, TO> outs) {
     using VT = Vec<T>;
@@ -370,6 +371,9 @@ __global__ void __launch_bounds__(kBlock) k_combine(const T* __restrict__ R, siz
 #pragma unroll
                 for (int v = 0; v < VN; v++) o[v] = (TO)acc[m][v];
                 TO* dst = outs.p[m] + aos;
+                if (ADD)
+#pragma unroll
+                    for (int v = 0; v < VN; v++) o[v] += dst[v];
                 if (sizeof(TO) == sizeof(T)) store_vec<TO>(dst, o);
                 else {
 #pragma unroll
@@ -412,10 +416,6 @@ __global__ void k_to_float(const double* __restrict__ in, float* __restrict__ ou
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
         out[i] = (float)in[i];
 }
-__global__ void k_add_f2d(const float* __restrict__ in, double* __restrict__ out, size_t n) {
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        out[i] += (double)in[i];
-}
 __global__ void k_axpby64(double a, const double* __restrict__ x, double b, const double* __restrict__ y,
                           double* __restrict__ out, size_t n) {
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
@@ -439,11 +439,6 @@ static int elem_grid(const rmhmc_ctx* ctx, size_t n) {
 
 int to_float(rmhmc_ctx* ctx, const double* in, float* out, size_t n, cudaStream_t st) {
     k_to_float<<<elem_grid(ctx, n), kBlock, 0, st>>>(in, out, n); ++ctx->launches;
-    RM_LAUNCH_CHECK(ctx);
-    return RMHMC_OK;
-}
-int add_float_to_double(rmhmc_ctx* ctx, const float* in, double* out, size_t n, cudaStream_t st) {
-    k_add_f2d<<<elem_grid(ctx, n), kBlock, 0, st>>>(in, out, n); ++ctx->launches;
     RM_LAUNCH_CHECK(ctx);
     return RMHMC_OK;
 }
@@ -644,8 +639,9 @@ int krylov_run(rmhmc_ctx* ctx, const TI* b, double sigma0, double tol, int maxit
 }
 
 template <typename T, typename TO>
-int krylov_combine(rmhmc_ctx* ctx, const CombineSpec& spec, TO* const* outs, cudaStream_t st) {
+int krylov_combine(rmhmc_ctx* ctx, const CombineSpec& spec, TO* const* outs, cudaStream_t st, bool add) {
     if (spec.n == 0) {
+        if (add) return RMHMC_OK;
         for (int m = 0; m < spec.M; m++) RM_CHECK(ctx, cudaMemsetAsync(outs[m], 0, field_elems(ctx) * sizeof(TO), st));
         return RMHMC_OK;
     }
@@ -663,7 +659,8 @@ int krylov_combine(rmhmc_ctx* ctx, const CombineSpec& spec, TO* const* outs, cud
         OutPtrs<T, TO> op{};
         for (int m = 0; m < mc; m++) op.p[m] = outs[m0 + m];
         const double* c = dcoef + (size_t)m0 * spec.n;
-        if (mc == 1) k_combine<T, TO, 1><<<grid, kBlock, 0, st>>>(R, fs, nullptr, spec.n, c, spec.n, 1, op);
+        if (mc == 1 && add) k_combine<T, TO, 1, true><<<grid, kBlock, 0, st>>>(R, fs, nullptr, spec.n, c, spec.n, 1, op);
+        else if (mc == 1) k_combine<T, TO, 1><<<grid, kBlock, 0, st>>>(R, fs, nullptr, spec.n, c, spec.n, 1, op);
         else k_combine<T, TO, kChunk><<<grid, kBlock, 0, st>>>(R, fs, nullptr, spec.n, c, spec.n, mc, op);
         ++ctx->launches;
         RM_LAUNCH_CHECK(ctx);
@@ -698,9 +695,8 @@ template int krylov_run<float, double>(rmhmc_ctx*, const double*, double, double
 template int krylov_run<double, double>(rmhmc_ctx*, const double*, double, double, int, KrylovResult&, cudaStream_t);
 template float* krylov_basis<float>(rmhmc_ctx*);
 template double* krylov_basis<double>(rmhmc_ctx*);
-template int krylov_combine<float, float>(rmhmc_ctx*, const CombineSpec&, float* const*, cudaStream_t);
-template int krylov_combine<float, double>(rmhmc_ctx*, const CombineSpec&, double* const*, cudaStream_t);
-template int krylov_combine<double, double>(rmhmc_ctx*, const CombineSpec&, double* const*, cudaStream_t);
+template int krylov_combine<float, double>(rmhmc_ctx*, const CombineSpec&, double* const*, cudaStream_t, bool);
+template int krylov_combine<double, double>(rmhmc_ctx*, const CombineSpec&, double* const*, cudaStream_t, bool);
 
 // ------------------------------------------------------------------------------------------------
 // mass term parsing and the per-shift solve with float64 reliable updates
@@ -785,9 +781,7 @@ int solve_shifts(rmhmc_ctx* ctx, const MassTerm& m, const double* b, double tol,
     // the links, which stay fixed for the whole solve.
     double* r = !mixed ? (double*)workspace(ctx, "ss_r", sizeof(double) * fs * ns, &status) : nullptr;
     float* r32 = mixed ? (float*)workspace(ctx, "ss_r32", sizeof(float) * fs * ns, &status) : nullptr;
-    float* e32 = mixed ? (float*)workspace(ctx, "ss_e32", sizeof(float) * fs, &status) : nullptr;
-    double* e64 = !mixed ? (double*)workspace(ctx, "ss_e64", sizeof(double) * fs, &status) : nullptr;
-    if ((mixed && (!r32 || !e32)) || (!mixed && (!r || !e64))) return status;
+    if (mixed ? !r32 : !r) return status;
     float* adj = nullptr;
     if (mixed) RM_TRY(adjoint_table(ctx, &adj, st));
     std::vector<double> n2(ns);
@@ -820,18 +814,34 @@ int solve_shifts(rmhmc_ctx* ctx, const MassTerm& m, const double* b, double tol,
             tri.build(kr);
             CombineSpec spec;
             shifted_rows(tri, std::vector<double>{m.sigma[j]}, m.sigma[j], spec);
-            if (mixed) {
-                float* o[1] = {e32};
-                RM_TRY((krylov_combine<float, float>(ctx, spec, o, st)));
-                RM_TRY(add_float_to_double(ctx, e32, outs[j], fs, st));
-            } else {
-                double* o[1] = {e64};
-                RM_TRY((krylov_combine<double, double>(ctx, spec, o, st)));
-                RM_TRY(axpby64(ctx, 1.0, outs[j], 1.0, e64, outs[j], fs, st));
-            }
+            double* o[1] = {outs[j]};
+            if (mixed) RM_TRY((krylov_combine<float, double>(ctx, spec, o, st, true)));
+            else RM_TRY((krylov_combine<double, double>(ctx, spec, o, st, true)));
         }
     }
     if (iters) *iters = total;
+    return RMHMC_OK;
+}
+
+// y = c b + sum_j alpha_j x_j, every field read once (a pass per pole read and wrote y twelve times more)
+struct PoleWeights { double w[24]; };
+__global__ void k_rational_sum(double c, const double* b, const double* __restrict__ xs, PoleWeights w, int ns, double* y,
+                               size_t n) {
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        double v = c * b[i];
+#pragma unroll 4
+        for (int j = 0; j < ns; j++) v = fma(w.w[j], __ldg(xs + (size_t)j * n + i), v);
+        y[i] = v;
+    }
+}
+
+static int rational_sum(rmhmc_ctx* ctx, const MassTerm& m, const double* b, const double* xs, double* y, cudaStream_t st) {
+    PoleWeights w{};
+    for (int j = 0; j < m.npole(); j++) w.w[j] = m.alpha[j];
+    const size_t n = field_elems(ctx);
+    k_rational_sum<<<elem_grid(ctx, n), kBlock, 0, st>>>(m.c, b, xs, w, m.npole(), y, n);
+    ++ctx->launches;
+    RM_LAUNCH_CHECK(ctx);
     return RMHMC_OK;
 }
 
@@ -847,8 +857,7 @@ int rational_apply(rmhmc_ctx* ctx, const MassTerm& m, const double* b, double to
         if (!xs) return status;
         RM_TRY(solve_shifts(ctx, m, b, tol, maxiter, prec, xs, &it, nullptr, st));
     }
-    RM_TRY(axpby64(ctx, m.c, b, 0.0, nullptr, Y, fs, st));
-    for (int j = 0; j < ns; j++) RM_TRY(axpby64(ctx, 1.0, Y, m.alpha[j], xs + (size_t)j * fs, Y, fs, st));
+    RM_TRY(rational_sum(ctx, m, b, xs, Y, st));
     if (iters) *iters = it;
     return RMHMC_OK;
 }
@@ -1263,8 +1272,7 @@ extern "C" int rat_mass_solve(rmhmc_ctx* ctx, const double* U, const double* b, 
         int it = 0;
         RM_TRY(solve_shifts(ctx, m, bf, tol, maxiter, prec, x, &it, resid ? resid + (size_t)f * nshift : nullptr, stream));
         // y_f = c b_f + sum_j alpha_j x_fj (float64)
-        RM_TRY(axpby64(ctx, c, bf, 0.0, nullptr, yf, fs, stream));
-        for (int j = 0; j < nshift; j++) RM_TRY(axpby64(ctx, 1.0, yf, alpha[j], x + (size_t)j * fs, yf, fs, stream));
+        RM_TRY(rational_sum(ctx, m, bf, x, yf, stream));
         if (iters) *iters += it;
     }
     return RMHMC_OK;

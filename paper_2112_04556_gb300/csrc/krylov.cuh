@@ -65,9 +65,9 @@ int cg_run_launch(rmhmc_ctx* ctx, const typename LinksOf<T>::type& U, const TI* 
                   long long* iters, cudaStream_t st);
 // basis pointer of the last run
 template <typename T> T* krylov_basis(rmhmc_ctx* ctx);
-// out[m] = sum_k coef[m][k] r_k for m < M (outputs as float or double)
+// out[m] = sum_k coef[m][k] r_k for m < M; add (M = 1): the combination is added to out[0]
 template <typename T, typename TO>
-int krylov_combine(rmhmc_ctx* ctx, const CombineSpec& spec, TO* const* outs, cudaStream_t st);
+int krylov_combine(rmhmc_ctx* ctx, const CombineSpec& spec, TO* const* outs, cudaStream_t st, bool add = false);
 
 // per-field residuals r_f = b - (A + sigma_f) x_f in float64 (x_f float64 [nf][V][4][8]), their squared
 // norms to host norm2[nf]; r (nullable) stores the residual fields
@@ -80,9 +80,8 @@ int adjoint_table(rmhmc_ctx* ctx, float** tab, cudaStream_t st);
 int resid_df(rmhmc_ctx* ctx, const float* tab, const double* b, const double* x, int nf, const double* sigma, float* r,
              double* norm2, cudaStream_t st);
 
-// float64 -> float32 field conversion and float32 correction accumulation
+// float64 -> float32 field conversion
 int to_float(rmhmc_ctx* ctx, const double* in, float* out, size_t n, cudaStream_t st);
-int add_float_to_double(rmhmc_ctx* ctx, const float* in, double* out, size_t n, cudaStream_t st);
 int axpby64(rmhmc_ctx* ctx, double a, const double* x, double b, const double* y, double* out, size_t n, cudaStream_t st);
 // squared norm of a float64 field (deterministic float64 sum)
 int norm2_64(rmhmc_ctx* ctx, const double* x, size_t n, double* out, cudaStream_t st);

@@ -128,15 +128,14 @@ __global__ void __launch_bounds__(kBlock) k_resid_df(Geom g, const float* __rest
             load8(b + (size_t)site * 32 + mu * 8, bb);
             float xh[8], xl[8];
             ld_pair(xf + ((size_t)site * 4 + mu) * 16, xh, xl);
-            const double dg = -(sig[f] + 0.5);
-            const float dh = (float)dg, dl = (float)(dg - (double)dh);
+            const dfl d = df_split(-(sig[f] + 0.5));
 #pragma unroll
             for (int a = 0; a < 8; a++) {
-                const float bh = (float)bb[a];
-                s[a] = bh;
-                c[a] = (float)(bb[a] - (double)bh);
-                dot2_acc(dh, xh[a], s[a], c[a]);
-                c[a] = __fmaf_rn(dh, xl[a], __fmaf_rn(dl, xh[a], c[a]));
+                const dfl v = df_split(bb[a]);   // integer operations, as k_split_pairs
+                s[a] = v.hi;
+                c[a] = v.lo;
+                dot2_acc(d.hi, xh[a], s[a], c[a]);
+                c[a] = __fmaf_rn(d.hi, xl[a], __fmaf_rn(d.lo, xh[a], c[a]));
             }
         }
         int fwd[4], bwd[4];
