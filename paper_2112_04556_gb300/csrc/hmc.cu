@@ -1118,11 +1118,11 @@ static int md_graph_run(rmhmc_ctx* ctx, double* U, double* P, const rmhmc_params
     memcpy(st, ctx->h_pinned, sizeof st);
     memcpy(ints, (char*)ctx->h_pinned + 128, sizeof ints);
     *used = true;
-    // kernels the graph ran: links, gauge force (1 to 4 kernels), momenta; 5 and a gauge force per step outside the loops; 6
-    // per fixed-point iteration (7 with the velocity in a kernel of its own); 2 per Krylov iteration unless a run is one
+    // kernels the graph ran: links, gauge force (1 to 4 kernels), momenta; 5 and a gauge force per step outside the loops; 5
+    // per fixed-point iteration (6 with the velocity in a kernel of its own); 2 per Krylov iteration unless a run is one
     // kernel
     const int gk = ctx->g.V > kLoopsMax || ctx->loops_off ? 1 : p->c1 != 0.0 ? 4 : 2;
-    ctx->launches += 2 + gk + (5LL + gk) * p->nsteps + (ctx->lg_mode == kLgFused ? 6 : 7) * (st[1] + st[2]) +
+    ctx->launches += 2 + gk + (5LL + gk) * p->nsteps + (ctx->lg_mode == kLgFused ? 5 : 6) * (st[1] + st[2]) +
                      (cg_run_fits<float>(ctx) ? 0 : 2 * st[0]);
     ctx->krylov_iters += st[0];
     ctx->links_valid = true;

@@ -142,6 +142,7 @@ __global__ void __launch_bounds__(256) k_pair_matrix(const double* __restrict__ 
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n * n; idx += gridDim.x * blockDim.x) {
         const int k = idx / n, l = idx % n;
         double s = 0.0;
+#pragma unroll 4
         for (int j = 0; j < ns; j++) {
             const double* X = rows + (size_t)j * ldr;
             const double* Z = rows + (size_t)(ns + j) * ldr;
@@ -450,10 +451,12 @@ int link_grad_krylov_launch(rmhmc_ctx* ctx, const float* R, const double* rows, 
     int status = RMHMC_OK;
     double* S = (double*)workspace(ctx, "kf_pairs", sizeof(double) * kBasisCap * kBasisCap, &status);
     if (!S) return status;
-    PairWeights pw{};
-    for (int j = 0; j < ns; j++) pw.w[j] = alpha[j];
-    k_pair_matrix<<<ctx->num_sms / 4 > 1 ? ctx->num_sms / 4 : 1, 256, 0, st>>>(rows, ldr, ns, pw, flags, n, S, kBasisCap);
-    ++ctx->launches;
+    if (rows) {
+        PairWeights pw{};
+        for (int j = 0; j < ns; j++) pw.w[j] = alpha[j];
+        k_pair_matrix<<<ctx->num_sms / 4 > 1 ? ctx->num_sms / 4 : 1, 256, 0, st>>>(rows, ldr, ns, pw, flags, n, S, kBasisCap);
+        ++ctx->launches;
+    }
     if (ctx->lg_mode == kLgFused) {
         if (Vel && cen) return launch_basis<true, true>(ctx, R, flags, n, S, F, cvel, Vel, cen, slot, st);
         if (Vel) return launch_basis<true, false>(ctx, R, flags, n, S, F, cvel, Vel, cen, slot, st);

@@ -1034,21 +1034,27 @@ __global__ void __launch_bounds__(kBlock) k_cgg_B(T* __restrict__ R, size_t fs, 
 }
 
 // Lanczos post-processing on the device (one block): from alpha, beta, rho of the run, the Galerkin coefficient
-// vectors y_j = (T + D_j)^{-1} e1 |b|, g = R(T) e1 |b|, z_j = (T + D_j)^{-1} g, v = R(T) g, written as rows on the
-// stored residuals: rows j < ns: X_j, rows ns + j: Z_j, row 2 ns: V.  Row stride: kBasisCap.  A run that did not
-// converge (cap or NaN) is recorded in *status.
+// vectors y_j = (T + D_j)^{-1} e1 |b|, g = R(T) e1 |b|, z_j = (T + D_j)^{-1} g, v = R(T) g on the stored residuals: the
+// velocity's row to row 2 ns of `rows` (stride kBasisCap; rows j < ns: X_j, rows ns + j: Z_j) and the pair matrix
+// S_kl = sum_j alpha_j (X_jk Z_jl + Z_jk X_jl) to S (stride kBasisCap).  A run that did not converge (cap or NaN) is recorded
+// in *status.
+// What bounds it: one thread per pole walks the tridiagonal recurrences, a chain of float64 divisions.  Both solves of a
+// pole share one factorisation (a division per row, where two solves took four), and runs of up to kLzN keep everything in
+// shared memory.
 struct DevMass {
     int ns;
     double c;
     double alpha[24];
     double delta[24];
 };
+constexpr int kLzN = 32, kLzPoles = 15;   // 2 ns + 1 <= kMaxCombine
 
 __global__ void __launch_bounds__(128) k_lanczos_rows(const int* __restrict__ flags, const double* __restrict__ vals, int maxit,
                                                       DevMass m, double* __restrict__ rows, double* __restrict__ work,
-                                                      int* status) {
+                                                      double* __restrict__ S, int* status) {
     constexpr int N = 160;   // kBasisCap
     __shared__ double d[N], e[N], inv[N], g[N], v[N];
+    __shared__ double small[4 * kLzPoles * (kLzN + 1)];
     const int n = flags[1];
     const double* rho = vals;
     const double* alpha = vals + (maxit + 1) + maxit;
@@ -1061,42 +1067,58 @@ __global__ void __launch_bounds__(128) k_lanczos_rows(const int* __restrict__ fl
     }
     __syncthreads();
     const double bn = n > 0 ? sqrt(rho[0]) : 0.0;
-    // work: [ns][N] y_j, then [ns][N] z_j, then [ns][N] Thomas scratch
-    double* Y = work;
-    double* Z = work + (size_t)m.ns * N;
-    double* C = work + (size_t)2 * m.ns * N;
-    auto thomas = [&](double shift, const double* rhs, double* y, double* c) {
-        if (n == 0) return;
-        double den = d[0] + shift;
-        c[0] = n > 1 ? e[0] / den : 0.0;
-        y[0] = rhs[0] / den;
+    // [ns] rows of y_j, z_j, the factor's off-diagonals and inverse pivots
+    const bool in_shared = n <= kLzN;
+    const int ld = in_shared ? kLzN + 1 : N;
+    double* Y = in_shared ? small : work;
+    double *Z = Y + m.ns * ld, *C = Z + m.ns * ld, *I = C + m.ns * ld;
+    auto solve = [&](const double* rhs, double* y, const double* c, const double* p) {
+        double t = rhs[0] * p[0];
+        y[0] = t;
         for (int k = 1; k < n; k++) {
-            den = d[k] + shift - e[k - 1] * c[k - 1];
-            c[k] = k < n - 1 ? e[k] / den : 0.0;
-            y[k] = (rhs[k] - e[k - 1] * y[k - 1]) / den;
+            t = fma(-e[k - 1], t, rhs[k]) * p[k];
+            y[k] = t;
         }
-        for (int k = n - 2; k >= 0; k--) y[k] -= c[k] * y[k + 1];
+        for (int k = n - 2; k >= 0; k--) {
+            t = fma(-c[k], t, y[k]);
+            y[k] = t;
+        }
     };
     for (int k = threadIdx.x; k < n; k += blockDim.x) v[k] = k == 0 ? bn : 0.0;   // e1 |b| (scratch)
     __syncthreads();
-    if (threadIdx.x < m.ns) thomas(m.delta[threadIdx.x], v, Y + (size_t)threadIdx.x * N, C + (size_t)threadIdx.x * N);
+    if (threadIdx.x < m.ns && n > 0) {
+        double *c = C + threadIdx.x * ld, *p = I + threadIdx.x * ld;
+        const double shift = m.delta[threadIdx.x];
+        double q = 0.0;
+        for (int k = 0; k < n; k++) {
+            const double r = 1.0 / (k > 0 ? fma(-e[k - 1], q, d[k] + shift) : d[0] + shift);
+            q = e[k] * r;
+            p[k] = r;
+            c[k] = q;
+        }
+        solve(v, Y + threadIdx.x * ld, c, p);
+    }
     __syncthreads();
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
         double t = m.c * (k == 0 ? bn : 0.0);
-        for (int j = 0; j < m.ns; j++) t += m.alpha[j] * Y[(size_t)j * N + k];
+        for (int j = 0; j < m.ns; j++) t += m.alpha[j] * Y[j * ld + k];
         g[k] = t;
     }
     __syncthreads();
-    if (threadIdx.x < m.ns) thomas(m.delta[threadIdx.x], g, Z + (size_t)threadIdx.x * N, C + (size_t)threadIdx.x * N);
+    if (threadIdx.x < m.ns && n > 0)
+        solve(g, Z + threadIdx.x * ld, C + threadIdx.x * ld, I + threadIdx.x * ld);
     __syncthreads();
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
         double t = m.c * g[k];
-        for (int j = 0; j < m.ns; j++) t += m.alpha[j] * Z[(size_t)j * N + k];
+        for (int j = 0; j < m.ns; j++) t += m.alpha[j] * Z[j * ld + k];
         rows[(size_t)(2 * m.ns) * N + k] = t * inv[k];
-        for (int j = 0; j < m.ns; j++) {
-            rows[(size_t)j * N + k] = Y[(size_t)j * N + k] * inv[k];
-            rows[(size_t)(m.ns + j) * N + k] = Z[(size_t)j * N + k] * inv[k];
-        }
+    }
+    for (int i = threadIdx.x; i < n * n; i += blockDim.x) {
+        const int k = i / n, l = i - k * n;
+        double t = 0.0;
+        for (int j = 0; j < m.ns; j++)
+            t = fma(m.alpha[j], fma(Y[j * ld + k], Z[j * ld + l], Z[j * ld + k] * Y[j * ld + l]), t);
+        S[(size_t)k * N + l] = t * (inv[k] * inv[l]);
     }
 }
 
@@ -1152,7 +1174,7 @@ static int kin_graph_bufs(rmhmc_ctx* ctx, int ns, int maxit, KinGraphBufs& b) {
     b.q = (float*)workspace(ctx, "kg_q32", sizeof(float) * fs, &status);
     void* sc = workspace(ctx, "kg_scal", 64 + sizeof(double) * 4 * (size_t)(kBasisCap + 2), &status);
     b.rows = (double*)workspace(ctx, "kg_rows", sizeof(double) * kBasisCap * (size_t)(2 * ns + 1), &status);
-    b.work = (double*)workspace(ctx, "kg_work", sizeof(double) * kBasisCap * (size_t)(3 * ns + 1), &status);
+    b.work = (double*)workspace(ctx, "kg_work", sizeof(double) * kBasisCap * (size_t)(4 * ns), &status);
     b.pairs = (double*)workspace(ctx, "kf_pairs", sizeof(double) * kBasisCap * kBasisCap, &status);
     if (!b.R || !b.q || !sc || !b.rows || !b.work || !b.pairs) return status;
     b.flags = (int*)sc;
@@ -1221,7 +1243,7 @@ int kinetic_enqueue(rmhmc_ctx* ctx, const MassTerm& m, const double* P, double t
             RM_CHECK(ctx, cudaStreamEndCapture(aux, &tmp));
         }
     }
-    k_lanczos_rows<<<1, 128, 0, st>>>(b.flags, b.vals, b.maxit, dm, b.rows, b.work, status); ++ctx->launches;
+    k_lanczos_rows<<<1, 128, 0, st>>>(b.flags, b.vals, b.maxit, dm, b.rows, b.work, b.pairs, status); ++ctx->launches;
     RM_LAUNCH_CHECK(ctx);
     const double* cvel = b.rows + (size_t)2 * ns * kBasisCap;
     if (ctx->lg_mode != kLgFused) {
@@ -1232,8 +1254,9 @@ int kinetic_enqueue(rmhmc_ctx* ctx, const MassTerm& m, const double* P, double t
         ++ctx->launches;
         RM_LAUNCH_CHECK(ctx);
     }
-    return link_grad_krylov_launch(ctx, b.R, b.rows, kBasisCap, ns, m.alpha.data(), b.flags, 0, F, cvel, Vel, nullptr,
-                                   kSlotNorm, st);
+    // the pair matrix is in place: no rows to form it from
+    return link_grad_krylov_launch(ctx, b.R, nullptr, kBasisCap, ns, nullptr, b.flags, 0, F, cvel, Vel, nullptr, kSlotNorm,
+                                   st);
 }
 
 }  // namespace rm

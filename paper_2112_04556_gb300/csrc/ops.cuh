@@ -47,6 +47,7 @@ int link_update_launch(rmhmc_ctx* ctx, const double* Uin, const double* V, doubl
 // kinetic force G = sum_j alpha_j d<Z_j, A X_j>/dw straight from the float32 Krylov basis R (n vectors), with
 // X_j, Z_j given as rows of basis coefficients (rows j and ns + j, row stride ldr, device float64); n is
 // read on the device from flags[1] when flags is not null.  G float64 [V][4][8].
+// rows may be null: the pair matrix is then in the workspace "kf_pairs" already.
 // With cvel, cen (coefficients on the basis) the velocity sum_k cvel[k] r_k goes to Vel and |sum_k cen[k] r_k|^2 to the
 // reduction slot in the same pass, if that kernel is selected (ctx->lg_mode == kLgFused; the other one computes G only).
 constexpr int kLgFused = 4;
