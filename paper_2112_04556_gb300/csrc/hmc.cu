@@ -1081,21 +1081,30 @@ static int md_graph_run(rmhmc_ctx* ctx, double* U, double* P, const rmhmc_params
             ctx->md_exec = nullptr;
         }
         const long long saved = ctx->launches;
-        cudaGraph_t g = nullptr;
-        const int s = md_graph_capture(ctx, p, m, gb, w, lg, &g);
-        ctx->launches = saved;
-        if (s != RMHMC_OK) {
-            ctx->graph_note = "capture failed: " + ctx->err;
+        // a second attempt without the cooperative Krylov run: a device shared through MPS does not take cooperative kernels
+        // inside conditional nodes
+        for (int attempt = 0; !ctx->md_exec; attempt++) {
+            const bool last = attempt == 1 || !cg_run_fits<float>(ctx);
+            cudaGraph_t g = nullptr;
+            const int s = md_graph_capture(ctx, p, m, gb, w, lg, &g);
+            ctx->launches = saved;
+            cudaError_t e = cudaSuccess;
+            if (s == RMHMC_OK) {
+                e = cudaGraphInstantiate(&ctx->md_exec, g, 0);
+                cudaGraphDestroy(g);
+                if (e == cudaSuccess) break;
+                cudaGetLastError();
+                ctx->md_exec = nullptr;
+            }
+            if (!last) {
+                ctx->cg_run_off = true;
+                ctx->err.clear();
+                RM_TRY(kinetic_graph_prepare(ctx, m, p->maxiter));   // the two-kernel form's shape, before the capture
+                continue;
+            }
+            ctx->graph_note = s != RMHMC_OK ? "capture failed: " + ctx->err
+                                            : std::string("instantiate failed: ") + cudaGetErrorString(e);
             ctx->err.clear();
-            ctx->use_graphs = false;
-            return RMHMC_OK;
-        }
-        const cudaError_t e = cudaGraphInstantiate(&ctx->md_exec, g, 0);
-        cudaGraphDestroy(g);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            ctx->md_exec = nullptr;
-            ctx->graph_note = std::string("instantiate failed: ") + cudaGetErrorString(e);
             ctx->use_graphs = false;
             return RMHMC_OK;
         }
