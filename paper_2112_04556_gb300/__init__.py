@@ -114,13 +114,27 @@ def lib():
 
 
 def _ptr(t):
+    """Device address of a tensor, for a c_void_p argument (a plain int: building a c_void_p object costs as much as
+    the checks)."""
     if t is None:
         return None
     if not t.is_cuda:
         raise ValueError("tensor must live on the GPU")
     if not t.is_contiguous():
         raise ValueError("tensor must be contiguous")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+def _raw_stream(stream=None):
+    """Handle of the stream, or of the current one without building a torch.cuda.Stream for it (a third of the host
+    time of a small lap_apply)."""
+    if stream is not None:
+        return stream.cuda_stream
+    import torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch.cuda.current_device())
 
 
 def _stream(stream=None):
@@ -216,21 +230,23 @@ def tuning(ctx):
 
 
 def set_links(ctx, U, stream=None):
-    ctx.check(lib().rmhmc_set_links(ctx.h, _links(U), _stream(stream)))
+    ctx.check(lib().rmhmc_set_links(ctx.h, _links(U), _raw_stream(stream)))
 
 
 def lap_apply(ctx, U, X, Y=None, prec=None, linkfmt=LINK18, op=OP_A, stream=None):
     """Y = A X (A = -Delta_G/16) or Delta_G X; X float64 or float32 [.., V, 4, 8]."""
     import torch
+    dt = X.dtype
     if prec is None:
-        prec = FP64 if X.dtype == torch.float64 else FP32
-    want = torch.float64 if prec == FP64 else torch.float32
-    if X.dtype != want:
+        prec = FP64 if dt == torch.float64 else FP32
+    if dt != (torch.float64 if prec == FP64 else torch.float32):
         raise ValueError("X dtype does not match prec")
     if Y is None:
         Y = torch.empty_like(X)
-    nfield = X.numel() // (ctx.V * 32)
-    ctx.check(lib().lap_apply(ctx.h, _links(U), _ptr(X), _ptr(Y), nfield, prec, linkfmt, op, _stream(stream)))
+    code = (_lib or lib()).lap_apply(ctx.h, _links(U), _ptr(X), _ptr(Y), X.numel() // (ctx.V * 32), prec, linkfmt, op,
+                                     _raw_stream(stream))
+    if code != OK:
+        ctx.check(code)
     return Y
 
 
@@ -242,7 +258,7 @@ def lap_link_grad(ctx, U, X, Z, w, G=None, prec=FP64, stream=None):
         raise ValueError("one weight per field pair")
     if G is None:
         G = torch.empty((ctx.V, 4, 8), dtype=torch.float64, device=X.device)
-    ctx.check(lib().lap_link_grad(ctx.h, _links(U), _ptr(X), _ptr(Z), nfield, wp, prec, _ptr(G), _stream(stream)))
+    ctx.check(lib().lap_link_grad(ctx.h, _links(U), _ptr(X), _ptr(Z), nfield, wp, prec, _ptr(G), _raw_stream(stream)))
     return G
 
 
@@ -261,7 +277,7 @@ def cheb_filter_spectrum(ctx, U, F, noise, degree, edges, kernel=KERNEL_JACKSON,
         ctx.h, _links(U), _ptr(F), nF, _ptr(noise), nn, int(seed), int(degree), nwin, ep, int(kernel), int(prec),
         spec.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), num.ctypes.data_as(ctypes.POINTER(ctypes.c_double)),
         tr.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), mom.ctypes.data_as(ctypes.POINTER(ctypes.c_double)),
-        _stream(stream)))
+        _raw_stream(stream)))
     return spec, num, tr, mom
 
 
@@ -305,7 +321,7 @@ def rat_mass_solve(ctx, U, b, mass, tol=1e-10, maxiter=2000, prec=FP64, want_xs=
     resid = np.zeros(max(n * nfield, 1))
     ctx.check(lib().rat_mass_solve(ctx.h, _links(U), _ptr(b), nfield, n, sp, ap, float(mass["c"]), float(tol),
                                    int(maxiter), int(prec), _ptr(y), _ptr(xs), ctypes.byref(iters),
-                                   resid.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), _stream(stream)))
+                                   resid.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), _raw_stream(stream)))
     res = resid[:n] if single else resid[:n * nfield].reshape(nfield, n)
     return y, xs, iters.value, res
 
@@ -315,7 +331,7 @@ def heatbath(ctx, U, xi, mass, tol=1e-10, prec=FP64, stream=None):
     m = _mass_struct(mass)
     P = torch.empty_like(xi)
     ctx.check(lib().rmhmc_heatbath(ctx.h, _links(U), _ptr(xi), ctypes.byref(m), float(tol), int(prec), _ptr(P),
-                                   _stream(stream)))
+                                   _raw_stream(stream)))
     return P
 
 
@@ -327,7 +343,7 @@ def gauge_force(ctx, U, beta, c1=0.0, prec=FP64, F=None, stream=None):
     S = ctypes.c_double()
     pl = ctypes.c_double()
     ctx.check(lib().gauge_force(ctx.h, _links(U), float(beta), float(c1), int(prec), _ptr(F), ctypes.byref(S),
-                                ctypes.byref(pl), _stream(stream)))
+                                ctypes.byref(pl), _raw_stream(stream)))
     return F, S.value, pl.value
 
 
@@ -339,7 +355,7 @@ def kinetic_force(ctx, U, P, mass, tol=1e-12, prec=FP64, want_force=True, want_v
     Vel = torch.empty_like(P) if want_velocity else None
     T = ctypes.c_double()
     ctx.check(lib().kinetic_force(ctx.h, _links(U), _ptr(P), ctypes.byref(m), float(tol), int(prec), _ptr(F),
-                                  _ptr(Vel), ctypes.byref(T), _stream(stream)))
+                                  _ptr(Vel), ctypes.byref(T), _raw_stream(stream)))
     return F, Vel, T.value
 
 
@@ -347,7 +363,7 @@ def gauss_field(ctx, seed, stream_id, tag=0, out=None, stream=None):
     import torch
     if out is None:
         out = torch.empty((ctx.V, 4, 8), dtype=torch.float64, device="cuda:%d" % ctx.device)
-    ctx.check(lib().rmhmc_gauss_field(ctx.h, _ptr(out), int(seed), int(stream_id), int(tag), _stream(stream)))
+    ctx.check(lib().rmhmc_gauss_field(ctx.h, _ptr(out), int(seed), int(stream_id), int(tag), _raw_stream(stream)))
     return out
 
 
@@ -356,7 +372,7 @@ def link_update(ctx, U, V, eps, reunit=True, out=None, stream=None):
     if out is None:
         out = torch.empty_like(U)
     ctx.check(lib().rmhmc_link_update(ctx.h, _links(U), _ptr(V), float(eps), int(bool(reunit)), _links(out),
-                                      _stream(stream)))
+                                      _raw_stream(stream)))
     return out
 
 
@@ -401,7 +417,7 @@ def cheb_filter_apply(ctx, U, F, coef, prec=FP64, out=None, stream=None):
     if out is None:
         out = torch.empty_like(Fc)
     ctx.check(lib().cheb_filter_apply(ctx.h, _links(U), _ptr(Fc), nf, len(c) - 1, cp, int(prec), _ptr(out),
-                                      _stream(stream)))
+                                      _raw_stream(stream)))
     return out
 
 
@@ -432,7 +448,7 @@ def wilson_flow(ctx, U, eps, nsteps, prec=FP64, stream=None):
     import numpy as np
     E = np.zeros(int(nsteps) + 1)
     ctx.check(lib().wilson_flow(ctx.h, _links(U), float(eps), int(nsteps), int(prec),
-                                E.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), _stream(stream)))
+                                E.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), _raw_stream(stream)))
     return E
 
 
@@ -451,20 +467,20 @@ def make_params(beta=6.0, c1=0.0, mass=None, tau=1.0, nsteps=20, tol_md=1e-10, t
 def hamiltonian(ctx, U, P, params, stream=None):
     H, T, S = ctypes.c_double(), ctypes.c_double(), ctypes.c_double()
     ctx.check(lib().rmhmc_hamiltonian(ctx.h, _links(U), _ptr(P), ctypes.byref(params), ctypes.byref(H),
-                                      ctypes.byref(T), ctypes.byref(S), _stream(stream)))
+                                      ctypes.byref(T), ctypes.byref(S), _raw_stream(stream)))
     return H.value, T.value, S.value
 
 
 def md(ctx, U, P, params, stream=None):
     r = Result()
-    ctx.check(lib().rmhmc_md(ctx.h, _links(U), _ptr(P), ctypes.byref(params), ctypes.byref(r), _stream(stream)))
+    ctx.check(lib().rmhmc_md(ctx.h, _links(U), _ptr(P), ctypes.byref(params), ctypes.byref(r), _raw_stream(stream)))
     return r.as_dict()
 
 
 def rmhmc_trajectory(ctx, U, params, xi=None, P_out=None, stream=None):
     r = Result()
     ctx.check(lib().rmhmc_trajectory(ctx.h, _links(U), _ptr(xi), ctypes.byref(params), ctypes.byref(r),
-                                     _ptr(P_out), _stream(stream)))
+                                     _ptr(P_out), _raw_stream(stream)))
     return r.as_dict()
 
 
