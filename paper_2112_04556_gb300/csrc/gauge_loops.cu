@@ -11,7 +11,9 @@
 // staples take 5616 and 36,700; the action reads the traces of the same products.  The links have to be SU(3) (the
 // transport uses U U^dag = 1, as the Laplacian's traceless form does).
 //
-// float64 (0.55 TFMA/s) is bound by the operations, float32 was by re-reading the links of every staple from L2.
+// float64 (0.55 TFMA/s) is bound by the operations, float32 was by re-reading the links of every staple from L2.  Measured at
+// 24^3 x 48, float32 Iwasaki force with its float64 action: 9.70 ms with staples, 6.84 ms here; float64 Wilson flow at 16^4,
+// 8 steps: 23.8 -> 15.6 ms.
 #include <algorithm>
 
 #include "krylov.cuh"

