@@ -58,11 +58,9 @@ DH_BAR = 1e-3
 # setting's trajectories use 64 steps
 PAIR_NSTEPS = 40
 ACCEPT_NSTEPS = 64
-# DRAM bytes (read + write) of one k_cg_A<float,18> launch at 32^4, mean of three consecutive CG iterations of
-# one ncu capture per launch shape (dram__bytes_read.sum + dram__bytes_write.sum;
-# profiles/k_cg_A_fp32_32x32x32x32.md), keyed by the tuned shape (components per lane, threads per block); a
-# shape without a capture reports null
-CG_TRAFFIC_32 = {(1, 256): 880.3e6, (2, 256): 885.9e6, (1, 128): 877.0e6, (0, 128): 936.9e6, (0, 256): 936.9e6}
+# DRAM bytes (read + write) of one k_cg_A<float,18> launch at 32^4 by ncu (dram__bytes_read.sum + dram__bytes_write.sum), keyed
+# by the tuned shape (components per lane, threads per block); a shape without a capture of the kernel as it is reports null
+CG_TRAFFIC_32 = {}
 # algorithmic bytes per site of the conjugate-gradient stencil k_cg_A<float,18> (float32, 18-real links):
 # read r_k (128 B) and q_{k-1} (128 B), write q_k (128 B), four links of 72 B
 CG_BYTES_PER_SITE = 3 * 128 + 4 * 72
