@@ -27,7 +27,10 @@ struct PairWeights { double w[kMaxPairs]; };
 // so that a pair costs two outer products per component (576 operations per link with the weights) and the conjugation
 // by U comes once, for C.  The form above takes two conjugations and two matrix products per pair and component, 2016 FMA
 // a link, which float64 (0.55 TFMA/s) is bound by: float64 at 16^4, 12 pairs 11.5 -> 3.5 ms, one pair 1.01 -> 0.7 ms.
-// Four lanes per link, two columns d of C each; the contraction with f meets in shared memory.
+// Four lanes per link, two columns d of C each; the contraction with f meets in shared memory.  Where the stencils have the
+// table of R (LF = kLinkAd; built once per set of links) a column costs its 64 FMA instead of a conjugation's 108 and its
+// expansions: differentiated Laplacian at 16^4 1.623 -> 1.590 ms, kinetic force with 12 pairs 13.35 -> 13.20 ms, and the error
+// against 64 bits 4.6e-16 -> 3.5e-16.
 template <typename T, int LF>
 __global__ void __launch_bounds__(kBlock) k_link_grad(Geom g, typename LinksOf<T>::type U, const T* __restrict__ X,
                                                        const T* __restrict__ Z, size_t fs, int nf, PairWeights w,
@@ -40,7 +43,6 @@ __global__ void __launch_bounds__(kBlock) k_link_grad(Geom g, typename LinksOf<T
     T* const rc = rcs[threadIdx.x >> 2];
     if (live) {
         const size_t yo = (size_t)y * 32 + 2 * q, yn = (size_t)step_site(g, y, nu, 1) * 32;
-        const mat3<T> u = LinkLoad<T, LF>::load(U, y, nu);
         T C[2][8];
 #pragma unroll
         for (int i = 0; i < 2; i++)
@@ -62,15 +64,37 @@ __global__ void __launch_bounds__(kBlock) k_link_grad(Geom g, typename LinksOf<T
                 }
             }
         }
+        T r[2][8];
+        if constexpr (LF == kLinkAd) {
+            const double2* t = U.ad + (size_t)nu * 32 * U.V + y;
 #pragma unroll
-        for (int i = 0; i < 2; i++) {
-            T r[8];
-            herm<T> E = h_zero<T>();
-            acc_uxud_tl(E, u, coef_to_herm2(C[i]));
-            herm2_to_coef_tl(E, r);
+            for (int i = 0; i < 2; i++)
 #pragma unroll
-            for (int c = 0; c < 8; c++) rc[c * 8 + 2 * q + i] = r[c];
+                for (int c = 0; c < 8; c++) r[i][c] = 0.0;
+#pragma unroll
+            for (int b = 0; b < 8; b++)
+#pragma unroll
+                for (int a = 0; a < 4; a++) {
+                    const double2 v = __ldg(t + (size_t)(4 * b + a) * U.V);
+#pragma unroll
+                    for (int i = 0; i < 2; i++) {
+                        r[i][2 * a] = fma(v.x, C[i][b], r[i][2 * a]);
+                        r[i][2 * a + 1] = fma(v.y, C[i][b], r[i][2 * a + 1]);
+                    }
+                }
+        } else {
+            const mat3<T> u = LinkLoad<T, LF>::load(U, y, nu);
+#pragma unroll
+            for (int i = 0; i < 2; i++) {
+                herm<T> E = h_zero<T>();
+                acc_uxud_tl(E, u, coef_to_herm2(C[i]));
+                herm2_to_coef_tl(E, r[i]);
+            }
         }
+#pragma unroll
+        for (int i = 0; i < 2; i++)
+#pragma unroll
+            for (int c = 0; c < 8; c++) rc[c * 8 + 2 * q + i] = r[i][c];
     }
     __syncwarp();
     if (live) {
@@ -94,10 +118,16 @@ int link_grad_launch(rmhmc_ctx* ctx, int prec, const void* X, const void* Z, int
     PairWeights pw{};
     for (int f = 0; f < nf; f++) pw.w[f] = w[f];
     const dim3 grid(lane_blocks(ctx), 4);
-    if (prec == RMHMC_FP64)
-        k_link_grad<double, 18><<<grid, kBlock, 0, st>>>(ctx->g, links64(ctx), (const double*)X, (const double*)Z,
-                                                         field_elems(ctx), nf, pw, G);
-    else
+    if (prec == RMHMC_FP64) {
+        Links64 U = links64(ctx);
+        RM_TRY(links64_adjoint(ctx, &U, st));
+        if (U.ad)
+            k_link_grad<double, kLinkAd><<<grid, kBlock, 0, st>>>(ctx->g, U, (const double*)X, (const double*)Z,
+                                                                  field_elems(ctx), nf, pw, G);
+        else
+            k_link_grad<double, 18><<<grid, kBlock, 0, st>>>(ctx->g, U, (const double*)X, (const double*)Z,
+                                                             field_elems(ctx), nf, pw, G);
+    } else
         k_link_grad<float, 18><<<grid, kBlock, 0, st>>>(ctx->g, links32(ctx), (const float*)X, (const float*)Z,
                                                         field_elems(ctx), nf, pw, G);
     ++ctx->launches;
