@@ -58,9 +58,11 @@ DH_BAR = 1e-3
 # setting's trajectories use 64 steps
 PAIR_NSTEPS = 40
 ACCEPT_NSTEPS = 64
-# DRAM bytes (read + write) of one k_cg_A<float,18> launch at 32^4 by ncu (dram__bytes_read.sum + dram__bytes_write.sum), keyed
-# by the tuned shape (components per lane, threads per block); a shape without a capture of the kernel as it is reports null
-CG_TRAFFIC_32 = {}
+# DRAM bytes (read + write) of one k_cg_A<float,18> launch at 32^4, mean of three consecutive CG iterations of
+# one ncu capture per launch shape (dram__bytes_read.sum + dram__bytes_write.sum;
+# profiles/k_cg_A_fp32_32x32x32x32.md), keyed by the tuned shape (components per lane, threads per block); a
+# shape without a capture reports null
+CG_TRAFFIC_32 = {(2, 256): 907.0e6, (4, 256): 811.7e6, (1, 256): 871.6e6, (2, 128): 904.7e6}
 # algorithmic bytes per site of the conjugate-gradient stencil k_cg_A<float,18> (float32, 18-real links):
 # read r_k (128 B) and q_{k-1} (128 B), write q_k (128 B), four links of 72 B
 CG_BYTES_PER_SITE = 3 * 128 + 4 * 72
