@@ -264,17 +264,20 @@ template <typename T> bool cg_run_fits(const rmhmc_ctx* ctx) {
 // the barrier words (64 bytes; they wrap and count on from launch to launch) and two arrays of partials
 int cg_run_reset(rmhmc_ctx* ctx, cudaStream_t st) {
     auto it = ctx->bufs.find("cg_run");
-    if (it != ctx->bufs.end()) RM_CHECK(ctx, cudaMemsetAsync(it->second.p, 0, 64, st));
+    if (it != ctx->bufs.end() && it->second.p) RM_CHECK(ctx, cudaMemsetAsync(it->second.p, 0, 64, st));
     return RMHMC_OK;
 }
 
-int cg_run_prepare(rmhmc_ctx* ctx) {
-    if (ctx->bufs.count("cg_run")) return RMHMC_OK;
+int cg_run_prepare(rmhmc_ctx* ctx, unsigned** bar) {
     int status = RMHMC_OK;
+    const unsigned long long gen = ctx->ws_gen;
     void* p = workspace(ctx, "cg_run", 64 + sizeof(double) * 2 * ctx->num_sms, &status);
     if (!p) return status;
-    RM_CHECK(ctx, cudaMemset(p, 0, 64));
-    RM_CHECK(ctx, cudaDeviceSynchronize());   // the caller's stream may not follow the legacy stream
+    if (ctx->ws_gen != gen) {   // a new buffer
+        RM_CHECK(ctx, cudaMemset(p, 0, 64));
+        RM_CHECK(ctx, cudaDeviceSynchronize());   // the caller's stream may not follow the legacy stream
+    }
+    if (bar) *bar = (unsigned*)p;
     return RMHMC_OK;
 }
 
@@ -282,8 +285,8 @@ template <typename T, typename TI>
 int cg_run_launch(rmhmc_ctx* ctx, const typename LinksOf<T>::type& links, const TI* b, T* R, double diag, int* flags, double* vals, int maxit, double tol2,
                   long long* iters, cudaStream_t st) {
     const CgRunShape s = cg_run_shape<T>(ctx);
-    RM_TRY(cg_run_prepare(ctx));
-    unsigned* bar = (unsigned*)ctx->bufs["cg_run"].p;
+    unsigned* bar = nullptr;
+    RM_TRY(cg_run_prepare(ctx, &bar));
     double* part = (double*)((char*)bar + 64);
     typename LinksOf<T>::type U = links;
     Geom g = ctx->g;

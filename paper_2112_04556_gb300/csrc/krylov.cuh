@@ -57,7 +57,7 @@ int krylov_run(rmhmc_ctx* ctx, const TI* b, double sigma0, double tol, int maxit
 // form at 262,144 sites in float32, 2 % at 122,880 in float64
 constexpr int kCgRunMax32 = 1 << 18, kCgRunMax64 = 1 << 17;
 template <typename T> bool cg_run_fits(const rmhmc_ctx* ctx);
-int cg_run_prepare(rmhmc_ctx* ctx);
+int cg_run_prepare(rmhmc_ctx* ctx, unsigned** bar = nullptr);
 int cg_run_reset(rmhmc_ctx* ctx, cudaStream_t st);
 template <typename T> struct LinksOf;
 template <typename T, typename TI>

@@ -1,0 +1,93 @@
+"""The library's host side without a GPU: linked with a stand-in for the CUDA runtime (tests/fake/cudart.cpp: host memory,
+kernels recorded but not run), the entry points choose their routes, allocate and report errors as they do on the device.
+Allocations, cooperative launches and the device's size are the test's to set."""
+import ctypes
+import glob
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.fixture(scope="module")
+def fake_library(tmp_path_factory):
+    import __graft_entry__ as ge
+    ge.build_library()
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
+    so = str(tmp_path_factory.mktemp("fake") / "librmhmc_fake.so")
+    srcs = {os.path.basename(f) for f in glob.glob(os.path.join(ROOT, "paper_2112_04556_gb300", "csrc", "*.c*"))}
+    objs = [o for o in glob.glob(os.path.join(ROOT, "paper_2112_04556_gb300", "_build", "*.o"))
+            if os.path.basename(o)[:-2] in srcs]
+    subprocess.run(["g++", "-shared", "-fPIC", "-O1", "-std=c++17", "-I", inc, "-Wl,-Bsymbolic", "-Wl,--no-undefined",
+                    "-o", so, os.path.join(ROOT, "tests", "fake", "cudart.cpp")] + objs, check=True)
+    return so
+
+
+@pytest.fixture
+def rm(fake_library, monkeypatch):
+    import paper_2112_04556_gb300 as rm
+    monkeypatch.setattr(rm, "_SO", fake_library)
+    monkeypatch.setattr(rm, "_lib", None)
+    L = rm.lib()
+    L.fake_report.restype = ctypes.c_char_p
+    L.fake_watched.restype = L.fake_held.restype = ctypes.c_longlong
+    L.fake_device.argtypes = [ctypes.c_int, ctypes.c_longlong]
+    L.fake_room.argtypes = [ctypes.c_longlong]
+    L.fake_reset()
+    return rm
+
+
+# caller's buffers: the stand-in touches at most the first megabyte of a block
+_SPACE = np.zeros((4, (1 << 17) + 2))
+LINKS, FIELD, OUT, OUT2 = (a.ctypes.data + -a.ctypes.data % 16 for a in _SPACE)
+
+
+def launched(rm):
+    """Names of the kernels launched since the last call."""
+    names = rm.lib().fake_report().decode().split()
+    rm.lib().fake_clear_report()
+    return names
+
+
+def context(rm, L):
+    ctx = rm.Context(L)
+    ctx.check(rm.lib().rmhmc_set_links(ctx.h, LINKS, None))
+    rm.lib().fake_poke(b"k_cg_run", 6, 0, 1)     # every Krylov run ends at once, converged with no iteration
+    rm.lib().fake_poke(b"k_cg_start", 3, 0, 1)
+    launched(rm)
+    return ctx
+
+
+def kinetic(rm, ctx, prec, mass=None):
+    m = rm._mass_struct(mass or rm.mass_fit(12, 0.9))
+    T = ctypes.c_double()
+    return rm.lib().kinetic_force(ctx.h, None, FIELD, ctypes.byref(m), 1e-6, prec, OUT, OUT2, ctypes.byref(T), None)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_a_failed_allocation_leaves_the_context_usable(rm, prec):
+    """Whichever allocation of a kinetic evaluation fails, the call says ENOMEM (or does without the buffer) and the
+    next one runs on buffers that exist: the barrier of the cooperative run (arguments 12 and 13) among them."""
+    n = 0
+    while True:
+        n += 1
+        with context(rm, (4, 4, 4, 4)) as ctx:
+            rm.lib().fake_fail_at(n)
+            code = kinetic(rm, ctx, prec)
+            reached = not rm.lib().fake_fail_pending()
+            rm.lib().fake_fail_at(0)
+            assert code in (rm.OK, rm.ENOMEM)
+            for arg in (12, 13):
+                rm.lib().fake_watch(b"k_cg_run", arg)
+                launched(rm)
+                assert kinetic(rm, ctx, prec) == rm.OK
+                if any("k_cg_run" in k for k in launched(rm)):
+                    assert rm.lib().fake_watched() > 0, (n, arg)
+        if not reached:
+            break
+    assert n > 4
