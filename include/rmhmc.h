@@ -180,6 +180,11 @@ int rmhmc_get_counters(rmhmc_ctx* ctx, long long* launches, long long* krylov_it
  * on by default. */
 int rmhmc_set_graphs(rmhmc_ctx* ctx, int on);
 
+/* Limit of the device-side waits (the grid barriers of a Krylov run on up to 2^18 sites): a block that has polled
+ * a barrier this many times gives up, the run ends, and the call that made it returns RMHMC_ETIMEOUT; the context stays
+ * usable.  The default, 2^21, is about two seconds; 0 gives up every wait.  RMHMC_EINVAL for polls < 0. */
+int rmhmc_set_wait_limit(rmhmc_ctx* ctx, int polls);
+
 /* Text report of the stencil launch shapes the autotuner chose in this context (components per lane and
  * threads per block for each precision and link format, with the measured times of every candidate),
  * written NUL-terminated into buf[len]. */

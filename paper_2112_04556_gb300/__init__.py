@@ -95,6 +95,7 @@ def lib():
         "rmhmc_set_profiling": ([P, I], I),
         "rmhmc_tuning": ([P, ctypes.c_char_p, I], I),
         "rmhmc_set_graphs": ([P, I], I),
+        "rmhmc_set_wait_limit": ([P, I], I),
         "rmhmc_set_stencil_shape": ([P, I, I, I, I, I], I),
         "wilson_flow": ([P, P, D, I, I, DP, P], I),
         "cheb_window_coeffs": ([I, DP, I, I, DP], I),
@@ -212,6 +213,11 @@ def counters(ctx, reset=False):
 def set_graphs(ctx, on=True):
     """Run the mixed-precision MD as one CUDA graph (default) or host-driven."""
     ctx.check(lib().rmhmc_set_graphs(ctx.h, int(bool(on))))
+
+
+def set_wait_limit(ctx, polls=1 << 21):
+    """Polls after which a device-side wait gives up (ETIMEOUT)."""
+    ctx.check(lib().rmhmc_set_wait_limit(ctx.h, int(polls)))
 
 
 SHAPE_LAP, SHAPE_CG, SHAPE_KFORCE, SHAPE_LINKUPDATE, SHAPE_ADJOINT = 0, 1, 2, 3, 4

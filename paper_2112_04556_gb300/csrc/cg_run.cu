@@ -20,21 +20,20 @@
 
 namespace rm {
 
-// polls of a grid barrier before a block gives up (each at least one L2 round trip: about two seconds); a cooperative
-// launch has all its blocks resident, so that only a lost block can run it out
-constexpr int kSpinLimit = 1 << 21;
-
 // Grid barrier with the sum of the blocks' values v (valid in thread 0) returned to all threads; the blocks' global
 // writes before it are visible after it.  The partials are added by the first warp of every block in a fixed order.
 // bar[0] counts arrivals (wrapping), bar[1] is the generation; part holds two arrays of gridDim.x, used in turn (a block
 // that runs ahead writes the other one, and comes back to this one only after all have left it).  Returns false in
 // every thread of a block whose wait ran out.  (Polling the partials themselves, tagged with the generation, saves the
-// counter's round trip but floods L2: 350 against 333 us for a kinetic evaluation at 8^4.)
+// counter's round trip but floods L2: 350 against 333 us for a kinetic evaluation at 8^4.)  limit: polls before a block
+// gives up (the default, kWaitPolls, is about two seconds at an L2 round trip each); a cooperative launch has all its
+// blocks resident, so that only a lost block can run it out.
 struct GridSum {
     unsigned* bar;
     double* part;
+    int limit;
     unsigned gen;
-    __device__ __forceinline__ GridSum(unsigned* b, double* p) : bar(b), part(p) {
+    __device__ __forceinline__ GridSum(unsigned* b, double* p, int l) : bar(b), part(p), limit(l) {
         gen = *reinterpret_cast<volatile unsigned*>(bar + 1);   // cannot change before this block has arrived
     }
     __device__ __forceinline__ bool operator()(double v, double& sum, double* sh) {
@@ -48,11 +47,9 @@ struct GridSum {
                 __threadfence();
                 asm volatile("st.release.gpu.u32 [%0], %1;" ::"l"(bar + 1), "r"(gen + 1) : "memory");
             } else {
-                unsigned now;
-                int n = 0;
-                do {
+                unsigned now = gen;
+                for (int n = 0; n < limit && now == gen; n++)
                     asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(now) : "l"(bar + 1) : "memory");
-                } while (now == gen && ++n < kSpinLimit);
                 if (now == gen) failed = 1;
             }
             __threadfence();
@@ -114,15 +111,17 @@ template <typename T> __device__ __forceinline__ double block_total(T x, double*
 }
 
 // NMU: 1, or 0 with the neighbours of a unit loaded ahead (hop_sum_shape); BLOCK: largest block; iters (nullable) counts
-// iterations; status 4: a barrier gave up
+// iterations.  flags[0] is the largest of what the blocks say, 4 (a barrier gave up) above every outcome of block 0: a block
+// can give up on a barrier that the others still pass.  (Block 0 clears it first.  A 4 from before that is lost only
+// where all blocks then pass the first barrier, and with it the run if it ends there: its work is complete.)
 template <typename T, typename TI, int NMU, int BLOCK>
 __global__ void __launch_bounds__(BLOCK, 1)
     k_cg_run(Geom g, typename LinksOf<T>::type U, const TI* __restrict__ b, T* R, size_t fs, T diag, int* flags, double* vals,
-             int maxit, double tol2, long long* iters, int units_per_block, double* part, unsigned* bar) {
+             int maxit, double tol2, long long* iters, int units_per_block, double* part, unsigned* bar, int limit) {
     extern __shared__ __align__(16) unsigned char cgs[];
     T* const qs = reinterpret_cast<T*>(cgs);   // [item][chunk][thread][4]
     __shared__ double shw[BLOCK / 32], sh[3];
-    GridSum gsum(bar, part);
+    GridSum gsum(bar, part, limit);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
     const int nunit = (g.V + 31) / 32 * 4;
     const int u0 = blockIdx.x * units_per_block + warp, u1 = min(nunit, (blockIdx.x + 1) * units_per_block);
@@ -131,6 +130,7 @@ __global__ void __launch_bounds__(BLOCK, 1)
     double* const alpha = gamma + maxit;
     double* const beta = alpha + maxit;
     const bool writer = blockIdx.x == 0 && threadIdx.x == 0;
+    if (writer) flags[0] = flags[1] = 0;   // readers of the vectors' number see 0 or the run's
     // r_0 = b in T, |r_0|^2 accurate to float64
     double rr;
     {
@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(BLOCK, 1)
         }
         const double t = block_total(sizeof(T) == 4 ? sf.value() : sd, shw);
         if (!gsum(t, rr, sh)) {
-            if (threadIdx.x == 0) { flags[1] = 0; flags[0] = 4; }
+            if (threadIdx.x == 0) atomicMax(flags, 4);
             return;
         }
     }
@@ -230,10 +230,10 @@ __global__ void __launch_bounds__(BLOCK, 1)
         else if (k >= maxit) done = 2;
     }
     if (done == 4) {
-        if (threadIdx.x == 0) { flags[1] = 0; flags[0] = 4; }
+        if (threadIdx.x == 0) atomicMax(flags, 4);
     } else if (writer) {
         flags[1] = k;
-        flags[0] = done;
+        atomicMax(flags, done);
         if (iters) *iters += k;
     }
 }
@@ -292,8 +292,8 @@ int cg_run_launch(rmhmc_ctx* ctx, const typename LinksOf<T>::type& links, const 
     Geom g = ctx->g;
     size_t fs = field_elems(ctx);
     T d = (T)diag;
-    int units = s.units;
-    void* args[] = {&g, &U, &b, &R, &fs, &d, &flags, &vals, &maxit, &tol2, &iters, &units, &part, &bar};
+    int units = s.units, limit = ctx->wait_limit;
+    void* args[] = {&g, &U, &b, &R, &fs, &d, &flags, &vals, &maxit, &tol2, &iters, &units, &part, &bar, &limit};
     const void* kern = (const void*)k_cg_run<T, TI, sizeof(T) == 8 ? 1 : 0, 256>;
     if constexpr (sizeof(T) == 4) {
         if (s.maxw == 24) kern = (const void*)k_cg_run<T, TI, 0, 768>;

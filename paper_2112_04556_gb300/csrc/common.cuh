@@ -312,6 +312,8 @@ __device__ __forceinline__ bool grid_sum_finish(const double* v, double* partial
 // ------------------------------------------------------------------------------------------------
 struct DevBuf { void* p = nullptr; size_t bytes = 0; };
 
+constexpr int kWaitPolls = 1 << 21;
+
 }  // namespace rm
 
 // ------------------------------------------------------------------------------------------------
@@ -369,7 +371,9 @@ struct rmhmc_ctx {
     int ad_slab = 0;
     // set when the device refuses the cooperative CG run
     bool cg_run_off = false;
-    // incremented by every rmhmc_set_stencil_shape: part of the key of a captured trajectory graph
+    // polls of a device-side wait before it gives up (rmhmc_set_wait_limit)
+    int wait_limit = rm::kWaitPolls;
+    // incremented by every rmhmc_set_stencil_shape and rmhmc_set_wait_limit: part of the key of a captured trajectory graph
     int shape_gen = 0;
     std::string tune_report;
     // counters: kernels launched; optional timing of the conjugate-gradient stencil launches

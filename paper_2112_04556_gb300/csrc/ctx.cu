@@ -226,6 +226,15 @@ extern "C" int rmhmc_tuning(const rmhmc_ctx* ctx, char* buf, int len) {
     return RMHMC_OK;
 }
 
+extern "C" int rmhmc_set_wait_limit(rmhmc_ctx* ctx, int polls) {
+    if (!ctx) return RMHMC_EINVAL;
+    ctx->err.clear();
+    if (polls < 0) return set_err(ctx, RMHMC_EINVAL, "wait limit: polls must be >= 0");
+    ctx->wait_limit = polls;
+    ctx->shape_gen++;
+    return RMHMC_OK;
+}
+
 extern "C" int rmhmc_set_stencil_shape(rmhmc_ctx* ctx, int kernel, int prec, int linkfmt, int nmu, int block) {
     if (!ctx) return RMHMC_EINVAL;
     ctx->err.clear();

@@ -1055,7 +1055,7 @@ __global__ void __launch_bounds__(128) k_lanczos_rows(const int* __restrict__ fl
     constexpr int N = 160;   // kBasisCap
     __shared__ double d[N], e[N], inv[N], g[N], v[N];
     __shared__ double small[4 * kLzPoles * (kLzN + 1)];
-    const int n = flags[1];
+    const int n = flags[0] == 4 ? 0 : flags[1];   // a run that gave up has no vectors
     const double* rho = vals;
     const double* alpha = vals + (maxit + 1) + maxit;
     const double* beta = alpha + maxit;

@@ -266,3 +266,28 @@ def test_cg_run_matches_two_kernel_form(L, prec, tol, bound):
         y2, _, iters2, _ = rm.rat_mass_solve(ctx, None, bd, m, tol=tol, prec=prec)
     assert rel_l2(host(y), host(y2)) <= bound
     assert abs(iters - iters2) <= 2 + iters // 20
+
+
+@pytest.mark.parametrize("L", [(4, 4, 4, 4), (8, 8, 8, 9), (12, 12, 14, 16)])
+@pytest.mark.parametrize("prec,tol", [(0, 1e-12), (1, 1e-10)])
+def test_wait_that_runs_out_is_reported(L, prec, tol):
+    """With a wait limit of no polls every block of the cooperative Krylov run but the last to arrive gives up at the
+    first barrier, and that one at the second: the call returns ETIMEOUT (whatever block 0 makes of the run), and with the
+    limit back the same context solves as before, bit for bit."""
+    import paper_2112_04556_gb300 as rm
+    b = inputs.gaussian_fields(L, 1, seed=34)[0]
+    m = rm.mass_fit(12, 0.9)
+    with rm.Context(L) as ctx:
+        Ud, bd = dev(inputs.random_links(L, eps=0.4, seed=33)), dev(b)
+        want = host(rm.rat_mass_solve(ctx, Ud, bd, m, tol=tol, prec=prec)[0])
+        rm.set_wait_limit(ctx, 0)
+        for call in (lambda: rm.rat_mass_solve(ctx, None, bd, m, tol=tol, prec=prec),
+                     lambda: rm.kinetic_force(ctx, None, bd, m, tol=1e-6, prec=prec)):
+            with pytest.raises(rm.RmhmcError) as e:
+                call()
+            assert e.value.code == rm.ETIMEOUT
+        rm.set_wait_limit(ctx)
+        assert np.array_equal(host(rm.rat_mass_solve(ctx, None, bd, m, tol=tol, prec=prec)[0]), want)
+        with pytest.raises(rm.RmhmcError) as e:
+            rm.set_wait_limit(ctx, -1)
+        assert e.value.code == rm.EINVAL
