@@ -114,10 +114,13 @@ template <typename T> __device__ __forceinline__ double block_total(T x, double*
 // iterations.  flags[0] is the largest of what the blocks say, 4 (a barrier gave up) above every outcome of block 0: a block
 // can give up on a barrier that the others still pass.  (Block 0 clears it first.  A 4 from before that is lost only
 // where all blocks then pass the first barrier, and with it the run if it ends there: its work is complete.)
+// status (nullable): the trajectory's status word.  After a run that gave up the barrier's counter is off until the host
+// clears it, so that the graph's later runs return at once.
 template <typename T, typename TI, int NMU, int BLOCK>
 __global__ void __launch_bounds__(BLOCK, 1)
     k_cg_run(Geom g, typename LinksOf<T>::type U, const TI* __restrict__ b, T* R, size_t fs, T diag, int* flags, double* vals,
-             int maxit, double tol2, long long* iters, int units_per_block, double* part, unsigned* bar, int limit) {
+             int maxit, double tol2, long long* iters, int units_per_block, double* part, unsigned* bar, int limit,
+             const int* status) {
     extern __shared__ __align__(16) unsigned char cgs[];
     T* const qs = reinterpret_cast<T*>(cgs);   // [item][chunk][thread][4]
     __shared__ double shw[BLOCK / 32], sh[3];
@@ -130,6 +133,7 @@ __global__ void __launch_bounds__(BLOCK, 1)
     double* const alpha = gamma + maxit;
     double* const beta = alpha + maxit;
     const bool writer = blockIdx.x == 0 && threadIdx.x == 0;
+    if (status && *status == kStatusGaveUp) return;   // flags still say so
     if (writer) flags[0] = flags[1] = 0;   // readers of the vectors' number see 0 or the run's
     // r_0 = b in T, |r_0|^2 accurate to float64
     double rr;
@@ -283,7 +287,7 @@ int cg_run_prepare(rmhmc_ctx* ctx, unsigned** bar) {
 
 template <typename T, typename TI>
 int cg_run_launch(rmhmc_ctx* ctx, const typename LinksOf<T>::type& links, const TI* b, T* R, double diag, int* flags, double* vals, int maxit, double tol2,
-                  long long* iters, cudaStream_t st) {
+                  long long* iters, cudaStream_t st, const int* status) {
     const CgRunShape s = cg_run_shape<T>(ctx);
     unsigned* bar = nullptr;
     RM_TRY(cg_run_prepare(ctx, &bar));
@@ -293,7 +297,7 @@ int cg_run_launch(rmhmc_ctx* ctx, const typename LinksOf<T>::type& links, const 
     size_t fs = field_elems(ctx);
     T d = (T)diag;
     int units = s.units, limit = ctx->wait_limit;
-    void* args[] = {&g, &U, &b, &R, &fs, &d, &flags, &vals, &maxit, &tol2, &iters, &units, &part, &bar, &limit};
+    void* args[] = {&g, &U, &b, &R, &fs, &d, &flags, &vals, &maxit, &tol2, &iters, &units, &part, &bar, &limit, &status};
     const void* kern = (const void*)k_cg_run<T, TI, sizeof(T) == 8 ? 1 : 0, 256>;
     if constexpr (sizeof(T) == 4) {
         if (s.maxw == 24) kern = (const void*)k_cg_run<T, TI, 0, 768>;
@@ -314,8 +318,8 @@ int cg_run_launch(rmhmc_ctx* ctx, const typename LinksOf<T>::type& links, const 
 
 template bool cg_run_fits<float>(const rmhmc_ctx*);
 template bool cg_run_fits<double>(const rmhmc_ctx*);
-template int cg_run_launch<float, float>(rmhmc_ctx*, const Links32&, const float*, float*, double, int*, double*, int, double, long long*, cudaStream_t);
-template int cg_run_launch<float, double>(rmhmc_ctx*, const Links32&, const double*, float*, double, int*, double*, int, double, long long*, cudaStream_t);
-template int cg_run_launch<double, double>(rmhmc_ctx*, const Links64&, const double*, double*, double, int*, double*, int, double, long long*, cudaStream_t);
+template int cg_run_launch<float, float>(rmhmc_ctx*, const Links32&, const float*, float*, double, int*, double*, int, double, long long*, cudaStream_t, const int*);
+template int cg_run_launch<float, double>(rmhmc_ctx*, const Links32&, const double*, float*, double, int*, double*, int, double, long long*, cudaStream_t, const int*);
+template int cg_run_launch<double, double>(rmhmc_ctx*, const Links64&, const double*, double*, double, int*, double*, int, double, long long*, cudaStream_t, const int*);
 
 }  // namespace rm

@@ -898,7 +898,8 @@ static int md_run(rmhmc_ctx* ctx, double* U, double* P, const rmhmc_params* p, c
 // the molecular dynamics as one CUDA graph (mixed precision): the fixed points and the Krylov runs are
 // conditional WHILE nodes whose conditions the kernels set on the device, so a whole MD trajectory is one
 // graph launch with no host round trip.  Status codes written on the device: 1 Krylov cap, 2 Krylov NaN,
-// 3 fixed point without convergence, 4 fixed point NaN.
+// 3 fixed point without convergence, 4 fixed point NaN, 5 (kStatusGaveUp) a Krylov run's barrier gave up: the runs that
+// follow return at once and every fixed point ends with its first pass, so that the graph ends soon.
 // ------------------------------------------------------------------------------------------------
 // iter[0]: iterations of this fixed point; iter[1]: iterations still to run after convergence (-1 before it)
 __global__ void k_fp_decide(double* dmax, int* iter, int cap, double tol, int extra, cudaGraphConditionalHandle h,
@@ -913,9 +914,10 @@ __global__ void k_fp_decide(double* dmax, int* iter, int cap, double tol, int ex
     const bool done = rem == 0;
     if (rem > 0) rem--;
     iter[1] = rem;
+    const bool gave_up = *status == kStatusGaveUp;
     if (bad) atomicMax(status, 4);
     else if (!done && it >= cap) atomicMax(status, 3);
-    cudaGraphSetConditional(h, (!done && !bad && it < cap) ? 1u : 0u);
+    cudaGraphSetConditional(h, (!done && !bad && !gave_up && it < cap) ? 1u : 0u);
     *dmax = 0.0;
 }
 
@@ -1145,7 +1147,7 @@ static int md_graph_run(rmhmc_ctx* ctx, double* U, double* P, const rmhmc_params
     switch (ints[0]) {
         case 0: return RMHMC_OK;
         case 1: return set_err(ctx, RMHMC_ENOCONV, "MD graph: a Krylov run hit its iteration cap");
-        case 5:
+        case kStatusGaveUp:
             RM_TRY(cg_run_reset(ctx, stream));
             return set_err(ctx, RMHMC_ETIMEOUT, "MD graph: a grid barrier of a Krylov run gave up");
         case 3: return set_err(ctx, RMHMC_ENOCONV, "MD graph: a fixed point did not converge in %d iterations", p->fp_maxit);

@@ -1059,7 +1059,7 @@ __global__ void __launch_bounds__(128) k_lanczos_rows(const int* __restrict__ fl
     const double* rho = vals;
     const double* alpha = vals + (maxit + 1) + maxit;
     const double* beta = alpha + maxit;
-    if (threadIdx.x == 0 && flags[0] >= 2) atomicMax(status, flags[0] == 2 ? 1 : flags[0] == 4 ? 5 : 2);
+    if (threadIdx.x == 0 && flags[0] >= 2) atomicMax(status, flags[0] == 2 ? 1 : flags[0] == 4 ? kStatusGaveUp : 2);
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
         d[k] = 1.0 / alpha[k] + (k > 0 ? beta[k - 1] / alpha[k - 1] : 0.0);
         e[k] = k < n - 1 ? -sqrt(beta[k]) / alpha[k] : 0.0;
@@ -1192,7 +1192,7 @@ int kinetic_graph_prepare(rmhmc_ctx* ctx, const MassTerm& m, int maxiter) {
 
 // Enqueue (on a capturing stream) one mixed-precision kinetic evaluation at the context's links:
 // F_K (float64) and the velocity M^{-1} P (float64), every decision taken on the device.  stats[0] counts
-// Krylov iterations; *status records a Krylov run that hit its cap (1) or produced NaN (2).  aux is a second
+// Krylov iterations; *status records a Krylov run that hit its cap (1), produced NaN (2) or gave up on a barrier (5).  aux is a second
 // stream used to capture the body of the CG loop.
 int kinetic_enqueue(rmhmc_ctx* ctx, const MassTerm& m, const double* P, double tol, int maxiter, double* F, double* Vel,
                     long long* stats, int* status, cudaStream_t st, cudaStream_t aux) {
@@ -1211,7 +1211,7 @@ int kinetic_enqueue(rmhmc_ctx* ctx, const MassTerm& m, const double* P, double t
         dm.delta[j] = m.sigma[j] - s0;
     }
     if (cg_run_fits<float>(ctx)) {
-        RM_TRY((cg_run_launch<float, double>(ctx, links32(ctx), P, b.R, 0.5 + s0, b.flags, b.vals, b.maxit, tol * tol, stats, st)));
+        RM_TRY((cg_run_launch<float, double>(ctx, links32(ctx), P, b.R, 0.5 + s0, b.flags, b.vals, b.maxit, tol * tol, stats, st, status)));
         if (ctx->cg_run_off) return set_err(ctx, RMHMC_ECUDA, "cooperative launch refused");
     } else {
         const int nb = capped_grid(ctx, nvec, kBlock);

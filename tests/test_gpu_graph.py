@@ -66,3 +66,36 @@ def test_graph_fixed_point_cap_reports_noconv():
         with pytest.raises(rm.RmhmcError) as e:
             rm.md(ctx, dev(U), dev(P), _params(rm, rm.mass_fit(12, 0.9), fp_maxit=1, fp_tol=1e-15))
         assert e.value.code == rm.ENOCONV
+
+
+@pytest.mark.parametrize("logdet", [0, 1])
+def test_wait_that_runs_out_ends_the_graph(logdet):
+    """A Krylov run whose barrier gives up (a wait limit of no polls) ends the captured trajectory: each of the 2 x 4 fixed
+    points stops after its first pass, the call returns ETIMEOUT with the links as they were, and with the limit
+    back the context gives the trajectory it gave before."""
+    import ctypes
+    import paper_2112_04556_gb300 as rm
+    L = (8, 8, 8, 8)
+    U = inputs.random_links(L, eps=0.3, seed=77)
+    P = inputs.gaussian_fields(L, 1, seed=78)[0]
+    m = rm.mass_fit(12, 0.9)
+    p = _params(rm, m, logdet=logdet)
+    with rm.Context(L) as ctx:
+        def trajectory():
+            Ud = dev(U)
+            r = rm.rmhmc_trajectory(ctx, Ud, p)
+            return host(Ud), r
+        want, r = trajectory()
+        assert "md graph captured" in rm.tuning(ctx)
+        rm.set_wait_limit(ctx, 0)
+        Ud, Pd, res = dev(U), dev(P), rm.Result()
+        code = rm.lib().rmhmc_md(ctx.h, Ud.data_ptr(), Pd.data_ptr(), ctypes.byref(p), ctypes.byref(res), None)
+        assert code == rm.ETIMEOUT
+        assert res.fp_iters_p == 4 and res.fp_iters_u == 4
+        Ud = dev(U)
+        with pytest.raises(rm.RmhmcError) as e:
+            rm.rmhmc_trajectory(ctx, Ud, p)
+        assert e.value.code == rm.ETIMEOUT and np.array_equal(host(Ud), U)
+        rm.set_wait_limit(ctx)
+        again, r2 = trajectory()
+    assert np.array_equal(again, want) and r2["dH"] == r["dH"]
