@@ -260,9 +260,14 @@ template <typename T> static CgRunShape cg_run_shape(const rmhmc_ctx* ctx) {
     return s;
 }
 
+// static shared memory of the kernel (the block's partial sums and the barrier's words), rounded up
+constexpr size_t kCgRunStatic = 1024;
+
+// q has to fit next to it: ceil(units / warps) rounds of 1 or 2 KB a warp, which depends on how many SMs share the sites
 template <typename T> bool cg_run_fits(const rmhmc_ctx* ctx) {
     return !ctx->cg_run_off && !ctx->prof && !ctx->tune.count(10000 + (int)sizeof(T) * 100 + 18) &&
-           ctx->g.V <= (sizeof(T) == 4 ? kCgRunMax32 : kCgRunMax64);
+           ctx->g.V <= (sizeof(T) == 4 ? kCgRunMax32 : kCgRunMax64) &&
+           cg_run_shape<T>(ctx).smem + kCgRunStatic <= ctx->smem_optin;
 }
 
 // the barrier words (64 bytes; they wrap and count on from launch to launch) and two arrays of partials
@@ -303,9 +308,10 @@ int cg_run_launch(rmhmc_ctx* ctx, const typename LinksOf<T>::type& links, const 
         if (s.maxw == 24) kern = (const void*)k_cg_run<T, TI, 0, 768>;
         if (s.maxw == 16) kern = (const void*)k_cg_run<T, TI, 1, 512>;
     }
-    RM_CHECK(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem));
-    const cudaError_t e = cudaLaunchCooperativeKernel(kern, dim3(s.grid), dim3(s.warps * 32), args, s.smem, st);
-    if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem);
+    const bool refused = e != cudaSuccess;
+    if (!refused) e = cudaLaunchCooperativeKernel(kern, dim3(s.grid), dim3(s.warps * 32), args, s.smem, st);
+    if (refused || e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
         // fewer SMs than the device reports are ours (a partitioned GPU): the two-kernel form from here on
         cudaGetLastError();
         ctx->cg_run_off = true;

@@ -342,6 +342,7 @@ struct rmhmc_ctx {
     // workspace pool
     std::map<std::string, rm::DevBuf> bufs;
     size_t num_sms = 0;
+    size_t smem_optin = 0;              // most shared memory a block may have
     // pinned upload ring (kRingSlots slots of kRingBytes) and the events that guard slot reuse
     char* ring = nullptr;
     cudaEvent_t ring_ev[4] = {};

@@ -134,6 +134,9 @@ extern "C" int rmhmc_create(const int dims[4], int device, rmhmc_ctx** out) {
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     ctx->num_sms = sms;
+    int optin = 0;
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+    ctx->smem_optin = optin;
     // the most blocks any reduced launch uses: four lanes per site in blocks of kBlockMin, or one float32
     // float4 per thread (8 per site) in blocks of kBlock
     ctx->max_blocks = (int)std::max((4 * V + kBlockMin - 1) / kBlockMin, (8 * V + kBlock - 1) / kBlock);

@@ -53,8 +53,8 @@ int krylov_run(rmhmc_ctx* ctx, const TI* b, double sigma0, double tol, int maxit
 // the same run as one cooperative launch (cg_run.cu), for lattices of up to kCgRunMax32 / kCgRunMax64 sites (float32 /
 // float64) in contexts whose CG stencil is neither pinned nor being timed.  flags[0] as KScal::done, or 4 if a grid
 // barrier gave up (cg_run_reset then); where the device refuses the launch, ctx->cg_run_off is set and nothing has run
-// The limits are what q leaves of the shared memory (227 KB an SM) and was measured: still 7 % faster than the two-kernel
-// form at 262,144 sites in float32, 2 % at 122,880 in float64
+// The limits are what q leaves of the shared memory (227 KB an SM) on 152 SMs and was measured: still 7 % faster than the
+// two-kernel form at 262,144 sites in float32, 2 % at 122,880 in float64; with fewer SMs the run takes fewer sites
 constexpr int kCgRunMax32 = 1 << 18, kCgRunMax64 = 1 << 17;
 template <typename T> bool cg_run_fits(const rmhmc_ctx* ctx);
 int cg_run_prepare(rmhmc_ctx* ctx, unsigned** bar = nullptr);

@@ -291,3 +291,27 @@ def test_wait_that_runs_out_is_reported(L, prec, tol):
         with pytest.raises(rm.RmhmcError) as e:
             rm.set_wait_limit(ctx, -1)
         assert e.value.code == rm.EINVAL
+
+
+@pytest.mark.parametrize("prec,L", [(1, (13, 31, 26, 25)), (1, (32, 32, 16, 16)), (1, (33, 32, 16, 16)),
+                                    (0, (11, 23, 22, 23)), (0, (16, 16, 16, 32)), (0, (17, 16, 16, 32))])
+def test_cg_run_at_its_limits(prec, L):
+    """Just below, at and above the largest lattices of the cooperative run (2^18 sites in float32, 2^17 in float64: 13
+    or 14 rounds of units), against the two-kernel form that a pinned CG stencil selects.  Both solve to relative
+    residual tol, so the sums differ by less than ten times tol, as on the small lattices."""
+    import paper_2112_04556_gb300 as rm
+    from perf import cases
+    m = rm.mass_fit(12, 0.9)
+    tol = 1e-10
+    U, b = cases._links(L, 35), cases._field(L, 35, 2)
+    with rm.Context(L) as ctx:
+        y, _, iters, resid = rm.rat_mass_solve(ctx, U, b, m, tol=tol, prec=prec)
+        assert np.all(resid <= tol)
+        F, V, T = rm.kinetic_force(ctx, None, b, m, tol=1e-6, prec=prec)
+    with rm.Context(L) as ctx:
+        rm.set_stencil_shape(ctx, rm.SHAPE_CG, rm.FP64 if prec == 0 else rm.FP32, 18, 1, 128)
+        y2, _, iters2, _ = rm.rat_mass_solve(ctx, U, b, m, tol=tol, prec=prec)
+        F2, V2, T2 = rm.kinetic_force(ctx, None, b, m, tol=1e-6, prec=prec)
+    assert rel_l2(host(y), host(y2)) <= 1e-9
+    assert abs(iters - iters2) <= 2 + iters // 20
+    assert rel_l2(host(F), host(F2)) <= 1e-5 and rel_l2(host(V), host(V2)) <= 1e-5 and abs(T - T2) <= 1e-5 * T

@@ -91,3 +91,28 @@ def test_a_failed_allocation_leaves_the_context_usable(rm, prec):
         if not reached:
             break
     assert n > 4
+
+
+SMEM = 232448   # shared memory a block of sm_103 may have
+
+
+@pytest.mark.parametrize("prec,L", [(1, (64, 64, 8, 8)), (1, (32, 16, 16, 16)), (0, (32, 16, 16, 16))])
+def test_cooperative_run_only_where_q_fits(rm, prec, L):
+    """On a device of any size a Krylov run on the largest lattices of the cooperative form either fits its shared
+    memory or takes the two-kernel form; so does one whose launch the device refuses."""
+    seen = set()
+    for sms in (152, 148, 147, 146, 145, 144, 132, 76, 38, 19, 1):
+        rm.lib().fake_device(sms, SMEM)
+        with context(rm, L) as ctx:
+            assert kinetic(rm, ctx, prec) == rm.OK, sms
+            seen.add((sms, any("k_cg_run" in k for k in launched(rm))))
+    assert (152, True) in seen and (1, False) in seen
+    rm.lib().fake_device(152, SMEM)
+    for error in (720, 801):   # cooperative launch too large, not supported
+        with context(rm, L) as ctx:
+            rm.lib().fake_coop_error(error)
+            assert kinetic(rm, ctx, prec) == rm.OK
+            assert any("k_cg_start" in k for k in launched(rm))
+            rm.lib().fake_coop_error(0)
+            assert kinetic(rm, ctx, prec) == rm.OK   # not asked again
+            assert not any("k_cg_run" in k for k in launched(rm))
