@@ -264,8 +264,8 @@ template <typename T> static CgRunShape cg_run_shape(const rmhmc_ctx* ctx) {
 constexpr size_t kCgRunStatic = 1024;
 
 // q has to fit next to it: ceil(units / warps) rounds of 1 or 2 KB a warp, which depends on how many SMs share the sites
-template <typename T> bool cg_run_fits(const rmhmc_ctx* ctx) {
-    return !ctx->cg_run_off && !ctx->prof && !ctx->tune.count(10000 + (int)sizeof(T) * 100 + 18) &&
+template <typename T> bool cg_run_fits(const rmhmc_ctx* ctx, bool captured) {
+    return !ctx->cg_run_off && (captured || !ctx->prof) && !ctx->pinned.count(10000 + (int)sizeof(T) * 100 + 18) &&
            ctx->g.V <= (sizeof(T) == 4 ? kCgRunMax32 : kCgRunMax64) &&
            cg_run_shape<T>(ctx).smem + kCgRunStatic <= ctx->smem_optin;
 }
@@ -322,8 +322,8 @@ int cg_run_launch(rmhmc_ctx* ctx, const typename LinksOf<T>::type& links, const 
     return RMHMC_OK;
 }
 
-template bool cg_run_fits<float>(const rmhmc_ctx*);
-template bool cg_run_fits<double>(const rmhmc_ctx*);
+template bool cg_run_fits<float>(const rmhmc_ctx*, bool);
+template bool cg_run_fits<double>(const rmhmc_ctx*, bool);
 template int cg_run_launch<float, float>(rmhmc_ctx*, const Links32&, const float*, float*, double, int*, double*, int, double, long long*, cudaStream_t, const int*);
 template int cg_run_launch<float, double>(rmhmc_ctx*, const Links32&, const double*, float*, double, int*, double*, int, double, long long*, cudaStream_t, const int*);
 template int cg_run_launch<double, double>(rmhmc_ctx*, const Links64&, const double*, double*, double, int*, double*, int, double, long long*, cudaStream_t, const int*);

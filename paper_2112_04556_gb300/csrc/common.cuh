@@ -7,6 +7,7 @@
 
 #include <algorithm>
 #include <map>
+#include <set>
 #include <string>
 #include <vector>
 
@@ -355,6 +356,7 @@ struct rmhmc_ctx {
     // captured for, capture streams, and whether graphs are used (fallback reason when not)
     cudaGraphExec_t md_exec = nullptr;
     std::string md_key;
+    bool md_cg_run = false;             // its Krylov runs are cooperative (one kernel each)
     unsigned long long md_gen = 0;
     unsigned long long ws_gen = 0;      // bumped whenever a workspace buffer is (re)allocated
     cudaStream_t cap_st[3] = {};
@@ -362,6 +364,7 @@ struct rmhmc_ctx {
     std::string graph_note;
     // autotuned stencil shapes per (precision bytes * 100 + link format): components per lane, block size
     std::map<int, std::pair<int, int>> tune;
+    std::set<int> pinned;              // keys of tune that the caller set (rmhmc_set_stencil_shape)
     // kernel of the kinetic-force contraction (rmhmc_set_stencil_shape, RMHMC_SHAPE_KFORCE): 4 the fused one (the default),
     // 0 four lanes per link
     int lg_mode = 4;

@@ -280,6 +280,7 @@ extern "C" int rmhmc_set_stencil_shape(rmhmc_ctx* ctx, int kernel, int prec, int
     const int key = (kernel == RMHMC_SHAPE_CG ? 10000 : 0) + bytes * 100 + linkfmt;
     if (kernel == RMHMC_SHAPE_CG && !ctx->tune.count(bytes * 100 + 18)) ctx->tune[bytes * 100 + 18] = {2, 256};
     ctx->tune[key] = {nmu, block};
+    ctx->pinned.insert(key);
     char line[96];
     snprintf(line, sizeof line, "%s%s %s LF%d pinned -> nmu %d block %d", ctx->tune_report.empty() ? "" : "; ",
              kernel == RMHMC_SHAPE_CG ? "cg" : "lap", bytes == 8 ? "fp64" : "fp32", linkfmt, nmu, block);

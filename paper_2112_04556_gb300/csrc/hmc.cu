@@ -1086,7 +1086,7 @@ static int md_graph_run(rmhmc_ctx* ctx, double* U, double* P, const rmhmc_params
         // a second attempt without the cooperative Krylov run: a device shared through MPS does not take cooperative kernels
         // inside conditional nodes
         for (int attempt = 0; !ctx->md_exec; attempt++) {
-            const bool last = attempt == 1 || !cg_run_fits<float>(ctx);
+            const bool last = attempt == 1 || !cg_run_fits<float>(ctx, true);
             cudaGraph_t g = nullptr;
             const int s = md_graph_capture(ctx, p, m, gb, w, lg, &g);
             ctx->launches = saved;
@@ -1111,6 +1111,7 @@ static int md_graph_run(rmhmc_ctx* ctx, double* U, double* P, const rmhmc_params
             return RMHMC_OK;
         }
         ctx->md_key = key;
+        ctx->md_cg_run = cg_run_fits<float>(ctx, true);
         ctx->md_gen = ctx->ws_gen;
         ctx->graph_note = "md graph captured";
     }
@@ -1134,7 +1135,7 @@ static int md_graph_run(rmhmc_ctx* ctx, double* U, double* P, const rmhmc_params
     // kernel
     const int gk = ctx->g.V > kLoopsMax || ctx->loops_off ? 1 : p->c1 != 0.0 ? 4 : 2;
     ctx->launches += 2 + gk + (5LL + gk) * p->nsteps + (ctx->lg_mode == kLgFused ? 5 : 6) * (st[1] + st[2]) +
-                     (cg_run_fits<float>(ctx) ? 0 : 2 * st[0]);
+                     (ctx->md_cg_run ? 0 : 2 * st[0]);
     ctx->krylov_iters += st[0];
     ctx->links_valid = true;
     if (r) {

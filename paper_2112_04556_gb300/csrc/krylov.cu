@@ -550,7 +550,7 @@ int krylov_run(rmhmc_ctx* ctx, const TI* b, double sigma0, double tol, int maxit
     bool run = cg_run_fits<T>(ctx);
     if constexpr (sizeof(T) == 8) {
         U = links64(ctx);
-        if (!ctx->tune.count(10818)) RM_TRY(links64_adjoint(ctx, &U, st));
+        if (!ctx->pinned.count(10818)) RM_TRY(links64_adjoint(ctx, &U, st));
         run = run && U.ad;
     } else {
         U = links32(ctx);
@@ -1187,7 +1187,7 @@ int kinetic_graph_prepare(rmhmc_ctx* ctx, const MassTerm& m, int maxiter) {
     RM_TRY(kin_graph_bufs(ctx, m.npole(), maxiter, b));
     RM_TRY(cg_run_prepare(ctx));
     StencilShape shp;
-    return cg_run_fits<float>(ctx) ? RMHMC_OK : cg_shape<float>(ctx, 0, shp);
+    return cg_run_fits<float>(ctx, true) ? RMHMC_OK : cg_shape<float>(ctx, 0, shp);
 }
 
 // Enqueue (on a capturing stream) one mixed-precision kinetic evaluation at the context's links:
@@ -1210,7 +1210,7 @@ int kinetic_enqueue(rmhmc_ctx* ctx, const MassTerm& m, const double* P, double t
         dm.alpha[j] = m.alpha[j];
         dm.delta[j] = m.sigma[j] - s0;
     }
-    if (cg_run_fits<float>(ctx)) {
+    if (cg_run_fits<float>(ctx, true)) {
         RM_TRY((cg_run_launch<float, double>(ctx, links32(ctx), P, b.R, 0.5 + s0, b.flags, b.vals, b.maxit, tol * tol, stats, st, status)));
         if (ctx->cg_run_off) return set_err(ctx, RMHMC_ECUDA, "cooperative launch refused");
     } else {

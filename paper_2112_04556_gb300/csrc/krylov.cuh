@@ -56,7 +56,8 @@ int krylov_run(rmhmc_ctx* ctx, const TI* b, double sigma0, double tol, int maxit
 // The limits are what q leaves of the shared memory (227 KB an SM) on 152 SMs and was measured: still 7 % faster than the
 // two-kernel form at 262,144 sites in float32, 2 % at 122,880 in float64; with fewer SMs the run takes fewer sites
 constexpr int kCgRunMax32 = 1 << 18, kCgRunMax64 = 1 << 17;
-template <typename T> bool cg_run_fits(const rmhmc_ctx* ctx);
+// captured: in a trajectory's graph, whose launches are not timed
+template <typename T> bool cg_run_fits(const rmhmc_ctx* ctx, bool captured = false);
 int cg_run_prepare(rmhmc_ctx* ctx, unsigned** bar = nullptr);
 int cg_run_reset(rmhmc_ctx* ctx, cudaStream_t st);
 template <typename T> struct LinksOf;

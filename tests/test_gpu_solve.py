@@ -315,3 +315,27 @@ def test_cg_run_at_its_limits(prec, L):
     assert rel_l2(host(y), host(y2)) <= 1e-9
     assert abs(iters - iters2) <= 2 + iters // 20
     assert rel_l2(host(F), host(F2)) <= 1e-5 and rel_l2(host(V), host(V2)) <= 1e-5 and abs(T - T2) <= 1e-5 * T
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_profiling_in_between_changes_nothing(prec):
+    """A solve and a trajectory before and after a profiled solve agree bit for bit (16,384 sites: the size from which
+    the profiled two-kernel form tunes its stencil)."""
+    import paper_2112_04556_gb300 as rm
+    L = (16, 8, 8, 16)
+    U = dev(inputs.random_links(L, eps=0.3, seed=36))
+    b = dev(inputs.gaussian_fields(L, 1, seed=37)[0])
+    m = rm.mass_fit(12, 0.9)
+    p = rm.make_params(beta=6.0, mass=m, tau=0.1, nsteps=2, tol_md=1e-6, tol_h=1e-10, fp_tol=1e-6, maxiter=400,
+                       prec=rm.MIXED, seed=5, metropolis=False)
+    out = []
+    with rm.Context(L) as ctx:
+        for on in (False, True, False):
+            rm.set_profiling(ctx, on)
+            y = rm.rat_mass_solve(ctx, U, b, m, tol=1e-10, prec=prec)[0]
+            V = U.clone()
+            r = rm.rmhmc_trajectory(ctx, V, p)
+            out.append((host(y), host(V), r["dH"], rm.counters(ctx)["cg_count"]))
+    assert out[0][3] == 0 and out[1][3] > 0 and out[2][3] == out[1][3]
+    assert np.array_equal(out[0][0], out[2][0]) and np.array_equal(out[0][1], out[2][1]) and out[0][2] == out[2][2]
+    assert rel_l2(out[1][0], out[0][0]) <= 1e-9

@@ -116,3 +116,54 @@ def test_cooperative_run_only_where_q_fits(rm, prec, L):
             rm.lib().fake_coop_error(0)
             assert kinetic(rm, ctx, prec) == rm.OK   # not asked again
             assert not any("k_cg_run" in k for k in launched(rm))
+
+
+def krylov_forms(names):
+    return {f for f in ("k_cg_run", "k_cg_start", "k_cgg_start") for k in names if f in k}
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_profiling_does_not_outlast_itself(rm, prec):
+    """While profiling is on the two-kernel form runs (its stencil launches are what is timed, in a tuned shape); before
+    and after it the cooperative one.  A pinned stencil shape selects the two-kernel form for good."""
+    with context(rm, (16, 8, 8, 16)) as ctx:
+        forms = []
+        for on in (0, 1, 0):
+            rm.set_profiling(ctx, on)
+            assert kinetic(rm, ctx, prec) == rm.OK
+            forms.append(krylov_forms(launched(rm)))
+        assert forms == [{"k_cg_run"}, {"k_cg_start"}, {"k_cg_run"}]
+        rm.set_stencil_shape(ctx, rm.SHAPE_CG, rm.FP64 if prec == 0 else rm.FP32, 18, 1, 128)
+        assert kinetic(rm, ctx, prec) == rm.OK
+        assert krylov_forms(launched(rm)) == {"k_cg_start"}
+
+
+def trajectory_md(rm, ctx):
+    p = rm.make_params(beta=6.0, mass=rm.mass_fit(12, 0.9), tau=0.1, nsteps=2, prec=rm.MIXED)
+    return rm.lib().rmhmc_md(ctx.h, LINKS, FIELD, ctypes.byref(p), None, None)
+
+
+@pytest.mark.parametrize("L,form", [((4, 4, 4, 4), "k_cg_run"), ((64, 64, 8, 9), "k_cgg_start")])
+def test_captured_trajectory_is_kept(rm, L, form):
+    """The graph of a trajectory is captured once: profiling in between neither changes it nor what is counted for it,
+    and one whose first capture the device refuses (a cooperative run in a conditional node) is captured without."""
+    with context(rm, L) as ctx:
+        counted = []
+        for on in (0, 1, 0):
+            rm.set_profiling(ctx, on)
+            rm.counters(ctx, reset=True)
+            assert trajectory_md(rm, ctx) == rm.OK
+            counted.append(rm.counters(ctx)["launches"])
+            names = launched(rm)
+            assert ("instantiate" in names) == (len(counted) == 1) and "graph" in names
+            assert krylov_forms(names) == ({form} if len(counted) == 1 else set())
+        assert counted[1] == counted[2] > 0
+    rm.lib().fake_instantiate_errors(1)
+    with context(rm, L) as ctx:
+        assert trajectory_md(rm, ctx) == rm.OK
+        if form == "k_cg_run":
+            assert krylov_forms(launched(rm)) == {"k_cg_run", "k_cgg_start"}   # two captures
+            assert "graphs: on" in rm.tuning(ctx)
+            assert trajectory_md(rm, ctx) == rm.OK and "instantiate" not in launched(rm)
+        else:
+            assert "graphs: off" in rm.tuning(ctx)
