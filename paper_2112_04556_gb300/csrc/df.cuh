@@ -26,10 +26,12 @@ __device__ __forceinline__ dfl quick_two_sum(float a, float b) {
     const float s = __fadd_rn(a, b);
     return df_make(s, __fsub_rn(b, __fsub_rn(s, a)));
 }
-// float64-accurate running sum of squares in float32 arithmetic: the rounding errors of the products (fma) and of the
-// sum (TwoSum) are collected in c; values whose squares leave float32's range go to a float64 sum
+// running sum of squares in float32 arithmetic, no less accurate than a float64 sum: the rounding errors of the products
+// (fma) and of the sum (TwoSum) are added up in c with TwoSum again, whose errors go to e.  What e loses is 2^-72 of the
+// sum a term, so that the result is off by the roundings of value() alone, 2^-52; with the errors in c added up plainly it
+// was 1e-14.  Values whose squares leave float32's range go to a float64 sum
 struct SumSq32 {
-    float s = 0.f, c = 0.f;
+    float s = 0.f, c = 0.f, e = 0.f;
     double d = 0.0;
     __device__ __forceinline__ void add(float x) {
         const float m = fabsf(x);
@@ -37,12 +39,13 @@ struct SumSq32 {
             d = fma((double)x, (double)x, d);
             return;
         }
-        const float p = __fmul_rn(x, x), e = __fmaf_rn(x, x, -p);
-        const dfl t = two_sum(s, p);
+        const float p = __fmul_rn(x, x);
+        const dfl t = two_sum(s, p), u = two_sum(c, t.lo), v = two_sum(u.hi, __fmaf_rn(x, x, -p));
         s = t.hi;
-        c = __fadd_rn(c, __fadd_rn(t.lo, e));
+        c = v.hi;
+        e = __fadd_rn(e, __fadd_rn(u.lo, v.lo));
     }
-    __device__ __forceinline__ double value() const { return (double)s + (double)c + d; }
+    __device__ __forceinline__ double value() const { return ((double)e + (double)c) + (double)s + d; }
 };
 
 // Conversions between float64 and float pairs from the IEEE-754 bit fields, with integer operations and no

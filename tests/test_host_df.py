@@ -1,0 +1,54 @@
+"""The float32-pair arithmetic of csrc/df.cuh, built by the host compiler (every operation is one IEEE-754 float32
+operation, so that host and device agree bit for bit), against exact rational arithmetic."""
+import ctypes
+import os
+import subprocess
+from fractions import Fraction
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+SRC = r"""
+#include "df.cuh"
+using namespace rm;
+extern "C" double sum_squares(const float* x, int n) {
+    SumSq32 a;
+    for (int i = 0; i < n; i++) a.add(x[i]);
+    return a.value();
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def df(tmp_path_factory):
+    d = tmp_path_factory.mktemp("df")
+    (d / "df.cpp").write_text(SRC)
+    subprocess.run(["g++", "-shared", "-fPIC", "-O1", "-std=c++17", "-ffp-contract=off", "-I",
+                    os.path.join(ROOT, "tests", "fake", "host"), "-I",
+                    os.path.join(ROOT, "paper_2112_04556_gb300", "csrc"), "-o", str(d / "df.so"), str(d / "df.cpp")],
+                   check=True)
+    L = ctypes.CDLL(str(d / "df.so"))
+    L.sum_squares.restype = ctypes.c_double
+    return L
+
+
+@pytest.mark.parametrize("n", [1, 2, 32, 448, 4096])
+@pytest.mark.parametrize("spread", [0.0, 8.0, 30.0])
+def test_sum_of_squares_is_float64_accurate(df, n, spread):
+    """Sums of squares of one lane (448 terms: the largest lattice of the cooperative Krylov run; 4096: beyond any),
+    normal values times 2^k, |k| <= spread (30: some squares leave float32's range and go through the float64 sum).  A
+    float64 sum of n squares may be off by n 2^-53; this one by its last three additions and, where the float64 part
+    holds some of the terms, theirs: 4 2^-53 and n 2^-53 of that part."""
+    worst = 0.0
+    for seed in range(20):
+        rng = np.random.default_rng(seed)
+        x = (rng.standard_normal(n) * 2.0 ** rng.uniform(-spread, spread, n)).astype(np.float32)
+        got = df.sum_squares(x.ctypes.data_as(ctypes.c_void_p), n)
+        want = sum(Fraction(float(v)) ** 2 for v in x)
+        wide = sum(Fraction(float(v)) ** 2 for v in x if not 2.0 ** -40 <= abs(v) <= 2.0 ** 40)
+        bound = (4 * want + n * wide) / 2 ** 53
+        assert abs(Fraction(got) - want) <= bound, (seed, float(abs(Fraction(got) - want) / want))
+        worst = max(worst, float(abs(Fraction(got) - want) / want))
+    assert worst < 1e-12
