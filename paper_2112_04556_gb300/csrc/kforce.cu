@@ -31,40 +31,40 @@ struct PairWeights { double w[kMaxPairs]; };
 // table of R (LF = kLinkAd; built once per set of links) a column costs its 64 FMA instead of a conjugation's 108 and its
 // expansions: differentiated Laplacian at 16^4 1.623 -> 1.590 ms, kinetic force with 12 pairs 13.35 -> 13.20 ms, and the error
 // against 64 bits 4.6e-16 -> 3.5e-16.
-template <typename T, int LF>
-__global__ void __launch_bounds__(kBlock) k_link_grad(Geom g, typename LinksOf<T>::type U, const T* __restrict__ X,
-                                                       const T* __restrict__ Z, size_t fs, int nf, PairWeights w,
+template <int LF>
+__global__ void __launch_bounds__(kBlock) k_link_grad(Geom g, Links64 U, const double* __restrict__ X,
+                                                       const double* __restrict__ Z, size_t fs, int nf, PairWeights w,
                                                        double* __restrict__ G) {
-    __shared__ T rcs[kBlock / 4][65];   // R C of the block's links
+    __shared__ double rcs[kBlock / 4][65];   // R C of the block's links
     const int lane = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = lane >> 2, q = lane & 3;
     const int nu = blockIdx.y;
     const bool live = y < g.V;
-    T* const rc = rcs[threadIdx.x >> 2];
+    double* const rc = rcs[threadIdx.x >> 2];
     if (live) {
         const size_t yo = (size_t)y * 32 + 2 * q, yn = (size_t)step_site(g, y, nu, 1) * 32;
-        T C[2][8];
+        double C[2][8];
 #pragma unroll
         for (int i = 0; i < 2; i++)
 #pragma unroll
-            for (int b = 0; b < 8; b++) C[i][b] = T(0);
+            for (int b = 0; b < 8; b++) C[i][b] = 0.0;
         for (int f = 0; f < nf; f++) {
-            const T wf = (T)w.w[f];
-            const T *Xf = X + f * fs, *Zf = Z + f * fs;
+            const double wf = w.w[f];
+            const double *Xf = X + f * fs, *Zf = Z + f * fs;
 #pragma unroll 2
             for (int mu = 0; mu < 4; mu++) {
-                T xp[8], zp[8];
+                double xp[8], zp[8];
                 load8(Xf + yn + mu * 8, xp);
                 load8(Zf + yn + mu * 8, zp);
 #pragma unroll
                 for (int i = 0; i < 2; i++) {
-                    const T x = wf * __ldg(Xf + yo + mu * 8 + i), z = wf * __ldg(Zf + yo + mu * 8 + i);
+                    const double x = wf * __ldg(Xf + yo + mu * 8 + i), z = wf * __ldg(Zf + yo + mu * 8 + i);
 #pragma unroll
                     for (int b = 0; b < 8; b++) C[i][b] = fma(xp[b], z, fma(zp[b], x, C[i][b]));
                 }
             }
         }
-        T r[2][8];
+        double r[2][8];
         if constexpr (LF == kLinkAd) {
             const double2* t = U.ad + (size_t)nu * 32 * U.V + y;
 #pragma unroll
@@ -83,10 +83,10 @@ __global__ void __launch_bounds__(kBlock) k_link_grad(Geom g, typename LinksOf<T
                     }
                 }
         } else {
-            const mat3<T> u = LinkLoad<T, LF>::load(U, y, nu);
+            const mat3<double> u = LinkLoad<double, LF>::load(U, y, nu);
 #pragma unroll
             for (int i = 0; i < 2; i++) {
-                herm<T> E = h_zero<T>();
+                herm<double> E = h_zero<double>();
                 acc_uxud_tl(E, u, coef_to_herm2(C[i]));
                 herm2_to_coef_tl(E, r[i]);
             }
@@ -101,14 +101,74 @@ __global__ void __launch_bounds__(kBlock) k_link_grad(Geom g, typename LinksOf<T
         double* out = G + (size_t)y * 32 + nu * 8 + 2 * q;
 #pragma unroll
         for (int i = 0; i < 2; i++) {
-            T v = T(0);
+            double v = 0.0;
 #pragma unroll
             for (int t = 0; t < 4; t++) {
                 const FTerm f = kFTerms[2 * q + i][t];
-                if (f.v != 0.0) v = fma((T)f.v, rc[f.c * 8 + f.d] - rc[f.d * 8 + f.c], v);
+                if (f.v != 0.0) v = fma(f.v, rc[f.c * 8 + f.d] - rc[f.d * 8 + f.c], v);
             }
-            out[i] = (double)v * (1.0 / 16.0);
+            out[i] = v * (1.0 / 16.0);
         }
+    }
+}
+
+// The form of the file's head, four lanes per link with a component each, for float32: there the operations are not what bounds
+// it, and a lane reads its own component's rows only, where a lane of the kernel above reads all four.  The form above took
+// 1.3 to 1.4 times as long at any number of pairs: 24^3 x 48 672 against 499 us for one pair, 4547 against 3524 us for 12;
+// 16^4 76 against 57 us; 8^4 with 12 pairs 45 against 35 us
+template <int LF>
+__global__ void __launch_bounds__(kBlock) k_link_grad_direct(Geom g, Links32 U, const float* __restrict__ X,
+                                                              const float* __restrict__ Z, size_t fs, int nf, PairWeights w,
+                                                              double* __restrict__ G) {
+    const int lane = blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = lane >> 2, mu = lane & 3;
+    const int nu = blockIdx.y;
+    const bool live = y < g.V;
+    float k[8];
+#pragma unroll
+    for (int a = 0; a < 8; a++) k[a] = 0.f;
+    if (live) {
+        int fwd[4], bwd[4];
+        neighbours(g, y, fwd, bwd);
+        const int yp = fwd[nu];
+        const mat3<float> u = LinkLoad<float, LF>::load(U, y, nu);
+        for (int f = 0; f < nf; f++) {
+            const float wf = (float)w.w[f];
+            const float* Xf = X + f * fs;
+            const float* Zf = Z + f * fs;
+            float xb[8];
+            load8(Xf + (size_t)yp * 32 + mu * 8, xb);
+            herm<float> W1 = h_zero<float>();
+            acc_uxud(W1, u, coef_to_herm2(xb));          // 2 W1
+            load8(Zf + (size_t)yp * 32 + mu * 8, xb);
+            herm<float> W2 = h_zero<float>();
+            acc_uxud(W2, u, coef_to_herm2(xb));          // 2 W2
+            load8(Zf + (size_t)y * 32 + mu * 8, xb);
+            const mat3<float> Zy = herm_full(coef_to_herm2(xb));   // 2 Z(y)
+            load8(Xf + (size_t)y * 32 + mu * 8, xb);
+            const mat3<float> Xy = herm_full(coef_to_herm2(xb));   // 2 X(y)
+            mat3<float> M = m_mul(herm_full(W1), Zy);              // 4 W1 Z
+            const mat3<float> M2 = m_mul(Xy, herm_full(W2));       // 4 X W2
+#pragma unroll
+            for (int i = 0; i < 3; i++)
+#pragma unroll
+                for (int j = 0; j < 3; j++) M.e[i][j] = csub(M.e[i][j], M2.e[i][j]);
+            float kk[8];
+            antiherm_coef(M, kk);                               // 4 coef(M)
+#pragma unroll
+            for (int a = 0; a < 8; a++) k[a] = fma(wf, kk[a], k[a]);
+        }
+    }
+#pragma unroll
+    for (int a = 0; a < 8; a++) {
+        k[a] += __shfl_xor_sync(0xffffffffu, k[a], 1);
+        k[a] += __shfl_xor_sync(0xffffffffu, k[a], 2);
+    }
+    if (live && mu == 0) {
+        double* out = G + (size_t)y * 32 + nu * 8;
+        // d<Z,AX>/dw = (1/8) coef(M) and the doubled expansions gave 4 coef(M): scale by 1/32
+#pragma unroll
+        for (int a = 0; a < 8; a++) out[a] = (double)k[a] * (1.0 / 32.0);
     }
 }
 
@@ -122,13 +182,13 @@ int link_grad_launch(rmhmc_ctx* ctx, int prec, const void* X, const void* Z, int
         Links64 U = links64(ctx);
         RM_TRY(links64_adjoint(ctx, &U, st));
         if (U.ad)
-            k_link_grad<double, kLinkAd><<<grid, kBlock, 0, st>>>(ctx->g, U, (const double*)X, (const double*)Z,
+            k_link_grad<kLinkAd><<<grid, kBlock, 0, st>>>(ctx->g, U, (const double*)X, (const double*)Z,
                                                                   field_elems(ctx), nf, pw, G);
         else
-            k_link_grad<double, 18><<<grid, kBlock, 0, st>>>(ctx->g, U, (const double*)X, (const double*)Z,
+            k_link_grad<18><<<grid, kBlock, 0, st>>>(ctx->g, U, (const double*)X, (const double*)Z,
                                                              field_elems(ctx), nf, pw, G);
     } else
-        k_link_grad<float, 18><<<grid, kBlock, 0, st>>>(ctx->g, links32(ctx), (const float*)X, (const float*)Z,
+        k_link_grad_direct<18><<<grid, kBlock, 0, st>>>(ctx->g, links32(ctx), (const float*)X, (const float*)Z,
                                                         field_elems(ctx), nf, pw, G);
     ++ctx->launches;
     RM_LAUNCH_CHECK(ctx);

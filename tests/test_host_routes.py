@@ -167,3 +167,13 @@ def test_captured_trajectory_is_kept(rm, L, form):
             assert trajectory_md(rm, ctx) == rm.OK and "instantiate" not in launched(rm)
         else:
             assert "graphs: off" in rm.tuning(ctx)
+
+
+@pytest.mark.parametrize("prec,kernel", [(0, "k_link_grad"), (1, "k_link_grad_direct")])
+def test_link_derivative_kernel_by_precision(rm, prec, kernel):
+    """float64 contracts in the adjoint representation, float32 takes the direct form, which is faster there."""
+    with context(rm, (4, 4, 4, 4)) as ctx:
+        w = np.ones(3)
+        ctx.check(rm.lib().lap_link_grad(ctx.h, None, FIELD, OUT, 3, w.ctypes.data_as(ctypes.POINTER(ctypes.c_double)),
+                                         prec, OUT2, None))
+        assert "%d%sI" % (len(kernel), kernel) in [k for k in launched(rm) if "k_link_grad" in k][-1]
