@@ -214,6 +214,13 @@ int rmhmc_tuning(const rmhmc_ctx* ctx, char* buf, int len);
                                    per pass and parity, 2 or 3 (0: timed on first use, the default); block = the
                                    z-extent of the slabs in which the grid sweeps t, 1 .. L2 (0: L2, i.e.
                                    lexicographic order, the default) */
+#define RMHMC_SHAPE_LOOPS 5     /* gauge force and action (prec RMHMC_FP64, linkfmt 18, block 128): nmu 1 (the default) from
+                                   shared plaquettes and rectangles, on up to 2^22 sites; nmu 0 from the staples of each
+                                   link.  Applies to both precisions */
+#define RMHMC_SHAPE_TABLE 6     /* float64 stencils and link derivative (prec RMHMC_FP64, linkfmt 18, block 128): nmu 1 (the
+                                   default) from a table of the links' adjoint matrices (2 KB a site, on up to 2^22
+                                   sites); nmu 0 by 3x3 products.  A pinned RMHMC_SHAPE_LAP or RMHMC_SHAPE_CG of
+                                   float64 takes the latter for its own kernel */
 int rmhmc_set_stencil_shape(rmhmc_ctx* ctx, int kernel, int prec, int linkfmt, int nmu, int block);
 
 /* ---------------------------------------------------------------------------------------------- */

@@ -220,7 +220,7 @@ def set_wait_limit(ctx, polls=1 << 21):
     ctx.check(lib().rmhmc_set_wait_limit(ctx.h, int(polls)))
 
 
-SHAPE_LAP, SHAPE_CG, SHAPE_KFORCE, SHAPE_LINKUPDATE, SHAPE_ADJOINT = 0, 1, 2, 3, 4
+SHAPE_LAP, SHAPE_CG, SHAPE_KFORCE, SHAPE_LINKUPDATE, SHAPE_ADJOINT, SHAPE_LOOPS, SHAPE_TABLE = 0, 1, 2, 3, 4, 5, 6
 
 
 def set_stencil_shape(ctx, kernel, prec, linkfmt, nmu, block):

@@ -370,6 +370,8 @@ struct rmhmc_ctx {
     int lg_mode = 4;
     // float64 link update in float-float arithmetic (rmhmc_set_stencil_shape, RMHMC_SHAPE_LINKUPDATE)
     bool link_update_ff = true;
+    // gauge force from shared loops, float64 stencils from the table of adjoint matrices (RMHMC_SHAPE_LOOPS, _TABLE)
+    bool use_loops = true, use_table = true;
     // z-extent of the multi-field adjoint kernel's slabs (rmhmc_set_stencil_shape, RMHMC_SHAPE_ADJOINT); 0 chosen
     // from the lattice and the field count
     int ad_slab = 0;

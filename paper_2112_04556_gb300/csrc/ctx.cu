@@ -255,6 +255,12 @@ extern "C" int rmhmc_set_stencil_shape(rmhmc_ctx* ctx, int kernel, int prec, int
         ctx->lg_mode = nmu == kLgFused ? kLgFused : 0;   // 1, 2 and 3 name former variants of 0
         return RMHMC_OK;
     }
+    if (kernel == RMHMC_SHAPE_LOOPS || kernel == RMHMC_SHAPE_TABLE) {
+        if (prec != RMHMC_FP64 || linkfmt != 18 || (nmu != 0 && nmu != 1) || block != 128)
+            return set_err(ctx, RMHMC_EINVAL, "loops and table: RMHMC_FP64, 18, nmu 0 or 1, block 128");
+        (kernel == RMHMC_SHAPE_LOOPS ? ctx->use_loops : ctx->use_table) = nmu == 1;
+        return RMHMC_OK;
+    }
     if (kernel == RMHMC_SHAPE_ADJOINT) {
         if (prec != RMHMC_FP32 || (linkfmt != 12 && linkfmt != 18) || (nmu != 0 && nmu != 2 && nmu != 3) ||
             block < 0 || block > ctx->g.L[2])

@@ -175,10 +175,8 @@ __global__ void __launch_bounds__(kBlock) k_action(Geom g, Links64 U64, double b
     grid_sum_finish<2>(v, partials, counter, out, gridDim.x, blockIdx.x, sh);
 }
 
-int gauge_force_launch(rmhmc_ctx* ctx, double beta, double c1, int prec, double* F, cudaStream_t st) {
-    bool used = false;
-    RM_TRY(gauge_loops_launch(ctx, beta, c1, prec, F, false, &used, st));
-    if (used) return RMHMC_OK;
+// force and action from the staples and loops of each link
+static int force_staples(rmhmc_ctx* ctx, double beta, double c1, int prec, double* F, cudaStream_t st) {
     const dim3 grid(site_blocks(ctx), 4);
     const double c0 = 1.0 - 8.0 * c1;
     if (prec == RMHMC_FP64)
@@ -190,25 +188,7 @@ int gauge_force_launch(rmhmc_ctx* ctx, double beta, double c1, int prec, double*
     return RMHMC_OK;
 }
 
-int gauge_force_action(rmhmc_ctx* ctx, double beta, double c1, double* F, double* S, double* plaq, cudaStream_t st) {
-    bool used = false;
-    RM_TRY(gauge_loops_launch(ctx, beta, c1, RMHMC_FP64, F, true, &used, st));
-    if (!used) {
-        if (F) RM_TRY(gauge_force_launch(ctx, beta, c1, RMHMC_FP64, F, st));
-        return action_launch(ctx, beta, c1, S, plaq, st);
-    }
-    double out[3];
-    RM_TRY(fetch(ctx, red_slot_out(ctx, kSlotLoops), out, 3, st));
-    if (S) *S = beta * ((1.0 - 8.0 * c1) * out[0] + (c1 != 0.0 ? c1 * out[2] : 0.0));
-    if (plaq) *plaq = out[1] / (6.0 * ctx->g.V);
-    return RMHMC_OK;
-}
-
-int action_launch(rmhmc_ctx* ctx, double beta, double c1, double* S, double* plaq, cudaStream_t st) {
-    if (ctx->g.V <= kLoopsMax && !ctx->loops_off) {
-        RM_TRY(gauge_force_action(ctx, beta, c1, nullptr, S, plaq, st));
-        if (!ctx->loops_off) return RMHMC_OK;
-    }
+static int action_loops(rmhmc_ctx* ctx, double beta, double c1, double* S, double* plaq, cudaStream_t st) {
     k_action<<<capped_grid(ctx, ctx->g.V, kBlock), kBlock, 0, st>>>(ctx->g, links64(ctx), beta, 1.0 - 8.0 * c1, c1,
                                                   red_slot_partials(ctx, kSlotAction), red_slot_counter(ctx, kSlotAction),
                                                   red_slot_out(ctx, kSlotAction)); ++ctx->launches;
@@ -218,6 +198,30 @@ int action_launch(rmhmc_ctx* ctx, double beta, double c1, double* S, double* pla
     if (S) *S = out[0];
     if (plaq) *plaq = out[1] / (6.0 * ctx->g.V);
     return RMHMC_OK;
+}
+
+int gauge_force_launch(rmhmc_ctx* ctx, double beta, double c1, int prec, double* F, cudaStream_t st) {
+    bool used = false;
+    RM_TRY(gauge_loops_launch(ctx, beta, c1, prec, F, false, &used, st));
+    return used ? RMHMC_OK : force_staples(ctx, beta, c1, prec, F, st);
+}
+
+int gauge_force_action(rmhmc_ctx* ctx, double beta, double c1, double* F, double* S, double* plaq, cudaStream_t st) {
+    bool used = false;
+    RM_TRY(gauge_loops_launch(ctx, beta, c1, RMHMC_FP64, F, true, &used, st));
+    if (!used) {
+        if (F) RM_TRY(force_staples(ctx, beta, c1, RMHMC_FP64, F, st));
+        return action_loops(ctx, beta, c1, S, plaq, st);
+    }
+    double out[3];
+    RM_TRY(fetch(ctx, red_slot_out(ctx, kSlotLoops), out, 3, st));
+    if (S) *S = beta * ((1.0 - 8.0 * c1) * out[0] + (c1 != 0.0 ? c1 * out[2] : 0.0));
+    if (plaq) *plaq = out[1] / (6.0 * ctx->g.V);
+    return RMHMC_OK;
+}
+
+int action_launch(rmhmc_ctx* ctx, double beta, double c1, double* S, double* plaq, cudaStream_t st) {
+    return gauge_force_action(ctx, beta, c1, nullptr, S, plaq, st);
 }
 
 }  // namespace rm

@@ -286,7 +286,7 @@ static int loops_t(rmhmc_ctx* ctx, const typename LinksOf<T>::type& U, double be
 int gauge_loops_launch(rmhmc_ctx* ctx, double beta, double c1, int prec, double* F, bool act, bool* used,
                        cudaStream_t st) {
     *used = false;
-    if (ctx->g.V > kLoopsMax || ctx->loops_off) return RMHMC_OK;
+    if (!loops_usable(ctx)) return RMHMC_OK;
     const int s = prec == RMHMC_FP64 ? loops_t<double>(ctx, links64(ctx), beta, c1, F, act, st)
                                      : loops_t<float>(ctx, links32(ctx), beta, c1, F, false, st);
     if (s == RMHMC_ENOMEM) {
@@ -301,7 +301,7 @@ int gauge_loops_launch(rmhmc_ctx* ctx, double beta, double c1, int prec, double*
 }
 
 int gauge_loops_prepare(rmhmc_ctx* ctx, double c1, int prec) {
-    if (ctx->g.V > kLoopsMax || ctx->loops_off) return RMHMC_OK;
+    if (!loops_usable(ctx)) return RMHMC_OK;
     LoopBufs<float> f;
     LoopBufs<double> d;
     const int s = prec == RMHMC_FP64 ? loop_bufs<double>(ctx, c1 != 0.0, true, d) : loop_bufs<float>(ctx, c1 != 0.0, true, f);

@@ -1133,7 +1133,7 @@ static int md_graph_run(rmhmc_ctx* ctx, double* U, double* P, const rmhmc_params
     // kernels the graph ran: links, gauge force (1 to 4 kernels), momenta; 5 and a gauge force per step outside the loops; 5
     // per fixed-point iteration (6 with the velocity in a kernel of its own); 2 per Krylov iteration unless a run is one
     // kernel
-    const int gk = ctx->g.V > kLoopsMax || ctx->loops_off ? 1 : p->c1 != 0.0 ? 4 : 2;
+    const int gk = !loops_usable(ctx) ? 1 : p->c1 != 0.0 ? 4 : 2;
     ctx->launches += 2 + gk + (5LL + gk) * p->nsteps + (ctx->lg_mode == kLgFused ? 5 : 6) * (st[1] + st[2]) +
                      (ctx->md_cg_run ? 0 : 2 * st[0]);
     ctx->krylov_iters += st[0];

@@ -31,6 +31,7 @@ int action_launch(rmhmc_ctx* ctx, double beta, double c1, double* S, double* pla
 // scratch (before a capture)
 constexpr int kLoopsMax = 1 << 22;
 constexpr int kSlotLoops = 41, kSlotLoopsEnd = 128;   // the partials may run on into the unused slots
+inline bool loops_usable(const rmhmc_ctx* ctx) { return ctx->use_loops && !ctx->loops_off && ctx->g.V <= kLoopsMax; }
 int gauge_loops_launch(rmhmc_ctx* ctx, double beta, double c1, int prec, double* F, bool act, bool* used, cudaStream_t st);
 int gauge_loops_prepare(rmhmc_ctx* ctx, double c1, int prec);
 // float64 force with action and average plaquette (each pointer nullable) of the context's links

@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(kBlock) k_adjoint_table64(Links64 U, double2* 
 }
 
 int links64_adjoint(rmhmc_ctx* ctx, Links64* U, cudaStream_t st) {
-    if (ctx->g.V > kAdTableMax || ctx->adj64_off) return RMHMC_OK;
+    if (ctx->g.V > kAdTableMax || ctx->adj64_off || !ctx->use_table) return RMHMC_OK;
     int status = RMHMC_OK;
     const unsigned long long ws = ctx->ws_gen;
     double2* t = (double2*)workspace(ctx, "ad_table64", sizeof(double2) * (size_t)ctx->g.V * 128, &status);

@@ -50,3 +50,29 @@ def test_gauge_force_full_size_sampled(L, c1):
     if L == (16, 16, 16, 16):
         S_ref, pl_ref = oracle.action(L, U, 6.0, c1)
         assert abs(S - S_ref) <= 1e-12 * abs(S_ref) and abs(pl - pl_ref) <= 1e-13
+
+
+@pytest.mark.parametrize("L", [(2, 2, 2, 2), (5, 3, 4, 7), (2, 3, 33, 2)])
+@pytest.mark.parametrize("c1", [0.0, -0.331])
+def test_staples_and_loops(L, c1):
+    """The staples of each link (the form above 2^22 sites and without memory for the loops) and the shared loops
+    against the oracle and each other, both precisions, with the bounds of the parity test."""
+    import paper_2112_04556_gb300 as rm
+    U = inputs.random_links(L, eps=0.6, seed=12)
+    ref = oracle.gauge_force(L, U, 6.0, c1)
+    S_ref, pl_ref = oracle.action(L, U, 6.0, c1)
+    with rm.Context(L) as ctx:
+        for loops in (0, 1, 0):
+            rm.set_stencil_shape(ctx, rm.SHAPE_LOOPS, rm.FP64, 18, loops, 128)
+            rm.counters(ctx, reset=True)
+            F, S, pl = rm.gauge_force(ctx, dev(U), 6.0, c1, prec=rm.FP64)
+            if not loops:   # links, staples, action
+                assert rm.counters(ctx)["launches"] == 3
+            assert rel_l2(host(F), ref) <= 1e-12
+            assert abs(S - S_ref) <= 1e-12 * abs(S_ref) and abs(pl - pl_ref) <= 1e-13
+            F32, S32, _ = rm.gauge_force(ctx, None, 6.0, c1, prec=rm.FP32)
+            assert rel_l2(host(F32), ref) <= 1e-5 and abs(S32 - S_ref) <= 1e-12 * abs(S_ref)
+        for bad in ((rm.FP32, 18, 1, 128), (rm.FP64, 12, 1, 128), (rm.FP64, 18, 2, 128), (rm.FP64, 18, 1, 64)):
+            for kernel in (rm.SHAPE_LOOPS, rm.SHAPE_TABLE):
+                with pytest.raises(rm.RmhmcError):
+                    rm.set_stencil_shape(ctx, kernel, *bad)

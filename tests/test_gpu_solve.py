@@ -339,3 +339,27 @@ def test_profiling_in_between_changes_nothing(prec):
     assert out[0][3] == 0 and out[1][3] > 0 and out[2][3] == out[1][3]
     assert np.array_equal(out[0][0], out[2][0]) and np.array_equal(out[0][1], out[2][1]) and out[0][2] == out[2][2]
     assert rel_l2(out[1][0], out[0][0]) <= 1e-9
+
+
+@pytest.mark.parametrize("L", [(2, 2, 2, 2), (5, 3, 4, 7), (6, 4, 5, 9)])
+def test_float64_without_the_table(L):
+    """float64 stencil, residuals, link derivative and kinetic force by 3x3 products (the form above 2^22 sites and
+    without memory for the table of adjoint matrices) and from the table, against the oracle with the bounds of the
+    parity tests."""
+    import paper_2112_04556_gb300 as rm
+    U = inputs.random_links(L, eps=0.5, seed=38)
+    X, Z = inputs.gaussian_fields(L, 2, seed=39)
+    m = fit.mass_term(12, 0.9)
+    y_ref, _ = oracle.rational_apply(L, U, X, m, tol=1e-14)
+    lap_ref, grad_ref = oracle.lap(L, U, X), oracle.lap_link_grad(L, U, X, Z, [0.7])
+    _, F_ref, V_ref = oracle.kinetic(L, U, X, m, tol=1e-13)
+    with rm.Context(L) as ctx:
+        Ud, Xd, Zd = dev(U), dev(X), dev(Z)
+        for table in (0, 1, 0):
+            rm.set_stencil_shape(ctx, rm.SHAPE_TABLE, rm.FP64, 18, table, 128)
+            assert rel_l2(host(rm.lap_apply(ctx, Ud, Xd)), lap_ref) <= 1e-13
+            assert rel_l2(host(rm.lap_link_grad(ctx, None, Xd, Zd, [0.7])), grad_ref) <= 1e-12
+            y, _, _, resid = rm.rat_mass_solve(ctx, None, Xd, m, tol=1e-12, prec=rm.FP64)
+            assert np.all(resid <= 1e-12) and rel_l2(host(y), y_ref) <= 1e-10
+            F, V, _ = rm.kinetic_force(ctx, None, Xd, m, tol=1e-12, prec=rm.FP64)
+            assert rel_l2(host(F), F_ref) <= 1e-9 and rel_l2(host(V), V_ref) <= 1e-9
