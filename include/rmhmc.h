@@ -127,8 +127,8 @@ typedef struct {
                            iteration has left shrinks by the contraction factor at every further iteration:
                            extra iterations remove that systematic part, so the mixed trajectory follows the
                            float64 one to the noise level. */
-    int fg_fp64;        /* gauge force inside the mixed-precision MD: 0 float32 staples from the float32 link
-                           copies, 1 float64 staples from the float64 links (the float64 MD always uses float64);
+    int fg_fp64;        /* gauge force inside the mixed-precision MD: 0 in float32 from the float32 link
+                           copies, 1 in float64 from the float64 links (the float64 MD always uses float64);
                            any other value: RMHMC_EINVAL */
 } rmhmc_params;
 
@@ -215,8 +215,8 @@ int rmhmc_tuning(const rmhmc_ctx* ctx, char* buf, int len);
                                    z-extent of the slabs in which the grid sweeps t, 1 .. L2 (0: L2, i.e.
                                    lexicographic order, the default) */
 #define RMHMC_SHAPE_LOOPS 5     /* gauge force and action (prec RMHMC_FP64, linkfmt 18, block 128): nmu 1 (the default) from
-                                   shared plaquettes and rectangles, on up to 2^22 sites; nmu 0 from the staples of each
-                                   link.  Applies to both precisions */
+                                   shared plaquettes and rectangles, for unitary links on up to 2^22 sites; nmu 0 from
+                                   the staples of each link.  Applies to both precisions */
 #define RMHMC_SHAPE_TABLE 6     /* float64 stencils and link derivative (prec RMHMC_FP64, linkfmt 18, block 128): nmu 1 (the
                                    default) from a table of the links' adjoint matrices (2 KB a site, on up to 2^22
                                    sites); nmu 0 by 3x3 products.  A pinned RMHMC_SHAPE_LAP or RMHMC_SHAPE_CG of
@@ -332,7 +332,8 @@ int rmhmc_action_noalloc(const int dims[4], const double* U, double beta, double
  *   S = beta sum_x [ c0 sum_{mu<nu} (1 - ReTr P_{mu nu}/3) + c1 sum_{mu!=nu} (1 - ReTr R_{mu nu}/3) ],
  * c0 = 1 - 8 c1 (c1 = 0: Wilson plaquette action), R the 1x2 rectangles.  action and plaq (host,
  * nullable) receive S and the average plaquette ReTr P/3, both summed in float64.
- * prec: RMHMC_FP64, or RMHMC_FP32 (float32 staples, float64 action). */
+ * prec: RMHMC_FP64, or RMHMC_FP32 (force in float32 arithmetic, float64 action).  U may be any matrices: unitary
+ * ones (to 2^-43, looked at once per import) share their loops, others take the staples of each link. */
 int gauge_force(rmhmc_ctx* ctx, const double* U, double beta, double c1, int prec, double* F,
                 double* action, double* plaq, cudaStream_t stream);
 

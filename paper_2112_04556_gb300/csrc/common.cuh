@@ -330,6 +330,10 @@ struct rmhmc_ctx {
     float2* u32b = nullptr;
     bool links_valid = false;
     unsigned long long link_gen = 1;   // bumped whenever the internal link copies change
+    unsigned long long import_gen = 0; // bumped by every import of the caller's links
+    unsigned long long su3_gen = 0;    // import_gen whose links were last looked at, and whether they are unitary (links_su3)
+    bool su3 = false;
+    bool own_capture = false;          // the library's streams are capturing a trajectory
     unsigned long long adj_gen = 0;    // link_gen the float32-pair adjoint table was built for
     unsigned long long adj64_gen = 0;  // and the float64 one
     bool loops_off = false;            // no memory for the gauge force's loops
@@ -357,6 +361,7 @@ struct rmhmc_ctx {
     cudaGraphExec_t md_exec = nullptr;
     std::string md_key;
     bool md_cg_run = false;             // its Krylov runs are cooperative (one kernel each)
+    bool md_loops = false;              // its gauge forces come from shared loops
     unsigned long long md_gen = 0;
     unsigned long long ws_gen = 0;      // bumped whenever a workspace buffer is (re)allocated
     cudaStream_t cap_st[3] = {};

@@ -100,6 +100,7 @@ int import_links(rmhmc_ctx* ctx, const double* U, cudaStream_t st) {
     RM_LAUNCH_CHECK(ctx);
     ctx->links_valid = true;
     ctx->link_gen++;
+    if (!ctx->own_capture) ctx->import_gen++;
     return RMHMC_OK;
 }
 

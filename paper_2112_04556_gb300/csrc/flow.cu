@@ -41,7 +41,7 @@ extern "C" int wilson_flow(rmhmc_ctx* ctx, double* U, double eps, int nsteps, in
         // the energy at the step's links comes with its first force (float64) or before it
         if (E && prec == RMHMC_FP64) {
             double plaq = 0.0;
-            RM_TRY(gauge_force_action(ctx, 1.0, 0.0, Z0, nullptr, &plaq, stream));
+            RM_TRY(gauge_force_action(ctx, 1.0, 0.0, RMHMC_FP64, Z0, nullptr, &plaq, stream));
             E[n] = 36.0 * (1.0 - plaq);
         } else {
             if (E) RM_TRY(energy(E + n));

@@ -10,7 +10,7 @@
 
 namespace rm {
 
-constexpr int kSlotAction = 40;
+constexpr int kSlotAction = 39;
 
 // index of the site c + n1 e_d1 + n2 e_d2 (|n1|, |n2| <= 2, d1 != d2 or n2 = 0), periodic, without division
 __device__ __forceinline__ int site_at(const Geom& g, const int c[4], int d1, int n1, int d2, int n2) {
@@ -202,26 +202,46 @@ static int action_loops(rmhmc_ctx* ctx, double beta, double c1, double* S, doubl
 
 int gauge_force_launch(rmhmc_ctx* ctx, double beta, double c1, int prec, double* F, cudaStream_t st) {
     bool used = false;
-    RM_TRY(gauge_loops_launch(ctx, beta, c1, prec, F, false, &used, st));
+    RM_TRY(gauge_loops_launch(ctx, beta, c1, prec, F, false, false, &used, st));
     return used ? RMHMC_OK : force_staples(ctx, beta, c1, prec, F, st);
 }
 
-int gauge_force_action(rmhmc_ctx* ctx, double beta, double c1, double* F, double* S, double* plaq, cudaStream_t st) {
-    bool used = false;
-    RM_TRY(gauge_loops_launch(ctx, beta, c1, RMHMC_FP64, F, true, &used, st));
-    if (!used) {
-        if (F) RM_TRY(force_staples(ctx, beta, c1, RMHMC_FP64, F, st));
-        return action_loops(ctx, beta, c1, S, plaq, st);
+int gauge_force_action(rmhmc_ctx* ctx, double beta, double c1, int prec, double* F, double* S, double* plaq,
+                       cudaStream_t st, bool su3) {
+    bool force = !F, act = false;
+    const bool check = (su3 || F || c1 != 0.0) && loops_usable(ctx) && su3_unknown(ctx);
+    if (check) RM_TRY(su3_check_launch(ctx, st));
+    if (F && prec != RMHMC_FP64) {
+        RM_TRY(gauge_loops_launch(ctx, beta, c1, prec, F, false, true, &force, st));
+        RM_TRY(gauge_loops_launch(ctx, beta, c1, RMHMC_FP64, nullptr, true, true, &act, st));
+    } else {
+        RM_TRY(gauge_loops_launch(ctx, beta, c1, RMHMC_FP64, F, true, true, &act, st));
+        force = force || act;
     }
-    double out[3];
-    RM_TRY(fetch(ctx, red_slot_out(ctx, kSlotLoops), out, 3, st));
+    double buf[8 + 3];
+    if (check || act) {
+        // the count of links that are not unitary, in the slot before the loops' sums
+        RM_TRY(fetch(ctx, red_slot_out(ctx, kSlotSu3), buf, 8 + 3, st));
+        if (check) {
+            su3_known(ctx, buf[0] == 0.0);
+            if (!ctx->su3) {
+                force = !F;
+                act = act && c1 == 0.0;
+            }
+        }
+    }
+    const bool staples = !force;
+    if (staples) RM_TRY(force_staples(ctx, beta, c1, prec, F, st));
+    if (!act) return action_loops(ctx, beta, c1, S, plaq, st);
+    if (staples) RM_CHECK(ctx, cudaStreamSynchronize(st));   // the staples run after the transfer
+    const double* out = buf + 8;
     if (S) *S = beta * ((1.0 - 8.0 * c1) * out[0] + (c1 != 0.0 ? c1 * out[2] : 0.0));
     if (plaq) *plaq = out[1] / (6.0 * ctx->g.V);
     return RMHMC_OK;
 }
 
 int action_launch(rmhmc_ctx* ctx, double beta, double c1, double* S, double* plaq, cudaStream_t st) {
-    return gauge_force_action(ctx, beta, c1, nullptr, S, plaq, st);
+    return gauge_force_action(ctx, beta, c1, RMHMC_FP64, nullptr, S, plaq, st);
 }
 
 }  // namespace rm
@@ -235,8 +255,6 @@ extern "C" int gauge_force(rmhmc_ctx* ctx, const double* U, double beta, double 
     if (prec != RMHMC_FP64 && prec != RMHMC_FP32) return set_err(ctx, RMHMC_EINVAL, "gauge_force: bad prec");
     if (!F && !action && !plaq) return set_err(ctx, RMHMC_EINVAL, "gauge_force: nothing to compute");
     RM_TRY(ensure_links(ctx, U, stream));
-    if (F && prec == RMHMC_FP64 && (action || plaq)) return gauge_force_action(ctx, beta, c1, F, action, plaq, stream);
-    if (F) RM_TRY(gauge_force_launch(ctx, beta, c1, prec, F, stream));
-    if (action || plaq) RM_TRY(action_launch(ctx, beta, c1, action, plaq, stream));
-    return RMHMC_OK;
+    if (action || plaq) return gauge_force_action(ctx, beta, c1, prec, F, action, plaq, stream);
+    return gauge_force_launch(ctx, beta, c1, prec, F, stream);
 }

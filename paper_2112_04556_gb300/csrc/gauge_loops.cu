@@ -8,14 +8,16 @@
 // Sorting the loops that hold U_m(y) by their base point gives, with -(beta/6) in front,
 //   F_m = sum_n { c0 (1 - T_n) k_mn + c1 [ (1 + T_m)(1 - T_n) r_mn - r_nm + T_n T_n r_nm ] }(y).
 // Per site that is 6 x 324 + 12 x 108 = 3240 FMA for the plaquette action and about 10,200 with rectangles, where the
-// staples take 5616 and 36,700; the action reads the traces of the same products.  The links have to be SU(3) (the
-// transport uses U U^dag = 1, as the Laplacian's traceless form does).
+// staples take 5616 and 36,700; the action reads the traces of the same products.  The transport and the rectangles use
+// U U^dag = 1: links that are not unitary to 2^-43 (say, read from single precision) keep the staples, which take any
+// matrices (links_su3; 173 us once per import at 24^3 x 48).
 //
 // float64 (0.55 TFMA/s) is bound by the operations, float32 was by re-reading the links of every staple from L2.  Measured at
 // 24^3 x 48, float32 Iwasaki force with its float64 action: 9.70 ms with staples, 6.84 ms here; float64 Wilson flow at 16^4,
 // 8 steps: 23.8 -> 15.6 ms.
 #include <algorithm>
 
+#include "df.cuh"
 #include "krylov.cuh"
 #include "ops.cuh"
 #include "stencil.cuh"
@@ -283,10 +285,71 @@ static int loops_t(rmhmc_ctx* ctx, const typename LinksOf<T>::type& U, double be
     return RMHMC_OK;
 }
 
-int gauge_loops_launch(rmhmc_ctx* ctx, double beta, double c1, int prec, double* F, bool act, bool* used,
+// Number of links with an entry of U U^dag - 1 above 2^-43 or not a number.  Thread per link; float-float (errors of about
+// 1e-14), since float64 would take 0.35 ms at 24^3 x 48 (this: 0.17 ms).
+__global__ void __launch_bounds__(kBlock) k_su3_check(Links64 U, double* partials, unsigned* counter, double* out) {
+    int bad = 0;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 4 * U.V; i += gridDim.x * blockDim.x) {
+        const int mu = i / U.V, s = i - mu * U.V;
+        cdfl u[9];
+#pragma unroll
+        for (int e = 0; e < 9; e++) {
+            const double2 v = __ldg(U.u + (size_t)(mu * 9 + e) * U.V + s);
+            u[e] = cdf_make(df_split(v.x), df_split(v.y));
+        }
+        bool ok = true;
+        auto within = [&](dfl x) { ok = ok && fabsf(x.hi + x.lo) <= 0x1p-43f; };
+#pragma unroll
+        for (int a = 0; a < 3; a++)
+#pragma unroll
+            for (int b = a; b < 3; b++) {
+                cdfl t = cdf_mul(u[3 * a], cdf_conj(u[3 * b]));
+                t = cdf_add(t, cdf_mul(u[3 * a + 1], cdf_conj(u[3 * b + 1])));
+                t = cdf_add(t, cdf_mul(u[3 * a + 2], cdf_conj(u[3 * b + 2])));
+                within(a == b ? df_sub(t.re, df_make(1.f, 0.f)) : t.re);
+                if (a != b) within(t.im);
+            }
+        bad += !ok;
+    }
+    __shared__ double sh[kBlock / 32];
+    double v[1] = {(double)bad};
+    block_sum<1>(v, sh);
+    grid_sum_finish<1>(v, partials, counter, out, gridDim.x, blockIdx.x, sh);
+}
+
+int su3_check_launch(rmhmc_ctx* ctx, cudaStream_t st) {
+    k_su3_check<<<capped_grid(ctx, (size_t)4 * ctx->g.V, kBlock), kBlock, 0, st>>>(
+        links64(ctx), red_slot_partials(ctx, kSlotSu3), red_slot_counter(ctx, kSlotSu3), red_slot_out(ctx, kSlotSu3));
+    ++ctx->launches;
+    RM_LAUNCH_CHECK(ctx);
+    return RMHMC_OK;
+}
+
+void su3_known(rmhmc_ctx* ctx, bool su3) {
+    ctx->su3 = su3;
+    ctx->su3_gen = ctx->import_gen;
+}
+
+int links_su3(rmhmc_ctx* ctx, cudaStream_t st, bool* su3) {
+    if (su3_unknown(ctx)) {
+        double bad = 0.0;
+        RM_TRY(su3_check_launch(ctx, st));
+        RM_TRY(fetch(ctx, red_slot_out(ctx, kSlotSu3), &bad, 1, st));
+        su3_known(ctx, bad == 0.0);
+    }
+    *su3 = ctx->su3;
+    return RMHMC_OK;
+}
+
+int gauge_loops_launch(rmhmc_ctx* ctx, double beta, double c1, int prec, double* F, bool act, bool defer, bool* used,
                        cudaStream_t st) {
     *used = false;
     if (!loops_usable(ctx)) return RMHMC_OK;
+    if (F || c1 != 0.0) {
+        bool su3 = true;
+        if (!defer || !su3_unknown(ctx)) RM_TRY(links_su3(ctx, st, &su3));
+        if (!su3) return RMHMC_OK;
+    }
     const int s = prec == RMHMC_FP64 ? loops_t<double>(ctx, links64(ctx), beta, c1, F, act, st)
                                      : loops_t<float>(ctx, links32(ctx), beta, c1, F, false, st);
     if (s == RMHMC_ENOMEM) {

@@ -960,6 +960,7 @@ static int md_graph_capture(rmhmc_ctx* ctx, const rmhmc_params* p, const MassTer
     const int gprec = md_gauge_prec(p);
     const bool ff = p->prec == RMHMC_MIXED;
     RM_CHECK(ctx, cudaStreamBeginCapture(st, cudaStreamCaptureModeRelaxed));
+    ctx->own_capture = true;
     int s = RMHMC_OK;
     do {
         // U-only potential force: gauge force, plus the auxiliary-field force as one more captured kinetic
@@ -1042,6 +1043,7 @@ static int md_graph_capture(rmhmc_ctx* ctx, const rmhmc_params* p, const MassTer
             if ((s = mom_update(ctx, gb.P, 0.5 * eps, w.FG, w.FK, nullptr, w.Q, nullptr, st)) != RMHMC_OK) break;
         }
     } while (0);
+    ctx->own_capture = false;
     cudaGraph_t g = nullptr;
     const cudaError_t e = cudaStreamEndCapture(st, &g);
     if (s != RMHMC_OK) {
@@ -1057,10 +1059,11 @@ static int md_graph_capture(rmhmc_ctx* ctx, const rmhmc_params* p, const MassTer
     return RMHMC_OK;
 }
 
+// imported: the context holds U already.
 // Runs the MD through the cached graph; returns RMHMC_OK, a status of the run, or a negative code of the
 // capture (the caller then falls back to the host-driven path)
 static int md_graph_run(rmhmc_ctx* ctx, double* U, double* P, const rmhmc_params* p, const MassTerm& m, rmhmc_result* r,
-                        cudaStream_t stream, bool* used, const AuxTerm* lg = nullptr) {
+                        cudaStream_t stream, bool* used, const AuxTerm* lg = nullptr, bool imported = false) {
     *used = false;
     if (!ctx->use_graphs || p->prec == RMHMC_FP64 || p->symplectic || m.npole() == 0 || 2 * m.npole() + 1 > 32)
         return RMHMC_OK;
@@ -1074,9 +1077,14 @@ static int md_graph_run(rmhmc_ctx* ctx, double* U, double* P, const rmhmc_params
         if (lg->inv.npole() == 0 || 2 * lg->inv.npole() + 1 > 32) return RMHMC_OK;
         RM_TRY(kinetic_graph_prepare(ctx, lg->inv, p->maxiter));
     }
+    bool su3 = false;
+    if (loops_usable(ctx)) {
+        if (!imported) RM_TRY(import_links(ctx, U, stream));
+        RM_TRY(links_su3(ctx, stream, &su3));
+    }
     for (int i = 0; i < 3; i++)
         if (!ctx->cap_st[i]) RM_CHECK(ctx, cudaStreamCreateWithFlags(&ctx->cap_st[i], cudaStreamNonBlocking));
-    const std::string key = md_key(ctx, p, m) + (lg ? "|logdet" : "");
+    const std::string key = md_key(ctx, p, m) + (lg ? "|logdet" : "") + (su3 ? "|loops" : "");
     if (!ctx->md_exec || ctx->md_key != key || ctx->md_gen != ctx->ws_gen) {
         if (ctx->md_exec) {
             cudaGraphExecDestroy(ctx->md_exec);
@@ -1112,6 +1120,7 @@ static int md_graph_run(rmhmc_ctx* ctx, double* U, double* P, const rmhmc_params
         }
         ctx->md_key = key;
         ctx->md_cg_run = cg_run_fits<float>(ctx, true);
+        ctx->md_loops = su3 && loops_usable(ctx);
         ctx->md_gen = ctx->ws_gen;
         ctx->graph_note = "md graph captured";
     }
@@ -1133,7 +1142,7 @@ static int md_graph_run(rmhmc_ctx* ctx, double* U, double* P, const rmhmc_params
     // kernels the graph ran: links, gauge force (1 to 4 kernels), momenta; 5 and a gauge force per step outside the loops; 5
     // per fixed-point iteration (6 with the velocity in a kernel of its own); 2 per Krylov iteration unless a run is one
     // kernel
-    const int gk = !loops_usable(ctx) ? 1 : p->c1 != 0.0 ? 4 : 2;
+    const int gk = !ctx->md_loops ? 1 : p->c1 != 0.0 ? 4 : 2;
     ctx->launches += 2 + gk + (5LL + gk) * p->nsteps + (ctx->lg_mode == kLgFused ? 5 : 6) * (st[1] + st[2]) +
                      (ctx->md_cg_run ? 0 : 2 * st[0]);
     ctx->krylov_iters += st[0];
@@ -1157,8 +1166,9 @@ static int md_graph_run(rmhmc_ctx* ctx, double* U, double* P, const rmhmc_params
 }
 
 // T = 1/2 |R(A) P|^2 with every shift at relative residual tol_h (float64 check), S, plaquette
+// (su3: the molecular dynamics follows, whose forces ask whether these links are unitary)
 static int hamiltonian_run(rmhmc_ctx* ctx, const double* U, const double* P, const rmhmc_params* p, const MassTerm& m,
-                           double* H, double* T, double* S, double* plaq, cudaStream_t st) {
+                           double* H, double* T, double* S, double* plaq, cudaStream_t st, bool su3 = false) {
     int status = RMHMC_OK;
     const size_t fs = field_elems(ctx);
     RM_TRY(import_links(ctx, U, st));
@@ -1167,7 +1177,7 @@ static int hamiltonian_run(rmhmc_ctx* ctx, const double* U, const double* P, con
     RM_TRY(rational_apply(ctx, m, P, p->tol_h, p->maxiter, p->prec, Y, nullptr, st));
     double y2 = 0.0, s = 0.0, pl = 0.0;
     RM_TRY(norm2_64(ctx, Y, fs, &y2, st));
-    RM_TRY(action_launch(ctx, p->beta, p->c1, &s, &pl, st));
+    RM_TRY(gauge_force_action(ctx, p->beta, p->c1, RMHMC_FP64, nullptr, &s, &pl, st, su3));
     const double t = 0.5 * y2;
     if (!isfinite(t) || !isfinite(s)) return set_err(ctx, RMHMC_ENAN, "NaN/Inf in the Hamiltonian");
     if (T) *T = t;
@@ -1291,11 +1301,11 @@ extern "C" int rmhmc_trajectory(rmhmc_ctx* ctx, double* U, const double* xi, con
     // start from the same momenta
     int s = heatbath_apply(ctx, m, X, p->tol_h, p->maxiter, p->prec, P, stream);
     if (s != RMHMC_OK) return restore(s);
-    s = hamiltonian_run(ctx, U, P, p, m, &res.H0, &res.T0, &res.S0, nullptr, stream);
+    s = hamiltonian_run(ctx, U, P, p, m, &res.H0, &res.T0, &res.S0, nullptr, stream, true);
     if (s == RMHMC_OK) s = aux_action(&res.A0);
     if (s != RMHMC_OK) return restore(s);
     bool used = false;
-    s = md_graph_run(ctx, U, P, p, m, &res, stream, &used, lg);
+    s = md_graph_run(ctx, U, P, p, m, &res, stream, &used, lg, true);
     if (s == RMHMC_OK && !used) s = md_run(ctx, U, P, p, m, &res, stream, lg);
     if (s != RMHMC_OK) return restore(s);
     s = hamiltonian_run(ctx, U, P, p, m, &res.H1, &res.T1, &res.S1, &res.plaq, stream);

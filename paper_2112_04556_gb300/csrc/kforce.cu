@@ -87,8 +87,8 @@ __global__ void __launch_bounds__(kBlock) k_link_grad(Geom g, Links64 U, const d
 #pragma unroll
             for (int i = 0; i < 2; i++) {
                 herm<double> E = h_zero<double>();
-                acc_uxud_tl(E, u, coef_to_herm2(C[i]));
-                herm2_to_coef_tl(E, r[i]);
+                acc_uxud(E, u, coef_to_herm2(C[i]));   // (with its trace: exact for any matrix, as the table)
+                herm2_to_coef(E, r[i]);
             }
         }
 #pragma unroll

@@ -25,17 +25,29 @@ constexpr int kAdMinFields = 6;
 int gauge_force_launch(rmhmc_ctx* ctx, double beta, double c1, int prec, double* F, cudaStream_t st);
 // action S and average plaquette (float64, deterministic) from the context's float64 links
 int action_launch(rmhmc_ctx* ctx, double beta, double c1, double* S, double* plaq, cudaStream_t st);
+// Whether the links imported last are unitary to 2^-43 (the rounding a long chain of updates leaves; what the library's own
+// updates make of them keeps that property).  Looked at once per import; synchronises the stream then.
+int links_su3(rmhmc_ctx* ctx, cudaStream_t st, bool* su3);
+int su3_check_launch(rmhmc_ctx* ctx, cudaStream_t st);   // the number of other links to the slot kSlotSu3
+void su3_known(rmhmc_ctx* ctx, bool su3);
+inline bool su3_unknown(const rmhmc_ctx* ctx) { return ctx->su3_gen != ctx->import_gen; }
+constexpr int kSlotSu3 = 40;
 // Force (F not null) and, in float64, the loop sums of the action (act) from shared loops (gauge_loops.cu), on lattices of up
 // to kLoopsMax sites (scratch: up to 4.5 KB a site in float64); *used tells whether it ran.  The sums go to the slot kSlotLoops:
-// sum (1 - ReTr P/3), sum ReTr P/3 over plaquettes, sum (1 - ReTr R/3) over rectangles.  gauge_loops_prepare allocates the
+// sum (1 - ReTr P/3), sum ReTr P/3 over plaquettes, sum (1 - ReTr R/3) over rectangles.  The force and the rectangles need
+// unitary links; where that is not known yet it is looked at first or, with defer, left to the caller's fetch (the slot
+// kSlotSu3).  gauge_loops_prepare allocates the
 // scratch (before a capture)
 constexpr int kLoopsMax = 1 << 22;
 constexpr int kSlotLoops = 41, kSlotLoopsEnd = 128;   // the partials may run on into the unused slots
 inline bool loops_usable(const rmhmc_ctx* ctx) { return ctx->use_loops && !ctx->loops_off && ctx->g.V <= kLoopsMax; }
-int gauge_loops_launch(rmhmc_ctx* ctx, double beta, double c1, int prec, double* F, bool act, bool* used, cudaStream_t st);
+int gauge_loops_launch(rmhmc_ctx* ctx, double beta, double c1, int prec, double* F, bool act, bool defer, bool* used,
+                       cudaStream_t st);
 int gauge_loops_prepare(rmhmc_ctx* ctx, double c1, int prec);
-// float64 force with action and average plaquette (each pointer nullable) of the context's links
-int gauge_force_action(rmhmc_ctx* ctx, double beta, double c1, double* F, double* S, double* plaq, cudaStream_t st);
+// force (in prec's arithmetic) with float64 action and average plaquette (each pointer nullable) of the context's links; su3:
+// the answer of links_su3 with the same transfer, for a later force
+int gauge_force_action(rmhmc_ctx* ctx, double beta, double c1, int prec, double* F, double* S, double* plaq,
+                       cudaStream_t st, bool su3 = false);
 // G = sum_f w_f d<Z_f, A X_f>/dw (X, Z in the arithmetic precision, [nf][V][4][8]); G float64 [V][4][8]
 int link_grad_launch(rmhmc_ctx* ctx, int prec, const void* X, const void* Z, int nf, const double* w, double* G,
                      cudaStream_t st);
