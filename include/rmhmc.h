@@ -25,6 +25,11 @@
  *  Streams  Every call takes a cudaStream_t (0 = legacy default stream) and enqueues its work there.
  *           Calls that return host scalars synchronise that stream before returning.
  *  Threads  A context is not thread-safe: use one context per host thread / stream.
+ *  Capture  Calls that return nothing to the host (rmhmc_set_links, lap_apply, lap_link_grad in float64, gauge_force without
+ *           action and plaq, rmhmc_link_update, rmhmc_gauss_field) may be captured into a CUDA graph of the caller's
+ *           once their buffers exist (after one call outside a capture).  A replay reads the context's links of its own
+ *           time.  Captured float64 calls take the forms that keep nothing derived from the links (3x3 products,
+ *           staples); once a set of links has been imported by a captured call, so do the context's other calls.
  *  Errors   Every entry point returns RMHMC_OK (0) or a negative status.  rmhmc_last_error(ctx) gives
  *           a message.  On error the contents of output buffers are unspecified, except that
  *           rmhmc_trajectory leaves U unchanged.

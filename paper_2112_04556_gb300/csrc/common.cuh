@@ -334,6 +334,7 @@ struct rmhmc_ctx {
     unsigned long long su3_gen = 0;    // import_gen whose links were last looked at, and whether they are unitary (links_su3)
     bool su3 = false;
     bool own_capture = false;          // the library's streams are capturing a trajectory
+    bool links_in_graph = false;       // a graph of the caller's imports links: the host no longer sees when they change
     unsigned long long adj_gen = 0;    // link_gen the float32-pair adjoint table was built for
     unsigned long long adj64_gen = 0;  // and the float64 one
     bool loops_off = false;            // no memory for the gauge force's loops
@@ -428,8 +429,17 @@ inline int capped_grid(const rmhmc_ctx* ctx, size_t threads, int block) {
     return (int)std::min(cap, (g + sms - 1) / sms * sms);   // whole blocks per SM
 }
 inline Links64 links64(const rmhmc_ctx* ctx) { return Links64{ctx->u64, ctx->g.V, nullptr}; }
+// whether st is being captured into a graph of the caller's: such a graph reads the links it finds when it is replayed, so
+// that it must not hold what the host derived from those of today (the float64 table, whether they are unitary)
+inline bool caller_captures(const rmhmc_ctx* ctx, cudaStream_t st) {
+    if (ctx->own_capture) return false;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) cudaGetLastError();   // (the legacy stream beside a capture)
+    return cs == cudaStreamCaptureStatusActive;
+}
+inline bool links_tracked(const rmhmc_ctx* ctx, cudaStream_t st) { return !ctx->links_in_graph && !caller_captures(ctx, st); }
 // the links with their float64 adjoint table, built if the links changed since; ad is null where a table is not used
-// (more than kAdTableMax sites, or no memory for it)
+// (more than kAdTableMax sites, no memory for it, links that change behind the host's back)
 constexpr int kAdTableMax = 1 << 22;   // 2 KB a site
 int links64_adjoint(rmhmc_ctx* ctx, Links64* U, cudaStream_t st);
 inline Links32 links32(const rmhmc_ctx* ctx) { return Links32{ctx->u32a, ctx->u32b, ctx->g.V}; }

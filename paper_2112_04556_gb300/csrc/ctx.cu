@@ -96,6 +96,7 @@ __global__ void k_import_links(const double* __restrict__ U, double2* __restrict
 
 int import_links(rmhmc_ctx* ctx, const double* U, cudaStream_t st) {
     if (((uintptr_t)U) % 16) return set_err(ctx, RMHMC_EINVAL, "links must be 16-byte aligned");
+    if (caller_captures(ctx, st)) ctx->links_in_graph = true;
     k_import_links<<<site_blocks(ctx), kBlock, 0, st>>>(U, ctx->u64, ctx->u32a, ctx->u32b, ctx->g.V); ++ctx->launches;
     RM_LAUNCH_CHECK(ctx);
     ctx->links_valid = true;

@@ -209,7 +209,7 @@ int gauge_force_launch(rmhmc_ctx* ctx, double beta, double c1, int prec, double*
 int gauge_force_action(rmhmc_ctx* ctx, double beta, double c1, int prec, double* F, double* S, double* plaq,
                        cudaStream_t st, bool su3) {
     bool force = !F, act = false;
-    const bool check = (su3 || F || c1 != 0.0) && loops_usable(ctx) && su3_unknown(ctx);
+    const bool check = (su3 || F || c1 != 0.0) && loops_usable(ctx) && su3_unknown(ctx) && links_tracked(ctx, st);
     if (check) RM_TRY(su3_check_launch(ctx, st));
     if (F && prec != RMHMC_FP64) {
         RM_TRY(gauge_loops_launch(ctx, beta, c1, prec, F, false, true, &force, st));

@@ -344,7 +344,7 @@ int links_su3(rmhmc_ctx* ctx, cudaStream_t st, bool* su3) {
 int gauge_loops_launch(rmhmc_ctx* ctx, double beta, double c1, int prec, double* F, bool act, bool defer, bool* used,
                        cudaStream_t st) {
     *used = false;
-    if (!loops_usable(ctx)) return RMHMC_OK;
+    if (!loops_usable(ctx) || !links_tracked(ctx, st)) return RMHMC_OK;
     if (F || c1 != 0.0) {
         bool su3 = true;
         if (!defer || !su3_unknown(ctx)) RM_TRY(links_su3(ctx, st, &su3));

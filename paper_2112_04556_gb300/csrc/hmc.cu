@@ -1078,7 +1078,7 @@ static int md_graph_run(rmhmc_ctx* ctx, double* U, double* P, const rmhmc_params
         RM_TRY(kinetic_graph_prepare(ctx, lg->inv, p->maxiter));
     }
     bool su3 = false;
-    if (loops_usable(ctx)) {
+    if (loops_usable(ctx) && links_tracked(ctx, stream)) {
         if (!imported) RM_TRY(import_links(ctx, U, stream));
         RM_TRY(links_su3(ctx, stream, &su3));
     }

@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(kBlock) k_adjoint_table64(Links64 U, double2* 
 }
 
 int links64_adjoint(rmhmc_ctx* ctx, Links64* U, cudaStream_t st) {
-    if (ctx->g.V > kAdTableMax || ctx->adj64_off || !ctx->use_table) return RMHMC_OK;
+    if (ctx->g.V > kAdTableMax || ctx->adj64_off || !ctx->use_table || !links_tracked(ctx, st)) return RMHMC_OK;
     int status = RMHMC_OK;
     const unsigned long long ws = ctx->ws_gen;
     double2* t = (double2*)workspace(ctx, "ad_table64", sizeof(double2) * (size_t)ctx->g.V * 128, &status);
@@ -219,7 +219,7 @@ int adjoint_table(rmhmc_ctx* ctx, float** tab, cudaStream_t st) {
     *tab = t;
     // the table of the current links is kept until they change (a heatbath and the Hamiltonian that follows
     // share it)
-    if (ctx->adj_gen == ctx->link_gen && ws == ctx->ws_gen) return RMHMC_OK;
+    if (ctx->adj_gen == ctx->link_gen && ws == ctx->ws_gen && !ctx->links_in_graph) return RMHMC_OK;
     const dim3 grid(site_blocks(ctx), 4);
     k_adjoint_table<<<grid, kBlock, 0, st>>>(links64(ctx), ctx->g.V, t); ++ctx->launches;
     RM_LAUNCH_CHECK(ctx);

@@ -3,6 +3,8 @@ points and every Krylov run, decided on the device) against the host-driven path
 import numpy as np
 import pytest
 
+import oracle
+
 from gpu_util import dev, host, rel_l2, torch_cuda
 from paper_2112_04556_gb300 import inputs
 
@@ -99,3 +101,58 @@ def test_wait_that_runs_out_ends_the_graph(logdet):
         rm.set_wait_limit(ctx)
         again, r2 = trajectory()
     assert np.array_equal(again, want) and r2["dH"] == r["dH"]
+
+
+@pytest.mark.parametrize("L", [(4, 4, 4, 4), (5, 3, 4, 7)])
+def test_graph_of_the_callers(L):
+    """Calls captured into the caller's own graph read the links of the replay: float64 stencil, link derivative and force,
+    with the links set between replays, and with an import in the graph, after which
+    the context's other calls see the links of the last replay too.  Bounds of the parity tests."""
+    import paper_2112_04556_gb300 as rm
+    torch = torch_cuda()
+    Us = [inputs.random_links(L, eps=0.5, seed=s) for s in (81, 82)]
+    X, Z = inputs.gaussian_fields(L, 2, seed=84)
+    m = rm.mass_fit(12, 0.9)
+    with rm.Context(L) as ctx:
+        Ud, Xd, Zd = dev(Us[0]), dev(X), dev(Z)
+        Y, G, F = (torch.empty_like(Xd) for _ in range(3))
+
+        def calls(links=None):
+            rm.lap_apply(ctx, links, Xd, Y)
+            rm.lap_link_grad(ctx, None, Xd, Zd, [0.7], G=G)
+            ctx.check(rm.lib().gauge_force(ctx.h, None, 6.0, -0.331, rm.FP64, F.data_ptr(), None, None, rm._raw_stream()))
+
+        def check(U):
+            assert rel_l2(host(Y), oracle.lap(L, U, X)) <= 1e-12
+            assert rel_l2(host(G), oracle.lap_link_grad(L, U, X, Z, [0.7])) <= 1e-12
+            assert rel_l2(host(F), oracle.gauge_force(L, U, 6.0, -0.331)) <= 1e-12
+
+        calls(Ud)
+        check(Us[0])
+        held, bringing = torch.cuda.CUDAGraph(), torch.cuda.CUDAGraph()
+        with torch.cuda.graph(held):
+            calls()
+        for U in Us + Us[:1]:
+            rm.set_links(ctx, dev(U))
+            for t in (Y, G, F):
+                t.zero_()
+            held.replay()
+            torch.cuda.synchronize()
+            check(U)
+        rm.set_links(ctx, dev(Us[1]))
+        calls()                     # outside the graph again: table and loops of the present links
+        check(Us[1])
+        with torch.cuda.graph(bringing):
+            calls(Ud)
+        for U in (Us[1], Us[0]):
+            Ud.copy_(dev(U))
+            bringing.replay()
+            torch.cuda.synchronize()
+            check(U)
+            for t in (Y, G, F):
+                t.zero_()
+            calls()
+            check(U)
+            y, _, _, resid = rm.rat_mass_solve(ctx, None, Xd, m, tol=1e-11, prec=rm.MIXED)
+            assert np.all(resid <= 1e-11)
+            assert rel_l2(host(y), oracle.rational_apply(L, U, X, m, tol=1e-13)[0]) <= 1e-9

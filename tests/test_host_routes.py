@@ -177,3 +177,33 @@ def test_link_derivative_kernel_by_precision(rm, prec, kernel):
         ctx.check(rm.lib().lap_link_grad(ctx.h, None, FIELD, OUT, 3, w.ctypes.data_as(ctypes.POINTER(ctypes.c_double)),
                                          prec, OUT2, None))
         assert "%d%sI" % (len(kernel), kernel) in [k for k in launched(rm) if "k_link_grad" in k][-1]
+
+
+def test_captured_calls_keep_nothing_derived_from_the_links(rm):
+    """Under a capture of the caller's the float64 stencil and link derivative run by 3x3 products and the gauge force on
+    staples, nothing is timed or allocated, and the calls after it go on from the table and the loops; a captured import
+    ends both for the context."""
+    def calls():
+        one = np.ones(1).ctypes.data_as(ctypes.POINTER(ctypes.c_double))
+        ctx.check(rm.lib().lap_apply(ctx.h, None, FIELD, OUT, 1, rm.FP64, 18, 0, None))
+        ctx.check(rm.lib().lap_link_grad(ctx.h, None, FIELD, OUT, 1, one, rm.FP64, OUT2, None))
+        ctx.check(rm.lib().gauge_force(ctx.h, None, 6.0, 0.0, rm.FP64, OUT2, None, None, None))
+        names = " ".join(launched(rm))
+        return ["k_lapIdLi64E" in names, "k_link_gradILi64E" in names, "k_loop_force" in names]
+    derived, direct = [True] * 3, [False] * 3
+    with context(rm, (4, 4, 4, 4)) as ctx:
+        rm.lib().fake_capturing(1)
+        held = rm.lib().fake_held()
+        assert calls() == direct and rm.lib().fake_held() == held
+        rm.lib().fake_capturing(0)
+        assert calls() == derived
+        rm.lib().fake_capturing(1)
+        assert calls() == direct
+        rm.lib().fake_capturing(0)
+        assert calls() == derived
+        rm.lib().fake_capturing(1)
+        ctx.check(rm.lib().rmhmc_set_links(ctx.h, LINKS, None))
+        rm.lib().fake_capturing(0)
+        assert calls() == direct
+        assert trajectory_md(rm, ctx) == rm.OK
+        assert not any("k_plaquettes" in k for k in launched(rm))
