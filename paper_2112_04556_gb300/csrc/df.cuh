@@ -52,13 +52,14 @@ struct SumSq32 {
 // float64 arithmetic (float64 runs at a small fraction of the float32 rate on this part).  df_split: hi = x
 // rounded to 24 significant bits (its 29 low significand bits dropped, rounding half away from zero, a carry
 // moving into the exponent), lo = the signed remainder (at most 2^28 units of x's last place) as a float times
-// 2^(e - 52); |lo| <= ulp(hi) / 2 and hi + lo = x to 2^-49 |x|.  |x| below 2^-126 gives 0 and |x|
-// near or above 2^128 gives +-inf (NaN too); lo keeps what float32's subnormals hold of it.
+// 2^(e - 52); |lo| <= ulp(hi) / 2 and hi + lo = x to 2^-49 |x|.  |x| below 2^-126 takes the conversion instruction (hi the
+// nearest subnormal, lo 0) and |x| near or above 2^128 gives +-inf (NaN too); lo keeps what float32's subnormals hold of
+// it.
 __device__ __forceinline__ dfl df_split(double x) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
     const int e = (int)((b >> 52) & 0x7ff);
-    if (e < 1023 - 126) return df_make(__uint_as_float(sign), __uint_as_float(sign));
+    if (e < 1023 - 126) return df_make((float)x, 0.f);
     const unsigned long long m = b & 0x1fffffffull;
     const bool up = m >= (1ull << 28);
     const unsigned long long bh = (b & ~0x1fffffffull) + (up ? (1ull << 29) : 0ull);
@@ -70,25 +71,24 @@ __device__ __forceinline__ dfl df_split(double x) {
         const int r = up ? (int)m - (1 << 29) : (int)m;
         lo = __int2float_rn(r) * __uint_as_float((unsigned)(e - 948) << 23);
         if (sign) lo = -lo;
-    } else {   // 2^(e - 1075) in two steps: lo may end among the subnormals
-        const int r = up ? (int)m - (1 << 29) : (int)m;
-        lo = __int2float_rn(r) * __uint_as_float((unsigned)(e - 884) << 23) * 0x1p-64f;
-        if (sign) lo = -lo;
+    } else {   // lo may end among the subnormals: rounded once, by the instruction
+        lo = (float)(x - (double)hi);
     }
     return df_make(hi, lo);
 }
-// the nearest float of a value, without a float64 conversion (|x| below 2^-126 gives 0)
+// the nearest float of a value, without a float64 conversion but for |x| below 2^-126 (float32's subnormals: a field that
+// small must not turn into a field of zeros, which every solve would call solved)
 __device__ __forceinline__ float to_f32(float x) { return x; }
 __device__ __forceinline__ float to_f32(double x) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
     const int e = (int)((b >> 52) & 0x7ff);
-    if (e < 1023 - 126) return __uint_as_float(sign);
+    if (e < 1023 - 126) return (float)x;
     if (e > 1023 + 127) return __uint_as_float(sign | (e == 0x7ff && (b << 12) ? 0x7fc00000u : 0x7f800000u));
     // round half to even at bit 29; a carry moves into the exponent (up to infinity)
     const unsigned long long m = b & 0x7fffffffffffffffull;
     const unsigned long long r = m + 0x0fffffffull + ((m >> 29) & 1ull);
-    return __uint_as_float(sign | (unsigned)((r >> 29) - (unsigned long long)((1023 - 127) << 23)));
+    return __uint_as_float(sign | ((unsigned)(r >> 29) - ((1023u - 127u) << 23)));
 }
 // a float as a double, from its bit fields (normal numbers, zero, inf and NaN; subnormals give 0)
 __device__ __forceinline__ double f_to_d_bits(float f) {

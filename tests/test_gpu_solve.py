@@ -363,3 +363,25 @@ def test_float64_without_the_table(L):
             assert np.all(resid <= 1e-12) and rel_l2(host(y), y_ref) <= 1e-10
             F, V, _ = rm.kinetic_force(ctx, None, Xd, m, tol=1e-12, prec=rm.FP64)
             assert rel_l2(host(F), F_ref) <= 1e-9 and rel_l2(host(V), V_ref) <= 1e-9
+
+
+@pytest.mark.parametrize("scale", [1e-39, 1e-42])
+def test_fields_below_float32s_normal_range(scale):
+    """A right-hand side or momenta whose values are float32 subnormals: the float32 recurrence cannot hold their squares and
+    says so (ENAN); they are not taken for zero and called solved."""
+    import paper_2112_04556_gb300 as rm
+    L = (4, 4, 4, 4)
+    b = dev(scale * inputs.gaussian_fields(L, 1, seed=46)[0])
+    m = rm.mass_fit(12, 0.9)
+    with rm.Context(L) as ctx:
+        rm.set_links(ctx, dev(inputs.random_links(L, eps=0.4, seed=45)))
+        for pinned in (False, True):
+            if pinned:   # the two-kernel form
+                rm.set_stencil_shape(ctx, rm.SHAPE_CG, rm.FP32, 18, 1, 128)
+            for call in (lambda: rm.rat_mass_solve(ctx, None, b, m, tol=1e-10, prec=rm.MIXED),
+                         lambda: rm.kinetic_force(ctx, None, b, m, tol=1e-6, prec=rm.MIXED)):
+                with pytest.raises(rm.RmhmcError) as e:
+                    call()
+                assert e.value.code == rm.ENAN
+        y, _, _, resid = rm.rat_mass_solve(ctx, None, b, m, tol=1e-10, prec=rm.FP64)
+        assert np.all(resid <= 1e-10) and float(y.abs().max()) > 0.0

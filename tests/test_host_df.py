@@ -18,6 +18,14 @@ extern "C" double sum_squares(const float* x, int n) {
     for (int i = 0; i < n; i++) a.add(x[i]);
     return a.value();
 }
+extern "C" void convert(const double* x, int n, float* f, float* hi, float* lo) {
+    for (int i = 0; i < n; i++) {
+        f[i] = to_f32(x[i]);
+        const dfl d = df_split(x[i]);
+        hi[i] = d.hi;
+        lo[i] = d.lo;
+    }
+}
 """
 
 
@@ -52,3 +60,22 @@ def test_sum_of_squares_is_float64_accurate(df, n, spread):
         assert abs(Fraction(got) - want) <= bound, (seed, float(abs(Fraction(got) - want) / want))
         worst = max(worst, float(abs(Fraction(got) - want) / want))
     assert worst < 1e-12
+
+
+def test_conversions_over_all_exponents(df):
+    """to_f32 rounds as the conversion instruction does, subnormals, infinities and NaN included; df_split's pair holds a
+    value to 2^-49 of it (2^-150 absolute among the subnormals), the high part a float next to it."""
+    rng = np.random.default_rng(1)
+    x = np.concatenate([((1.0 + rng.random(40)) * s * 2.0 ** e) for e in range(-1022, 1023) for s in (1, -1)])
+    tie = np.float64(np.float32(1.0 + rng.random(200))) + 2.0 ** -24   # halves of a last place, either way
+    x = np.concatenate([x, tie, -tie, tie * 2.0 ** -126, tie * 2.0 ** -127, [0.0, -0.0, 5e-324, np.inf, -np.inf, np.nan]])
+    f, hi, lo = (np.empty(x.size, dtype=np.float32) for _ in range(3))
+    ptr = [a.ctypes.data_as(ctypes.c_void_p) for a in (x, f, hi, lo)]
+    df.convert(ptr[0], x.size, *ptr[1:])
+    with np.errstate(over="ignore"):
+        want = x.astype(np.float32)
+    assert np.array_equal(f, want, equal_nan=True) and np.array_equal(np.signbit(f), np.signbit(want))
+    ok = np.abs(x) < 2.0 ** 127
+    h, l, v = hi[ok].astype(np.float64), lo[ok].astype(np.float64), x[ok]
+    assert np.all(np.abs((v - h) - l) <= np.maximum(2.0 ** -49 * np.abs(v), 2.0 ** -150))
+    assert np.all(np.abs(l) <= 0.5 * np.spacing(np.abs(hi[ok])).astype(np.float64))
