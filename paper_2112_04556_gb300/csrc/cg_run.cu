@@ -148,10 +148,10 @@ __global__ void __launch_bounds__(BLOCK, 1)
                 TI v[4];
                 T x[4];
                 load4(b + (size_t)s * 32 + mu * 8 + h * 4, v);
+                if constexpr (sizeof(T) == 4) to_f32_n(v, x);
 #pragma unroll
                 for (int a = 0; a < 4; a++) {
                     if constexpr (sizeof(T) == 4) {
-                        x[a] = to_f32(v[a]);
                         sf.add(x[a]);
                     } else {
                         x[a] = v[a];

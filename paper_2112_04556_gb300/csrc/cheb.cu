@@ -36,10 +36,10 @@ __global__ void k_copy_norms(const double* __restrict__ in, T* __restrict__ out,
         double v[4];
         T x[4];
         load4(in + f * fs + i * 4, v);
+        if constexpr (sizeof(T) == 4) to_f32_n(v, x);
 #pragma unroll
         for (int k = 0; k < 4; k++) {
             if constexpr (sizeof(T) == 4) {
-                x[k] = to_f32(v[k]);
                 sf.add(x[k]);
             } else {
                 x[k] = v[k];

@@ -52,14 +52,14 @@ struct SumSq32 {
 // float64 arithmetic (float64 runs at a small fraction of the float32 rate on this part).  df_split: hi = x
 // rounded to 24 significant bits (its 29 low significand bits dropped, rounding half away from zero, a carry
 // moving into the exponent), lo = the signed remainder (at most 2^28 units of x's last place) as a float times
-// 2^(e - 52); |lo| <= ulp(hi) / 2 and hi + lo = x to 2^-49 |x|.  |x| below 2^-126 takes the conversion instruction (hi the
-// nearest subnormal, lo 0) and |x| near or above 2^128 gives +-inf (NaN too); lo keeps what float32's subnormals hold of
-// it.
+// 2^(e - 52); |lo| <= ulp(hi) / 2 and hi + lo = x to 2^-49 |x|.  |x| below 2^-74 has lo = 0, |x| below 2^-126 gives 0 and
+// |x| near or above 2^128 gives +-inf (NaN too): enough for links, whose entries have to be accurate to 2^-48 of 1.  Fields,
+// whose scale is the caller's, go through df_split_n.
 __device__ __forceinline__ dfl df_split(double x) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
     const int e = (int)((b >> 52) & 0x7ff);
-    if (e < 1023 - 126) return df_make((float)x, 0.f);
+    if (e < 1023 - 126) return df_make(__uint_as_float(sign), __uint_as_float(sign));
     const unsigned long long m = b & 0x1fffffffull;
     const bool up = m >= (1ull << 28);
     const unsigned long long bh = (b & ~0x1fffffffull) + (up ? (1ull << 29) : 0ull);
@@ -71,24 +71,64 @@ __device__ __forceinline__ dfl df_split(double x) {
         const int r = up ? (int)m - (1 << 29) : (int)m;
         lo = __int2float_rn(r) * __uint_as_float((unsigned)(e - 948) << 23);
         if (sign) lo = -lo;
-    } else {   // lo may end among the subnormals: rounded once, by the instruction
-        lo = (float)(x - (double)hi);
     }
     return df_make(hi, lo);
 }
-// the nearest float of a value, without a float64 conversion but for |x| below 2^-126 (float32's subnormals: a field that
-// small must not turn into a field of zeros, which every solve would call solved)
-__device__ __forceinline__ float to_f32(float x) { return x; }
+// whether x is not zero and below 2^(e0 - 1023): the conversions that use no float64 operation lose (part of) it.  (Values
+// below 2^-1042 count as zero: they are zero as floats.)
+__device__ __forceinline__ bool df_small(double x, unsigned e0) {
+    return ((unsigned)((unsigned long long)__double_as_longlong(x) >> 32) & 0x7fffffffu) - 1u < (e0 << 20) - 1u;
+}
+// df_split of N values of a field; where one is small, those that are take the float64 instructions.  (One branch for all:
+// a branch each is turned into predicated float64 instructions, 4 % of a mass solve.)
+template <int N>
+__device__ __forceinline__ void df_split_n(const double (&x)[N], float (&hi)[N], float (&lo)[N]) {
+    bool small = false;
+#pragma unroll
+    for (int a = 0; a < N; a++) {
+        const dfl d = df_split(x[a]);
+        hi[a] = d.hi;
+        lo[a] = d.lo;
+        small = small || df_small(x[a], 949);
+    }
+    if (small) {
+#pragma unroll
+        for (int a = 0; a < N; a++)
+            if (df_small(x[a], 949)) {
+                hi[a] = (float)x[a];
+                lo[a] = (float)(x[a] - (double)hi[a]);
+            }
+    }
+}
+// the nearest floats of N values of a field, by integer operations, or by the instruction among float32's subnormals: a field
+// that small must not turn into zeros, which every solve would call solved
 __device__ __forceinline__ float to_f32(double x) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
     const int e = (int)((b >> 52) & 0x7ff);
-    if (e < 1023 - 126) return (float)x;
+    if (e < 1023 - 126) return __uint_as_float(sign);
     if (e > 1023 + 127) return __uint_as_float(sign | (e == 0x7ff && (b << 12) ? 0x7fc00000u : 0x7f800000u));
     // round half to even at bit 29; a carry moves into the exponent (up to infinity)
     const unsigned long long m = b & 0x7fffffffffffffffull;
     const unsigned long long r = m + 0x0fffffffull + ((m >> 29) & 1ull);
     return __uint_as_float(sign | ((unsigned)(r >> 29) - ((1023u - 127u) << 23)));
+}
+template <int N> __device__ __forceinline__ void to_f32_n(const float (&x)[N], float (&f)[N]) {
+#pragma unroll
+    for (int a = 0; a < N; a++) f[a] = x[a];
+}
+template <int N> __device__ __forceinline__ void to_f32_n(const double (&x)[N], float (&f)[N]) {
+    bool small = false;
+#pragma unroll
+    for (int a = 0; a < N; a++) {
+        f[a] = to_f32(x[a]);
+        small = small || df_small(x[a], 897);
+    }
+    if (small) {
+#pragma unroll
+        for (int a = 0; a < N; a++)
+            if (df_small(x[a], 897)) f[a] = (float)x[a];
+    }
 }
 // a float as a double, from its bit fields (normal numbers, zero, inf and NaN; subnormals give 0)
 __device__ __forceinline__ double f_to_d_bits(float f) {

@@ -48,10 +48,10 @@ __device__ __forceinline__ double start_pass(const TI* __restrict__ b, T* __rest
         TI v[4];
         load4(b + i * 4, v);
         T x[4];
+        if constexpr (sizeof(T) == 4) to_f32_n(v, x);
 #pragma unroll
         for (int k = 0; k < 4; k++) {
             if constexpr (sizeof(T) == 4) {
-                x[k] = to_f32(v[k]);
                 sf.add(x[k]);
             } else {
                 x[k] = v[k];

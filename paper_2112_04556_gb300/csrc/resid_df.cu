@@ -80,12 +80,7 @@ __global__ void k_split_pairs(const double* __restrict__ x, float* __restrict__ 
         double v[8];
         load8(x + i * 8, v);
         float h[8], l[8];
-#pragma unroll
-        for (int a = 0; a < 8; a++) {
-            const dfl p = df_split(v[a]);   // integer operations: the float64 pipe held this pass at a third of its bandwidth
-            h[a] = p.hi;
-            l[a] = p.lo;
-        }
+        df_split_n(v, h, l);   // integer operations: the float64 pipe held this pass at a third of its bandwidth
         store8(out + i * 16, h);
         store8(out + i * 16 + 8, l);
     }
@@ -129,11 +124,9 @@ __global__ void __launch_bounds__(kBlock) k_resid_df(Geom g, const float* __rest
             float xh[8], xl[8];
             ld_pair(xf + ((size_t)site * 4 + mu) * 16, xh, xl);
             const dfl d = df_split(-(sig[f] + 0.5));
+            df_split_n(bb, s, c);   // integer operations, as k_split_pairs
 #pragma unroll
             for (int a = 0; a < 8; a++) {
-                const dfl v = df_split(bb[a]);   // integer operations, as k_split_pairs
-                s[a] = v.hi;
-                c[a] = v.lo;
                 dot2_acc(d.hi, xh[a], s[a], c[a]);
                 c[a] = __fmaf_rn(d.hi, xl[a], __fmaf_rn(d.lo, xh[a], c[a]));
             }

@@ -19,11 +19,14 @@ extern "C" double sum_squares(const float* x, int n) {
     return a.value();
 }
 extern "C" void convert(const double* x, int n, float* f, float* hi, float* lo) {
-    for (int i = 0; i < n; i++) {
-        f[i] = to_f32(x[i]);
-        const dfl d = df_split(x[i]);
-        hi[i] = d.hi;
-        lo[i] = d.lo;
+    for (int i = 0; i < n; i++) {   // each value beside its neighbours, as a thread converts them
+        const double v[3] = {x[i], x[(i + 1) % n], x[(i + 41) % n]};
+        float a[3], h[3], l[3];
+        to_f32_n(v, a);
+        df_split_n(v, h, l);
+        f[i] = a[0];
+        hi[i] = h[0];
+        lo[i] = l[0];
     }
 }
 """
