@@ -12,6 +12,7 @@
 //
 // Work: units of 32 consecutive sites and one component, a contiguous range of units per block, one warp per unit.
 #include <algorithm>
+#include <type_traits>
 
 #include "df.cuh"
 #include "krylov.cuh"
@@ -121,6 +122,8 @@ __global__ void __launch_bounds__(BLOCK, 1)
     k_cg_run(Geom g, typename LinksOf<T>::type U, const TI* __restrict__ b, T* R, size_t fs, T diag, int* flags, double* vals,
              int maxit, double tol2, long long* iters, int units_per_block, double* part, unsigned* bar, int limit,
              const int* status) {
+    // float32 blocks of 256 and 768 threads have a unit per warp and nothing to add up
+    using Sum = std::conditional_t<sizeof(T) == 4 && BLOCK == 512, CompSum, PlainSum<T>>;
     extern __shared__ __align__(16) unsigned char cgs[];
     T* const qs = reinterpret_cast<T*>(cgs);   // [item][chunk][thread][4]
     __shared__ double shw[BLOCK / 32], sh[3];
@@ -175,7 +178,7 @@ __global__ void __launch_bounds__(BLOCK, 1)
         const SrcShared<T> src{R + (size_t)k * fs, g.V};
         T* const rn = R + (size_t)(k + 1) * fs;
         const T bt = (T)bk;
-        T dot = T(0);
+        Sum dot;
         T* q = qs + threadIdx.x * 4;
         for (int u = u0; u < u1; u += wpb, q += 8 * blockDim.x) {
             const int s = u / 4 * 32 + lane, mu = u & 3;
@@ -188,20 +191,22 @@ __global__ void __launch_bounds__(BLOCK, 1)
                 q_load(q, o);
                 q_load(q + 4 * blockDim.x, o + 4);
             }
+            T d = T(0);
 #pragma unroll
             for (int a = 0; a < 8; a++) {
                 y[a] = fma(T(-0.0625), h[a], diag * x[a]);
                 if (k > 0) y[a] = fma(bt, o[a], y[a]);
-                dot = fma(x[a], y[a], dot);
+                d = fma(x[a], y[a], d);
             }
+            dot.add(d);
             store4(q, y);
             store4(q + 4 * blockDim.x, y + 4);
         }
         double gm;
-        if (!gsum(block_total(dot, shw), gm, sh + 1)) { done = 4; break; }
+        if (!gsum(block_total(dot.value(), shw), gm, sh + 1)) { done = 4; break; }
         const double al = rr / gm;
         const T at = (T)al;
-        dot = T(0);
+        dot = Sum();
         q = qs + threadIdx.x * 4;
         for (int u = u0; u < u1; u += wpb, q += 8 * blockDim.x) {
             const int s = u / 4 * 32 + lane, mu = u & 3;
@@ -210,16 +215,18 @@ __global__ void __launch_bounds__(BLOCK, 1)
             src(s, mu, x);
             q_load(q, o);
             q_load(q + 4 * blockDim.x, o + 4);
+            T d = T(0);
 #pragma unroll
             for (int a = 0; a < 8; a++) {
                 x[a] = fma(-at, o[a], x[a]);
-                dot = fma(x[a], x[a], dot);
+                d = fma(x[a], x[a], d);
             }
+            dot.add(d);
             store4(plane_at(rn, g.V, s, 2 * mu), x);
             store4(plane_at(rn, g.V, s, 2 * mu + 1), x + 4);
         }
         double rn2;
-        if (!gsum(block_total(dot, shw), rn2, sh + 2)) { done = 4; break; }
+        if (!gsum(block_total(dot.value(), shw), rn2, sh + 2)) { done = 4; break; }
         bk = rn2 / rr;
         if (writer) {
             gamma[k] = gm;

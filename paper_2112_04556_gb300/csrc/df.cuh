@@ -48,6 +48,24 @@ struct SumSq32 {
     __device__ __forceinline__ double value() const { return ((double)e + (double)c) + (double)s + d; }
 };
 
+// running sum of a few dozen float32 values without the growth of their rounding errors: TwoSum's go to c.  (A lane of the
+// cooperative Krylov run adds up to 14 units of 8 products; a lane of the two-kernel form has at most four.)
+struct CompSum {
+    float s = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float x) {
+        const dfl t = two_sum(s, x);
+        s = t.hi;
+        c = __fadd_rn(c, t.lo);
+    }
+    __device__ __forceinline__ float value() const { return __fadd_rn(s, c); }
+};
+// the plain sum
+template <typename T> struct PlainSum {
+    T s = T(0);
+    __device__ __forceinline__ void add(T x) { s += x; }
+    __device__ __forceinline__ T value() const { return s; }
+};
+
 // Conversions between float64 and float pairs from the IEEE-754 bit fields, with integer operations and no
 // float64 arithmetic (float64 runs at a small fraction of the float32 rate on this part).  df_split: hi = x
 // rounded to 24 significant bits (its 29 low significand bits dropped, rounding half away from zero, a carry

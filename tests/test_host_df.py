@@ -18,6 +18,11 @@ extern "C" double sum_squares(const float* x, int n) {
     for (int i = 0; i < n; i++) a.add(x[i]);
     return a.value();
 }
+extern "C" float sum_floats(const float* x, int n) {
+    CompSum a;
+    for (int i = 0; i < n; i++) a.add(x[i]);
+    return a.value();
+}
 extern "C" void convert(const double* x, int n, float* f, float* hi, float* lo) {
     for (int i = 0; i < n; i++) {   // each value beside its neighbours, as a thread converts them
         const double v[3] = {x[i], x[(i + 1) % n], x[(i + 41) % n]};
@@ -42,6 +47,7 @@ def df(tmp_path_factory):
                    check=True)
     L = ctypes.CDLL(str(d / "df.so"))
     L.sum_squares.restype = ctypes.c_double
+    L.sum_floats.restype = ctypes.c_float
     return L
 
 
@@ -82,3 +88,15 @@ def test_conversions_over_all_exponents(df):
     h, l, v = hi[ok].astype(np.float64), lo[ok].astype(np.float64), x[ok]
     assert np.all(np.abs((v - h) - l) <= np.maximum(2.0 ** -49 * np.abs(v), 2.0 ** -150))
     assert np.all(np.abs(l) <= 0.5 * np.spacing(np.abs(hi[ok])).astype(np.float64))
+
+
+@pytest.mark.parametrize("n", [1, 2, 14, 100])
+def test_sums_of_a_lane_do_not_lose_with_their_length(df, n):
+    """A lane's sum over its units, values of either sign: rounded once (2^-24 of the result) and n^2 2^-48 of the sum of
+    the magnitudes (n errors of 2^-24 of partial sums, added up in float32), at any of the lengths a run has."""
+    for seed in range(50):
+        rng = np.random.default_rng(seed)
+        x = (rng.standard_normal(n) * 2.0 ** rng.uniform(-6, 6, n)).astype(np.float32)
+        got = Fraction(float(df.sum_floats(x.ctypes.data_as(ctypes.c_void_p), n)))
+        want, size = sum(Fraction(float(v)) for v in x), sum(Fraction(abs(float(v))) for v in x)
+        assert abs(got - want) <= abs(want) / 2 ** 24 + n * n * size / 2 ** 48
