@@ -21,7 +21,10 @@
  *  Memory   All field and link pointers are DEVICE pointers on the context's device, owned by the
  *           caller; the library never frees them.  Small vectors marked (host) are host memory.
  *           The context owns its workspace: it is allocated by rmhmc_create or on the first call that
- *           needs it, and reused afterwards; nothing is allocated inside an iteration loop.
+ *           needs it, and reused afterwards; nothing is allocated inside an iteration loop.  What a call can do
+ *           without (the float64 table of adjoint matrices, 2 KB a site; the loops of the gauge force, up to 4.5 KB a
+ *           site) is given back when another allocation of the context fails; rmhmc_tuning says so, and setting
+ *           RMHMC_SHAPE_TABLE or RMHMC_SHAPE_LOOPS to 1 takes it up again.
  *  Streams  Every call takes a cudaStream_t (0 = legacy default stream) and enqueues its work there.
  *           Calls that return host scalars synchronise that stream before returning.
  *  Threads  A context is not thread-safe: use one context per host thread / stream.

@@ -409,6 +409,8 @@ int upload(rmhmc_ctx* ctx, void* dst, const void* src, size_t bytes, cudaStream_
 int set_err(rmhmc_ctx* ctx, int code, const char* fmt, ...);
 int cuda_check(rmhmc_ctx* ctx, cudaError_t e, const char* what);
 void* workspace(rmhmc_ctx* ctx, const char* name, size_t bytes, int* status);
+// a form that the context does without for want of memory (&ctx->adj64_off or &ctx->loops_off), noted in rmhmc_tuning
+void without(rmhmc_ctx* ctx, bool* off);
 int import_links(rmhmc_ctx* ctx, const double* U, cudaStream_t st);
 int ensure_links(rmhmc_ctx* ctx, const double* U, cudaStream_t st);
 inline size_t field_elems(const rmhmc_ctx* ctx) { return (size_t)ctx->g.V * 32; }

@@ -30,6 +30,31 @@ int cuda_check(rmhmc_ctx* ctx, cudaError_t e, const char* what) {
     return set_err(ctx, RMHMC_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
+// Buffers that a call can do without: the float64 adjoint table and the loops of the gauge force.  They give way to the
+// others: where an allocation fails they are freed, their forms are off for the context (set_stencil_shape puts them back)
+// and the allocation is tried again.  No call holds a pointer to one of them over a workspace() of something else.
+static bool optional_buffer(const std::string& name) { return name == "ad_table64" || name.compare(0, 3, "gl_") == 0; }
+
+static bool drop_optional(rmhmc_ctx* ctx) {
+    bool any = false;
+    cudaDeviceSynchronize();
+    for (auto& kv : ctx->bufs)
+        if (kv.second.p && optional_buffer(kv.first)) {
+            without(ctx, kv.first == "ad_table64" ? &ctx->adj64_off : &ctx->loops_off);
+            cudaFree(kv.second.p);
+            kv.second = DevBuf();
+            any = true;
+        }
+    if (any) ctx->ws_gen++;   // a captured trajectory may hold them
+    return any;
+}
+
+void without(rmhmc_ctx* ctx, bool* off) {
+    *off = true;
+    ctx->tune_report += ctx->tune_report.empty() ? "" : "; ";
+    ctx->tune_report += off == &ctx->loops_off ? "gauge loops off: no memory" : "float64 table off: no memory";
+}
+
 void* workspace(rmhmc_ctx* ctx, const char* name, size_t bytes, int* status) {
     DevBuf& b = ctx->bufs[name];
     if (b.bytes >= bytes && b.p) return b.p;
@@ -41,6 +66,10 @@ void* workspace(rmhmc_ctx* ctx, const char* name, size_t bytes, int* status) {
     }
     void* p = nullptr;
     cudaError_t e = cudaMalloc(&p, bytes);
+    if (e == cudaErrorMemoryAllocation && !optional_buffer(name) && drop_optional(ctx)) {
+        cudaGetLastError();
+        e = cudaMalloc(&p, bytes);
+    }
     if (e != cudaSuccess) {
         *status = cuda_check(ctx, e, name);
         return nullptr;
@@ -261,6 +290,7 @@ extern "C" int rmhmc_set_stencil_shape(rmhmc_ctx* ctx, int kernel, int prec, int
         if (prec != RMHMC_FP64 || linkfmt != 18 || (nmu != 0 && nmu != 1) || block != 128)
             return set_err(ctx, RMHMC_EINVAL, "loops and table: RMHMC_FP64, 18, nmu 0 or 1, block 128");
         (kernel == RMHMC_SHAPE_LOOPS ? ctx->use_loops : ctx->use_table) = nmu == 1;
+        (kernel == RMHMC_SHAPE_LOOPS ? ctx->loops_off : ctx->adj64_off) = false;
         return RMHMC_OK;
     }
     if (kernel == RMHMC_SHAPE_ADJOINT) {

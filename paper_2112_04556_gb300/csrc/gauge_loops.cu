@@ -355,7 +355,7 @@ int gauge_loops_launch(rmhmc_ctx* ctx, double beta, double c1, int prec, double*
     if (s == RMHMC_ENOMEM) {
         // no room for the loops: the staples serve as before
         ctx->err.clear();
-        ctx->loops_off = true;
+        without(ctx, &ctx->loops_off);
         return RMHMC_OK;
     }
     RM_TRY(s);
@@ -370,7 +370,7 @@ int gauge_loops_prepare(rmhmc_ctx* ctx, double c1, int prec) {
     const int s = prec == RMHMC_FP64 ? loop_bufs<double>(ctx, c1 != 0.0, true, d) : loop_bufs<float>(ctx, c1 != 0.0, true, f);
     if (s == RMHMC_ENOMEM) {
         ctx->err.clear();
-        ctx->loops_off = true;
+        without(ctx, &ctx->loops_off);
         return RMHMC_OK;
     }
     return s;

@@ -548,6 +548,7 @@ int krylov_run(rmhmc_ctx* ctx, const TI* b, double sigma0, double tol, int maxit
     bool done = false;
     typename LinksOf<T>::type U;
     bool run = cg_run_fits<T>(ctx);
+    if (run) RM_TRY(cg_run_prepare(ctx));   // before the table: an allocation may take it back
     if constexpr (sizeof(T) == 8) {
         U = links64(ctx);
         if (!ctx->pinned.count(10818)) RM_TRY(links64_adjoint(ctx, &U, st));

@@ -60,7 +60,7 @@ int links64_adjoint(rmhmc_ctx* ctx, Links64* U, cudaStream_t st) {
     if (status == RMHMC_ENOMEM) {
         // no room: the 3x3 form serves as before
         ctx->err.clear();
-        ctx->adj64_off = true;
+        without(ctx, &ctx->adj64_off);
         return RMHMC_OK;
     }
     if (!t) return status;

@@ -207,3 +207,49 @@ def test_captured_calls_keep_nothing_derived_from_the_links(rm):
         assert calls() == direct
         assert trajectory_md(rm, ctx) == rm.OK
         assert not any("k_plaquettes" in k for k in launched(rm))
+
+
+def test_optional_buffers_give_way(rm):
+    """The float64 table and the gauge force's loops are given back when another buffer of the context does not fit beside
+    them: the call that needs it runs, as it does in a context without them, and the forms that do without them serve
+    until the caller asks for the others again."""
+    def stencil(ctx):
+        ctx.check(rm.lib().lap_apply(ctx.h, None, FIELD, OUT, 1, rm.FP64, 18, 0, None))
+        ctx.check(rm.lib().gauge_force(ctx.h, None, 6.0, 0.0, rm.FP64, OUT2, None, None, None))
+        names = " ".join(launched(rm))
+        return "k_lapIdLi64E" in names, "k_loop_force" in names
+    for prec in (rm.FP64, rm.MIXED):
+        with context(rm, (4, 4, 4, 4)) as ctx:   # what the evaluation takes without the optional buffers
+            for kernel in (rm.SHAPE_TABLE, rm.SHAPE_LOOPS):
+                rm.set_stencil_shape(ctx, kernel, rm.FP64, 18, 0, 128)
+            held = rm.lib().fake_held()
+            assert kinetic(rm, ctx, prec) == rm.OK
+            need = rm.lib().fake_held() - held
+        with context(rm, (4, 4, 4, 4)) as ctx:
+            assert stencil(ctx) == (True, True)
+            assert "off" not in rm.tuning(ctx)
+            rm.lib().fake_room(need - 1024)
+            assert kinetic(rm, ctx, prec) == rm.OK
+            assert "float64 table off: no memory" in rm.tuning(ctx) and "gauge loops off" in rm.tuning(ctx)
+            assert stencil(ctx) == (False, False)
+            rm.lib().fake_room(1 << 40)
+            assert stencil(ctx) == (False, False)
+            for kernel in (rm.SHAPE_TABLE, rm.SHAPE_LOOPS):
+                rm.set_stencil_shape(ctx, kernel, rm.FP64, 18, 1, 128)
+            assert stencil(ctx) == (True, True)
+        rm.lib().fake_room(1 << 50)
+
+
+def test_a_trajectory_lets_go_of_its_loops(rm):
+    """A captured trajectory whose loops were given back is captured again, on staples."""
+    with context(rm, (4, 4, 4, 4)) as ctx:
+        assert trajectory_md(rm, ctx) == rm.OK
+        assert any("k_loop_force" in k for k in launched(rm))
+        rm.lib().fake_room(4096)
+        assert kinetic(rm, ctx, rm.FP64) == rm.ENOMEM     # far too large, with or without them
+        rm.lib().fake_room(1 << 40)
+        launched(rm)
+        assert trajectory_md(rm, ctx) == rm.OK
+        names = launched(rm)
+        assert "instantiate" in names and not any("k_loop_force" in k for k in names)
+        assert any("k_gauge_force" in k for k in names)
