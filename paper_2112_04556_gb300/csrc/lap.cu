@@ -95,7 +95,7 @@ static int launch_lap_t(rmhmc_ctx* ctx, const T* X, T* Y, int nfield, double a, 
     if constexpr (sizeof(T) == 8) {
         U = links64(ctx);
         // float64 with 18-real links, no shape pinned: the adjoint form, one component per lane (the arithmetic bounds every
-        // shape alike).  32^4: 3.66 ms and 2.46 ms for the table of new links, against 6.38 ms in the 3x3 form
+        // shape alike).  32^4: 3.65 ms and 2.26 ms for the table of new links, against 6.38 ms in the 3x3 form
         if (LF == 18 && !ctx->pinned.count(818)) {
             RM_TRY(links64_adjoint(ctx, &U, st));
             if (U.ad) {

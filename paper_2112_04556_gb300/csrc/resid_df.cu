@@ -39,17 +39,24 @@ __global__ void __launch_bounds__(kBlock) k_adjoint_table(Links64 U, int V, floa
     });
 }
 
-// the float64 table of Links64::ad: thread per (site, direction), consecutive sites adjacent in every plane
+// the float64 table of Links64::ad, consecutive sites adjacent in every plane: thread per site, direction (blockIdx.y) and
+// two of the eight columns (blockIdx.z).  A warp has half a float64 lane, so that a thread with all columns took 14 us on the
+// smallest lattice, where lap_apply with new links was then slower than by 3x3 products (39 us at 4^4): the table's part
+// there 14.5 -> 7 us, at 10^4 37 -> 29 us, at 32^4 2.46 -> 2.26 ms
 __global__ void __launch_bounds__(kBlock) k_adjoint_table64(Links64 U, double2* __restrict__ out) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     const int nu = blockIdx.y;
     if (s >= U.V) return;
     const mat3<double> u = LinkLoad<double, 18>::load(U, s, nu);
     double2* const o = out + (size_t)nu * 32 * U.V + s;
-    adjoint_columns(u, [&](int b, const double (&col)[8]) {
+    auto put = [&](int b, const double (&col)[8]) {
 #pragma unroll
         for (int h = 0; h < 4; h++) o[(size_t)(4 * b + h) * U.V] = make_double2(col[2 * h], col[2 * h + 1]);
-    });
+    };
+    if (blockIdx.z == 0) adjoint_pair_columns<double, 0>(u, put);
+    else if (blockIdx.z == 1) adjoint_pair_columns<double, 1>(u, put);
+    else if (blockIdx.z == 2) adjoint_pair_columns<double, 2>(u, put);
+    else adjoint_diagonal_columns(u, put);
 }
 
 int links64_adjoint(rmhmc_ctx* ctx, Links64* U, cudaStream_t st) {
@@ -65,7 +72,7 @@ int links64_adjoint(rmhmc_ctx* ctx, Links64* U, cudaStream_t st) {
     }
     if (!t) return status;
     if (ctx->adj64_gen != ctx->link_gen || ws != ctx->ws_gen) {
-        k_adjoint_table64<<<dim3(site_blocks(ctx), 4), kBlock, 0, st>>>(links64(ctx), t);
+        k_adjoint_table64<<<dim3(site_blocks(ctx), 4, 4), kBlock, 0, st>>>(links64(ctx), t);
         ++ctx->launches;
         RM_LAUNCH_CHECK(ctx);
         ctx->adj64_gen = ctx->link_gen;
