@@ -298,8 +298,8 @@ int cg_run_prepare(rmhmc_ctx* ctx, unsigned** bar) {
 }
 
 template <typename T, typename TI>
-int cg_run_launch(rmhmc_ctx* ctx, const typename LinksOf<T>::type& links, const TI* b, T* R, double diag, int* flags, double* vals, int maxit, double tol2,
-                  long long* iters, cudaStream_t st, const int* status) {
+int cg_run_launch(rmhmc_ctx* ctx, const typename LinksOf<T>::type& links, const TI* b, T* R, double diag, int* flags,
+                  double* vals, int maxit, double tol2, long long* iters, cudaStream_t st, const int* status) {
     const CgRunShape s = cg_run_shape<T>(ctx);
     unsigned* bar = nullptr;
     RM_TRY(cg_run_prepare(ctx, &bar));
@@ -331,8 +331,11 @@ int cg_run_launch(rmhmc_ctx* ctx, const typename LinksOf<T>::type& links, const 
 
 template bool cg_run_fits<float>(const rmhmc_ctx*, bool);
 template bool cg_run_fits<double>(const rmhmc_ctx*, bool);
-template int cg_run_launch<float, float>(rmhmc_ctx*, const Links32&, const float*, float*, double, int*, double*, int, double, long long*, cudaStream_t, const int*);
-template int cg_run_launch<float, double>(rmhmc_ctx*, const Links32&, const double*, float*, double, int*, double*, int, double, long long*, cudaStream_t, const int*);
-template int cg_run_launch<double, double>(rmhmc_ctx*, const Links64&, const double*, double*, double, int*, double*, int, double, long long*, cudaStream_t, const int*);
+template int cg_run_launch<float, float>(rmhmc_ctx*, const Links32&, const float*, float*, double, int*, double*, int, double,
+                                         long long*, cudaStream_t, const int*);
+template int cg_run_launch<float, double>(rmhmc_ctx*, const Links32&, const double*, float*, double, int*, double*, int, double,
+                                          long long*, cudaStream_t, const int*);
+template int cg_run_launch<double, double>(rmhmc_ctx*, const Links64&, const double*, double*, double, int*, double*, int,
+                                           double, long long*, cudaStream_t, const int*);
 
 }  // namespace rm

@@ -80,9 +80,9 @@ __global__ void __launch_bounds__(kBlock) k_cg_start(const TI* __restrict__ b, T
 // CG without the search direction: q_k = (A + sigma0) p_k is carried as q_k = (A + sigma0) r_k + beta_{k-1} q_{k-1}
 // (p_k = r_k + beta_{k-1} p_{k-1}), so the stencil reads only r_k; gamma_k = <p_k, A p_k> = <r_k, q_k> by
 // A-conjugacy of the directions, alpha_k = rho_k / gamma_k.  q is updated in place at the lane's own site.
-// At 32^4: 0.212 ms (two components per lane, 256 threads) against 0.225 ms with the vectors as site rows (one component,
-// four lanes a site); at 16^4 22.3 against 23.4 us.  What is left is DRAM traffic (1.25 times the 672 bytes a site) and the
-// latency of the neighbour loads.
+// At 32^4: 0.214 ms (two components per lane, 256 threads) against 0.225 ms with the vectors as site rows (one component,
+// four lanes a site); at 16^4 22.3 against 23.4 us.  What is left is DRAM traffic (1.29 times the 672 bytes a site in this
+// shape, 1.15 with four components, which is 0.229 ms) and the latency of the neighbour loads.
 // One lane per site and group of NC components: a warp holds 32 consecutive sites of one group, and the blocks run
 // through the groups of a site range together, so that its links come from DRAM once.
 template <typename T, int LF, int NMU>
@@ -154,8 +154,9 @@ static void launch_cg_A(rmhmc_ctx* ctx, const StencilShape& shp, typename LinksO
                         T diag, int* flags, double* vals, int maxit, cudaStream_t st) {
     // whole warps of 32 sites per group
     const size_t lanes = (size_t)((ctx->g.V + 31) / 32 * 32) * lanes_per_site(NMU);
-    k_cg_A<T, LF, NMU><<<std::min(capped_grid(ctx, lanes, shp.block), ctx->max_blocks * 2), shp.block, 0, st>>>(ctx->g, U, R, fs, q, diag, flags, vals, maxit,
-                                                                      red_slot_partials(ctx, 0), red_slot_counter(ctx, 0));
+    const int grid = std::min(capped_grid(ctx, lanes, shp.block), ctx->max_blocks * 2);
+    k_cg_A<T, LF, NMU><<<grid, shp.block, 0, st>>>(ctx->g, U, R, fs, q, diag, flags, vals, maxit, red_slot_partials(ctx, 0),
+                                                   red_slot_counter(ctx, 0));
     ++ctx->launches;
 }
 
@@ -566,8 +567,9 @@ int krylov_run(rmhmc_ctx* ctx, const TI* b, double sigma0, double tol, int maxit
         bool shaped = true;
         if constexpr (sizeof(T) == 8) shaped = !U.ad;
         if (shaped) RM_TRY(cg_shape<T>(ctx, st, shp));
-        k_cg_start<T, TI><<<capped_grid(ctx, fs / 4, kBlock), kBlock, 0, st>>>(b, R, ctx->g.V, w.flags, w.vals, red_slot_partials(ctx, kSlotRho),
-                                             red_slot_counter(ctx, kSlotRho)); ++ctx->launches;
+        k_cg_start<T, TI><<<capped_grid(ctx, fs / 4, kBlock), kBlock, 0, st>>>(
+            b, R, ctx->g.V, w.flags, w.vals, red_slot_partials(ctx, kSlotRho), red_slot_counter(ctx, kSlotRho));
+        ++ctx->launches;
         RM_LAUNCH_CHECK(ctx);
         const T diag = (T)(0.5 + sigma0);
         // iteration count of the previous run of the same operator and tolerance: the first chunk of launches

@@ -62,8 +62,8 @@ int cg_run_prepare(rmhmc_ctx* ctx, unsigned** bar = nullptr);
 int cg_run_reset(rmhmc_ctx* ctx, cudaStream_t st);
 template <typename T> struct LinksOf;
 template <typename T, typename TI>
-int cg_run_launch(rmhmc_ctx* ctx, const typename LinksOf<T>::type& U, const TI* b, T* R, double diag, int* flags, double* vals, int maxit, double tol2,
-                  long long* iters, cudaStream_t st, const int* status = nullptr);
+int cg_run_launch(rmhmc_ctx* ctx, const typename LinksOf<T>::type& U, const TI* b, T* R, double diag, int* flags,
+                  double* vals, int maxit, double tol2, long long* iters, cudaStream_t st, const int* status = nullptr);
 // value of a captured trajectory's status word after a run whose barrier gave up
 constexpr int kStatusGaveUp = 5;
 // basis pointer of the last run

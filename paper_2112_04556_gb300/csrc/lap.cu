@@ -69,8 +69,9 @@ __global__ void __launch_bounds__(kBlockMax, (stencil_min_blocks<T, NMU>())) k_l
 }
 
 template <typename T, int LF, int NMU>
-static void launch_lap_shape(rmhmc_ctx* ctx, const StencilShape& shp, const typename LinksOf<T>::type& U, const T* X, T* Y, int nfield, double a, double b,
-                             const T* W, double c, int slot, cudaStream_t st, double* dots = nullptr) {
+static void launch_lap_shape(rmhmc_ctx* ctx, const StencilShape& shp, const typename LinksOf<T>::type& U, const T* X, T* Y,
+                             int nfield, double a, double b, const T* W, double c, int slot, cudaStream_t st,
+                             double* dots = nullptr) {
     const dim3 grid(stencil_blocks(ctx, shp), nfield);
     const size_t fs = field_elems(ctx);
     const size_t ss = (size_t)ctx->max_blocks * 2;

@@ -40,8 +40,9 @@ inline size_t ad_smem_bytes(int nd) {
     return kAdSmemFloats * sizeof(float) + kAdSites * 8 * sizeof(int) + (size_t)(kAdThreads / 32) * nd * 2 * sizeof(double);
 }
 
-// CH: fields per pass of phase 2; MINB: resident blocks the register budget is compiled for.  (Nine or five fields a pass without the second operand
-// buffer read the adjoint records less often but are slower: 18 fields at 32^4 3.3-3.6 and 3.0 ms against 2.65 ms.)
+// CH: fields per pass of phase 2; MINB: resident blocks the register budget is compiled for.  (Nine or five fields a pass
+// without the second operand buffer read the adjoint records less often but are slower: 18 fields at 32^4 3.3-3.6 and
+// 3.0 ms against 2.65 ms.)
 template <int LF, bool HAS_W, bool DOTS, int CH, int MINB>
 __global__ void __launch_bounds__(kAdThreads, MINB) k_lap_ad(Geom g, Links32 U, const float* __restrict__ X,
                                                         float* __restrict__ Y, const float* __restrict__ W, int nf,

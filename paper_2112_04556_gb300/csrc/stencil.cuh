@@ -3,10 +3,11 @@
 // (the factor 2 comes from the doubled Hermitian expansion of the coefficients).  Every term is traceless, so
 // the sum is accumulated without its (2,2) entry (acc_*_tl) and read with herm2_to_coef_tl.
 //
-// Thread layout of the stencil kernels: 4 / NMU consecutive lanes own one site, each lane NMU of its four
+// Thread layout of the kernels on [V][4][8] fields: 4 / NMU consecutive lanes own one site, each lane NMU of its four
 // field components (NMU = 1: a warp covers 8 consecutive sites, its loads of X_mu at a neighbour are one
-// contiguous 1 KB segment of the [V][4][8] field and its link loads hit 8 consecutive entries of the
-// structure-of-arrays link copy).  NMU and the block size are chosen per context by the autotuner
+// contiguous 1 KB segment of the field and its link loads hit 8 consecutive entries of the structure-of-arrays
+// link copy).  The CG stencil (krylov.cu, cg_run.cu) reads chunk-planar vectors: a warp covers 32 consecutive sites of
+// one group of NMU components.  NMU and the block size are chosen per context by the autotuner
 // (tune.cuh): fewer lanes per site load each link fewer times but hold more registers.
 #pragma once
 #include "common.cuh"

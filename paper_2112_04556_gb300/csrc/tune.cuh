@@ -1,6 +1,6 @@
 // Autotuner of the stencil launch shape: components per lane (NMU = 1, 2, 4, i.e. 4, 2 or 1 lanes per
-// site, or the prefetching one-component variant) and threads per block (64, 128, 256).  On first use of a (precision, link format) in a context,
-// every shape is timed with CUDA events on the context's own lattice (a plain A X application on scratch
+// site, or the prefetching one-component variant) and threads per block (64, 128, 256).  On first use of a (precision,
+// link format) in a context, every shape is timed with CUDA events on the context's own lattice (a plain A X application on scratch
 // fields, three repetitions after a warm-up) and the fastest is kept for every stencil kernel of that
 // precision and link format.
 #pragma once
