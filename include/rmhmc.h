@@ -341,7 +341,8 @@ int rmhmc_action_noalloc(const int dims[4], const double* U, double beta, double
  * c0 = 1 - 8 c1 (c1 = 0: Wilson plaquette action), R the 1x2 rectangles.  action and plaq (host,
  * nullable) receive S and the average plaquette ReTr P/3, both summed in float64.
  * prec: RMHMC_FP64, or RMHMC_FP32 (force in float32 arithmetic, float64 action).  U may be any matrices: unitary
- * ones (to 2^-43, looked at once per import) share their loops, others take the staples of each link. */
+ * ones (to 2^-43, for the float32 force to 2^-20; looked at once per import) share their loops, others take the
+ * staples of each link. */
 int gauge_force(rmhmc_ctx* ctx, const double* U, double beta, double c1, int prec, double* F,
                 double* action, double* plaq, cudaStream_t stream);
 

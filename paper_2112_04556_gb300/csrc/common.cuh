@@ -331,8 +331,9 @@ struct rmhmc_ctx {
     bool links_valid = false;
     unsigned long long link_gen = 1;   // bumped whenever the internal link copies change
     unsigned long long import_gen = 0; // bumped by every import of the caller's links
-    unsigned long long su3_gen = 0;    // import_gen whose links were last looked at, and whether they are unitary (links_su3)
-    bool su3 = false;
+    // import_gen whose links were last looked at, and whether they are unitary, for float64 and float32 (links_su3)
+    unsigned long long su3_gen[2] = {0, 0};
+    bool su3[2] = {false, false};
     bool own_capture = false;          // the library's streams are capturing a trajectory
     bool links_in_graph = false;       // a graph of the caller's imports links: the host no longer sees when they change
     unsigned long long adj_gen = 0;    // link_gen the float32-pair adjoint table was built for

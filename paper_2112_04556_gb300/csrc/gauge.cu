@@ -207,33 +207,37 @@ int gauge_force_launch(rmhmc_ctx* ctx, double beta, double c1, int prec, double*
 }
 
 int gauge_force_action(rmhmc_ctx* ctx, double beta, double c1, int prec, double* F, double* S, double* plaq,
-                       cudaStream_t st, bool su3) {
-    bool force = !F, act = false;
-    const bool check = (su3 || F || c1 != 0.0) && loops_usable(ctx) && su3_unknown(ctx) && links_tracked(ctx, st);
-    if (check) RM_TRY(su3_check_launch(ctx, st));
+                       cudaStream_t st, int ask) {
+    // what has to be known of the links: launched before the loops, read with their sums
+    bool look[2] = {false, false};
+    if (loops_usable(ctx) && links_tracked(ctx, st)) {
+        look[RMHMC_FP64] = (c1 != 0.0 || (F && prec == RMHMC_FP64) || ask == RMHMC_FP64) && su3_state(ctx, RMHMC_FP64) < 0;
+        look[RMHMC_FP32] = ((F && prec == RMHMC_FP32) || ask == RMHMC_FP32) && !look[RMHMC_FP64] &&
+                           su3_state(ctx, RMHMC_FP32) < 0;
+    }
+    for (int q : {RMHMC_FP64, RMHMC_FP32})
+        if (look[q]) RM_TRY(su3_check_launch(ctx, q, st));
+    bool force = false, act = false;   // what the loops gave
     if (F && prec != RMHMC_FP64) {
         RM_TRY(gauge_loops_launch(ctx, beta, c1, prec, F, false, true, &force, st));
         RM_TRY(gauge_loops_launch(ctx, beta, c1, RMHMC_FP64, nullptr, true, true, &act, st));
     } else {
         RM_TRY(gauge_loops_launch(ctx, beta, c1, RMHMC_FP64, F, true, true, &act, st));
-        force = force || act;
+        force = act;
     }
-    double buf[8 + 3];
-    if (check || act) {
-        // the count of links that are not unitary, in the slot before the loops' sums
+    double buf[8 + 3];   // the slots kSlotSu3 and kSlotLoops
+    if (look[0] || look[1] || act) {
         RM_TRY(fetch(ctx, red_slot_out(ctx, kSlotSu3), buf, 8 + 3, st));
-        if (check) {
-            su3_known(ctx, buf[0] == 0.0);
-            if (!ctx->su3) {
-                force = !F;
-                act = act && c1 == 0.0;
-            }
-        }
+        for (int q : {RMHMC_FP64, RMHMC_FP32})
+            if (look[q]) su3_known(ctx, q, buf[q] == 0.0);
+        // (known by now, but for float32 where the links are not unitary to float64)
+        if (F && force) RM_TRY(links_su3(ctx, prec, st, &force));
+        if (act && c1 != 0.0) RM_TRY(links_su3(ctx, RMHMC_FP64, st, &act));
     }
-    const bool staples = !force;
+    const bool staples = F && !force;
     if (staples) RM_TRY(force_staples(ctx, beta, c1, prec, F, st));
     if (!act) return action_loops(ctx, beta, c1, S, plaq, st);
-    if (staples) RM_CHECK(ctx, cudaStreamSynchronize(st));   // the staples run after the transfer
+    if (staples) RM_CHECK(ctx, cudaStreamSynchronize(st));   // they run after the transfer
     const double* out = buf + 8;
     if (S) *S = beta * ((1.0 - 8.0 * c1) * out[0] + (c1 != 0.0 ? c1 * out[2] : 0.0));
     if (plaq) *plaq = out[1] / (6.0 * ctx->g.V);

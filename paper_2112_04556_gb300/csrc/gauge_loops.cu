@@ -9,8 +9,8 @@
 //   F_m = sum_n { c0 (1 - T_n) k_mn + c1 [ (1 + T_m)(1 - T_n) r_mn - r_nm + T_n T_n r_nm ] }(y).
 // Per site that is 6 x 324 + 12 x 108 = 3240 FMA for the plaquette action and about 10,200 with rectangles, where the
 // staples take 5616 and 36,700; the action reads the traces of the same products.  The transport and the rectangles use
-// U U^dag = 1: links that are not unitary to 2^-43 (say, read from single precision) keep the staples, which take any
-// matrices (links_su3; 173 us once per import at 24^3 x 48).
+// U U^dag = 1: links that are not unitary to 2^-43 (say, read from single precision; 2^-20 for the float32 force) keep the
+// staples, which take any matrices (links_su3; once per import, 24^3 x 48: 170 us, float32 45 us).
 //
 // float64 (0.55 TFMA/s) is bound by the operations, float32 was by re-reading the links of every staple from L2.  Measured at
 // 24^3 x 48, float32 Iwasaki force with its float64 action: 9.70 ms with staples, 6.84 ms here; float64 Wilson flow at 16^4,
@@ -317,27 +317,60 @@ __global__ void __launch_bounds__(kBlock) k_su3_check(Links64 U, double* partial
     grid_sum_finish<1>(v, partials, counter, out, gridDim.x, blockIdx.x, sh);
 }
 
-int su3_check_launch(rmhmc_ctx* ctx, cudaStream_t st) {
-    k_su3_check<<<capped_grid(ctx, (size_t)4 * ctx->g.V, kBlock), kBlock, 0, st>>>(
-        links64(ctx), red_slot_partials(ctx, kSlotSu3), red_slot_counter(ctx, kSlotSu3), red_slot_out(ctx, kSlotSu3));
+// the same of the float32 copies, above 2^-20 (the sums here are off by less than 2^-21)
+__global__ void __launch_bounds__(kBlock) k_su3_check32(Links32 U, double* partials, unsigned* counter, double* out) {
+    int bad = 0;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 4 * U.V; i += gridDim.x * blockDim.x) {
+        const int mu = i / U.V, s = i - mu * U.V;
+        const mat3<float> u = LinkLoad<float, 18>::load(U, s, mu);
+        const mat3<float> p = m_mul_nd(u, u);
+        bool ok = true;
+#pragma unroll
+        for (int e = 0; e < 9; e++) {
+            const cplx<float> z = p.e[e / 3][e % 3];
+            ok = ok && fabsf(z.re - (e % 4 == 0 ? 1.f : 0.f)) <= 0x1p-20f && fabsf(z.im) <= 0x1p-20f;
+        }
+        bad += !ok;
+    }
+    __shared__ double sh[kBlock / 32];
+    double v[1] = {(double)bad};
+    block_sum<1>(v, sh);
+    grid_sum_finish<1>(v, partials, counter, out, gridDim.x, blockIdx.x, sh);
+}
+
+int su3_check_launch(rmhmc_ctx* ctx, int prec, cudaStream_t st) {
+    const int grid = capped_grid(ctx, (size_t)4 * ctx->g.V, kBlock);
+    double* part = red_slot_partials(ctx, kSlotSu3);
+    unsigned* cnt = red_slot_counter(ctx, kSlotSu3);
+    double* out = red_slot_out(ctx, kSlotSu3) + prec;
+    if (prec == RMHMC_FP64) k_su3_check<<<grid, kBlock, 0, st>>>(links64(ctx), part, cnt, out);
+    else k_su3_check32<<<grid, kBlock, 0, st>>>(links32(ctx), part, cnt, out);
     ++ctx->launches;
     RM_LAUNCH_CHECK(ctx);
     return RMHMC_OK;
 }
 
-void su3_known(rmhmc_ctx* ctx, bool su3) {
-    ctx->su3 = su3;
-    ctx->su3_gen = ctx->import_gen;
+void su3_known(rmhmc_ctx* ctx, int prec, bool su3) {
+    ctx->su3[prec] = su3;
+    ctx->su3_gen[prec] = ctx->import_gen;
 }
 
-int links_su3(rmhmc_ctx* ctx, cudaStream_t st, bool* su3) {
-    if (su3_unknown(ctx)) {
+int su3_state(const rmhmc_ctx* ctx, int prec) {
+    const bool known64 = ctx->su3_gen[RMHMC_FP64] == ctx->import_gen, known32 = ctx->su3_gen[RMHMC_FP32] == ctx->import_gen;
+    if (prec == RMHMC_FP64) return known64 ? ctx->su3[RMHMC_FP64] : known32 && !ctx->su3[RMHMC_FP32] ? 0 : -1;
+    return known32 ? ctx->su3[RMHMC_FP32] : known64 && ctx->su3[RMHMC_FP64] ? 1 : -1;
+}
+
+int links_su3(rmhmc_ctx* ctx, int prec, cudaStream_t st, bool* su3) {
+    int state = su3_state(ctx, prec);
+    if (state < 0) {
         double bad = 0.0;
-        RM_TRY(su3_check_launch(ctx, st));
-        RM_TRY(fetch(ctx, red_slot_out(ctx, kSlotSu3), &bad, 1, st));
-        su3_known(ctx, bad == 0.0);
+        RM_TRY(su3_check_launch(ctx, prec, st));
+        RM_TRY(fetch(ctx, red_slot_out(ctx, kSlotSu3) + prec, &bad, 1, st));
+        su3_known(ctx, prec, bad == 0.0);
+        state = bad == 0.0;
     }
-    *su3 = ctx->su3;
+    *su3 = state == 1;
     return RMHMC_OK;
 }
 
@@ -347,7 +380,7 @@ int gauge_loops_launch(rmhmc_ctx* ctx, double beta, double c1, int prec, double*
     if (!loops_usable(ctx) || !links_tracked(ctx, st)) return RMHMC_OK;
     if (F || c1 != 0.0) {
         bool su3 = true;
-        if (!defer || !su3_unknown(ctx)) RM_TRY(links_su3(ctx, st, &su3));
+        if (!defer || su3_state(ctx, prec) >= 0) RM_TRY(links_su3(ctx, prec, st, &su3));
         if (!su3) return RMHMC_OK;
     }
     const int s = prec == RMHMC_FP64 ? loops_t<double>(ctx, links64(ctx), beta, c1, F, act, st)

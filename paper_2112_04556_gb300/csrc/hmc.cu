@@ -1080,7 +1080,7 @@ static int md_graph_run(rmhmc_ctx* ctx, double* U, double* P, const rmhmc_params
     bool su3 = false;
     if (loops_usable(ctx) && links_tracked(ctx, stream)) {
         if (!imported) RM_TRY(import_links(ctx, U, stream));
-        RM_TRY(links_su3(ctx, stream, &su3));
+        RM_TRY(links_su3(ctx, md_gauge_prec(p), stream, &su3));
     }
     for (int i = 0; i < 3; i++)
         if (!ctx->cap_st[i]) RM_CHECK(ctx, cudaStreamCreateWithFlags(&ctx->cap_st[i], cudaStreamNonBlocking));
@@ -1166,9 +1166,9 @@ static int md_graph_run(rmhmc_ctx* ctx, double* U, double* P, const rmhmc_params
 }
 
 // T = 1/2 |R(A) P|^2 with every shift at relative residual tol_h (float64 check), S, plaquette
-// (su3: the molecular dynamics follows, whose forces ask whether these links are unitary)
+// (ask: as gauge_force_action, for the forces of the molecular dynamics that follows)
 static int hamiltonian_run(rmhmc_ctx* ctx, const double* U, const double* P, const rmhmc_params* p, const MassTerm& m,
-                           double* H, double* T, double* S, double* plaq, cudaStream_t st, bool su3 = false) {
+                           double* H, double* T, double* S, double* plaq, cudaStream_t st, int ask = -1) {
     int status = RMHMC_OK;
     const size_t fs = field_elems(ctx);
     RM_TRY(import_links(ctx, U, st));
@@ -1177,7 +1177,7 @@ static int hamiltonian_run(rmhmc_ctx* ctx, const double* U, const double* P, con
     RM_TRY(rational_apply(ctx, m, P, p->tol_h, p->maxiter, p->prec, Y, nullptr, st));
     double y2 = 0.0, s = 0.0, pl = 0.0;
     RM_TRY(norm2_64(ctx, Y, fs, &y2, st));
-    RM_TRY(gauge_force_action(ctx, p->beta, p->c1, RMHMC_FP64, nullptr, &s, &pl, st, su3));
+    RM_TRY(gauge_force_action(ctx, p->beta, p->c1, RMHMC_FP64, nullptr, &s, &pl, st, ask));
     const double t = 0.5 * y2;
     if (!isfinite(t) || !isfinite(s)) return set_err(ctx, RMHMC_ENAN, "NaN/Inf in the Hamiltonian");
     if (T) *T = t;
@@ -1301,7 +1301,8 @@ extern "C" int rmhmc_trajectory(rmhmc_ctx* ctx, double* U, const double* xi, con
     // start from the same momenta
     int s = heatbath_apply(ctx, m, X, p->tol_h, p->maxiter, p->prec, P, stream);
     if (s != RMHMC_OK) return restore(s);
-    s = hamiltonian_run(ctx, U, P, p, m, &res.H0, &res.T0, &res.S0, nullptr, stream, true);
+    s = hamiltonian_run(ctx, U, P, p, m, &res.H0, &res.T0, &res.S0, nullptr, stream,
+                        md_gauge_prec(p));
     if (s == RMHMC_OK) s = aux_action(&res.A0);
     if (s != RMHMC_OK) return restore(s);
     bool used = false;

@@ -25,12 +25,13 @@ constexpr int kAdMinFields = 6;
 int gauge_force_launch(rmhmc_ctx* ctx, double beta, double c1, int prec, double* F, cudaStream_t st);
 // action S and average plaquette (float64, deterministic) from the context's float64 links
 int action_launch(rmhmc_ctx* ctx, double beta, double c1, double* S, double* plaq, cudaStream_t st);
-// Whether the links imported last are unitary to 2^-43 (the rounding a long chain of updates leaves; what the library's own
-// updates make of them keeps that property).  Looked at once per import; synchronises the stream then.
-int links_su3(rmhmc_ctx* ctx, cudaStream_t st, bool* su3);
-int su3_check_launch(rmhmc_ctx* ctx, cudaStream_t st);   // the number of other links to the slot kSlotSu3
-void su3_known(rmhmc_ctx* ctx, bool su3);
-inline bool su3_unknown(const rmhmc_ctx* ctx) { return ctx->su3_gen != ctx->import_gen; }
+// Whether the links imported last are unitary: to 2^-43 for float64 (the rounding a long chain of updates leaves), to 2^-20
+// for float32 (any links rounded to float32 are off by up to 2^-21).  What the library's own updates make of them keeps
+// that property.  Looked at once per import and precision; synchronises the stream then.
+int links_su3(rmhmc_ctx* ctx, int prec, cudaStream_t st, bool* su3);
+int su3_check_launch(rmhmc_ctx* ctx, int prec, cudaStream_t st);   // the number of other links to the slot kSlotSu3, at prec
+void su3_known(rmhmc_ctx* ctx, int prec, bool su3);
+int su3_state(const rmhmc_ctx* ctx, int prec);                     // 1, 0, or -1: not looked at yet
 constexpr int kSlotSu3 = 40;
 // Force (F not null) and, in float64, the loop sums of the action (act) from shared loops (gauge_loops.cu), on lattices of up
 // to kLoopsMax sites (scratch: up to 4.5 KB a site in float64); *used tells whether it ran.  The sums go to the slot kSlotLoops:
@@ -44,10 +45,10 @@ inline bool loops_usable(const rmhmc_ctx* ctx) { return ctx->use_loops && !ctx->
 int gauge_loops_launch(rmhmc_ctx* ctx, double beta, double c1, int prec, double* F, bool act, bool defer, bool* used,
                        cudaStream_t st);
 int gauge_loops_prepare(rmhmc_ctx* ctx, double c1, int prec);
-// force (in prec's arithmetic) with float64 action and average plaquette (each pointer nullable) of the context's links; su3:
-// the answer of links_su3 with the same transfer, for a later force
+// force (in prec's arithmetic) with float64 action and average plaquette (each pointer nullable) of the context's links; ask:
+// the answer of links_su3 for that precision with the same transfer, for a later force (-1: none)
 int gauge_force_action(rmhmc_ctx* ctx, double beta, double c1, int prec, double* F, double* S, double* plaq,
-                       cudaStream_t st, bool su3 = false);
+                       cudaStream_t st, int ask = -1);
 // G = sum_f w_f d<Z_f, A X_f>/dw (X, Z in the arithmetic precision, [nf][V][4][8]); G float64 [V][4][8]
 int link_grad_launch(rmhmc_ctx* ctx, int prec, const void* X, const void* Z, int nf, const double* w, double* G,
                      cudaStream_t st);

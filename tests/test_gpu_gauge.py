@@ -145,3 +145,30 @@ def test_where_links_count_as_unitary(shift, loops):
         rm.counters(ctx, reset=True)
         rm.gauge_force(ctx, None, 6.0, -0.331)
         assert rm.counters(ctx)["launches"] == (4 if loops else 2)
+
+
+@pytest.mark.parametrize("shift,loops32,loops64", [(0.0, True, True), (2.0 ** -23, True, False), (2.0 ** -19, False, False)])
+@pytest.mark.parametrize("first", [0, 1])
+def test_where_links_count_as_unitary_in_float32(shift, loops32, loops64, first):
+    """The float32 force of links off by 2 shift shares its loops up to 2^-20, whatever was asked before it: a float64
+    force (first = 0) or nothing.  The Iwasaki force takes four kernels from loops and one from staples; both are within
+    float32 rounding of the oracle's."""
+    import paper_2112_04556_gb300 as rm
+    L = (4, 6, 4, 4)
+    U = inputs.random_links(L, eps=0.6, seed=17) * (1.0 + shift)
+    ref = oracle.gauge_force(L, U, 6.0, -0.331)
+    S_ref, _ = oracle.action(L, U, 6.0, -0.331)
+    with rm.Context(L) as ctx:
+        if first == 0:
+            F64, S64, _ = rm.gauge_force(ctx, dev(U), 6.0, -0.331, prec=rm.FP64)
+            assert rel_l2(host(F64), ref) <= 1e-12
+        else:
+            rm.set_links(ctx, dev(U))
+        F32, S, _ = rm.gauge_force(ctx, None, 6.0, -0.331, prec=rm.FP32)
+        assert rel_l2(host(F32), ref) <= 1e-5 and abs(S - S_ref) <= 1e-12 * abs(S_ref)
+        for prec, loops in ((rm.FP32, loops32), (rm.FP64, loops64)):
+            F = dev(np.zeros((int(np.prod(L)), 4, 8)))
+            rm.counters(ctx, reset=True)
+            ctx.check(rm.lib().gauge_force(ctx.h, None, 6.0, -0.331, prec, F.data_ptr(), None, None, rm._raw_stream()))
+            assert rm.counters(ctx)["launches"] == (4 if loops else 1), prec
+            assert rel_l2(host(F), ref) <= (1e-12 if prec == rm.FP64 else 1e-5)
