@@ -414,6 +414,7 @@ void* workspace(rmhmc_ctx* ctx, const char* name, size_t bytes, int* status);
 void without(rmhmc_ctx* ctx, bool* off);
 int import_links(rmhmc_ctx* ctx, const double* U, cudaStream_t st);
 int ensure_links(rmhmc_ctx* ctx, const double* U, cudaStream_t st);
+void links_imported(rmhmc_ctx* ctx);
 inline size_t field_elems(const rmhmc_ctx* ctx) { return (size_t)ctx->g.V * 32; }
 inline int site_blocks(const rmhmc_ctx* ctx) { return (ctx->g.V + kBlock - 1) / kBlock; }
 // blocks of the stencil kernels: four lanes per site (one per field component mu)
@@ -445,6 +446,11 @@ inline bool links_tracked(const rmhmc_ctx* ctx, cudaStream_t st) { return !ctx->
 // (more than kAdTableMax sites, no memory for it, links that change behind the host's back)
 constexpr int kAdTableMax = 1 << 22;   // 2 KB a site
 int links64_adjoint(rmhmc_ctx* ctx, Links64* U, cudaStream_t st);
+// ensure_links for a call that goes on to use the table (table): on up to kImportTableMax sites new links and their table come
+// from one launch (float64 lap_apply with links, two launches -> one: 4^4 37.0 -> 30.9 us, 8^4 46.2 -> 41.1, 12^4 153 -> 148;
+// by 3x3 products 39.0, 40.3 and 162 us)
+constexpr int kImportTableMax = 1 << 15;
+int ensure_links_table(rmhmc_ctx* ctx, const double* U, bool table, cudaStream_t st);
 inline Links32 links32(const rmhmc_ctx* ctx) { return Links32{ctx->u32a, ctx->u32b, ctx->g.V}; }
 double* red_slot_partials(rmhmc_ctx* ctx, int slot);
 unsigned* red_slot_counter(rmhmc_ctx* ctx, int slot);

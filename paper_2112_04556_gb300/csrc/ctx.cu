@@ -128,10 +128,14 @@ int import_links(rmhmc_ctx* ctx, const double* U, cudaStream_t st) {
     if (caller_captures(ctx, st)) ctx->links_in_graph = true;
     k_import_links<<<site_blocks(ctx), kBlock, 0, st>>>(U, ctx->u64, ctx->u32a, ctx->u32b, ctx->g.V); ++ctx->launches;
     RM_LAUNCH_CHECK(ctx);
+    links_imported(ctx);
+    return RMHMC_OK;
+}
+
+void links_imported(rmhmc_ctx* ctx) {
     ctx->links_valid = true;
     ctx->link_gen++;
     if (!ctx->own_capture) ctx->import_gen++;
-    return RMHMC_OK;
 }
 
 int ensure_links(rmhmc_ctx* ctx, const double* U, cudaStream_t st) {

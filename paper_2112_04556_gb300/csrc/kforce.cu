@@ -690,7 +690,7 @@ extern "C" int lap_link_grad(rmhmc_ctx* ctx, const double* U, const double* X, c
     if (!X || !Z || !G || (nfield > 0 && !w)) return set_err(ctx, RMHMC_EINVAL, "lap_link_grad: null argument");
     if (nfield < 0 || nfield > kMaxPairs) return set_err(ctx, RMHMC_EINVAL, "lap_link_grad: nfield in [0, %d]", kMaxPairs);
     if (prec != RMHMC_FP64 && prec != RMHMC_FP32) return set_err(ctx, RMHMC_EINVAL, "lap_link_grad: bad prec");
-    RM_TRY(ensure_links(ctx, U, stream));
+    RM_TRY(ensure_links_table(ctx, U, prec == RMHMC_FP64 && nfield > 0, stream));
     const size_t fs = field_elems(ctx);
     if (nfield == 0) {
         RM_CHECK(ctx, cudaMemsetAsync(G, 0, sizeof(double) * fs, stream));

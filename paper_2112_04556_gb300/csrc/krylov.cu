@@ -38,7 +38,7 @@ template <> struct Vec<double> {
 
 // r_0 = b rounded to T and re-laid from [V][4][8] to the planes, rho_0 = |r_0|^2; thread: four colours of a component.
 // The sum of a float32 run and the rounding use no float64 arithmetic, which took longer than the bytes (32^4: a
-// conversion pass of 75 us and this one of 139 us, together 60 us of traffic)
+// conversion pass of 75 us and this one of 139 us, together 60 us of traffic; now 88 us)
 template <typename T, typename TI>
 __device__ __forceinline__ double start_pass(const TI* __restrict__ b, T* __restrict__ r0, int V) {
     const size_t n4 = (size_t)V * 8;

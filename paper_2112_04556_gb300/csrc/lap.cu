@@ -222,7 +222,8 @@ extern "C" int lap_apply(rmhmc_ctx* ctx, const double* U, const void* X, void* Y
     const size_t bytes = field_elems(ctx) * (prec == RMHMC_FP64 ? 8 : 4) * (size_t)nfield;
     const char *xb = (const char*)X, *yb = (const char*)Y;
     if (xb < yb + bytes && yb < xb + bytes) return set_err(ctx, RMHMC_EINVAL, "lap_apply: X and Y overlap");
-    RM_TRY(ensure_links(ctx, U, stream));
+    const bool table = prec == RMHMC_FP64 && linkfmt == 18 && nfield > 0 && !ctx->pinned.count(818);
+    RM_TRY(ensure_links_table(ctx, U, table, stream));
     if (nfield == 0) return RMHMC_OK;
     const double a = op == RMHMC_OP_A ? 0.5 : -8.0;
     const double b = op == RMHMC_OP_A ? -1.0 / 16.0 : 1.0;

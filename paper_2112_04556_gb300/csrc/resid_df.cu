@@ -43,15 +43,11 @@ __global__ void __launch_bounds__(kBlock) k_adjoint_table(Links64 U, int V, floa
 // two of the eight columns (blockIdx.z).  A warp has half a float64 lane, so that a thread with all columns took 14 us on the
 // smallest lattice, where lap_apply with new links was then slower than by 3x3 products (39 us at 4^4): the table's part
 // there 14.5 -> 7 us, at 10^4 37 -> 29 us, at 32^4 2.46 -> 2.26 ms
-__global__ void __launch_bounds__(kBlock) k_adjoint_table64(Links64 U, double2* __restrict__ out) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    const int nu = blockIdx.y;
-    if (s >= U.V) return;
-    const mat3<double> u = LinkLoad<double, 18>::load(U, s, nu);
-    double2* const o = out + (size_t)nu * 32 * U.V + s;
+// columns of part blockIdx.z of a link's matrix to its planes o (stride V)
+__device__ __forceinline__ void table64_part(const mat3<double>& u, double2* o, int V) {
     auto put = [&](int b, const double (&col)[8]) {
 #pragma unroll
-        for (int h = 0; h < 4; h++) o[(size_t)(4 * b + h) * U.V] = make_double2(col[2 * h], col[2 * h + 1]);
+        for (int h = 0; h < 4; h++) o[(size_t)(4 * b + h) * V] = make_double2(col[2 * h], col[2 * h + 1]);
     };
     if (blockIdx.z == 0) adjoint_pair_columns<double, 0>(u, put);
     else if (blockIdx.z == 1) adjoint_pair_columns<double, 1>(u, put);
@@ -59,18 +55,65 @@ __global__ void __launch_bounds__(kBlock) k_adjoint_table64(Links64 U, double2* 
     else adjoint_diagonal_columns(u, put);
 }
 
-int links64_adjoint(rmhmc_ctx* ctx, Links64* U, cudaStream_t st) {
+__global__ void __launch_bounds__(kBlock) k_adjoint_table64(Links64 U, double2* __restrict__ out) {
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    const int nu = blockIdx.y;
+    if (s >= U.V) return;
+    const mat3<double> u = LinkLoad<double, 18>::load(U, s, nu);
+    table64_part(u, out + (size_t)nu * 32 * U.V + s, U.V);
+}
+
+// The import of the caller's links (k_import_links) and the table in one launch, for small lattices, where each of the two
+// is latency: the copies are shared out among the parts.
+__global__ void __launch_bounds__(kBlock) k_import_table64(const double2* __restrict__ in, double2* __restrict__ u64,
+                                                           float4* __restrict__ u32a, float2* __restrict__ u32b, int V,
+                                                           double2* __restrict__ out) {
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    const int nu = blockIdx.y;
+    if (s >= V) return;
+    mat3<double> u;
+#pragma unroll
+    for (int e = 0; e < 9; e++) {
+        const double2 v = __ldg(in + ((size_t)s * 4 + nu) * 9 + e);
+        u.e[e / 3][e % 3] = cmk(v.x, v.y);
+    }
+    auto f2 = [&](int e) { return make_float2((float)u.e[e / 3][e % 3].re, (float)u.e[e / 3][e % 3].im); };
+    if (blockIdx.z == 0) {
+#pragma unroll
+        for (int e = 0; e < 9; e++) u64[(size_t)(nu * 9 + e) * V + s] = make_double2(u.e[e / 3][e % 3].re, u.e[e / 3][e % 3].im);
+    } else if (blockIdx.z == 1) {
+#pragma unroll
+        for (int r = 0; r < 3; r++) {
+            const float2 a = f2(2 * r), b = f2(2 * r + 1);
+            u32a[(size_t)(nu * 3 + r) * V + s] = make_float4(a.x, a.y, b.x, b.y);
+        }
+    } else if (blockIdx.z == 2) {
+#pragma unroll
+        for (int j = 0; j < 3; j++) u32b[(size_t)(nu * 3 + j) * V + s] = f2(6 + j);
+    }
+    table64_part(u, out + (size_t)nu * 32 * V + s, V);
+}
+
+// the table's buffer; null where a table is not used
+static int table64(rmhmc_ctx* ctx, double2** t, cudaStream_t st) {
+    *t = nullptr;
     if (ctx->g.V > kAdTableMax || ctx->adj64_off || !ctx->use_table || !links_tracked(ctx, st)) return RMHMC_OK;
     int status = RMHMC_OK;
-    const unsigned long long ws = ctx->ws_gen;
-    double2* t = (double2*)workspace(ctx, "ad_table64", sizeof(double2) * (size_t)ctx->g.V * 128, &status);
+    *t = (double2*)workspace(ctx, "ad_table64", sizeof(double2) * (size_t)ctx->g.V * 128, &status);
     if (status == RMHMC_ENOMEM) {
         // no room: the 3x3 form serves as before
         ctx->err.clear();
         without(ctx, &ctx->adj64_off);
         return RMHMC_OK;
     }
-    if (!t) return status;
+    return status;
+}
+
+int links64_adjoint(rmhmc_ctx* ctx, Links64* U, cudaStream_t st) {
+    const unsigned long long ws = ctx->ws_gen;
+    double2* t;
+    RM_TRY(table64(ctx, &t, st));
+    if (!t) return RMHMC_OK;
     if (ctx->adj64_gen != ctx->link_gen || ws != ctx->ws_gen) {
         k_adjoint_table64<<<dim3(site_blocks(ctx), 4, 4), kBlock, 0, st>>>(links64(ctx), t);
         ++ctx->launches;
@@ -78,6 +121,19 @@ int links64_adjoint(rmhmc_ctx* ctx, Links64* U, cudaStream_t st) {
         ctx->adj64_gen = ctx->link_gen;
     }
     U->ad = t;
+    return RMHMC_OK;
+}
+
+int ensure_links_table(rmhmc_ctx* ctx, const double* U, bool table, cudaStream_t st) {
+    double2* t = nullptr;
+    if (U && table && ctx->g.V <= kImportTableMax && (uintptr_t)U % 16 == 0) RM_TRY(table64(ctx, &t, st));
+    if (!t) return ensure_links(ctx, U, st);
+    k_import_table64<<<dim3(site_blocks(ctx), 4, 4), kBlock, 0, st>>>((const double2*)U, ctx->u64, ctx->u32a, ctx->u32b,
+                                                                      ctx->g.V, t);
+    ++ctx->launches;
+    RM_LAUNCH_CHECK(ctx);
+    links_imported(ctx);
+    ctx->adj64_gen = ctx->link_gen;
     return RMHMC_OK;
 }
 

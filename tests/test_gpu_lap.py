@@ -231,3 +231,31 @@ def test_lap_fp64_adjoint_table_matches_3x3_form(L, nf):
             ref = host(rm.lap_apply(b, dev(U), dev(X)))
             assert rel_l2(y, ref) <= 1e-14
             assert rel_l2(y[0], oracle.lap(L, U, X[0])) <= 1e-12
+
+
+@pytest.mark.parametrize("L", [(2, 2, 2, 2), (5, 3, 4, 7), (33, 2, 3, 2), (16, 16, 8, 16), (17, 16, 8, 16)])
+def test_links_and_table_in_one_launch(L):
+    """A float64 call that brings its links (one launch for their copies and the table on up to 2^15 sites, two above)
+    leaves the same links and table behind as set_links and a call without links: the float64 stencil and link
+    derivative, the float32 stencil in both link formats and the gauge force agree bit for bit."""
+    import paper_2112_04556_gb300 as rm
+    X, Z = (dev(f) for f in inputs.gaussian_fields(L, 2, seed=62))
+    Us = [dev(inputs.random_links(L, eps=0.5, seed=60 + i)) for i in range(2)]
+    X32 = X.float()
+
+    def rest(ctx):
+        out = [rm.lap_apply(ctx, None, X), rm.lap_link_grad(ctx, None, X, Z, [0.7]), rm.lap_apply(ctx, None, X32),
+               rm.lap_apply(ctx, None, X32, linkfmt=12), rm.gauge_force(ctx, None, 6.0, 0.0)[0]]
+        return [host(t) for t in out]
+    with rm.Context(L) as a, rm.Context(L) as b:
+        for ctx in (a, b):
+            rm.set_stencil_shape(ctx, rm.SHAPE_LAP, rm.FP32, 18, 1, 128)
+            rm.set_stencil_shape(ctx, rm.SHAPE_LAP, rm.FP32, 12, 1, 128)
+        for U in Us + Us[:1]:
+            rm.set_links(a, U)
+            want = rest(a)
+            y = host(rm.lap_apply(b, U, X))
+            assert np.array_equal(y, want[0])
+            for g, w in zip(rest(b), want):
+                assert np.array_equal(g, w)
+            assert np.array_equal(host(rm.lap_link_grad(b, U, X, Z, [0.7])), want[1])
